@@ -97,7 +97,7 @@ extern "C" {
                                    through NP_E_DEVICE instead of touching memory */
 #define NP_F_DIRECT_LOADS    2  /* sparse MLP: plain 16-byte global loads instead of the
                                    shared-memory staged kernel (for comparison runs) */
-#define NP_F_NO_TENSOR_CORES 8  /* np_predict with B > 4: ALU kernel instead of the tcgen05 GEMM
+#define NP_F_NO_TENSOR_CORES 8  /* np_predict with B > 1: ALU kernels instead of the tcgen05 GEMMs
                                    (for comparison runs) */
 #define NP_F_LAYER_LAUNCHES  4  /* np_step / np_mlp_chain: one kernel launch per layer instead
                                    of resident kernels spanning runs of layers */
@@ -258,7 +258,7 @@ const char* np_last_error(const np_ctx* ctx);
 /* Stage 1 + 2: predictor forward and per-layer top-k (Section 3.1 step 2; the
  * workload's predictor is logits = W2 * relu(W1 * x), no biases).
  *   x_bf16       dev bf16 [B][D]   layer-0 hidden states
- *   logits_out   dev fp32 [B][L][M] or NULL (kept internally either way)
+ *   logits_out   dev fp32 [B][L][M] or NULL (then kept internally)
  *   bitmap_out   dev uint32 [L][W] or NULL: union over the B sequences of each
  *                sequence's k highest logits per layer; order = fp32 value
  *                descending (+0 above -0), ties to the lower neuron index
@@ -439,7 +439,7 @@ int np_last_step_times(np_ctx* ctx, float* out_us);
  *   w1 dev bf16 [d_pred][d_model], w2 dev bf16 [n_layers*d_ffn][d_pred], x_bf16 dev bf16 [B][d_model]
  *   logits_out dev fp32 [B][n_layers][d_ffn]   (all caller-owned, 16-byte aligned)
  * Bit-identical to np_predict's logits in a context created with NP_F_NO_TENSOR_CORES (the same
- * plain-core kernels); a default context takes the tensor-core kernel for B > 4, whose rounding
+ * plain-core kernels); a default context takes the tensor-core kernels for B > 1, whose rounding
  * differs (both are within rel-L2 1e-5 of the exact product).  Calls no cudaMalloc / cudaFree or
  * allocating library routine.  Every call first clears the status words in the scratch; a kernel
  * whose bounded wait runs out records a bit there, leaves part of logits_out unwritten and the

@@ -279,12 +279,10 @@ int check_config(const np_config* c, np_ctx* ctx) {
   if (c->record_format == NP_REC_INT8 && c->d_model % 16)
     return fail(ctx, NP_E_INVAL, "8-bit records need d_model % 16 == 0");
   {
-    // batches the tensor-core predictor does not take (B <= 4, no tensor cores, or a width
-    // outside its K blocks) run the ring kernel, whose shared memory holds the batch's hidden
-    // vectors beside at least two stages of W2 rows
-    Dims pd = {};
-    pd.H = c->d_pred;
-    const bool tc = c->max_batch > 4 && !(c->flags & NP_F_NO_TENSOR_CORES) && pred_tc_supported(pd);
+    // batches the tensor-core predictor does not take (no tensor cores, or a width whose hidden terms do not fit
+    // beside its stages; np_init knows) run the ring kernel, whose shared memory holds the batch's hidden vectors
+    // beside at least two stages of W2 rows
+    const bool tc = c->max_batch > 4 && !(c->flags & NP_F_NO_TENSOR_CORES) && c->d_pred % 64 == 0;
     const int b_ring = tc ? 4 : c->max_batch;
     if (b_ring >= 2 && !pred_l2_ring_fits(c->d_pred, b_ring))
       return fail(ctx, NP_E_INVAL, "max_batch=%d with d_pred=%d: the hidden vectors of %d sequences do not fit the "
@@ -520,7 +518,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   const size_t o_spid = take(LC), o_spsl = take(LC), o_spcnt = take((size_t)d.L * NP_N_COUNTERS), o_spcand = take(LW);
   const size_t o_sfix = take(2 * chain_slices::zfix_words(d)), o_sbar = take(chain_slices::bar_words()), o_sxch = take(2 * chain_slices::xch_words(d, ctx->sm_count));
   const size_t o_rz = take(chain_rows::z_floats(d)), o_rcnt = take(4);
-  const size_t o_l1p = take(cfg->max_batch > 4 ? (size_t)kPredL1Parts * 16 * d.H : 1);
+  const size_t o_l1p = take(cfg->max_batch >= kPredTcMinBatch ? (size_t)kPredL1Parts * 16 * d.H : 1);
   const size_t o_xt = take(cfg->max_batch >= kTcMinBatch ? mlp_tc_xterms_bytes(d) / 4 : 1);
   NP_INIT_CUDA(cudaMalloc(&ctx->slab, off));
   char* base = static_cast<char*>(ctx->slab);
@@ -618,12 +616,12 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   // tensor-core predictor for batches: tensor maps over W2 and the split hidden terms
   ctx->mlp_tc = cfg->max_batch >= kTcMinBatch && !(cfg->flags & (NP_F_NO_TENSOR_CORES | NP_F_DIRECT_LOADS)) &&
                 mlp_tc_supported(d, ctx->sm_count);
-  if (cfg->max_batch > 4 && !(cfg->flags & NP_F_NO_TENSOR_CORES))
+  if (cfg->max_batch >= kPredTcMinBatch && !(cfg->flags & NP_F_NO_TENSOR_CORES))
     pred_tc_prepare(d, b->w1, b->w2, ctx->ws.hsplit, reinterpret_cast<float*>(static_cast<char*>(ctx->slab) + o_l1p), ctx->sm_count, &ctx->tc);
   {
     // batches the tensor-core predictor does not take go through the ring kernel, whose shared
     // memory holds the batch's hidden vectors beside at least two stages of W2 rows
-    const int b_ring = ctx->tc.ready ? std::min(cfg->max_batch, 4) : cfg->max_batch;
+    const int b_ring = ctx->tc.ready ? 1 : cfg->max_batch;
     if (b_ring >= 2 && !pred_l2_ring_fits(d.H, b_ring)) {
       np_destroy(ctx);
       return fail(nullptr, NP_E_INVAL,
@@ -713,7 +711,7 @@ int np_predict(np_ctx* ctx, const void* x_bf16, int32_t B, float* logits_out, ui
   const Dims& d = ctx->d;
   // batches: both layers on the tensor cores where the shapes allow (layer 1 leaves partial sums that layer 2's
   // split kernel adds up)
-  const bool l1_tc = B > 4 && ctx->tc.ready && ctx->tc.l1_ready && d.dense == 0;
+  const bool l1_tc = B >= kPredTcMinBatch && ctx->tc.ready && ctx->tc.l1_ready;
   if (l1_tc)
     NP_LAUNCH(ctx, launch_pred_l1_tc(d, ctx->tc, x_bf16, B, ctx->t.status, s));
   else
@@ -726,23 +724,27 @@ int np_predict(np_ctx* ctx, const void* x_bf16, int32_t B, float* logits_out, ui
   const int skip_layers = B == 1 ? d.dense : 0;
   ds.L = d.L - skip_layers;
   const size_t skip_rows = (size_t)skip_layers * d.M;
-  float* logits = ctx->ws.logits + skip_rows;
+  // scores and sets go where the caller wants them; the context's own bitmap is written beside the caller's
+  float* logits = (logits_out ? logits_out : ctx->ws.logits) + skip_rows;
+  uint32_t* pred = ctx->t.pred + (size_t)skip_layers * d.W;
+  uint32_t* pred2 = bitmap_out ? bitmap_out + (size_t)skip_layers * d.W : nullptr;
   if (ds.L > 0) {
-    if (B > 4 && ctx->tc.ready) {
+    const bool l2_tc = B >= kPredTcMinBatch && ctx->tc.ready;
+    if (l2_tc) {
       ctx->launches += 1;  // split kernel + GEMM kernel
-      NP_LAUNCH(ctx, launch_pred_l2_tc(d, ctx->tc, ctx->ws.hidden, B, ctx->ws.logits, ctx->t.status, s, ctx->sm_count,
-                                       l1_tc ? ctx->tc.l1_parts : 0));
+      NP_LAUNCH(ctx, launch_pred_l2_tc(d, ctx->tc, ctx->ws.hidden, B, logits, ctx->t.status, s, ctx->sm_count,
+                                       l1_tc ? ctx->tc.l1_parts : 0, pred, pred2));
     } else {
       NP_LAUNCH(ctx, launch_pred_l2(ds, static_cast<const char*>(ctx->bufs.w2) + skip_rows * d.H * 2, ctx->ws.hidden,
                                   B, logits, ctx->t.status, s, ctx->sm_count));
     }
-    NP_LAUNCH(ctx, launch_topk(ds, logits, B, ctx->t.pred + (size_t)skip_layers * d.W, s));
+    NP_LAUNCH(ctx, launch_topk(ds, logits, B, pred, pred2, l2_tc, s));
   }
-  if (d.dense > 0) NP_CUDA(ctx, cudaMemsetAsync(ctx->t.pred, 0, (size_t)d.dense * d.W * 4, s));
-  const size_t nlog = (size_t)B * ds.L * d.M * 4, nbm = (size_t)d.L * d.W * 4;
-  if (logits_out && nlog)
-    NP_CUDA(ctx, cudaMemcpyAsync(logits_out + skip_rows, logits, nlog, cudaMemcpyDeviceToDevice, s));
-  if (bitmap_out) NP_CUDA(ctx, cudaMemcpyAsync(bitmap_out, ctx->t.pred, nbm, cudaMemcpyDeviceToDevice, s));
+  if (d.dense > 0) {
+    const size_t nbm = (size_t)d.dense * d.W * 4;
+    NP_CUDA(ctx, cudaMemsetAsync(ctx->t.pred, 0, nbm, s));
+    if (bitmap_out) NP_CUDA(ctx, cudaMemsetAsync(bitmap_out, 0, nbm, s));
+  }
   ctx->have_pred = true;
   return NP_OK;
 }
@@ -757,7 +759,7 @@ int np_topk(np_ctx* ctx, const float* logits, int32_t B, uint32_t* bitmap_out, v
   ds.L = d.L - skip_layers;
   if (ds.L > 0)
     NP_LAUNCH(ctx, launch_topk(ds, logits + (size_t)skip_layers * d.M, B, bitmap_out + (size_t)skip_layers * d.W,
-                               as_stream(stream)));
+                               nullptr, false, as_stream(stream)));
   if (d.dense > 0) NP_CUDA(ctx, cudaMemsetAsync(bitmap_out, 0, (size_t)d.dense * d.W * 4, as_stream(stream)));
   return NP_OK;
 }
@@ -1516,7 +1518,7 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
     ds.k = std::min(d.M, d.k + ctx->cfg.spec_rows);
     if (ds.L > 0)
       NP_LAUNCH(ctx, launch_topk(ds, ctx->ws.logits + (size_t)skip_layers * d.M, B,
-                                 ctx->t.spec_cand + (size_t)skip_layers * d.W, s));
+                                 ctx->t.spec_cand + (size_t)skip_layers * d.W, nullptr, false, s));
     if (d.dense > 0) NP_CUDA(ctx, cudaMemsetAsync(ctx->t.spec_cand, 0, (size_t)d.dense * d.W * 4, s));
     rc = np_speculate(ctx, ctx->t.spec_cand, ctx->cfg.spec_rows, stream);
     if (rc < 0) return rc;

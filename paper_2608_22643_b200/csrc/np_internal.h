@@ -75,6 +75,10 @@ cudaError_t launch_pred_l2(const Dims& d, const void* w2, const float* hidden, i
 // whether the ring form of layer 2 (batches without the tensor-core kernel) has room for B hidden vectors of H values
 bool pred_l2_ring_fits(int H, int B);
 // Tensor-core form of predictor layer 2 for batches (np_predict_tc.cu).
+// Batches from two sequences on run it: the plain-core kernels read the hidden vectors from shared memory once per
+// weight and sequence, and that, not the weights, is what bounds them (np_predict for three sequences of the 13B-shaped
+// stack, 708 MB of weights: 330 us on them, 131 us on the tensor cores).
+constexpr int kPredTcMinBatch = 2;
 constexpr int kPredL1Parts = 16;  // K ranges (partial sums) of the tensor-core layer 1, at most
 struct PredTcState {
   alignas(64) unsigned char map_w2[128];  // CUtensorMap of W2 [L*M][H]
@@ -90,10 +94,14 @@ struct PredTcState {
 bool pred_tc_supported(const Dims& d);
 bool pred_tc_prepare(const Dims& d, const void* w1, const void* w2, void* hsplit, float* l1_part, int sm_count, PredTcState* st);
 cudaError_t launch_pred_l1_tc(const Dims& d, const PredTcState& st, const void* x_bf16, int B, int32_t* status, cudaStream_t s);
+// clear / clear2 (may be NULL): bitmaps of L * W words that the split kernel zeroes for the selection behind it
 cudaError_t launch_pred_l2_tc(const Dims& d, const PredTcState& st, float* hidden, int B, float* logits,
-                              int32_t* status, cudaStream_t s, int sm_count, int l1_parts);
+                              int32_t* status, cudaStream_t s, int sm_count, int l1_parts, uint32_t* clear, uint32_t* clear2);
 
-cudaError_t launch_topk(const Dims& d, const float* logits, int B, uint32_t* bitmap, cudaStream_t s);
+// bitmap2 (may be NULL) receives the same words; `cleared`: an earlier kernel of the stream has zeroed both (a batch's
+// selections are ORed into them)
+cudaError_t launch_topk(const Dims& d, const float* logits, int B, uint32_t* bitmap, uint32_t* bitmap2, bool cleared,
+                        cudaStream_t s);
 
 // Centroid heads -> arg-max -> bank lookup -> gate AND up (np_centroid.cu).
 cudaError_t launch_centroid_select(const Dims& d, const float* logits, int B, int K, const uint32_t* bank,

@@ -1,13 +1,15 @@
-// Stage 1b for batched sequences (B > 4): the predictor's second layer as a real dense
+// Stage 1b for batched sequences (B >= 2): the predictor's second layer as a real dense
 // contraction on the 5th-generation tensor cores.
 //
 //   logits[b][r] = sum_m W2[r][m] * hidden[b][m]        r over all L*M rows, b < B <= 16
 //
 // (One predictor pass scores every FFN neuron of every downstream layer, Section 3.1 step 2;
-// the batch is the workload's batch-16 case.)  With 16 sequences the ALU kernel needs
-// 16 FMAs per weight element and becomes instruction-bound; here a 128-row tile of W2 is
-// the M side of a tcgen05.mma (bf16 x bf16 -> fp32 in tensor memory) and the sequences are
-// the N side.  The kernel is still bound by the single pass over W2:
+// the batch is the workload's batch-16 case.)  The ALU kernels read every hidden value once per
+// weight from shared memory and need an FMA per weight and sequence: three sequences of the
+// 13B-shaped stack (708 MB of weights) took 330 us that way, 131 us here (5.5 TB/s), and
+// sixteen are worse.  Here a 128-row tile of W2 is the M side of a tcgen05.mma
+// (bf16 x bf16 -> fp32 in tensor memory) and the sequences are the N side.  The kernel is
+// still bound by the single pass over W2:
 //
 //   * W2 tiles [128 rows x 64 k] come in by tiled TMA (128-byte swizzle, the layout the MMA
 //     shared-memory descriptor expects) through a ring of 16 KB stages, one producer lane.
@@ -47,6 +49,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst_smem, const CUtensorMap* m
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
           "r"(npp::smem_addr(dst_smem)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(npp::smem_addr(bar))
+      : "memory");
+}
+
+// the same for data that is read once: evict-first in the L2
+__device__ __forceinline__ void tma_load_2d_stream(void* dst_smem, const CUtensorMap* map, int x, int y, uint64_t* bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::
+          "r"(npp::smem_addr(dst_smem)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(npp::smem_addr(bar)), "l"(policy)
       : "memory");
 }
 
@@ -90,11 +101,17 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 // hidden fp32 [B][H] -> three bf16 terms, rows [term * 16 + b] of a [48][H] array (zero for b >= B).
 // n_part > 0: `hidden` holds n_part partial sums [n_part][16][H] of layer 1 (one per K range of the tensor-core
 // kernel below); they are added in a fixed order, the ReLU is applied, and the result is also stored to `sum_out`.
+// The words of `clear` and `clear2` (may be NULL) are zeroed on the way: the selection behind layer 2 ORs into them, and a
+// memset in front of it would keep its blocks from starting early.
 __global__ void k_split_hidden(const float* __restrict__ hidden, __nv_bfloat16* __restrict__ out, int H, int B, int n_part,
-                               float* __restrict__ sum_out) {
+                               float* __restrict__ sum_out, uint32_t* __restrict__ clear, uint32_t* __restrict__ clear2, int n_clear) {
   npp::pdl_launch_dependents();
   npp::pdl_wait_prior();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int w = i; w < n_clear; w += gridDim.x * blockDim.x) {
+    clear[w] = 0u;
+    if (clear2) clear2[w] = 0u;
+  }
   if (i >= 16 * H) return;
   const int b = i / H, m = i - b * H;
   float v = 0.f;
@@ -126,7 +143,7 @@ k_pred_l2_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant__
   __shared__ uint32_t s_tmem_base;
 
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int n_kb = H / kTcKBlock;
+  const int n_kb = (H + kTcKBlock - 1) / kTcKBlock;  // a last block past H reads zeros on both sides
   // shared memory: [ring of W2 stages][hidden terms: n_kb blocks of 48 rows x 128 B]
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tsm) + 1023) & ~(uintptr_t)1023);
   unsigned char* ring = base;
@@ -166,6 +183,7 @@ k_pred_l2_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant__
     if (lane == 0) {
       // W2 does not depend on the previous kernels: start streaming at once; the hidden
       // terms are written by the kernel just before this one
+      const uint64_t pol = npp::policy_evict_first();
       int it = 0;
       bool ok = true;
       const int prefill = min(n_stages, my_tiles * n_kb);
@@ -173,9 +191,10 @@ k_pred_l2_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant__
         const int kb = it % n_kb;
         const long long tile = t_begin + it / n_kb;
         npp::mbar_expect_tx(&full_bar[it], kTcStageBytes);
-        tma_load_2d(ring + (size_t)it * kTcStageBytes, &map_w2, kb * kTcKBlock, (int)(tile * kTcTileRows), &full_bar[it]);
+        tma_load_2d_stream(ring + (size_t)it * kTcStageBytes, &map_w2, kb * kTcKBlock, (int)(tile * kTcTileRows), &full_bar[it], pol);
       }
       npp::pdl_wait_prior();
+      npp::pdl_launch_dependents();  // the selection's blocks take the SMs as this grid's blocks leave them
       npp::mbar_expect_tx(&h_bar, (uint32_t)n_kb * h_block_bytes);
       for (int kb = 0; kb < n_kb; ++kb) tma_load_2d(hsm + (size_t)kb * h_block_bytes, &map_h, kb * kTcKBlock, 0, &h_bar);
       const int total = my_tiles * n_kb;
@@ -190,7 +209,7 @@ k_pred_l2_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant__
         const int kb = it % n_kb;
         const long long tile = t_begin + it / n_kb;
         npp::mbar_expect_tx(&full_bar[s], kTcStageBytes);
-        tma_load_2d(ring + (size_t)s * kTcStageBytes, &map_w2, kb * kTcKBlock, (int)(tile * kTcTileRows), &full_bar[s]);
+        tma_load_2d_stream(ring + (size_t)s * kTcStageBytes, &map_w2, kb * kTcKBlock, (int)(tile * kTcTileRows), &full_bar[s], pol);
       }
     }
   } else if (wid == 1) {
@@ -395,19 +414,22 @@ bool make_map(CUtensorMap* map, const void* gptr, uint64_t inner, uint64_t outer
 
 }  // namespace
 
-bool pred_tc_supported(const Dims& d) { return d.H % kTcKBlock == 0 && d.H >= kTcKBlock; }
+// Any width the configuration takes (a multiple of 8: rows start on 16-byte boundaries): the tensor maps fill what
+// lies past a row's end with zeros, so the last K block may be ragged.  What can still be missing is shared memory
+// for the hidden terms beside two stages (pred_tc_prepare).
+bool pred_tc_supported(const Dims& d) { return d.H % 8 == 0; }
 
 bool pred_tc_prepare(const Dims& d, const void* w1, const void* w2, void* hsplit, float* l1_part, int sm_count, PredTcState* st) {
   static_assert(sizeof(CUtensorMap) <= sizeof(st->map_w2), "tensor map blob too small");
   st->ready = 0;
   st->l1_ready = 0;
   if (!pred_tc_supported(d)) return false;
-  // layer 1 on the tensor cores: whole row tiles of W1 and whole K blocks, and room for the partial sums
-  if (l1_part && d.H % kTcTileRows == 0 && d.D % kTcKBlock == 0) {
+  // layer 1 on the tensor cores, ragged row tiles and K blocks included: it needs room for the partial sums
+  if (l1_part) {
     CUtensorMap w;
     if (make_map(&w, w1, (uint64_t)d.D, (uint64_t)d.H, kTcKBlock, kTcTileRows)) {
       memcpy(st->map_w1, &w, sizeof w);
-      const int n_kb = d.D / kTcKBlock, n_mt = d.H / kTcTileRows;
+      const int n_kb = (d.D + kTcKBlock - 1) / kTcKBlock, n_mt = (d.H + kTcTileRows - 1) / kTcTileRows;
       // K ranges: enough blocks to fill the machine, at most kPredL1Parts partial sums, at most kL1MaxKb K blocks each
       int parts = std::min(std::min(n_kb, kPredL1Parts), std::max(1, sm_count / n_mt));
       int per = (n_kb + parts - 1) / parts;
@@ -425,7 +447,7 @@ bool pred_tc_prepare(const Dims& d, const void* w1, const void* w2, void* hsplit
   if (!make_map(&b, hsplit, (uint64_t)d.H, kTcN, kTcKBlock, kTcN)) return false;
   memcpy(st->map_w2, &a, sizeof a);
   memcpy(st->map_h, &b, sizeof b);
-  const size_t h_bytes = (size_t)(d.H / kTcKBlock) * kTcN * kTcKBlock * 2;
+  const size_t h_bytes = (size_t)((d.H + kTcKBlock - 1) / kTcKBlock) * kTcN * kTcKBlock * 2;
   const size_t budget = 220 * 1024 - 1024;  // alignment slack
   if (h_bytes + 2 * kTcStageBytes > budget) return false;
   st->n_stages = (int)std::min<size_t>(kTcMaxStages, (budget - h_bytes) / kTcStageBytes);
@@ -444,23 +466,32 @@ cudaError_t launch_pred_l1_tc(const Dims& d, const PredTcState& st, const void* 
   const size_t smem = (size_t)st.l1_kb_per_block * kL1StageBytes + 1024;
   cudaError_t e = cudaFuncSetAttribute(k_pred_l1_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_pred_l1_tc<<<dim3(d.H / kTcTileRows, st.l1_parts), kTcThreads, smem, s>>>(w, x, st.l1_part, d.H, d.D / kTcKBlock, st.l1_kb_per_block,
-                                                                              status);
+  k_pred_l1_tc<<<dim3((d.H + kTcTileRows - 1) / kTcTileRows, st.l1_parts), kTcThreads, smem, s>>>(
+      w, x, st.l1_part, d.H, (d.D + kTcKBlock - 1) / kTcKBlock, st.l1_kb_per_block, status);
   return cudaGetLastError();
 }
 
 // l1_parts > 0: layer 1 ran on the tensor cores and left that many partial sums; the split kernel adds them up,
 // applies the ReLU and stores the hidden vectors to `hidden` as the other layer-1 kernels do.
 cudaError_t launch_pred_l2_tc(const Dims& d, const PredTcState& st, float* hidden, int B, float* logits,
-                              int32_t* status, cudaStream_t s, int sm_count, int l1_parts) {
+                              int32_t* status, cudaStream_t s, int sm_count, int l1_parts, uint32_t* clear, uint32_t* clear2) {
   if (!st.ready) return cudaErrorInvalidValue;
   CUtensorMap a, b;
   memcpy(&a, st.map_w2, sizeof a);
   memcpy(&b, st.map_h, sizeof b);
   const int n = 16 * d.H;
-  k_split_hidden<<<(n + 255) / 256, 256, 0, s>>>(l1_parts > 0 ? st.l1_part : hidden, static_cast<__nv_bfloat16*>(st.hsplit), d.H, B,
-                                                 l1_parts, hidden);
-  cudaError_t e = cudaGetLastError();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t scfg = {};
+  scfg.gridDim = dim3((n + 255) / 256);
+  scfg.blockDim = dim3(256);
+  scfg.stream = s;
+  scfg.attrs = attr;
+  scfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&scfg, k_split_hidden, static_cast<const float*>(l1_parts > 0 ? st.l1_part : hidden),
+                                     static_cast<__nv_bfloat16*>(st.hsplit), d.H, B, l1_parts, hidden, clear, clear2,
+                                     clear ? d.L * d.W : 0);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_pred_l2_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st.smem);
   if (e != cudaSuccess) return e;
@@ -471,9 +502,6 @@ cudaError_t launch_pred_l2_tc(const Dims& d, const PredTcState& st, float* hidde
   cfg.blockDim = dim3(kTcThreads);
   cfg.dynamicSmemBytes = st.smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_pred_l2_tc, a, b, logits, rows, d.H, B, st.n_stages, status);

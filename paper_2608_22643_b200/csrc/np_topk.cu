@@ -46,6 +46,7 @@ __device__ __forceinline__ uint32_t order_key(uint32_t b) { return (b & 0x800000
 template <int KPT>
 __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__ logits,  // [B][L][M]
                                                        uint32_t* __restrict__ bitmap,     // [L][W]
+                                                       uint32_t* __restrict__ bitmap2,    // a second copy, or NULL
                                                        int L, int M, int k, int use_atomic) {
   extern __shared__ __align__(16) int wsm[];  // [W] per word: selected keys of the deciding bin / count of threshold-equal keys
   __shared__ __align__(16) int hist[kTopkHist];
@@ -59,6 +60,19 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const float* z = logits + ((size_t)b * L + layer) * M;
   uint32_t* out = bitmap + (size_t)layer * W;
+  uint32_t* out2 = bitmap2 ? bitmap2 + (size_t)layer * W : nullptr;
+  // a word of the result: stored (one sequence), or ORed into what the other sequences left (a batch)
+  auto put = [&](int w, uint32_t word) {
+    if (use_atomic) {
+      if (word) {
+        atomicOr(out + w, word);
+        if (out2) atomicOr(out2 + w, word);
+      }
+    } else {
+      out[w] = word;
+      if (out2) out2[w] = word;
+    }
+  };
 
   TK(0);
   npp::pdl_launch_dependents();
@@ -66,15 +80,11 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   TK(1);
 
   if (k <= 0) {  // nothing selected
-    if (!use_atomic)
-      for (int w = tid; w < W; w += kTopkThreads) out[w] = 0u;
+    for (int w = tid; w < W; w += kTopkThreads) put(w, 0u);
     return;
   }
   if (k >= M) {
-    for (int w = tid; w < W; w += kTopkThreads) {
-      if (use_atomic) atomicOr(out + w, 0xffffffffu);
-      else out[w] = 0xffffffffu;
-    }
+    for (int w = tid; w < W; w += kTopkThreads) put(w, 0xffffffffu);
     return;
   }
 
@@ -156,13 +166,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
         const int w = wid + 32 * j;  // the word of neurons 32 w .. 32 w + 31: this warp's logits of round j
         const int bn = i < M ? bin_of(__uint_as_float(zb[j])) : -1;
         const uint32_t gt = __ballot_sync(0xffffffffu, bn > bstar);
-        if (lane == 0 && w < W) {
-          if (use_atomic) {
-            if (gt) atomicOr(out + w, gt);
-          } else {
-            out[w] = gt;
-          }
-        }
+        if (lane == 0 && w < W) put(w, gt);
         if (bn == bstar) {
           const int q = atomicAdd(&s_ncand, 1);
           ckey[q] = order_key(zb[j]);
@@ -179,7 +183,10 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
           const uint32_t qk = ckey[q];
           rank += (qk > mk || (qk == mk && cidx[q] < mi)) ? 1 : 0;
         }
-        if (rank < need) atomicOr(out + (mi >> 5), 1u << (mi & 31));
+        if (rank < need) {
+          atomicOr(out + (mi >> 5), 1u << (mi & 31));
+          if (out2) atomicOr(out2 + (mi >> 5), 1u << (mi & 31));
+        }
       }
       TK(16);
       return;
@@ -275,18 +282,13 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
     const uint32_t gt = __ballot_sync(0xffffffffu, valid && key > thr);
     const uint32_t eq = __ballot_sync(0xffffffffu, valid && key == thr);
     if (lane == 0 && w < W) {
-      const uint32_t word = gt | (surplus ? lowest_bits(eq, admit - wsm[w]) : eq);
-      if (use_atomic) {
-        if (word) atomicOr(out + w, word);
-      } else {
-        out[w] = word;
-      }
+      put(w, gt | (surplus ? lowest_bits(eq, admit - wsm[w]) : eq));
     }
   }
 }
 
 template <int KPT>
-static cudaError_t topk_launch(const Dims& d, const float* logits, int B, uint32_t* bitmap, int use_atomic, cudaStream_t s) {
+static cudaError_t topk_launch(const Dims& d, const float* logits, int B, uint32_t* bitmap, uint32_t* bitmap2, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(d.L, B);
   cfg.blockDim = dim3(kTopkThreads);
@@ -297,20 +299,22 @@ static cudaError_t topk_launch(const Dims& d, const float* logits, int B, uint32
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_topk<KPT>, logits, bitmap, d.L, d.M, d.k, use_atomic);
+  return cudaLaunchKernelEx(&cfg, k_topk<KPT>, logits, bitmap, bitmap2, d.L, d.M, d.k, B > 1 ? 1 : 0);
 }
 
-cudaError_t launch_topk(const Dims& d, const float* logits, int B, uint32_t* bitmap, cudaStream_t s) {
-  const int use_atomic = B > 1 ? 1 : 0;
-  if (use_atomic) {
-    cudaError_t e = cudaMemsetAsync(bitmap, 0, (size_t)d.L * d.W * 4, s);
+cudaError_t launch_topk(const Dims& d, const float* logits, int B, uint32_t* bitmap, uint32_t* bitmap2, bool cleared,
+                        cudaStream_t s) {
+  if (B > 1 && !cleared) {
+    const size_t bytes = (size_t)d.L * d.W * 4;
+    cudaError_t e = cudaMemsetAsync(bitmap, 0, bytes, s);
+    if (e == cudaSuccess && bitmap2) e = cudaMemsetAsync(bitmap2, 0, bytes, s);
     if (e != cudaSuccess) return e;
   }
   const int kpt = (d.M + kTopkThreads - 1) / kTopkThreads;
-  if (kpt <= 12) return topk_launch<12>(d, logits, B, bitmap, use_atomic, s);
-  if (kpt <= 16) return topk_launch<16>(d, logits, B, bitmap, use_atomic, s);
-  if (kpt <= 28) return topk_launch<28>(d, logits, B, bitmap, use_atomic, s);
-  if (kpt <= 40) return topk_launch<40>(d, logits, B, bitmap, use_atomic, s);
+  if (kpt <= 12) return topk_launch<12>(d, logits, B, bitmap, bitmap2, s);
+  if (kpt <= 16) return topk_launch<16>(d, logits, B, bitmap, bitmap2, s);
+  if (kpt <= 28) return topk_launch<28>(d, logits, B, bitmap, bitmap2, s);
+  if (kpt <= 40) return topk_launch<40>(d, logits, B, bitmap, bitmap2, s);
   return cudaErrorInvalidValue;  // d_ffn > 40960 is rejected by np_init
 }
 

@@ -1,0 +1,53 @@
+"""np_predict for batches on the tensor cores: ragged widths of both layers, and the caller's outputs."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import np_oracle as O
+from paper_2608_22643_b200 import binding as nb
+from paper_2608_22643_b200 import synth
+from tests.harness import Pair, rel_l2, u16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D,H", [(8, 8), (72, 64), (1000, 136), (2064, 200), (8192, 128), (8200, 64)])
+@pytest.mark.parametrize("B", [2, 5, 16])
+def test_ragged_widths_match_the_oracle(D, H, B):
+    """K blocks of 64 and row tiles of 128 that end past the matrix, one and many K ranges, a width (8200) whose
+    layer 1 is outside the tensor-core kernel; 160 rows of layer 2 = a full tile and a quarter."""
+    L, M = 5, 32
+    p = Pair(synth.StackConfig("pb", L, D, M, H, 25, 50, 2, 43, 0.9), max_batch=B, with_oracle=False)
+    try:
+        x = synth.hidden_states(p.cfg, 1, batch=B)[0]
+        logits = torch.full((B, L, M), 7.0, dtype=torch.float32, device="cuda")
+        nb.np_predict(p.eng.ctx, x.cuda(), B, logits, None, p.eng.stream)
+        p.eng.counters()
+        z = O.predict(u16(p.w1_cpu), u16(p.w2_cpu), u16(x), L, M)
+        assert rel_l2(logits.cpu().numpy(), z) < 1e-5    # fp32 accumulation of at most 8200 products: below 1e-6
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("B", [1, 2, 16])
+@pytest.mark.parametrize("k", [0, 7, 96])
+def test_bitmap_handed_out_is_the_one_kept(B, k):
+    """The selection writes the caller's words and the context's own, each call anew."""
+    L, M = 3, 96
+    p = Pair(synth.StackConfig("po", L, 64, M, 72, 25, 50, 4, 44, 0.5), max_batch=B, k=k, C=M, with_oracle=False)
+    try:
+        xs = synth.hidden_states(p.cfg, 3, batch=B)
+        logits = torch.empty((B, L, M), dtype=torch.float32, device="cuda")
+        words = torch.full((L, M // 32), -1, dtype=torch.int32, device="cuda")
+        for t in range(3):
+            nb.np_predict(p.eng.ctx, xs[t].cuda(), B, logits, words, p.eng.stream)
+            nb.np_delta(p.eng.ctx, None, p.eng.stream)
+            c = p.eng.counters()
+            want = O.topk_bitmap(logits.cpu().numpy(), k)
+            got = words.cpu().numpy().view(np.uint32)
+            assert (got == want).all(), t
+            for l in range(L):
+                active = p.eng.delta_lists(l, c[l])["active_ids"]
+                assert (active == np.flatnonzero(O.bitmap_to_bool(got[l], M))).all(), (t, l)
+    finally:
+        p.close()
