@@ -417,7 +417,9 @@ int np_chain_launches(np_ctx* ctx, int32_t* out);
 
 /* Name of the kernel np_mlp_chain / np_step run the sparse layers' MLP with for B sequences in this
  * context (a static string: "k_mlp_slices", "k_mlp_chain_alu", "k_mlp_tc_up + k_mlp_tc_down",
- * "k_sparse_mlp_pipe" or "k_sparse_mlp").  For reports; NULL if ctx is NULL or B is out of range. */
+ * "k_sparse_mlp_pipe" or "k_sparse_mlp").  "k_mlp_tc_up + k_mlp_tc_down" names the tensor-core form for batches: its
+ * two phases run as one resident kernel ("k_mlp_batch", the name for widths that only it covers) where that applies, as
+ * two kernels per layer elsewhere.  For reports; NULL if ctx is NULL or B is out of range. */
 const char* np_mlp_kernel_name(np_ctx* ctx, int32_t B);
 
 /* Timing of the last np_step in microseconds, host float [4]: predict+top-k,

@@ -205,6 +205,8 @@ struct np_ctx {
   chain_rows::State rows = {};  // cluster form of the resident MLP kernel (whole rows per block): its accumulators and counters
   bool use_rows = false;
   int chain_kernel_launches = 0;    // MLP kernel launches of the last np_mlp_chain / np_step
+  chain_batch::State batch = {};    // resident MLP kernel for batches
+  bool use_batch = false;           // np_mlp_chain / np_step run it for B >= 2
   size_t gu_bytes = 0;   // both dot-product accumulators of the batch MLP, contiguous
   bool mlp_tc = false;   // batches run the tensor-core MLP kernels
   std::string err;
@@ -330,6 +332,15 @@ size_t host_area_ints(const np_config& c) {
 size_t host_lists_ints(const np_config& c) { return 2 * host_area_ints(c); }
 
 cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
+
+// the batch kernel's counters and stamps, as np_init leaves them
+cudaError_t reset_batch_state(np_ctx* ctx, cudaStream_t s) {
+  if (!ctx->batch.cnt) return cudaSuccess;
+  ctx->batch.read_base = ctx->batch.add_base = ctx->batch.seq_base = 0;
+  cudaError_t e = cudaMemsetAsync(ctx->batch.cnt, 0, chain_batch::cnt_words() * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->batch.xch, 0, chain_batch::xch_words(ctx->sm_count) * 8, s);
+  return e;
+}
 
 int check_device_status(np_ctx* ctx, cudaStream_t s) {
   int32_t st[4];
@@ -518,6 +529,8 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   const size_t o_spid = take(LC), o_spsl = take(LC), o_spcnt = take((size_t)d.L * NP_N_COUNTERS), o_spcand = take(LW);
   const size_t o_sfix = take(2 * chain_slices::zfix_words(d)), o_sbar = take(chain_slices::bar_words()), o_sxch = take(2 * chain_slices::xch_words(d, ctx->sm_count));
   const size_t o_rz = take(chain_rows::z_floats(d)), o_rcnt = take(4);
+  const bool batches = cfg->max_batch >= kTcMinBatch;
+  const size_t o_bcnt = take(batches ? chain_batch::cnt_words() : 1), o_bxch = take(batches ? 2 * chain_batch::xch_words(ctx->sm_count) : 1);
   const size_t o_l1p = take(cfg->max_batch >= kPredTcMinBatch ? (size_t)kPredL1Parts * 16 * d.H : 1);
   const size_t o_xt = take(cfg->max_batch >= kTcMinBatch ? mlp_tc_xterms_bytes(d) / 4 : 1);
   NP_INIT_CUDA(cudaMalloc(&ctx->slab, off));
@@ -559,6 +572,11 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   ctx->rows.cnt_base = ctx->rows.seq = 0;
   NP_INIT_CUDA(cudaMemset(ctx->rows.z4, 0, chain_rows::z_floats(d) * 4));
   NP_INIT_CUDA(cudaMemset(ctx->rows.cnt, 0, 4 * 4));
+  if (batches) {
+    ctx->batch.cnt = reinterpret_cast<unsigned int*>(base + o_bcnt);
+    ctx->batch.xch = reinterpret_cast<unsigned long long*>(base + o_bxch);
+    NP_INIT_CUDA(reset_batch_state(ctx, nullptr));
+  }
   ctx->use_rows = (cfg->flags & NP_F_CLUSTER_ROWS) && !(cfg->flags & NP_F_ROW_CHAIN) && d.dense < d.L && chain_rows::prepare(d, ctx->sm_count, &ctx->rows);
 
   const WsLayout wl = ws_layout(*cfg);
@@ -616,6 +634,8 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   // tensor-core predictor for batches: tensor maps over W2 and the split hidden terms
   ctx->mlp_tc = cfg->max_batch >= kTcMinBatch && !(cfg->flags & (NP_F_NO_TENSOR_CORES | NP_F_DIRECT_LOADS)) &&
                 mlp_tc_supported(d, ctx->sm_count);
+  ctx->use_batch = cfg->max_batch >= kTcMinBatch && chain_batch::supported(d, ctx->sm_count) &&
+                   !(cfg->flags & (NP_F_NO_TENSOR_CORES | NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES | NP_F_TCGEN05_BATCH));
   if (cfg->max_batch >= kPredTcMinBatch && !(cfg->flags & NP_F_NO_TENSOR_CORES))
     pred_tc_prepare(d, b->w1, b->w2, ctx->ws.hsplit, reinterpret_cast<float*>(static_cast<char*>(ctx->slab) + o_l1p), ctx->sm_count, &ctx->tc);
   {
@@ -695,6 +715,7 @@ int np_reset(np_ctx* ctx, void* stream) {
   NP_CUDA(ctx, cudaMemsetAsync(ctx->rows.z4, 0, chain_rows::z_floats(ctx->d) * 4, as_stream(stream)));
   NP_CUDA(ctx, cudaMemsetAsync(ctx->rows.cnt, 0, 4 * 4, as_stream(stream)));
   ctx->rows.cnt_base = ctx->rows.seq = 0;
+  NP_CUDA(ctx, reset_batch_state(ctx, as_stream(stream)));
   ctx->have_delta = ctx->have_pred = ctx->have_step = ctx->have_spec = false;
   std::fill(ctx->install_pending.begin(), ctx->install_pending.end(), 0);
   ctx->step = 0;
@@ -1215,13 +1236,113 @@ static int mlp_layer(np_ctx* ctx, int layer, const float* xa, const float* xb, f
   return NP_OK;
 }
 
+enum { kChainAll = 0, kChainHead = 1, kChainTail = 2 };
+
+// Runs of the sparse layers in which a resident kernel takes them.  A run starts once its layers are installed, so what
+// the step waits for after its last row has landed is the last run: with chain_layers = 0 the runs shrink towards the end
+// (the tail is an eighth of the stack, the run before it a quarter, the first run takes the rest), which also makes fewer
+// launches than equal runs of a quarter each.
+static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
+  const Dims& d = ctx->d;
+  // layers whose rows have all landed already need no run of their own to wait in: they go into one
+  // first run (the whole stack when nothing is pending, as in np_mlp_chain on resident rows)
+  int landed = d.dense;
+  while (landed < d.L) {
+    if (ctx->install_pending[landed]) {
+      const cudaError_t q = cudaEventQuery(ctx->ev_installed[landed]);
+      if (q == cudaErrorNotReady) {
+        (void)cudaGetLastError();
+        break;
+      }
+      if (q != cudaSuccess) return fail(ctx, NP_E_CUDA, "cudaEventQuery failed: %s", cudaGetErrorString(q));
+      ctx->install_pending[landed] = 0;
+    }
+    ++landed;
+  }
+  const int ns = d.L - landed;  // layers that still wait for rows
+  if (ctx->cfg.chain_layers > 0) {
+    const int run = ctx->cfg.chain_layers;
+    for (int l0 = d.dense; l0 < d.L; l0 += run) runs->push_back(std::min(run, d.L - l0));
+    return NP_OK;
+  }
+  if (landed > d.dense) runs->push_back(landed - d.dense);
+  if (ns > 0) {
+    const int unit = std::max(1, (d.L - d.dense) / 8);
+    const int tail = std::min(ns, unit), mid = std::min(ns - tail, 2 * unit), first = ns - tail - mid;
+    if (first > 0) runs->push_back(first);
+    if (mid > 0) runs->push_back(mid);
+    runs->push_back(tail);
+  }
+  return NP_OK;
+}
+
+static int batch_run(np_ctx* ctx, const ChainArgs& a, float* x, int B, cudaStream_t s) {
+  int n = 0;
+  NP_CUDA(ctx, chain_batch::launch(ctx->d, a, x, B, &ctx->batch, s, ctx->sm_count, &n));
+  ctx->launches += n;
+  return NP_OK;
+}
+
+// The chain for a batch in the resident kernel: runs of layers as for one sequence, x in the kernel's own tiles
+// (the accumulators' space, which no other kernel of this chain uses).
+static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part) {
+  const Dims& d = ctx->d;
+  const size_t row_bytes = (size_t)d.D * 2;
+  float* x = ctx->ws.zbuf[0];
+  ChainArgs a = {};
+  a.status = ctx->t.status;
+  a.check = ctx->cfg.flags & NP_F_CHECK_BOUNDS;
+  a.counters = ctx->t.counters;
+  if (part != kChainTail) {
+    ctx->chain_kernel_launches = 0;
+    NP_LAUNCH(ctx, chain_batch::launch_in(d, x_bf16, x, B, s));
+    if (d.dense > 0) {
+      // runs, so that the sparse layers' installs advance between them (as for one sequence)
+      const char* dense = static_cast<const char*>(ctx->bufs.dense_buf);
+      a.gate = dense;
+      a.up = dense + row_bytes;
+      a.downT = dense + 2 * row_bytes;
+      a.active_slots = ctx->t.identity;
+      a.dense_rows = d.M;
+      const int dense_run = d.dense < d.L ? std::max(3, std::min(12, 2 * d.dense / (d.L - d.dense))) : d.dense;
+      for (int l0 = 0; l0 < d.dense; l0 += dense_run) {
+        a.l_begin = l0;
+        a.l_end = std::min(d.dense, l0 + dense_run);
+        const int rc = batch_run(ctx, a, x, B, s);
+        if (rc < 0) return rc;
+      }
+    }
+  }
+  if (part == kChainHead) return NP_OK;
+  const size_t shift = (size_t)d.dense * d.C * row_bytes;  // the sparse layers' buffers start at layer d
+  a.gate = static_cast<const char*>(ctx->bufs.gate_buf) - shift;
+  a.up = static_cast<const char*>(ctx->bufs.up_buf) - shift;
+  a.downT = static_cast<const char*>(ctx->bufs.downT_buf) - shift;
+  a.active_slots = ctx->t.active_slots;
+  a.dense_rows = 0;
+  std::vector<int> runs;
+  int rc = sparse_runs(ctx, &runs);
+  if (rc < 0) return rc;
+  int l0 = d.dense;
+  for (const int n : runs) {
+    for (int l = l0; l < l0 + n; ++l)
+      if (ctx->install_pending[l]) NP_CUDA(ctx, wait_install(ctx, l, s));
+    a.l_begin = l0;
+    a.l_end = l0 += n;
+    rc = batch_run(ctx, a, x, B, s);
+    if (rc < 0) return rc;
+  }
+  NP_LAUNCH(ctx, chain_batch::launch_out(d, x, x_out, B, s));
+  return NP_OK;
+}
+
 // residual chain: x_l = xbuf[(l+1)&1] + zbuf[(l-1)%3]; layer l accumulates MLP_l(x_l) into
 // zbuf[l%3], stores x_l to xbuf[l&1] and clears zbuf[(l+1)%3] for the next layer
 // `part`: kChainAll = the whole chain; kChainHead = its start up to the end of the dense prefix
 // (nothing there waits for an install, so np_step queues it before the host packs any rows);
 // kChainTail = the sparse layers and the result.
-enum { kChainAll = 0, kChainHead = 1, kChainTail = 2 };
 static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part = kChainAll) {
+  if (B >= kTcMinBatch && ctx->use_batch) return batch_chain(ctx, x_bf16, B, x_out, s, part);
   const Dims& d = ctx->d;
   const size_t n = (size_t)B * d.D;
   const bool persistent = B == 1 && !(ctx->cfg.flags & (NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES)) &&
@@ -1242,7 +1363,6 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
   if (persistent) {
     // runs of layers in one resident kernel each; a run starts once its layers are installed,
     // so the install of later runs still overlaps the compute of earlier ones
-    const int run = std::max(1, ctx->cfg.chain_layers > 0 ? ctx->cfg.chain_layers : (d.L + 3) / 4);
     const size_t row_bytes = (size_t)d.D * 2;
     ChainArgs a;
     for (int i = 0; i < 2; ++i) a.xbuf[i] = ctx->ws.xbuf[i];
@@ -1286,40 +1406,10 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
     a.downT = static_cast<const char*>(ctx->bufs.downT_buf) - shift;
     a.active_slots = ctx->t.active_slots;
     a.dense_rows = 0;
-    // Runs of the sparse layers.  A run starts once its layers are installed, so what the step waits for
-    // after its last row has landed is the last run: with chain_layers = 0 the runs shrink towards the end
-    // (the tail is an eighth of the stack, the run before it a quarter, the first run takes the rest), which
-    // also makes fewer launches than equal runs of a quarter each.
     std::vector<int> runs;
     if (part != kChainHead) {
-      // layers whose rows have all landed already need no run of their own to wait in: they go into one
-      // first run (the whole stack when nothing is pending, as in np_mlp_chain on resident rows)
-      int landed = d.dense;
-      while (landed < d.L) {
-        if (ctx->install_pending[landed]) {
-          const cudaError_t q = cudaEventQuery(ctx->ev_installed[landed]);
-          if (q == cudaErrorNotReady) {
-            (void)cudaGetLastError();
-            break;
-          }
-          if (q != cudaSuccess) return fail(ctx, NP_E_CUDA, "cudaEventQuery failed: %s", cudaGetErrorString(q));
-          ctx->install_pending[landed] = 0;
-        }
-        ++landed;
-      }
-      const int ns = d.L - landed;  // layers that still wait for rows
-      if (ctx->cfg.chain_layers > 0) {
-        for (int l0 = d.dense; l0 < d.L; l0 += run) runs.push_back(std::min(run, d.L - l0));
-      } else {
-        if (landed > d.dense) runs.push_back(landed - d.dense);
-        if (ns > 0) {
-          const int unit = std::max(1, (d.L - d.dense) / 8);
-          const int tail = std::min(ns, unit), mid = std::min(ns - tail, 2 * unit), first = ns - tail - mid;
-          if (first > 0) runs.push_back(first);
-          if (mid > 0) runs.push_back(mid);
-          runs.push_back(tail);
-        }
-      }
+      const int rc = sparse_runs(ctx, &runs);
+      if (rc < 0) return rc;
     }
     int l0 = d.dense;
     for (size_t ri = 0; ri < runs.size() && part != kChainHead; ++ri) {
@@ -1461,6 +1551,7 @@ const char* np_mlp_kernel_name(np_ctx* ctx, int32_t B) {
   }
   if (ctx->mlp_tc && B >= kTcMinBatch && !(flags & NP_F_DIRECT_LOADS))
     return ((flags & NP_F_TCGEN05_BATCH) && mlp_tc_up_on_tcgen05(d, ctx->sm_count)) ? "k_mlp_up5 + k_mlp_tc_down" : "k_mlp_tc_up + k_mlp_tc_down";
+  if (ctx->use_batch && B >= kTcMinBatch) return "k_mlp_batch";  // widths the pair does not cover
   return (flags & NP_F_DIRECT_LOADS) ? "k_sparse_mlp" : "k_sparse_mlp_pipe";
 }
 

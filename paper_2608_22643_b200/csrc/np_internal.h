@@ -209,6 +209,22 @@ size_t bar_words();
 cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s, int sm_count);
 }  // namespace chain_slices
 
+namespace chain_batch {  // resident form for two to sixteen sequences (np_mlp_batch.cu)
+// Library-owned device words and the host's running record of them; they only ever grow.
+struct State {
+  unsigned int* cnt;        // [cnt_words()] zero at init / reset
+  unsigned long long* xch;  // [xch_words(sm_count)] zero at init / reset
+  unsigned int read_base, add_base, seq_base;
+};
+bool supported(const Dims& d, int sm_count);
+size_t cnt_words();
+size_t xch_words(int sm_count);
+// x [D / 8][8 or 16 sequences][8] fp32: from the stack's bf16 input, updated by the layers, to the stack's fp32 result
+cudaError_t launch_in(const Dims& d, const void* x_bf16, float* x, int B, cudaStream_t s);
+cudaError_t launch(const Dims& d, const ChainArgs& a, float* x, int B, State* st, cudaStream_t s, int sm_count, int* launches);
+cudaError_t launch_out(const Dims& d, const float* x, float* out, int B, cudaStream_t s);
+}  // namespace chain_batch
+
 namespace chain_rows {  // whole rows per block, blocks in clusters (np_mlp_rows.cu); same hand-over of x
 // Library-owned device words and the host's running record of them: the counters only ever grow
 // and the accumulators are used in rotation, so nothing has to be cleared between launches.
