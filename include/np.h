@@ -57,21 +57,23 @@ extern "C" {
                                sums between layers in fixed point, resolution 2^-30); state is suspect */
 #define NP_E_IO        -6   /* a read of the store file failed or came up short */
 #define NP_W_OVERFLOW   1   /* some layer's predicted set did not fit capacity */
-#define NP_W_CHUNKED    2   /* some layer's delta exceeded staging and was split */
+#define NP_W_CHUNKED    2   /* some layer's delta is larger than the staging (rows that are staged were split) */
 
 /* eviction policies (np_config.evict_policy) */
 #define NP_EVICT_EXACT  0   /* Eq. 3: every row leaving the predicted set frees its slot */
 #define NP_EVICT_LRU    1   /* keep rows while capacity allows; evict least recently predicted,
                                ties by lower neuron index (not in the paper) */
 
-/* how np_install moves records (np_config.transfer_mode) */
-#define NP_XFER_MEMCPY_RUNS  0  /* one cudaMemcpyAsync per run of adjacent neuron IDs into
-                                   device staging, then the scatter kernel */
-#define NP_XFER_HOST_GATHER  1  /* host threads pack records into pinned staging, one
-                                   cudaMemcpyAsync per chunk, then the scatter kernel; the
-                                   staging buffers are used in up to four parts, round robin */
-#define NP_XFER_ZERO_COPY    2  /* the scatter kernel reads the pinned store directly by
-                                   neuron ID (the paper's mapped-staging idea); no host sync */
+/* how np_install moves records (np_config.transfer_mode).  The three modes with a pinned store differ in what the host
+   does; short runs of rows are pulled by a kernel that reads the store by neuron ID and places the rows (the paper's
+   mapped-staging idea without the staging: 51 GB/s on scattered records, on two SMs, no host core busy) in all of them. */
+#define NP_XFER_MEMCPY_RUNS  0  /* one cudaMemcpyAsync per run of adjacent neuron IDs into device staging, then the
+                                   scatter kernel, where the runs are long enough to pay a copy call (3.4 MB on
+                                   average); pulled otherwise */
+#define NP_XFER_HOST_GATHER  1  /* pulled, and the host waits for the counts to report warnings.  With
+                                   NP_F_MAPPED_STAGING host threads pack records into pinned staging, used in up to
+                                   four parts, round robin */
+#define NP_XFER_ZERO_COPY    2  /* pulled; no host synchronisation, so no warnings */
 #define NP_XFER_FILE         3  /* the store is a file (Section 3.5): the incoming IDs of a chunk,
                                    already ascending, are coalesced into ranges of adjacent
                                    records and read through io_uring (np_config.io_depth reads
@@ -113,11 +115,12 @@ extern "C" {
                                    sparse layers whose row width is a multiple of 256, other shapes keep the default.
                                    Results agree with the default to rounding order; measured slower at sixteen
                                    sequences, so off by default */
-#define NP_F_MAPPED_STAGING 16  /* NP_XFER_HOST_GATHER / NP_XFER_FILE: no staging copy; the scatter kernel
-                                   reads the records in the pinned staging buffer through its device
-                                   mapping (Section 3.5: the staging is page-aligned host memory registered
-                                   as mapped, so kernels reach it with no copy call in between).  host_staging
-                                   must be device-mapped pinned memory; np_buffers.staging is not used */
+#define NP_F_MAPPED_STAGING 16  /* NP_XFER_HOST_GATHER: host threads pack the records into host_staging and the scatter
+                                   kernel reads them there through its device mapping, instead of pulling them from the
+                                   store; NP_XFER_FILE: no staging copy, the scatter kernel reads the records the same
+                                   way (Section 3.5: the staging is page-aligned host memory registered as mapped, so
+                                   kernels reach it with no copy call in between).  host_staging must be device-mapped
+                                   pinned memory; np_buffers.staging is not used */
 
 /* per-layer counters written by np_delta (np_read_counters) */
 #define NP_CNT_PRED      0  /* |P|                      */
@@ -314,13 +317,13 @@ int np_read_records(int32_t fd, uint64_t base_offset, uint64_t rec_bytes, const 
  * (L, n) = bytes [(l*M + n)*REC, +REC) of the store to slot S[n] of the three
  * row buffers, on `copy_stream`, and mark each layer installed (np_sparse_mlp
  * orders itself after that mark).  The copy stream is first ordered after the
- * delta step.  Scatter kernels may run on streams the library owns; those are
+ * delta step.  Scatter kernels may run on a stream the library owns; those are
  * ordered after the work `copy_stream` held on entry and joined back into it
  * before the call returns, so work queued on `copy_stream` afterwards sees
  * every row installed.  With NP_XFER_MEMCPY_RUNS / NP_XFER_HOST_GATHER / NP_XFER_FILE this
  * call blocks the host until the delta lists of the last np_delta are readable (and, with
  * NP_XFER_FILE, until the last chunk's reads have completed); with NP_XFER_ZERO_COPY it
- * never blocks.  Deltas larger than staging_rows are split
+ * never blocks.  Staged rows beyond staging_rows are split
  * into chunks in list order (result unchanged).
  * Returns NP_W_OVERFLOW / NP_W_CHUNKED (OVERFLOW wins) where it can know.
  * Errors: NP_E_STATE (no np_delta since init/reset), NP_E_INVAL, NP_E_CUDA, NP_E_IO (a file

@@ -180,6 +180,7 @@ struct np_ctx {
   cudaEvent_t ev_delta = nullptr;
   cudaEvent_t ev_spec = nullptr;      // the lists of the last np_speculate are written
   std::vector<cudaEvent_t> ev_installed;
+  std::vector<cudaEvent_t> mark;      // the event behind a layer's rows: ev_installed of the last layer of its launch
   std::vector<char> install_pending;
   cudaEvent_t ev_half[kStageParts] = {};        // parts of the host / device staging in flight
   // library-owned side streams of the install path: [0] runs the scatter kernels behind the
@@ -348,6 +349,38 @@ int check_device_status(np_ctx* ctx, cudaStream_t s) {
   NP_CUDA(ctx, cudaStreamSynchronize(s));
   if (st[0]) return fail(ctx, NP_E_DEVICE, "kernel bounds check tripped (status bits 0x%x)", st[0]);
   return NP_OK;
+}
+
+// marks layers [l0, l1) installed by what `s` holds now
+cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
+  for (int l = l0; l < l1; ++l) {
+    ctx->mark[l] = ctx->ev_installed[l1 - 1];
+    ctx->install_pending[l] = 1;
+  }
+  return cudaEventRecord(ctx->ev_installed[l1 - 1], s);
+}
+
+// Orders `s` after the install marks of layers [l0, l1); marks that have already completed need no wait, and layers of
+// one launch share theirs.
+cudaError_t wait_installs(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
+  cudaEvent_t seen = nullptr;
+  bool landed = false;
+  for (int l = l0; l < l1; ++l) {
+    if (!ctx->install_pending[l]) continue;
+    if (ctx->mark[l] != seen) {
+      seen = ctx->mark[l];
+      const cudaError_t q = cudaEventQuery(seen);
+      if (q != cudaSuccess && q != cudaErrorNotReady) return q;
+      landed = q == cudaSuccess;
+      if (!landed) {
+        (void)cudaGetLastError();
+        const cudaError_t e = cudaStreamWaitEvent(s, seen, 0);
+        if (e != cudaSuccess) return e;
+      }
+    }
+    if (landed) ctx->install_pending[l] = 0;  // later calls need not ask again
+  }
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -596,6 +629,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_delta, cudaEventDisableTiming));
   NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_spec, cudaEventDisableTiming));
   ctx->ev_installed.assign(d.L, nullptr);
+  ctx->mark.assign(d.L, nullptr);
   ctx->install_pending.assign(d.L, 0);
   for (int l = 0; l < d.L; ++l)
     NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_installed[l], cudaEventDisableTiming));
@@ -609,7 +643,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   for (auto& e : ctx->ev_t) NP_INIT_CUDA(cudaEventCreate(&e));
   for (auto& e : ctx->ev_c) NP_INIT_CUDA(cudaEventCreate(&e));
 
-  if (cfg->transfer_mode == NP_XFER_HOST_GATHER || from_file) {
+  if (mapped_staging || from_file) {
     int n = cfg->host_threads;
     if (n == 0) {
       // the packing is what bounds the transfer (steps/s kept rising up to 14 of 16 cores); two
@@ -813,12 +847,8 @@ int np_delta(np_ctx* ctx, const uint32_t* pred_bitmap, void* stream) {
     pred_bitmap = ctx->t.pred;
   }
   // the previous step's installs must have landed before tables and slots are reused
-  for (int l = 0; l < ctx->d.L; ++l) {
-    if (ctx->install_pending[l]) {
-      NP_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_installed[l], 0));
-      ctx->install_pending[l] = 0;
-    }
-  }
+  NP_CUDA(ctx, wait_installs(ctx, 0, ctx->d.L, s));
+  std::fill(ctx->install_pending.begin(), ctx->install_pending.end(), 0);
   NP_LAUNCH(ctx, launch_delta(ctx->d, ctx->t, pred_bitmap, ctx->cfg.evict_policy, ctx->step, ctx->host_lists_dev,
                             ctx->cfg.flags & NP_F_CHECK_BOUNDS, s));
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_delta, s));
@@ -862,7 +892,7 @@ static int install_from_file(np_ctx* ctx, int layer_begin, int layer_end, cudaSt
       NP_CUDA(ctx, cudaEventRecord(ctx->ev_copied[c.h], cs));
       NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[0], ctx->ev_copied[c.h], 0));
     }
-    NP_LAUNCH(ctx, launch_scatter(d, dbuf, false, nullptr, ctx->t.delta_slots + (size_t)c.l * d.C,
+    NP_LAUNCH(ctx, launch_scatter(d, dbuf, ctx->t.delta_slots + (size_t)c.l * d.C,
                                 ctx->t.counters + (size_t)c.l * NP_N_COUNTERS + NP_CNT_DELTA, c.first, c.rows,
                                 static_cast<char*>(ctx->bufs.gate_buf) + (size_t)(c.l - d.dense) * d.C * row_bytes,
                                 static_cast<char*>(ctx->bufs.up_buf) + (size_t)(c.l - d.dense) * d.C * row_bytes,
@@ -871,8 +901,7 @@ static int install_from_file(np_ctx* ctx, int layer_begin, int layer_end, cudaSt
     NP_CUDA(ctx, cudaEventRecord(ctx->ev_half[c.h], ctx->aux[0]));  // both copies of the part are free again
     ctx->half_pending[c.h] = true;
     if (c.last) {
-      NP_CUDA(ctx, cudaEventRecord(ctx->ev_installed[c.l], ctx->aux[0]));
-      ctx->install_pending[c.l] = 1;
+      NP_CUDA(ctx, mark_installed(ctx, c.l, c.l + 1, ctx->aux[0]));
     }
     return NP_OK;
   };
@@ -893,8 +922,7 @@ static int install_from_file(np_ctx* ctx, int layer_begin, int layer_end, cudaSt
         queued.pop_front();
         if (rc < 0) return give_up(rc);
       }
-      NP_CUDA(ctx, cudaEventRecord(ctx->ev_installed[l], ctx->aux[0]));
-      ctx->install_pending[l] = 1;
+      NP_CUDA(ctx, mark_installed(ctx, l, l + 1, ctx->aux[0]));
       continue;
     }
     for (int first = 0; first < n; first += part_rows) {
@@ -940,20 +968,17 @@ static int install_from_file(np_ctx* ctx, int layer_begin, int layer_end, cudaSt
   return NP_OK;
 }
 
-// NP_XFER_HOST_GATHER: the pool packs the incoming records into a part of the pinned staging,
-// one cudaMemcpyAsync moves the part, scatter kernels place its rows.  The parts are used round
-// robin: one is packed while earlier ones are copied and scattered (the scatter kernels can fall
-// behind while a resident MLP launch holds the device; spare parts keep the host and the copy
-// engine going).  A part takes the rows of up to kGatherLayers consecutive layers: a copy has a
-// start-up cost, and a steady-state layer fills only a fraction of a part.
+// NP_XFER_HOST_GATHER with NP_F_MAPPED_STAGING: the pool packs the incoming records into a part of the pinned staging,
+// scatter kernels read the part through its device mapping and place its rows.  The parts are used round
+// robin: one is packed while earlier ones are scattered (the scatter kernels can fall behind while a resident MLP launch
+// holds the device; spare parts keep the host going).  A part takes the rows of up to kGatherLayers consecutive layers.
 constexpr int kGatherLayers = 2;
 
-static int install_host_gather(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_t cs, int* warn) {
+static int install_packed(np_ctx* ctx, int layer_begin, int layer_end, int* warn) {
   const Dims& d = ctx->d;
   const size_t rec = d.rec_bytes, row_bytes = (size_t)d.D * 2;
   const int check = ctx->cfg.flags & NP_F_CHECK_BOUNDS;
   const char* store = static_cast<const char*>(ctx->bufs.backing);
-  char* staging = static_cast<char*>(ctx->bufs.staging);
   char* hstage = static_cast<char*>(ctx->bufs.host_staging);
   const size_t per_layer = NP_N_COUNTERS + 2 * (size_t)d.C;
   const int parts = std::min(kStageParts, std::max(2, ctx->cfg.staging_rows / std::max(1, d.k / 4 + 1)));
@@ -964,8 +989,8 @@ static int install_host_gather(np_ctx* ctx, int layer_begin, int layer_end, cuda
   };
   std::vector<Piece> batch;
   int h = -1, used = 0, layers_in = 0, last_l = -1;
-  int flushed = 0;  // parts handed to the copy engine by this call
-  const int first_small = 1;  // the first part takes one layer: the copy engine starts sooner
+  int flushed = 0;  // parts scattered by this call
+  const int first_small = 1;  // the first part takes one layer: its rows are on their way sooner
   auto open_part = [&]() -> int {
     h = ctx->next_half % parts;
     ctx->next_half = (h + 1) % parts;
@@ -981,7 +1006,7 @@ static int install_host_gather(np_ctx* ctx, int layer_begin, int layer_end, cuda
   auto flush = [&]() -> int {
     if (batch.empty()) return NP_OK;
     char* hbuf = hstage + (size_t)h * part_rows * rec;
-    char* dbuf = staging + (size_t)h * part_rows * rec;
+    const char* dbuf = ctx->hstage_dev + (size_t)h * part_rows * rec;
     if (used > 0) {
       bool bad = false;
       const int nthreads = ctx->pool ? ctx->pool->size() + 1 : 1;
@@ -1004,27 +1029,17 @@ static int install_host_gather(np_ctx* ctx, int layer_begin, int layer_end, cuda
       if (ctx->pool) ctx->pool->parallel_for(jobs, body);
       else for (int job = 0; job < jobs; ++job) body(job);
       if (bad) return fail(ctx, NP_E_DEVICE, "layer %d: neuron id out of range", batch.front().l);
-      // the copies queue back to back on the caller's stream; the scatter kernels follow them
-      // on a side stream, so a copy never waits for the previous part's kernels
-      if (ctx->hstage_dev) {
-        dbuf = ctx->hstage_dev + (size_t)h * part_rows * rec;  // mapped staging: no staging copy
-      } else {
-        NP_CUDA(ctx, cudaMemcpyAsync(dbuf, hbuf, (size_t)used * rec, cudaMemcpyHostToDevice, cs));
-        NP_CUDA(ctx, cudaEventRecord(ctx->ev_copied[h], cs));
-        NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[0], ctx->ev_copied[h], 0));
-      }
     }
     for (const Piece& pc : batch) {
       if (pc.rows > 0)
-        NP_LAUNCH(ctx, launch_scatter(d, dbuf + (size_t)pc.at * rec, false, nullptr, ctx->t.delta_slots + (size_t)pc.l * d.C,
+        NP_LAUNCH(ctx, launch_scatter(d, dbuf + (size_t)pc.at * rec, ctx->t.delta_slots + (size_t)pc.l * d.C,
                                     ctx->t.counters + (size_t)pc.l * NP_N_COUNTERS + NP_CNT_DELTA, pc.first, pc.rows,
                                     static_cast<char*>(ctx->bufs.gate_buf) + (size_t)(pc.l - d.dense) * d.C * row_bytes,
                                     static_cast<char*>(ctx->bufs.up_buf) + (size_t)(pc.l - d.dense) * d.C * row_bytes,
                                     static_cast<char*>(ctx->bufs.downT_buf) + (size_t)(pc.l - d.dense) * d.C * row_bytes,
                                     ctx->t.status, check, ctx->aux[0], ctx->sm_count));
       if (pc.last) {
-        NP_CUDA(ctx, cudaEventRecord(ctx->ev_installed[pc.l], ctx->aux[0]));
-        ctx->install_pending[pc.l] = 1;
+        NP_CUDA(ctx, mark_installed(ctx, pc.l, pc.l + 1, ctx->aux[0]));
       }
     }
     if (used > 0) {
@@ -1065,86 +1080,98 @@ static int install_host_gather(np_ctx* ctx, int layer_begin, int layer_end, cuda
   return flush();
 }
 
-int np_install(np_ctx* ctx, int32_t layer_begin, int32_t layer_end, void* copy_stream) {
-  if (!ctx) return fail(nullptr, NP_E_INVAL, "ctx is NULL");
+// Rows of a part of the pinned staging.
+static int staging_part_rows(const np_ctx* ctx) {
+  const int parts = std::min(kStageParts, std::max(2, ctx->cfg.staging_rows / std::max(1, ctx->d.k / 4 + 1)));
+  return ctx->cfg.staging_rows / parts;
+}
+
+// The counts of the last np_delta (np_speculate), once the host can read them: what np_install reports.
+static int install_warnings(np_ctx* ctx, int layer_begin, int layer_end, int* warn) {
+  NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_delta));
   const Dims& d = ctx->d;
-  if (layer_begin < 0 || layer_end > d.L || layer_begin > layer_end)
-    return fail(ctx, NP_E_INVAL, "layer range [%d, %d) outside [0, %d)", layer_begin, layer_end, d.L);
-  if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_install needs a prior np_delta");
+  const int room = ctx->cfg.transfer_mode == NP_XFER_HOST_GATHER ? staging_part_rows(ctx) : ctx->cfg.staging_rows;
+  for (int l = std::max(layer_begin, d.dense); l < layer_end; ++l) {
+    const int32_t* cnt = ctx->host_lists + kHostHeaderInts + (size_t)l * (NP_N_COUNTERS + 2 * (size_t)d.C);
+    const int n = cnt[NP_CNT_DELTA];
+    if (n < 0 || n > d.C) return fail(ctx, NP_E_DEVICE, "layer %d: delta count %d outside [0, %d]", l, n, d.C);
+    if (cnt[NP_CNT_OVERFLOW] > 0) *warn = NP_W_OVERFLOW;
+    if (n > room && *warn == NP_OK) *warn = NP_W_CHUNKED;
+  }
+  return NP_OK;
+}
+
+// Rows pulled from the store by the device: launches of consecutive layers, in order, on the caller's copy stream.  Up to
+// eight launches, so that the MLP runs behind them (sparse_runs) can start as their own rows land, but none that is
+// expected to move less than 1 MB (about 20 us of the link): a launch and its mark cost the host and the device several
+// microseconds each.
+static int install_pull(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_t cs) {
+  const Dims& d = ctx->d;
+  const int n = layer_end - layer_begin;
+  if (n <= 0) return NP_OK;
+  const size_t expect = d.rec_bytes * (size_t)std::max(1, d.k / 8);  // bytes of a layer: an eighth of the set is new
+  const int least = (int)std::min<size_t>(n, ((1u << 20) + expect - 1) / expect);
+  const int launches = std::max(1, std::min(8, n / std::max(1, least)));
+  for (int g = 0; g < launches; ++g) {
+    const int l0 = layer_begin + (int)((long long)n * g / launches), l1 = layer_begin + (int)((long long)n * (g + 1) / launches);
+    NP_LAUNCH(ctx, launch_pull(d, ctx->t, ctx->backing_dev, ctx->bufs.gate_buf, ctx->bufs.up_buf, ctx->bufs.downT_buf, l0, l1,
+                               ctx->cfg.flags & NP_F_CHECK_BOUNDS, cs));
+    NP_CUDA(ctx, mark_installed(ctx, l0, l1, cs));
+  }
+  return NP_OK;
+}
+
+// NP_XFER_MEMCPY_RUNS: whether the copy engine moves the layers faster than the pull kernel.  A copy call costs 4.6 us and
+// its bytes cross at 55.1 GB/s, the kernel reads at 51.2: calls pay from about 3.4 MB each.  Runs are that long only where
+// most of a layer arrives at once.
+constexpr size_t kRunBytes = 3400000;
+static bool runs_by_copies(const np_ctx* ctx, int layer_begin, int layer_end) {
+  const Dims& d = ctx->d;
+  size_t rows = 0, runs = 0;
+  for (int l = layer_begin; l < layer_end; ++l) {
+    const int32_t* cnt = ctx->host_lists + kHostHeaderInts + (size_t)l * (NP_N_COUNTERS + 2 * (size_t)d.C);
+    const int32_t* ids = cnt + NP_N_COUNTERS;
+    const int n = cnt[NP_CNT_DELTA];
+    rows += n;
+    for (int i = 0; i < n; ++i) runs += i == 0 || ids[i] != ids[i - 1] + 1;
+  }
+  return runs > 0 && rows * d.rec_bytes >= runs * kRunBytes;
+}
+
+// Queues the transfer on a stream that is already ordered after the delta step.  *late: the warnings are to be collected
+// afterwards (install_warnings).
+static int install_enqueue(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_t cs, int* warn, bool* late) {
+  const Dims& d = ctx->d;
+  *late = false;
   layer_begin = std::max(layer_begin, d.dense);  // dense layers hold all their rows already
   layer_end = std::max(layer_end, layer_begin);
-  cudaStream_t cs = as_stream(copy_stream);
   const int check = ctx->cfg.flags & NP_F_CHECK_BOUNDS;
   const int mode = ctx->cfg.transfer_mode;
   const size_t rec = d.rec_bytes;
   const size_t row_bytes = (size_t)d.D * 2;
-  NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_delta, 0));
-  int warn = NP_OK;
-  // Side streams: ordered after everything the caller's copy stream holds so far, and joined
-  // back into it at the end, so the caller sees one stream's worth of ordering.
-  const bool forked = mode != NP_XFER_MEMCPY_RUNS;
-  if (forked) {
-    NP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, cs));
-    for (int i = 0; i < 2; ++i) NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[i], ctx->ev_fork, 0));
+  if (mode == NP_XFER_ZERO_COPY) return install_pull(ctx, layer_begin, layer_end, cs);
+  if (mode == NP_XFER_HOST_GATHER && !ctx->hstage_dev) {
+    *late = true;
+    return install_pull(ctx, layer_begin, layer_end, cs);
   }
-  auto join = [&]() -> cudaError_t {
-    for (int i = 0; i < 2; ++i) {
-      cudaError_t e = cudaEventRecord(ctx->ev_join[i], ctx->aux[i]);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ctx->ev_join[i], 0);
-      if (e != cudaSuccess) return e;
+  if (mode == NP_XFER_MEMCPY_RUNS) {
+    bool copies = false;
+    if ((size_t)d.C * rec >= kRunBytes) {  // else no run can be long enough, whatever the lists hold
+      const int rc = install_warnings(ctx, layer_begin, layer_end, warn);
+      if (rc < 0) return rc;
+      copies = runs_by_copies(ctx, layer_begin, layer_end);
+    } else {
+      *late = true;
     }
-    return cudaSuccess;
-  };
-
-  if (mode == NP_XFER_ZERO_COPY) {
-    // consecutive layers alternate between the two side streams: one kernel's tail (its last
-    // reads are still crossing PCIe) overlaps the next kernel's start
-    const int max_rows = d.C;
+    if (!copies) return install_pull(ctx, layer_begin, layer_end, cs);
+    const char* store = static_cast<const char*>(ctx->bufs.backing);
+    char* staging = static_cast<char*>(ctx->bufs.staging);
     for (int l = layer_begin; l < layer_end; ++l) {
-      cudaStream_t zs = ctx->aux[l & 1];
-      const char* store_l = ctx->backing_dev + (size_t)(l % d.Lp) * d.M * rec;
-      NP_LAUNCH(ctx, launch_scatter(d, store_l, true, ctx->t.delta_ids + (size_t)l * d.C,
-                                  ctx->t.delta_slots + (size_t)l * d.C,
-                                  ctx->t.counters + (size_t)l * NP_N_COUNTERS + NP_CNT_DELTA, 0, max_rows,
-                                  static_cast<char*>(ctx->bufs.gate_buf) + (size_t)(l - d.dense) * d.C * row_bytes,
-                                  static_cast<char*>(ctx->bufs.up_buf) + (size_t)(l - d.dense) * d.C * row_bytes,
-                                  static_cast<char*>(ctx->bufs.downT_buf) + (size_t)(l - d.dense) * d.C * row_bytes,
-                                  ctx->t.status, check, zs, ctx->sm_count));
-      NP_CUDA(ctx, cudaEventRecord(ctx->ev_installed[l], zs));
-      ctx->install_pending[l] = 1;
-    }
-    NP_CUDA(ctx, join());
-    return NP_OK;
-  }
-
-  // the host plans the copies: wait until the delta lists are readable
-  NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_delta));
-  if (mode == NP_XFER_FILE || mode == NP_XFER_HOST_GATHER) {
-    const int rc = mode == NP_XFER_FILE ? install_from_file(ctx, layer_begin, layer_end, cs, &warn)
-                                        : install_host_gather(ctx, layer_begin, layer_end, cs, &warn);
-    if (rc < 0) return rc;
-    NP_CUDA(ctx, join());
-    return warn;
-  }
-  const char* store = static_cast<const char*>(ctx->bufs.backing);
-  char* staging = static_cast<char*>(ctx->bufs.staging);
-  const size_t per_layer = NP_N_COUNTERS + 2 * (size_t)d.C;
-  for (int l = layer_begin; l < layer_end; ++l) {
-    const int32_t* cnt = ctx->host_lists + kHostHeaderInts + (size_t)l * per_layer;
-    const int32_t* ids = cnt + NP_N_COUNTERS;
-    const int n = cnt[NP_CNT_DELTA];
-    if (n < 0 || n > d.C) return fail(ctx, NP_E_DEVICE, "layer %d: delta count %d outside [0, %d]", l, n, d.C);
-    if (cnt[NP_CNT_OVERFLOW] > 0) warn = NP_W_OVERFLOW;
-    const char* store_l = store + (size_t)(l % d.Lp) * d.M * rec;
-    char* gate_l = static_cast<char*>(ctx->bufs.gate_buf) + (size_t)(l - d.dense) * d.C * row_bytes;
-    char* up_l = static_cast<char*>(ctx->bufs.up_buf) + (size_t)(l - d.dense) * d.C * row_bytes;
-    char* down_l = static_cast<char*>(ctx->bufs.downT_buf) + (size_t)(l - d.dense) * d.C * row_bytes;
-    const int32_t* slots_dev = ctx->t.delta_slots + (size_t)l * d.C;
-    const int32_t* count_dev = ctx->t.counters + (size_t)l * NP_N_COUNTERS + NP_CNT_DELTA;
-
-    if (mode == NP_XFER_MEMCPY_RUNS) {
-      const int cap = ctx->cfg.staging_rows;
-      if (n > cap && warn == NP_OK) warn = NP_W_CHUNKED;
+      const int32_t* cnt = ctx->host_lists + kHostHeaderInts + (size_t)l * (NP_N_COUNTERS + 2 * (size_t)d.C);
+      const int32_t* ids = cnt + NP_N_COUNTERS;
+      const int n = cnt[NP_CNT_DELTA], cap = ctx->cfg.staging_rows;
+      const char* store_l = store + (size_t)(l % d.Lp) * d.M * rec;
+      const size_t buf_l = (size_t)(l - d.dense) * d.C * row_bytes;
       for (int first = 0; first < n; first += cap) {
         const int rows = std::min(cap, n - first);
         // ascending IDs: adjacent IDs are adjacent records of the store -> one copy per run
@@ -1158,27 +1185,40 @@ int np_install(np_ctx* ctx, int32_t layer_begin, int32_t layer_end, void* copy_s
                                        cudaMemcpyHostToDevice, cs));
           r += len;
         }
-        NP_LAUNCH(ctx, launch_scatter(d, staging, false, nullptr, slots_dev, count_dev, first, rows, gate_l, up_l,
-                                    down_l, ctx->t.status, check, cs, ctx->sm_count));
+        NP_LAUNCH(ctx, launch_scatter(d, staging, ctx->t.delta_slots + (size_t)l * d.C,
+                                    ctx->t.counters + (size_t)l * NP_N_COUNTERS + NP_CNT_DELTA, first, rows,
+                                    static_cast<char*>(ctx->bufs.gate_buf) + buf_l, static_cast<char*>(ctx->bufs.up_buf) + buf_l,
+                                    static_cast<char*>(ctx->bufs.downT_buf) + buf_l, ctx->t.status, check, cs, ctx->sm_count));
       }
+      NP_CUDA(ctx, mark_installed(ctx, l, l + 1, cs));
     }
-    NP_CUDA(ctx, cudaEventRecord(ctx->ev_installed[l], cs));
-    ctx->install_pending[l] = 1;
+    return NP_OK;
   }
-  if (forked) NP_CUDA(ctx, join());
-  return warn;
+  // File reads and packed staging: the host plans the transfer, so it waits until the lists are readable.  The scatter
+  // kernels run on a side stream: ordered after everything the caller's copy stream holds so far, and joined back into it
+  // at the end, so the caller sees one stream's worth of ordering.
+  NP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, cs));
+  NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[0], ctx->ev_fork, 0));
+  NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_delta));
+  const int rc = mode == NP_XFER_FILE ? install_from_file(ctx, layer_begin, layer_end, cs, warn)
+                                      : install_packed(ctx, layer_begin, layer_end, warn);
+  if (rc < 0) return rc;
+  NP_CUDA(ctx, cudaEventRecord(ctx->ev_join[0], ctx->aux[0]));
+  NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_join[0], 0));
+  return NP_OK;
 }
 
-// Orders `s` after a layer's install mark; marks that have already completed need no wait.
-static cudaError_t wait_install(np_ctx* ctx, int layer, cudaStream_t s) {
-  const cudaError_t q = cudaEventQuery(ctx->ev_installed[layer]);
-  if (q == cudaSuccess) {
-    ctx->install_pending[layer] = 0;  // landed: later calls need not ask again
-    return cudaSuccess;
-  }
-  if (q != cudaErrorNotReady) return q;
-  (void)cudaGetLastError();
-  return cudaStreamWaitEvent(s, ctx->ev_installed[layer], 0);
+int np_install(np_ctx* ctx, int32_t layer_begin, int32_t layer_end, void* copy_stream) {
+  if (!ctx) return fail(nullptr, NP_E_INVAL, "ctx is NULL");
+  if (layer_begin < 0 || layer_end > ctx->d.L || layer_begin > layer_end)
+    return fail(ctx, NP_E_INVAL, "layer range [%d, %d) outside [0, %d)", layer_begin, layer_end, ctx->d.L);
+  if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_install needs a prior np_delta");
+  int warn = NP_OK;
+  bool late = false;
+  NP_CUDA(ctx, cudaStreamWaitEvent(as_stream(copy_stream), ctx->ev_delta, 0));
+  int rc = install_enqueue(ctx, layer_begin, layer_end, as_stream(copy_stream), &warn, &late);
+  if (rc >= 0 && late) rc = install_warnings(ctx, layer_begin, layer_end, &warn);
+  return rc < 0 ? rc : warn;
 }
 
 // gu_sel: which of the two dot-product accumulators this layer uses (the batch kernels clear the
@@ -1217,7 +1257,7 @@ static int mlp_layer(np_ctx* ctx, int layer, const float* xa, const float* xb, f
   a.status = ctx->t.status;
   a.gu = a.gu_next = a.ssq = a.ssq_next = nullptr;
   a.xterms = (ctx->cfg.flags & NP_F_TCGEN05_BATCH) ? ctx->xterms : nullptr;
-  if (ctx->install_pending[layer]) NP_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_installed[layer], 0));
+  NP_CUDA(ctx, wait_installs(ctx, layer, layer + 1, s));
   if (ctx->mlp_tc && B >= kTcMinBatch && !a.force_direct) {
     const int cur = gu_sel < 0 ? 0 : gu_sel;
     a.gu = ctx->ws.gu[cur];
@@ -1238,6 +1278,9 @@ static int mlp_layer(np_ctx* ctx, int layer, const float* xa, const float* xb, f
 
 enum { kChainAll = 0, kChainHead = 1, kChainTail = 2 };
 
+// Whether the install of this context's rows runs on the device itself (the pull kernel), not through staging.
+static bool pulls(const np_ctx* ctx) { return ctx->cfg.transfer_mode != NP_XFER_FILE && !ctx->hstage_dev; }
+
 // Runs of the sparse layers in which a resident kernel takes them.  A run starts once its layers are installed, so what
 // the step waits for after its last row has landed is the last run: with chain_layers = 0 the runs shrink towards the end
 // (the tail is an eighth of the stack, the run before it a quarter, the first run takes the rest), which also makes fewer
@@ -1247,19 +1290,32 @@ static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
   // layers whose rows have all landed already need no run of their own to wait in: they go into one
   // first run (the whole stack when nothing is pending, as in np_mlp_chain on resident rows)
   int landed = d.dense;
-  while (landed < d.L) {
-    if (ctx->install_pending[landed]) {
-      const cudaError_t q = cudaEventQuery(ctx->ev_installed[landed]);
+  cudaEvent_t ready = nullptr;
+  for (; landed < d.L; ++landed) {
+    if (!ctx->install_pending[landed]) continue;
+    if (ctx->mark[landed] != ready) {
+      const cudaError_t q = cudaEventQuery(ctx->mark[landed]);
       if (q == cudaErrorNotReady) {
         (void)cudaGetLastError();
         break;
       }
       if (q != cudaSuccess) return fail(ctx, NP_E_CUDA, "cudaEventQuery failed: %s", cudaGetErrorString(q));
-      ctx->install_pending[landed] = 0;
+      ready = ctx->mark[landed];
     }
-    ++landed;
+    ctx->install_pending[landed] = 0;
   }
   const int ns = d.L - landed;  // layers that still wait for rows
+  // Behind a dense prefix that takes longer than the rows do (an eighth of a set per layer at 50 GB/s, half as much again;
+  // a dense layer streams at 6 TB/s) there is nothing to wait for either.  (7B shape, 24 dense layers: 1.195 ms a step with
+  // one run, 1.215 with three; three such stacks stepping in turn 1.26 and 1.41: a resident launch of one context delays
+  // those of the others.)
+  if (pulls(ctx) && d.dense > 0 && ctx->cfg.chain_layers == 0 && d.dense < d.L) {
+    const double pull_s = 1.5 * ns * (d.k / 8.0) * (double)d.rec_bytes / 50e9, dense_s = d.dense * ((double)d.M * 6.0 * d.D / 6e12);
+    if (pull_s < dense_s) {
+      runs->push_back(d.L - d.dense);
+      return NP_OK;
+    }
+  }
   if (ctx->cfg.chain_layers > 0) {
     const int run = ctx->cfg.chain_layers;
     for (int l0 = d.dense; l0 < d.L; l0 += run) runs->push_back(std::min(run, d.L - l0));
@@ -1269,23 +1325,51 @@ static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
   if (ns > 0) {
     const int unit = std::max(1, (d.L - d.dense) / 8);
     const int tail = std::min(ns, unit), mid = std::min(ns - tail, 2 * unit), first = ns - tail - mid;
-    if (first > 0) runs->push_back(first);
-    if (mid > 0) runs->push_back(mid);
-    runs->push_back(tail);
+    int l1 = landed;
+    cudaEvent_t last = nullptr;
+    for (const int n : {first, mid, tail}) {
+      if (n == 0) continue;
+      l1 += n;
+      // rows that arrive with the last rows of the run before are no reason for another launch
+      const cudaEvent_t m = ctx->install_pending[l1 - 1] ? ctx->mark[l1 - 1] : nullptr;
+      if (m && m == last) runs->back() += n;
+      else runs->push_back(n);
+      last = m;
+    }
   }
   return NP_OK;
 }
 
-static int batch_run(np_ctx* ctx, const ChainArgs& a, float* x, int B, cudaStream_t s) {
+// SMs for a resident launch.  One that runs while rows are pulled leaves the pull kernel its SMs: on all of them it would
+// not start before the last row has landed.  Every launch of a step does so, also those that no pull of the same step runs
+// beside: other contexts pull, too, and a launch on all SMs would wait for them (2.7 % of the SMs; a step of the 7B shape
+// with 24 dense layers is 1.22 ms this way and 1.25 with the dense layers cut in two launches, the second on all SMs).
+static int resident_sms(const np_ctx* ctx, bool beside_pull, bool (*fits)(const Dims&, int)) {
+  const int n = ctx->sm_count - kPullReserve;
+  return beside_pull && pulls(ctx) && ctx->d.dense < ctx->d.L && n > 0 && fits(ctx->d, n) ? n : ctx->sm_count;
+}
+
+// Layers per launch of the dense prefix: all of them where the pull kernel installs the sparse layers' rows meanwhile.  The
+// scatter kernels of the staged modes do not run beside a resident launch: there the prefix runs in several launches, and
+// the installs advance between them.  The fewer sparse layers wait for rows, the longer a run may be (measured at the 7B
+// shape with packed staging: d = 20: 697 steps/s with runs of 3, 648 with 6; d = 24: 711 / 755 / 702 / 594 with runs of
+// 3 / 6 / 8 / 24; d = 28: 682 / 710 / 725 with 3 / 6 / 12).
+static int dense_run_layers(const np_ctx* ctx) {
+  const Dims& d = ctx->d;
+  if (pulls(ctx) || d.dense == d.L) return d.dense;
+  return std::max(3, std::min(12, 2 * d.dense / (d.L - d.dense)));
+}
+
+static int batch_run(np_ctx* ctx, const ChainArgs& a, float* x, int B, bool beside_pull, cudaStream_t s) {
   int n = 0;
-  NP_CUDA(ctx, chain_batch::launch(ctx->d, a, x, B, &ctx->batch, s, ctx->sm_count, &n));
+  NP_CUDA(ctx, chain_batch::launch(ctx->d, a, x, B, &ctx->batch, s, resident_sms(ctx, beside_pull, chain_batch::supported), &n));
   ctx->launches += n;
   return NP_OK;
 }
 
 // The chain for a batch in the resident kernel: runs of layers as for one sequence, x in the kernel's own tiles
 // (the accumulators' space, which no other kernel of this chain uses).
-static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part) {
+static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part, bool stepping) {
   const Dims& d = ctx->d;
   const size_t row_bytes = (size_t)d.D * 2;
   float* x = ctx->ws.zbuf[0];
@@ -1297,18 +1381,17 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
     ctx->chain_kernel_launches = 0;
     NP_LAUNCH(ctx, chain_batch::launch_in(d, x_bf16, x, B, s));
     if (d.dense > 0) {
-      // runs, so that the sparse layers' installs advance between them (as for one sequence)
       const char* dense = static_cast<const char*>(ctx->bufs.dense_buf);
       a.gate = dense;
       a.up = dense + row_bytes;
       a.downT = dense + 2 * row_bytes;
       a.active_slots = ctx->t.identity;
       a.dense_rows = d.M;
-      const int dense_run = d.dense < d.L ? std::max(3, std::min(12, 2 * d.dense / (d.L - d.dense))) : d.dense;
+      const int dense_run = dense_run_layers(ctx);
       for (int l0 = 0; l0 < d.dense; l0 += dense_run) {
         a.l_begin = l0;
         a.l_end = std::min(d.dense, l0 + dense_run);
-        const int rc = batch_run(ctx, a, x, B, s);
+        const int rc = batch_run(ctx, a, x, B, stepping, s);
         if (rc < 0) return rc;
       }
     }
@@ -1323,13 +1406,13 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
   std::vector<int> runs;
   int rc = sparse_runs(ctx, &runs);
   if (rc < 0) return rc;
+  const bool beside_pull = stepping || ctx->install_pending[d.L - 1];
   int l0 = d.dense;
   for (const int n : runs) {
-    for (int l = l0; l < l0 + n; ++l)
-      if (ctx->install_pending[l]) NP_CUDA(ctx, wait_install(ctx, l, s));
+    NP_CUDA(ctx, wait_installs(ctx, l0, l0 + n, s));
     a.l_begin = l0;
     a.l_end = l0 += n;
-    rc = batch_run(ctx, a, x, B, s);
+    rc = batch_run(ctx, a, x, B, beside_pull, s);
     if (rc < 0) return rc;
   }
   NP_LAUNCH(ctx, chain_batch::launch_out(d, x, x_out, B, s));
@@ -1341,8 +1424,9 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
 // `part`: kChainAll = the whole chain; kChainHead = its start up to the end of the dense prefix
 // (nothing there waits for an install, so np_step queues it before the host packs any rows);
 // kChainTail = the sparse layers and the result.
-static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part = kChainAll) {
-  if (B >= kTcMinBatch && ctx->use_batch) return batch_chain(ctx, x_bf16, B, x_out, s, part);
+// `stepping`: a launch of np_step, beside which rows are pulled.
+static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part, bool stepping) {
+  if (B >= kTcMinBatch && ctx->use_batch) return batch_chain(ctx, x_bf16, B, x_out, s, part, stepping);
   const Dims& d = ctx->d;
   const size_t n = (size_t)B * d.D;
   const bool persistent = B == 1 && !(ctx->cfg.flags & (NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES)) &&
@@ -1382,19 +1466,13 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
       a.downT = dense + 2 * row_bytes;
       a.active_slots = ctx->t.identity;
       a.dense_rows = d.M;
-      // Runs, not one launch: while a resident launch is on the device the install's scatter
-      // kernels do not run beside it (its blocks hold the register file), so the installs of the
-      // sparse layers advance between runs.  The fewer sparse layers wait for rows, the longer a
-      // run may be (measured at the 7B shape: d = 20: 697 steps/s with runs of 3, 648 with 6;
-      // d = 24: 711 / 755 / 702 / 594 with runs of 3 / 6 / 8 / 24; d = 28: 682 / 710 / 725 with
-      // 3 / 6 / 12).
-      const int dense_run = d.dense < d.L ? std::max(3, std::min(12, 2 * d.dense / (d.L - d.dense))) : 12;
+      const int dense_run = dense_run_layers(ctx);
       for (int l0 = 0; l0 < d.dense; l0 += dense_run) {
         a.l_begin = l0;
         a.l_end = std::min(d.dense, l0 + dense_run);
         if (dense_chain::supported(d, ctx->sm_count))
           NP_LAUNCH(ctx, dense_chain::launch(d, dense, d.M, a.xbuf, a.zbuf, a.grid_bar, a.status, a.l_begin, a.l_end, s,
-                                             ctx->sm_count));
+                                             resident_sms(ctx, stepping, dense_chain::supported)));
         else
           NP_LAUNCH(ctx, chain_alu::launch(d, a, s, ctx->sm_count));
       }
@@ -1411,11 +1489,11 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
       const int rc = sparse_runs(ctx, &runs);
       if (rc < 0) return rc;
     }
+    const bool beside_pull = stepping || ctx->install_pending[d.L - 1];
     int l0 = d.dense;
     for (size_t ri = 0; ri < runs.size() && part != kChainHead; ++ri) {
       const int l1 = l0 + runs[ri];
-      for (int l = l0; l < l1; ++l)
-        if (ctx->install_pending[l]) NP_CUDA(ctx, wait_install(ctx, l, s));
+      NP_CUDA(ctx, wait_installs(ctx, l0, l1, s));
       a.l_begin = l0;
       a.l_end = l1;
       if (ctx->use_rows) {
@@ -1423,17 +1501,18 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
         ctx->chain_kernel_launches += (l1 - l0 + rl - 1) / rl;
         NP_LAUNCH(ctx, chain_rows::launch(d, a, &ctx->rows, s));
       } else if (ctx->use_slices) {
+        const int sms = resident_sms(ctx, beside_pull, chain_slices::supported);
         chain_slices::Plan sp;
-        chain_slices::plan(d, ctx->sm_count, &sp);
+        chain_slices::plan(d, sms, &sp);
         ctx->chain_kernel_launches += (l1 - l0 + sp.run_layers - 1) / sp.run_layers;
         a.x_out = l1 == d.L ? x_out : nullptr;  // the run that ends the stack may leave the result itself
         if (lazy_clear && l0 == 0 && std::min(l1, sp.run_layers) == 1 && l1 != d.L)
           NP_CUDA(ctx, cudaMemsetAsync(ctx->ws.zbuf[0], 0, (size_t)kZRep * d.D * 4, s));
-        NP_LAUNCH(ctx, chain_slices::launch(d, a, &ctx->slices, s, ctx->sm_count));
+        NP_LAUNCH(ctx, chain_slices::launch(d, a, &ctx->slices, s, sms));
         out_written = a.x_out && ctx->slices.wrote_out;
       } else {
         ctx->chain_kernel_launches += 1;
-        NP_LAUNCH(ctx, chain_alu::launch(d, a, s, ctx->sm_count));
+        NP_LAUNCH(ctx, chain_alu::launch(d, a, s, resident_sms(ctx, beside_pull, chain_alu::supported)));
       }
       l0 = l1;
     }
@@ -1473,7 +1552,7 @@ int np_mlp_chain(np_ctx* ctx, const void* x_bf16, int32_t B, float* x_out, void*
   if ((uintptr_t)x_out % 16) return fail(ctx, NP_E_INVAL, "x_out must be 16-byte aligned");
   if (B < 1 || B > ctx->d.Bmax) return fail(ctx, NP_E_INVAL, "B=%d outside [1, max_batch=%d]", B, ctx->d.Bmax);
   if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_mlp_chain needs a prior np_delta");
-  return mlp_chain(ctx, x_bf16, B, x_out, as_stream(stream));
+  return mlp_chain(ctx, x_bf16, B, x_out, as_stream(stream), kChainAll, false);
 }
 
 int np_selftest_bounded_wait(np_ctx* ctx, void* stream) {
@@ -1491,8 +1570,7 @@ int np_speculate(np_ctx* ctx, const uint32_t* cand_bitmap, int32_t budget, void*
   if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_speculate needs a prior np_delta");
   cudaStream_t s = as_stream(stream);
   // rows brought in ahead of time by an earlier call must have landed before their tables move again
-  for (int l = 0; l < ctx->d.L; ++l)
-    if (ctx->have_spec && ctx->install_pending[l]) NP_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_installed[l], 0));
+  if (ctx->have_spec) NP_CUDA(ctx, wait_installs(ctx, 0, ctx->d.L, s));
   NP_LAUNCH(ctx, launch_speculate(ctx->d, ctx->t, cand_bitmap, std::min(budget, ctx->d.C),
                                   ctx->host_lists_dev + host_area_ints(ctx->cfg), s));
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_spec, s));
@@ -1617,23 +1695,28 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   // the dense prefix waits for no install: it is queued before the host starts on the rows
   const bool head_first = d.dense > 0;
   if (head_first) {
-    rc = mlp_chain(ctx, x_bf16, B, x_out, s, kChainHead);
+    rc = mlp_chain(ctx, x_bf16, B, x_out, s, kChainHead, true);
     if (rc < 0) return rc;
   }
-  // the copy stream is ordered after the delta step inside np_install
   NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_delta, 0));
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[0], cs));
-  const int warn = np_install(ctx, 0, d.L, copy_stream);
-  if (warn < 0) return warn;
+  int warn = NP_OK;
+  bool late = false;
+  rc = install_enqueue(ctx, 0, d.L, cs, &warn, &late);
+  if (rc < 0) return rc;
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[1], cs));
 
-  rc = mlp_chain(ctx, x_bf16, B, x_out, s, head_first ? kChainTail : kChainAll);
+  rc = mlp_chain(ctx, x_bf16, B, x_out, s, head_first ? kChainTail : kChainAll, true);
   if (rc < 0) return rc;
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_t[3], s));
   ctx->have_step = true;
   if (spec) {
     // the guessed rows cross behind the step's own rows, while its MLP launches run
     rc = np_install_speculative(ctx, copy_stream);
+    if (rc < 0) return rc;
+  }
+  if (late) {  // everything is queued: now the host may wait for the delta step's counts
+    rc = install_warnings(ctx, 0, d.L, &warn);
     if (rc < 0) return rc;
   }
   return warn;

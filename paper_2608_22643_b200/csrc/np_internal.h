@@ -113,12 +113,15 @@ cudaError_t launch_delta(const Dims& d, const Tables& t, const uint32_t* pred, i
 cudaError_t launch_speculate(const Dims& d, const Tables& t, const uint32_t* cand, int budget, int32_t* host_lists_dev,
                              cudaStream_t s);
 
-// src_is_store: records are read from the whole-layer store by neuron ID
-// (zero-copy); otherwise record r of `src` is the r-th entry of the lists.
-cudaError_t launch_scatter(const Dims& d, const void* src, bool src_is_store, const int32_t* ids,
-                           const int32_t* slots, const int32_t* count_ptr, int first, int max_rows,
-                           void* gate_l, void* up_l, void* downT_l, int32_t* status, int check,
+// record r of `src` (staged records) goes to the slot of entry first + r of the layer's list
+cudaError_t launch_scatter(const Dims& d, const void* src, const int32_t* slots, const int32_t* count_ptr, int first,
+                           int max_rows, void* gate_l, void* up_l, void* downT_l, int32_t* status, int check,
                            cudaStream_t s, int sm_count);
+// the incoming rows of layers [l_begin, l_end), read from the pinned store by neuron ID and placed
+cudaError_t launch_pull(const Dims& d, const Tables& t, const char* store_dev, void* gate, void* up, void* downT, int l_begin,
+                        int l_end, int check, cudaStream_t s);
+// SMs that resident kernels leave free where rows are pulled beside them: room for the pulls of two contexts
+constexpr int kPullReserve = 4;
 
 cudaError_t launch_dequant_dense_layer(const Dims& d, const void* store_l, const int32_t* identity, void* dense_l,
                                        int32_t* status, cudaStream_t s, int sm_count);

@@ -1045,10 +1045,14 @@ bool counted_handover(const Dims& d, int sm_count) {
   return plan(d, sm_count, &p) && p.ks <= kFixMaxKS;
 }
 
+// room for a launch on all SMs and for one beside the pull kernel
 size_t xch_words(const Dims& d, int sm_count) {
-  Plan p;
-  if (!plan(d, sm_count, &p)) return 16;
-  return (size_t)2 * (p.R * kQ) * p.xch_stride;
+  size_t most = 16;
+  for (const int n : {sm_count, sm_count - kPullReserve}) {
+    Plan p;
+    if (plan(d, n, &p)) most = std::max(most, (size_t)2 * (p.R * kQ) * p.xch_stride);
+  }
+  return most;
 }
 size_t zfix_words(const Dims& d) { return (size_t)2 * kFixRep * d.D; }
 size_t bar_words() { return (size_t)kQ * kBarStride; }

@@ -3,8 +3,8 @@
 // writes the three rows to the slot the delta step assigned, in the three
 // projection-specific resident buffers.  Pure 16-byte coalesced copies.
 //
-// The same kernel serves the zero-copy transfer mode, where `src` is the whole
-// layer of the pinned record store and records are addressed by neuron ID.
+// k_pull_rows does the same straight from the pinned record store, records addressed by neuron ID:
+// transfer and placement in one kernel, for several layers a launch.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -17,32 +17,19 @@ using namespace npd;
 
 constexpr int kScatterThreads = 256;
 
-template <bool kFromStore>
 __global__ void __launch_bounds__(kScatterThreads) k_deinterleave_scatter(
-    const uint4* __restrict__ src, const int32_t* __restrict__ ids, const int32_t* __restrict__ slots,
-    const int32_t* __restrict__ count_ptr, int first, int max_rows, uint4* __restrict__ gate,
-    uint4* __restrict__ up, uint4* __restrict__ downT, int row_chunks /* D*2/16 */, int M, int C,
-    int32_t* status, int check) {
+    const uint4* __restrict__ src, const int32_t* __restrict__ slots, const int32_t* __restrict__ count_ptr, int first,
+    int max_rows, uint4* __restrict__ gate, uint4* __restrict__ up, uint4* __restrict__ downT,
+    int row_chunks /* D*2/16 */, int C, int32_t* status, int check) {
   int n = *count_ptr - first;  // rows of this chunk
   if (n > max_rows) n = max_rows;
   for (int r = blockIdx.x; r < n; r += gridDim.x) {
     const int slot = slots[first + r];
-    size_t rec;
-    if (kFromStore) {
-      const int id = ids[first + r];
-      if (check && (id < 0 || id >= M)) {
-        if (threadIdx.x == 0) atomicOr(status, kStatBadNeuron);
-        continue;
-      }
-      rec = (size_t)id;
-    } else {
-      rec = (size_t)r;
-    }
     if (check && (slot < 0 || slot >= C)) {
       if (threadIdx.x == 0) atomicOr(status, kStatBadSlot);
       continue;
     }
-    const uint4* s = src + rec * 3 * row_chunks;
+    const uint4* s = src + (size_t)r * 3 * row_chunks;
     const size_t dst = (size_t)slot * row_chunks;
     // up to 4 loads in flight per thread per projection
     for (int c0 = threadIdx.x; c0 < row_chunks; c0 += kScatterThreads * 4) {
@@ -146,37 +133,148 @@ __global__ void __launch_bounds__(kScatterThreads) k_dequant_scatter(
   }
 }
 
-cudaError_t launch_scatter(const Dims& d, const void* src, bool src_is_store, const int32_t* ids,
-                           const int32_t* slots, const int32_t* count_ptr, int first, int max_rows,
-                           void* gate_l, void* up_l, void* downT_l, int32_t* status, int check,
+cudaError_t launch_scatter(const Dims& d, const void* src, const int32_t* slots, const int32_t* count_ptr, int first,
+                           int max_rows, void* gate_l, void* up_l, void* downT_l, int32_t* status, int check,
                            cudaStream_t s, int sm_count) {
   if (max_rows <= 0) return cudaSuccess;
-  const int row_chunks = d.D * 2 / 16;
-  int blocks = max_rows;
-  const int cap = sm_count * 8;
-  if (blocks > cap) blocks = cap;
-  if (d.rec_int8) {
-    if (src_is_store)
-      k_dequant_scatter<true><<<blocks, kScatterThreads, 0, s>>>(
-          static_cast<const unsigned char*>(src), ids, slots, count_ptr, first, max_rows, static_cast<uint4*>(gate_l),
-          static_cast<uint4*>(up_l), static_cast<uint4*>(downT_l), d.D, d.rec_bytes, d.M, d.C, (d.D >> 4) * 2, status,
-          check);
-    else
-      k_dequant_scatter<false><<<blocks, kScatterThreads, 0, s>>>(
-          static_cast<const unsigned char*>(src), ids, slots, count_ptr, first, max_rows, static_cast<uint4*>(gate_l),
-          static_cast<uint4*>(up_l), static_cast<uint4*>(downT_l), d.D, d.rec_bytes, d.M, d.C, (d.D >> 4) * 2, status,
-          check);
-    return cudaGetLastError();
+  const int blocks = std::min(max_rows, sm_count * 8);
+  if (d.rec_int8)
+    k_dequant_scatter<false><<<blocks, kScatterThreads, 0, s>>>(
+        static_cast<const unsigned char*>(src), nullptr, slots, count_ptr, first, max_rows, static_cast<uint4*>(gate_l),
+        static_cast<uint4*>(up_l), static_cast<uint4*>(downT_l), d.D, d.rec_bytes, d.M, d.C, (d.D >> 4) * 2, status, check);
+  else
+    k_deinterleave_scatter<<<blocks, kScatterThreads, 0, s>>>(
+        static_cast<const uint4*>(src), slots, count_ptr, first, max_rows, static_cast<uint4*>(gate_l),
+        static_cast<uint4*>(up_l), static_cast<uint4*>(downT_l), d.D * 2 / 16, d.C, status, check);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------
+// Transfer and placement in one: the incoming rows of several layers, read by neuron ID from the pinned store.
+//
+// What bounds it is the host link.  Reads of 128-byte lines, 512 bytes a warp instruction, 150 to 250 KB in flight over
+// the machine, reach 51.2 GB/s on random 24 KB records where one contiguous copy of the same bytes reaches 55.1; more in
+// flight gives nothing.  Packing the records with the host's cores and copying the packed parts gives 39 to 48 depending
+// on the host (the packing reads and writes every byte in host memory beside the copy's own reads), and a copy call per
+// record 5.4.  A step of the 7B shape (145 MB of incoming rows): 3.16 ms packed and copied, 2.97 pulled.
+//
+// Two SMs are enough for that, with 1024 threads each and six loads in flight per lane (four: 3.00 ms; one SM: 4.4 ms;
+// four SMs: 2.97 as well).  The others are left to the resident MLP kernels, which are launched narrower while rows are on
+// their way (kPullReserve).  A kernel on all SMs, small enough to fit beside the resident blocks, was no faster, and the
+// resident kernels lost 7 % by giving up the registers.  A piece is 384 units of 16 bytes (two rounds of loads), taken
+// from the 128-byte line the record starts in, so that a warp's accesses are whole lines also for records that are not a
+// multiple of 128 bytes; the last piece takes what is left.
+// ---------------------------------------------------------------------------------------
+constexpr int kPullThreads = 1024;
+constexpr int kPullBlocks = 2;
+constexpr int kPullUnits = 384;
+
+struct PullArgs {
+  const char* store;        // device alias of the pinned store
+  const int32_t* ids;       // [L][C]
+  const int32_t* slots;     // [L][C]
+  const int32_t* counters;  // [L][NP_N_COUNTERS]
+  char* gate;               // first sparse layer of each row buffer
+  char* up;
+  char* downT;
+  int32_t* status;
+  size_t rec_bytes;
+  int l_begin, l_end, dense, D, M, C, Lp, check;
+};
+
+template <bool kInt8>
+__global__ void __launch_bounds__(kPullThreads) k_pull_rows(PullArgs a) {
+  constexpr int U = 6;  // loads a lane has in flight
+  const int lane = threadIdx.x & 31;
+  const int nw = gridDim.x * (kPullThreads / 32);
+  const int row_units = kInt8 ? a.D >> 4 : a.D >> 3;             // 16-byte units of a source row
+  const int pieces = max(1, (3 * row_units + kPullUnits / 2) / kPullUnits);  // per record
+  // the first piece of the layer that is this warp's: the deal goes on where it stopped in the layer before
+  int i = blockIdx.x * (kPullThreads / 32) + (threadIdx.x >> 5);
+  for (int l = a.l_begin; l < a.l_end; ++l) {
+    const int total = min(max(a.counters[(size_t)l * NP_N_COUNTERS + NP_CNT_DELTA], 0), a.C) * pieces;
+    const int32_t* ids = a.ids + (size_t)l * a.C;
+    const int32_t* slots = a.slots + (size_t)l * a.C;
+    int next_id = 0, next_slot = 0;
+    if (i < total) next_id = ids[i / pieces], next_slot = slots[i / pieces];
+    for (; i < total; i += nw) {
+      const int p = i % pieces;
+      const int id = next_id, slot = next_slot;
+      if (i + nw < total) next_id = ids[(i + nw) / pieces], next_slot = slots[(i + nw) / pieces];  // on their way beside the rows
+      if (a.check && (id < 0 || id >= a.M || slot < 0 || slot >= a.C)) {
+        if (lane == 0) atomicOr(a.status, id < 0 || id >= a.M ? kStatBadNeuron : kStatBadSlot);
+        continue;
+      }
+      const char* rec = a.store + ((size_t)(l % a.Lp) * a.M + id) * a.rec_bytes;
+      const size_t dst = ((size_t)(l - a.dense) * a.C + slot) * a.D * 2;
+      const int mis = (int)((reinterpret_cast<uintptr_t>(rec) >> 4) & 7);  // units between the line's start and the record
+      const int end = p + 1 < pieces ? (p + 1) * kPullUnits - mis : 3 * row_units;
+      float sc[3];
+      if (kInt8) {
+        const uint4 s4 = ldg_stream(rec + (size_t)3 * a.D);
+        sc[0] = __uint_as_float(s4.x), sc[1] = __uint_as_float(s4.y), sc[2] = __uint_as_float(s4.z);
+      }
+#pragma unroll 1
+      for (int v0 = p * kPullUnits - mis + lane; v0 < end; v0 += U * 32) {
+        uint4 x[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const int v = v0 + 32 * j;
+          if (v >= 0 && v < end) x[j] = ldg_stream(rec + (size_t)v * 16);
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          int v = v0 + 32 * j;
+          if (v >= 0 && v < end) {
+            char* row = a.gate;
+            float scale = kInt8 ? sc[0] : 0.f;
+            if (v >= row_units) {
+              v -= row_units;
+              row = a.up;
+              if (kInt8) scale = sc[1];
+              if (v >= row_units) {
+                v -= row_units;
+                row = a.downT;
+                if (kInt8) scale = sc[2];
+              }
+            }
+            if (kInt8) {
+              uint4* o = reinterpret_cast<uint4*>(row + dst) + 2 * v;
+              o[0] = make_uint4(dequant2(x[j].x, 0, scale), dequant2(x[j].x, 16, scale), dequant2(x[j].y, 0, scale), dequant2(x[j].y, 16, scale));
+              o[1] = make_uint4(dequant2(x[j].z, 0, scale), dequant2(x[j].z, 16, scale), dequant2(x[j].w, 0, scale), dequant2(x[j].w, 16, scale));
+            } else {
+              reinterpret_cast<uint4*>(row + dst)[v] = x[j];
+            }
+          }
+        }
+      }
+    }
+    i -= total;  // >= 0 here; what is left of the round belongs to the next layer
   }
-  if (src_is_store) {
-    k_deinterleave_scatter<true><<<blocks, kScatterThreads, 0, s>>>(
-        static_cast<const uint4*>(src), ids, slots, count_ptr, first, max_rows, static_cast<uint4*>(gate_l),
-        static_cast<uint4*>(up_l), static_cast<uint4*>(downT_l), row_chunks, d.M, d.C, status, check);
-  } else {
-    k_deinterleave_scatter<false><<<blocks, kScatterThreads, 0, s>>>(
-        static_cast<const uint4*>(src), ids, slots, count_ptr, first, max_rows, static_cast<uint4*>(gate_l),
-        static_cast<uint4*>(up_l), static_cast<uint4*>(downT_l), row_chunks, d.M, d.C, status, check);
-  }
+}
+
+cudaError_t launch_pull(const Dims& d, const Tables& t, const char* store_dev, void* gate, void* up, void* downT, int l_begin,
+                        int l_end, int check, cudaStream_t s) {
+  PullArgs a;
+  a.store = store_dev;
+  a.ids = t.delta_ids;
+  a.slots = t.delta_slots;
+  a.counters = t.counters;
+  a.gate = static_cast<char*>(gate);
+  a.up = static_cast<char*>(up);
+  a.downT = static_cast<char*>(downT);
+  a.status = t.status;
+  a.rec_bytes = d.rec_bytes;
+  a.l_begin = l_begin;
+  a.l_end = l_end;
+  a.dense = d.dense;
+  a.D = d.D;
+  a.M = d.M;
+  a.C = d.C;
+  a.Lp = d.Lp;
+  a.check = check;
+  if (d.rec_int8) k_pull_rows<true><<<kPullBlocks, kPullThreads, 0, s>>>(a);
+  else k_pull_rows<false><<<kPullBlocks, kPullThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
