@@ -17,9 +17,10 @@
 // range of its outputs, so of x it only ever needs slice q.
 //
 //   up     Eight consumer warps.  A tile is 8 gate and 8 up pieces (the 16 rows of an MMA, mma.sync m16n8k16, bf16 x
-//          bf16 -> fp32).  The K blocks are dealt to the warps (NSG = 2: four warps per group of eight sequences), and a
-//          warp keeps the B operand of its K blocks -- x as three truncated bf16 terms, exact to 2^-24 -- in registers
-//          for the whole layer: x costs no shared memory, which all goes to rows in flight.
+//          bf16 -> fp32).  The K blocks are dealt to the warps, and a warp keeps the B operand of its K blocks -- x as
+//          three truncated bf16 terms, exact to 2^-24 -- in registers for the whole layer: x costs no shared memory,
+//          which all goes to rows in flight, and an A fragment read from shared memory serves all sequences (a tile read
+//          once per group of eight sequences kept shared memory busy for two thirds of the MMAs' time).
 //   chunk  Sixteen rows (two up tiles, one down tile).  Two groups of exchange warps take the chunks in turn: they add
 //          the consumers' partial dot products, trade them with the other slices of the row group through (value, stamp)
 //          words in global memory (one store, polled by the readers: no fence, no counter), form the activations and
@@ -140,6 +141,20 @@ __device__ __forceinline__ void warp_wait(uint64_t* bar, uint32_t parity, volati
   if (lane == 0) wait_or_flag(bar, parity, ok, status);
   __syncwarp();
 }
+// Whether the phase of that parity is complete, without waiting.  The consumers ask early and look at the answer when they
+// need it: asked at the point of use, the answer's way back is idle time of the tensor pipe (a warp per scheduler computes
+// while the other one waits, and both wait for the same tile).
+__device__ __forceinline__ uint32_t mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(npp::smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok;
+}
 // one lane: until the counter at `p` has reached `target` (modulo 2^32)
 __device__ __forceinline__ void wait_count(const unsigned int* p, unsigned int target, volatile int* ok, int32_t* status) {
   if (!*ok) return;
@@ -158,7 +173,7 @@ template <int NSG>
 __device__ __forceinline__ void exchange_chunk(const KArgs& a, const float4* part, const float* ssq_part, uint16_t* hs, int t, int rows,
                                                int q, int r, unsigned int area, unsigned int stamp, uint64_t* part_empty, int lane,
                                                volatile int* ok) {
-  constexpr int NS = 8 * NSG, KW = kWarps / NSG, NT = kExchWarps * 32;
+  constexpr int NS = 8 * NSG, NT = kExchWarps * 32;
   constexpr int NPAIR = kChunk * NS / NT;  // pairs of a thread
   constexpr int PB = 2, PQ = 4;            // pairs and slices whose words are polled together
   const int seq = t & (NS - 1), row0 = t / NS;
@@ -167,14 +182,14 @@ __device__ __forceinline__ void exchange_chunk(const KArgs& a, const float4* par
   float g[NPAIR], u[NPAIR], ss = 0.f;
   const float2* p2 = reinterpret_cast<const float2*>(part);
 #pragma unroll
-  for (int k = 0; k < KW; ++k) ss += ssq_part[k * 16 + seq];
+  for (int k = 0; k < kWarps; ++k) ss += ssq_part[k * 16 + seq];
 #pragma unroll
   for (int i = 0; i < NPAIR; ++i) {
     const int row = row0 + i * row_step;
     g[i] = u[i] = 0.f;
-    const float2* p = p2 + ((size_t)((row >> 3) * kWarps + (seq >> 3) * KW) * 32 + (row & 7) * 4 + ((seq & 7) >> 1)) * 2 + (seq & 1);
+    const float2* p = p2 + ((size_t)((row >> 3) * NSG + (seq >> 3)) * kWarps * 32 + (row & 7) * 4 + ((seq & 7) >> 1)) * 2 + (seq & 1);
 #pragma unroll
-    for (int k = 0; k < KW; ++k) {
+    for (int k = 0; k < kWarps; ++k) {
       const float2 v = p[k * 64];
       g[i] += v.x;
       u[i] += v.y;
@@ -272,6 +287,76 @@ __device__ __forceinline__ void exchange_chunk(const KArgs& a, const float4* par
   }
 }
 
+// acc += h . down of one chunk over PN pairs of 8-column tiles: pairs pair0, pair0 + kWarps, ... of the slice.  `bp`: the
+// lane's ldmatrix address of the tile's first pair.  Pairs past the slice's end are computed and never looked at.
+template <int NSG, int PN>
+__device__ __forceinline__ void down_mma(float (&acc)[2 * PN][4], const uint16_t* hc, uint32_t bp, int pair0, int nk, int lane) {
+  constexpr int HT = NSG == 2 ? 3 : 2;
+  uint32_t hf[HT][4];
+#pragma unroll
+  for (int e = 0; e < HT; ++e) {
+    const uint4 v = *reinterpret_cast<const uint4*>(hc + ((size_t)e * 32 + lane) * 8);
+    hf[e][0] = v.x;
+    hf[e][1] = NSG == 1 && e == 1 ? 0u : v.y;
+    hf[e][2] = v.z;
+    hf[e][3] = NSG == 1 && e == 1 ? 0u : v.w;
+  }
+#pragma unroll
+  for (int p0 = 0; p0 < PN; p0 += 4) {
+    uint32_t bf[4][4];
+#pragma unroll
+    for (int p = 0; p < 4 && p0 + p < PN; ++p) {
+      const int pair = pair0 + (p0 + p) * kWarps;
+      ldmatrix_x4_trans(bf[p], bp + (pair < nk ? (uint32_t)pair * 32u : 0u));
+    }
+#pragma unroll
+    for (int e = 0; e < HT; ++e)
+#pragma unroll
+      for (int p = 0; p < 4 && p0 + p < PN; ++p) {
+        mma_bf16(acc[2 * (p0 + p)], hf[e], bf[p][0], bf[p][1]);
+        mma_bf16(acc[2 * (p0 + p) + 1], hf[e], bf[p][2], bf[p][3]);
+      }
+  }
+}
+
+// x += acc for the same pairs
+template <int NSG, int PN>
+__device__ __forceinline__ void down_reds(const float (&acc)[2 * PN][4], float* xs, int pair0, int nk, int B, int lane) {
+  constexpr int NS = 8 * NSG;
+  const int g8 = lane >> 2, t4 = lane & 3;
+  const bool odd = t4 & 1;
+#pragma unroll
+  for (int p = 0; p < PN; ++p) {
+    const int pair = pair0 + p * kWarps;
+    if (pair >= nk) break;
+    float* tile = xs + (size_t)pair * 2 * NS * 8;
+    if (NSG == 2) {
+      // rows g8 / g8 + 8 = sequences; even lanes end up with four columns of sequence g8, odd lanes of 8 + g8
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float* v = acc[2 * p + j];
+        const float ra = __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[2], 1), rb = __shfl_xor_sync(0xffffffffu, odd ? v[1] : v[3], 1);
+        const int seq = odd ? 8 + g8 : g8;
+        float* dst = tile + (size_t)j * NS * 8 + seq * 8 + (t4 >> 1) * 4;
+        if (seq < B) {
+          if (odd) red_add_v4(dst, ra, rb, v[2], v[3]);
+          else red_add_v4(dst, v[0], v[1], ra, rb);
+        }
+      }
+    } else {
+      // rows g8 and g8 + 8 belong to one sequence; even lanes take the pair's first tile, odd lanes its second
+      const float a0 = acc[2 * p][0] + acc[2 * p][2], a1 = acc[2 * p][1] + acc[2 * p][3];
+      const float b0 = acc[2 * p + 1][0] + acc[2 * p + 1][2], b1 = acc[2 * p + 1][1] + acc[2 * p + 1][3];
+      const float ra = __shfl_xor_sync(0xffffffffu, odd ? a0 : b0, 1), rb = __shfl_xor_sync(0xffffffffu, odd ? a1 : b1, 1);
+      float* dst = tile + (size_t)(odd ? 1 : 0) * NS * 8 + g8 * 8 + (t4 >> 1) * 4;
+      if (g8 < B) {
+        if (odd) red_add_v4(dst, ra, rb, b0, b1);
+        else red_add_v4(dst, a0, a1, ra, rb);
+      }
+    }
+  }
+}
+
 // NSG: groups of eight sequences.  NP: pairs of 8-column output tiles per warp (= 16-wide K blocks per eight warps).
 template <int NSG, int NP>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
@@ -284,7 +369,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
   __shared__ unsigned int s_act[kExchGroups * kExchWarps];  // chunks each exchange warp has finished, ever growing
   __shared__ int lay_rb[kMaxLayers], lay_n[kMaxLayers], lay_pre[kMaxLayers + 1];
 
-  constexpr int NS = 8 * NSG, KW = kWarps / NSG, KPW = NP * NSG;
+  constexpr int NS = 8 * NSG;
+  constexpr int kPart = 2 * NSG * kWarps * 32;          // float4 of a chunk's partial dot products
   constexpr int HT = NSG == 2 ? 3 : 2;                  // A tiles per chunk
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int Q = a.Q, R = gridDim.x / Q;
@@ -295,8 +381,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
   const int nl = a.l_end - a.l_begin;
   const int max_chunks = (a.max_rows + kChunk - 1) / kChunk;
   // dynamic shared memory: ring | partial dot products, two chunks | activations of a layer | slots
-  float4* part = reinterpret_cast<float4*>(csm + (size_t)a.ng * a.slot_bytes);           // [2][2 tiles][8 warps][32]
-  uint16_t* hs = reinterpret_cast<uint16_t*>(part + 2 * 2 * kWarps * 32);                // [max_chunks][HT][32][4] words
+  float4* part = reinterpret_cast<float4*>(csm + (size_t)a.ng * a.slot_bytes);           // [2][2 tiles][NSG][8 warps][32]
+  uint16_t* hs = reinterpret_cast<uint16_t*>(part + 2 * kPart);                // [max_chunks][HT][32][4] words
   uint16_t* slot_cache = hs + (size_t)max_chunks * HT * 256;
   volatile int* ok = &s_ok;
   unsigned int* cnt_read = a.cnt + (size_t)q * kCntStride;
@@ -409,7 +495,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           const unsigned int buf = n & 1u, use = n >> 1, turn = n / kExchGroups;
           warp_wait(&part_full[buf], use & 1u, ok, a.status, lane);
           const unsigned int area = (unsigned int)e * 2u + (turn & 1u), stamp = a.seq_base + 1u + n;
-          const float4* pt = part + (size_t)buf * (2 * kWarps * 32);
+          const float4* pt = part + (size_t)buf * kPart;
           uint16_t* hc = hs + (size_t)c * HT * 256;
           const int rows = min(kChunk, nrows - c * kChunk);
           exchange_chunk<NSG>(a, pt, ssq_part, hc, t, rows, q, r, area, stamp, &part_empty[buf], lane, ok);
@@ -428,7 +514,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
   // =========================== consumer warps ===========================
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kConsumerRegs));
   const int g8 = lane >> 2, t4 = lane & 3;
-  const int sg = NSG == 2 ? wid / KW : 0, kw = wid % KW;  // this warp's sequences and K blocks kw, kw + KW, ...
   const uint32_t ring = npp::smem_addr(csm);
   const uint32_t up_off = (uint32_t)(lane & 15) * pstride + (uint32_t)(lane >> 4) * 16u;
   // transposed loads: matrices 0 / 1 = records 0-7 / 8-15 of an 8-column tile, 2 / 3 = the same of the next tile
@@ -446,162 +531,136 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
 
   for (int li = 0; li < nl; ++li) {
     const int nrows = lay_n[li], n_up = (nrows + 7) >> 3, nch = (nrows + kChunk - 1) / kChunk;
-    // ---- x_l: this warp's K blocks and sequences, straight into B fragments ----
-    uint32_t xb[KPW][3][2];
+    // ---- x_l: this warp's K blocks wid, wid + 8, ..., straight into B fragments ----
+    uint32_t xb[NP][NSG][3][2];
     {
       warp_wait(&x_ready, (uint32_t)li & 1u, ok, a.status, lane);
-      float2 lo[KPW], hi[KPW];
-      const float* xp = xs + (size_t)(sg * 8 + g8) * 8 + 2 * t4;
+      float2 lo[NP][NSG], hi[NP][NSG];
+      const float* xp = xs + (size_t)g8 * 8 + 2 * t4;
 #pragma unroll
-      for (int i = 0; i < KPW; ++i) {
-        const int kb = kw + i * KW;
-        lo[i] = hi[i] = make_float2(0.f, 0.f);
-        if (kb < nk) {
-          lo[i] = __ldcg(reinterpret_cast<const float2*>(xp + (size_t)kb * 2 * NS * 8));
-          hi[i] = __ldcg(reinterpret_cast<const float2*>(xp + (size_t)(kb * 2 + 1) * NS * 8));
+      for (int i = 0; i < NP; ++i) {
+        const int kb = wid + i * kWarps;
+#pragma unroll
+        for (int sg = 0; sg < NSG; ++sg) {
+          lo[i][sg] = hi[i][sg] = make_float2(0.f, 0.f);
+          if (kb < nk) {
+            lo[i][sg] = __ldcg(reinterpret_cast<const float2*>(xp + ((size_t)kb * 2 * NS + sg * 8) * 8));
+            hi[i][sg] = __ldcg(reinterpret_cast<const float2*>(xp + ((size_t)(kb * 2 + 1) * NS + sg * 8) * 8));
+          }
         }
       }
-      float ss = 0.f;
+      float ss[NSG];
 #pragma unroll
-      for (int i = 0; i < KPW; ++i) {
-        ss += lo[i].x * lo[i].x + lo[i].y * lo[i].y + hi[i].x * hi[i].x + hi[i].y * hi[i].y;
-        uint32_t s0[3], s1[3], s2[3], s3[3];
-        split3(lo[i].x, s0);
-        split3(lo[i].y, s1);
-        split3(hi[i].x, s2);
-        split3(hi[i].y, s3);
+      for (int sg = 0; sg < NSG; ++sg) {
+        ss[sg] = 0.f;
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-          xb[i][e][0] = pack2(s0[e], s1[e]);
-          xb[i][e][1] = pack2(s2[e], s3[e]);
+        for (int i = 0; i < NP; ++i) {
+          const float2 l2 = lo[i][sg], h2 = hi[i][sg];
+          ss[sg] += l2.x * l2.x + l2.y * l2.y + h2.x * h2.x + h2.y * h2.y;
+          uint32_t s0[3], s1[3], s2[3], s3[3];
+          split3(l2.x, s0);
+          split3(l2.y, s1);
+          split3(h2.x, s2);
+          split3(h2.y, s3);
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            xb[i][sg][e][0] = pack2(s0[e], s1[e]);
+            xb[i][sg][e][1] = pack2(s2[e], s3[e]);
+          }
         }
+        ss[sg] += __shfl_xor_sync(0xffffffffu, ss[sg], 1);
+        ss[sg] += __shfl_xor_sync(0xffffffffu, ss[sg], 2);
+        if (t4 == 0) ssq_part[wid * 16 + sg * 8 + g8] = ss[sg];
       }
-      ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-      ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-      if (t4 == 0) ssq_part[kw * 16 + sg * 8 + g8] = ss;
       __syncwarp();
       if (lane == 0) npp::mbar_arrive(&x_read);
     }
     // ---- up: partial dot products of the slice, a tile of 8 records at a time ----
+    uint32_t rdy = mbar_test(&full_bar[slot], par);
     for (int t = 0; t < n_up; ++t) {
       const unsigned int n = nx + (unsigned int)(t >> 1), buf = n & 1u;
-      if (!(t & 1) && n >= 2) warp_wait(&part_empty[buf], ((n >> 1) - 1u) & 1u, ok, a.status, lane);
-      warp_wait(&full_bar[slot], par, ok, a.status, lane);
+      if (!__all_sync(0xffffffffu, rdy)) warp_wait(&full_bar[slot], par, ok, a.status, lane);
       const uint32_t ap = ring + (uint32_t)slot * a.slot_bytes + up_off;
-      float c[3][4];
+      uint64_t* const done_bar = &empty_bar[slot];
+      next_slot();
+      rdy = mbar_test(&full_bar[slot], par);  // the next tile's
+      const uint32_t room = (t & 1) || n < 2 ? 1u : mbar_test(&part_empty[buf], ((n >> 1) - 1u) & 1u);
+      float c[NSG][3][4];
 #pragma unroll
-      for (int e = 0; e < 3; ++e) c[e][0] = c[e][1] = c[e][2] = c[e][3] = 0.f;
+      for (int sg = 0; sg < NSG; ++sg)
 #pragma unroll
-      for (int i0 = 0; i0 < KPW; i0 += 4) {
+        for (int e = 0; e < 3; ++e) c[sg][e][0] = c[sg][e][1] = c[sg][e][2] = c[sg][e][3] = 0.f;
+#pragma unroll
+      for (int i0 = 0; i0 < NP; i0 += 4) {
         uint32_t af[4][4];
 #pragma unroll
-        for (int i = 0; i < 4 && i0 + i < KPW; ++i) {
-          const int kb = kw + (i0 + i) * KW;  // past the slice's end: x is zero, any of the row's bytes do
+        for (int i = 0; i < 4 && i0 + i < NP; ++i) {
+          const int kb = wid + (i0 + i) * kWarps;  // past the slice's end: x is zero, any of the row's bytes do
           ldmatrix_x4(af[i], ap + (kb < nk ? (uint32_t)kb * 32u : 0u));
         }
 #pragma unroll
-        for (int i = 0; i < 4 && i0 + i < KPW; ++i)
+        for (int i = 0; i < 4 && i0 + i < NP; ++i)
 #pragma unroll
-          for (int e = 0; e < 3; ++e) mma_bf16(c[e], af[i], xb[i0 + i][e][0], xb[i0 + i][e][1]);
+          for (int e = 0; e < 3; ++e)
+#pragma unroll
+            for (int sg = 0; sg < NSG; ++sg) mma_bf16(c[sg][e], af[i], xb[i0 + i][sg][e][0], xb[i0 + i][sg][e][1]);
       }
       __syncwarp();
-      if (lane == 0) npp::mbar_arrive(&empty_bar[slot]);
-      next_slot();
-      // rows g8 (gate of record g8) and g8 + 8 (its up), sequences 2 t4, 2 t4 + 1
-      part[(size_t)(buf * 2 + (t & 1)) * (kWarps * 32) + wid * 32 + lane] =
-          make_float4(c[0][0] + c[1][0] + c[2][0], c[0][2] + c[1][2] + c[2][2], c[0][1] + c[1][1] + c[2][1], c[0][3] + c[1][3] + c[2][3]);
+      if (lane == 0) npp::mbar_arrive(done_bar);
+      if (!__all_sync(0xffffffffu, room)) warp_wait(&part_empty[buf], ((n >> 1) - 1u) & 1u, ok, a.status, lane);
+      // rows g8 (gate of record g8) and g8 + 8 (its up), sequences 8 sg + 2 t4, + 1
+#pragma unroll
+      for (int sg = 0; sg < NSG; ++sg)
+        part[(size_t)buf * kPart + (size_t)(((t & 1) * NSG + sg) * kWarps + wid) * 32 + lane] =
+            make_float4(c[sg][0][0] + c[sg][1][0] + c[sg][2][0], c[sg][0][2] + c[sg][1][2] + c[sg][2][2],
+                        c[sg][0][1] + c[sg][1][1] + c[sg][2][1], c[sg][0][3] + c[sg][1][3] + c[sg][2][3]);
       if ((t & 1) || t == n_up - 1) {
         __syncwarp();
         if (lane == 0) npp::mbar_arrive(&part_full[buf]);
       }
     }
     // ---- down: y[sequences][columns] += h . down, this warp's 16-column pairs wid, wid + 8, ... ----
-    float acc[2 * NP][4];
+    // A chunk is ready when both exchange warps of its group have left its activations and its rows have landed.
+    auto acts_there = [&](unsigned int n) {
+      const volatile unsigned int* done = &s_act[(n % kExchGroups) * kExchWarps];
+      const unsigned int target = n / kExchGroups + 1u;
+      bool there = true;
 #pragma unroll
-    for (int j = 0; j < 2 * NP; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-    for (int c = 0; c < nch; ++c) {
+      for (int w = 0; w < kExchWarps; ++w) there = there && (int)(done[w] - target) >= 0;  // one may be a chunk ahead
+      return there;
+    };
+    auto chunk_wait = [&](int c, int sl, uint32_t pr) {
       const unsigned int n = nx + (unsigned int)c;
-      if (lane == 0) {
-        const unsigned int target = n / kExchGroups + 1u;
-        for (int w = 0; w < kExchWarps; ++w) {  // a warp of the group may be a chunk ahead of the other
-          const volatile unsigned int* done = &s_act[(n % kExchGroups) * kExchWarps + w];
-          bool there = (int)(*done - target) >= 0;
-          for (uint32_t spin = 0; spin < npp::kSpinLimit * 16u && !there && *ok; ++spin) there = (int)(*done - target) >= 0;
+      if (!__all_sync(0xffffffffu, acts_there(n))) {
+        if (lane == 0) {
+          bool there = false;
+          for (uint32_t spin = 0; spin < npp::kSpinLimit * 16u && !there && *ok; ++spin) there = acts_there(n);
           if (!there && *ok) {
             *ok = 0;
             atomicOr(a.status, npp::kStatTimeout);
           }
         }
-        __threadfence_block();
-        wait_or_flag(&full_bar[slot], par, ok, a.status);
+        __syncwarp();
       }
-      __syncwarp();
-      uint32_t hf[HT][4];
+      __threadfence_block();
+      if (!__all_sync(0xffffffffu, mbar_test(&full_bar[sl], pr))) warp_wait(&full_bar[sl], pr, ok, a.status, lane);
+    };
+    {
+      float acc[2 * NP][4];
 #pragma unroll
-      for (int e = 0; e < HT; ++e) {
-        const uint4 v = *reinterpret_cast<const uint4*>(hs + ((size_t)(c * HT + e) * 32 + lane) * 8);
-        hf[e][0] = v.x;
-        hf[e][1] = NSG == 1 && e == 1 ? 0u : v.y;
-        hf[e][2] = v.z;
-        hf[e][3] = NSG == 1 && e == 1 ? 0u : v.w;
+      for (int j = 0; j < 2 * NP; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+      for (int c = 0; c < nch; ++c) {
+        chunk_wait(c, slot, par);
+        down_mma<NSG, NP>(acc, hs + (size_t)c * HT * 256, ring + (uint32_t)slot * a.slot_bytes + dn_off, wid, nk, lane);
+        __syncwarp();
+        if (lane == 0) npp::mbar_arrive(&empty_bar[slot]);
+        next_slot();
       }
-      const uint32_t bp = ring + (uint32_t)slot * a.slot_bytes + dn_off;
-#pragma unroll
-      for (int p0 = 0; p0 < NP; p0 += 4) {
-        uint32_t bf[4][4];
-#pragma unroll
-        for (int p = 0; p < 4 && p0 + p < NP; ++p) {
-          const int pair = wid + (p0 + p) * kWarps;  // past the slice's end: computed and never looked at
-          ldmatrix_x4_trans(bf[p], bp + (pair < nk ? (uint32_t)pair * 32u : 0u));
-        }
-#pragma unroll
-        for (int e = 0; e < HT; ++e)
-#pragma unroll
-          for (int p = 0; p < 4 && p0 + p < NP; ++p) {
-            mma_bf16(acc[2 * (p0 + p)], hf[e], bf[p][0], bf[p][1]);
-            mma_bf16(acc[2 * (p0 + p) + 1], hf[e], bf[p][2], bf[p][3]);
-          }
-      }
-      __syncwarp();
-      if (lane == 0) npp::mbar_arrive(&empty_bar[slot]);
-      next_slot();
+      // x += y in place, once every block of the slice has read x_l
+      warp_wait(&may_add, (uint32_t)li & 1u, ok, a.status, lane);
+      if (nrows > 0) down_reds<NSG, NP>(acc, xs, wid, nk, a.B, lane);
     }
     nx += (unsigned int)nch;
-    // ---- x += y in place, once every block of the slice has read x_l ----
-    warp_wait(&may_add, (uint32_t)li & 1u, ok, a.status, lane);
-    if (nrows > 0) {
-      const bool odd = t4 & 1;
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const int pair = wid + p * kWarps;
-        if (pair >= nk) break;
-        float* tile = xs + (size_t)pair * 2 * NS * 8;
-        if (NSG == 2) {
-          // rows g8 / g8 + 8 = sequences; even lanes end up with four columns of sequence g8, odd lanes of 8 + g8
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const float* v = acc[2 * p + j];
-            const float ra = __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[2], 1), rb = __shfl_xor_sync(0xffffffffu, odd ? v[1] : v[3], 1);
-            const int seq = odd ? 8 + g8 : g8;
-            float* dst = tile + (size_t)j * NS * 8 + seq * 8 + (t4 >> 1) * 4;
-            if (seq < a.B) {
-              if (odd) red_add_v4(dst, ra, rb, v[2], v[3]);
-              else red_add_v4(dst, v[0], v[1], ra, rb);
-            }
-          }
-        } else {
-          // rows g8 and g8 + 8 belong to one sequence; even lanes take the pair's first tile, odd lanes its second
-          const float a0 = acc[2 * p][0] + acc[2 * p][2], a1 = acc[2 * p][1] + acc[2 * p][3];
-          const float b0 = acc[2 * p + 1][0] + acc[2 * p + 1][2], b1 = acc[2 * p + 1][1] + acc[2 * p + 1][3];
-          const float ra = __shfl_xor_sync(0xffffffffu, odd ? a0 : b0, 1), rb = __shfl_xor_sync(0xffffffffu, odd ? a1 : b1, 1);
-          float* dst = tile + (size_t)(odd ? 1 : 0) * NS * 8 + g8 * 8 + (t4 >> 1) * 4;
-          if (g8 < a.B) {
-            if (odd) red_add_v4(dst, ra, rb, b0, b1);
-            else red_add_v4(dst, a0, a1, ra, rb);
-          }
-        }
-      }
-    }
     __syncwarp();
     if (lane == 0) {
       __threadfence();  // the warp's adds, then its arrival
@@ -652,7 +711,7 @@ bool make_plan(const Dims& d, int rows, bool dense, int nsg, int sm_count, Plan*
   const int max_chunks = (p->max_rows + kChunk - 1) / kChunk;
   p->slot_bytes = 16u * (uint32_t)(nk * 32 + kPad);
   const size_t budget = 227 * 1024 - 2560;  // static shared memory of the kernel
-  const size_t fixed = 2 * 2 * kWarps * 32 * 16 + (size_t)max_chunks * (nsg == 2 ? 3 : 2) * 512 + 256;
+  const size_t fixed = (size_t)2 * 2 * nsg * kWarps * 32 * 16 + (size_t)max_chunks * (nsg == 2 ? 3 : 2) * 512 + 256;
   const size_t cache_min = dense ? 0 : 2 * (size_t)p->max_rows * 8;
   if (fixed + cache_min + 3 * (size_t)p->slot_bytes > budget) return false;
   p->ng = (int)std::min<size_t>(kMaxSlots, (budget - fixed - cache_min) / p->slot_bytes);
