@@ -793,7 +793,7 @@ int np_predict(np_ctx* ctx, const void* x_bf16, int32_t B, float* logits_out, ui
       NP_LAUNCH(ctx, launch_pred_l2(ds, static_cast<const char*>(ctx->bufs.w2) + skip_rows * d.H * 2, ctx->ws.hidden,
                                   B, logits, ctx->t.status, s, ctx->sm_count));
     }
-    NP_LAUNCH(ctx, launch_topk(ds, logits, B, pred, pred2, l2_tc, s));
+    NP_LAUNCH(ctx, launch_topk(ds, logits, B, pred, pred2, l2_tc, s, ctx->sm_count));
   }
   if (d.dense > 0) {
     const size_t nbm = (size_t)d.dense * d.W * 4;
@@ -814,7 +814,7 @@ int np_topk(np_ctx* ctx, const float* logits, int32_t B, uint32_t* bitmap_out, v
   ds.L = d.L - skip_layers;
   if (ds.L > 0)
     NP_LAUNCH(ctx, launch_topk(ds, logits + (size_t)skip_layers * d.M, B, bitmap_out + (size_t)skip_layers * d.W,
-                               nullptr, false, as_stream(stream)));
+                               nullptr, false, as_stream(stream), ctx->sm_count));
   if (d.dense > 0) NP_CUDA(ctx, cudaMemsetAsync(bitmap_out, 0, (size_t)d.dense * d.W * 4, as_stream(stream)));
   return NP_OK;
 }
@@ -1687,7 +1687,7 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
     ds.k = std::min(d.M, d.k + ctx->cfg.spec_rows);
     if (ds.L > 0)
       NP_LAUNCH(ctx, launch_topk(ds, ctx->ws.logits + (size_t)skip_layers * d.M, B,
-                                 ctx->t.spec_cand + (size_t)skip_layers * d.W, nullptr, false, s));
+                                 ctx->t.spec_cand + (size_t)skip_layers * d.W, nullptr, false, s, ctx->sm_count));
     if (d.dense > 0) NP_CUDA(ctx, cudaMemsetAsync(ctx->t.spec_cand, 0, (size_t)d.dense * d.W * 4, s));
     rc = np_speculate(ctx, ctx->t.spec_cand, ctx->cfg.spec_rows, stream);
     if (rc < 0) return rc;

@@ -101,7 +101,7 @@ cudaError_t launch_pred_l2_tc(const Dims& d, const PredTcState& st, float* hidde
 // bitmap2 (may be NULL) receives the same words; `cleared`: an earlier kernel of the stream has zeroed both (a batch's
 // selections are ORed into them)
 cudaError_t launch_topk(const Dims& d, const float* logits, int B, uint32_t* bitmap, uint32_t* bitmap2, bool cleared,
-                        cudaStream_t s);
+                        cudaStream_t s, int sm_count);
 
 // Centroid heads -> arg-max -> bank lookup -> gate AND up (np_centroid.cu).
 cudaError_t launch_centroid_select(const Dims& d, const float* logits, int B, int K, const uint32_t* bank,

@@ -2,9 +2,9 @@
 // (The paper turns predictor outputs into one active set per layer, Section 3.4;
 // here the set is the k highest-scoring neurons, the K_max budget of Section 4.1.)
 //
-// One block of 1024 threads per (layer, sequence).  A layer is only 44 KB of logits: the
+// One block of 1024 (or 512) threads per (layer, sequence).  A layer is only 44 KB of logits: the
 // kernel is a chain of block-wide steps on one SM, and what it costs is the instructions of
-// those steps.  Every thread keeps its logits in registers, index tid + 1024 j, so that the 32
+// those steps.  Every thread keeps its logits in registers, index tid + threads * j, so that the 32
 // lanes of a warp hold the 32 neurons of one bitmap word and a ballot is a word.
 //
 // Fast path (finite logits that are not all equal): ONE histogram pass over 2048 bins that
@@ -26,7 +26,6 @@
 namespace npi {
 using namespace npd;
 
-constexpr int kTopkThreads = 1024;
 constexpr int kTopkHist = 8192;   // ints: 32 warps x 256 bins in the first radix pass, 4096 bins after; 2048 linear bins + candidate list
 constexpr int kLinBins = 2048;
 constexpr int kMaxCand = 1024;    // keys of the deciding bin that are ranked directly
@@ -42,12 +41,41 @@ extern "C" int np_debug_tk(void* out) { return (int)cudaMemcpyFromSymbol(out, np
 // bit pattern of an fp32 value -> order-preserving uint32 (larger float, larger key; +0 above -0)
 __device__ __forceinline__ uint32_t order_key(uint32_t b) { return (b & 0x80000000u) ? ~b : (b | 0x80000000u); }
 
-// KPT: keys per thread, ceil(M / 1024)
-template <int KPT>
-__global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__ logits,  // [B][L][M]
+// Inclusive scan of one int per thread in thread order over a block of T threads; wsum: 33 ints.  Two block-wide barriers; a
+// caller that scans again puts one between the calls.
+template <int T>
+__device__ __forceinline__ int block_inclusive_scan(int v, int* wsum, int lane, int wid) {
+  if (T == 1024) return block_inclusive_scan_1024(v, wsum, lane, wid);
+  constexpr int NW = T / 32;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += t;
+  }
+  if (lane == 31) wsum[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    const int ws = lane < NW ? wsum[lane] : 0;
+    int winc = ws;
+#pragma unroll
+    for (int o = 1; o < NW; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, winc, o);
+      if (lane >= o) winc += t;
+    }
+    if (lane < NW) wsum[lane] = winc - ws;
+  }
+  __syncthreads();
+  return wsum[wid] + inc;
+}
+
+// T: threads (512 or 1024).  KPT: keys per thread, ceil(M / T)
+template <int T, int KPT>
+__global__ void __launch_bounds__(T, 1024 / T) k_topk(const float* __restrict__ logits,  // [B][L][M]
                                                        uint32_t* __restrict__ bitmap,     // [L][W]
                                                        uint32_t* __restrict__ bitmap2,    // a second copy, or NULL
                                                        int L, int M, int k, int use_atomic) {
+  constexpr int NW = T / 32;
   extern __shared__ __align__(16) int wsm[];  // [W] per word: selected keys of the deciding bin / count of threshold-equal keys
   __shared__ __align__(16) int hist[kTopkHist];
   __shared__ int wsum[33];
@@ -80,11 +108,11 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   TK(1);
 
   if (k <= 0) {  // nothing selected
-    for (int w = tid; w < W; w += kTopkThreads) put(w, 0u);
+    for (int w = tid; w < W; w += T) put(w, 0u);
     return;
   }
   if (k >= M) {
-    for (int w = tid; w < W; w += kTopkThreads) put(w, 0xffffffffu);
+    for (int w = tid; w < W; w += T) put(w, 0xffffffffu);
     return;
   }
 
@@ -96,20 +124,20 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   const uint32_t* zbits = reinterpret_cast<const uint32_t*>(z);
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
-    const int i = tid + kTopkThreads * j;
+    const int i = tid + T * j;
     zb[j] = i < M ? zbits[i] : 0u;  // entries past the layer's end are never counted (every use tests the index)
   }
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
-    if (tid + kTopkThreads * j < M) {
+    if (tid + T * j < M) {
       bad |= (zb[j] & 0x7f800000u) == 0x7f800000u;  // infinity or NaN
       lo = fminf(lo, __uint_as_float(zb[j]));
       hi = fmaxf(hi, __uint_as_float(zb[j]));
     }
   }
-  hist[tid] = 0;
-  hist[tid + kTopkThreads] = 0;
-  for (int w = tid; w < W; w += kTopkThreads) wsm[w] = 0;
+#pragma unroll
+  for (int i = 0; i < kLinBins / T; ++i) hist[tid + T * i] = 0;
+  for (int w = tid; w < W; w += T) wsm[w] = 0;
   if (tid == 0) s_ncand = 0;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -122,8 +150,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   }
   TK(2);
   const int any_bad = __syncthreads_or(bad);
-  lo = wlo[lane];
-  hi = whi[lane];
+  lo = wlo[lane & (NW - 1)];
+  hi = whi[lane & (NW - 1)];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -139,19 +167,31 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
     auto bin_of = [&](float v) { return min(kLinBins - 1, (int)((v - lo) * scale)); };
 #pragma unroll
     for (int j = 0; j < KPT; ++j)
-      if (tid + kTopkThreads * j < M) atomicAdd(&hist[bin_of(__uint_as_float(zb[j]))], 1);
+      if (tid + T * j < M) atomicAdd(&hist[bin_of(__uint_as_float(zb[j]))], 1);
     __syncthreads();
     TK(4);
-    // the bin of the k-th largest key: thread t takes the two highest bins not taken by the threads below it
-    const int top = kLinBins - 1 - 2 * tid;
-    const int c_hi = hist[top], c_lo = hist[top - 1];
-    const int mine = c_hi + c_lo;
-    const int above = block_inclusive_scan_1024(mine, wsum, lane, wid) - mine;  // keys in higher bins
+    // the bin of the k-th largest key: thread t takes the highest bins not taken by the threads below it
+    constexpr int BPT = kLinBins / T;
+    const int top = kLinBins - 1 - BPT * tid;
+    int c[BPT], mine = 0;
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) mine += c[i] = hist[top - i];
+    const int above = block_inclusive_scan<T>(mine, wsum, lane, wid) - mine;  // keys in higher bins
     if (above < k && k <= above + mine) {  // exactly one thread
-      const bool first = k <= above + c_hi;
-      s_bin = first ? top : top - 1;
-      s_remaining = k - (first ? above : above + c_hi);
-      s_bin_count = first ? c_hi : c_lo;
+      int acc = above, i = 0;
+#pragma unroll
+      for (int q = 0; q < BPT - 1; ++q) {
+        if (i == q && k > acc + c[q]) {
+          acc += c[q];
+          i = q + 1;
+        }
+      }
+      int cnt = c[0];
+#pragma unroll
+      for (int q = 1; q < BPT; ++q) cnt = i == q ? c[q] : cnt;
+      s_bin = top - i;
+      s_remaining = k - acc;
+      s_bin_count = cnt;
     }
     __syncthreads();
     TK(5);
@@ -162,8 +202,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
       // one pass: the words of the keys above the bin go out, the keys inside it are listed
 #pragma unroll
       for (int j = 0; j < KPT; ++j) {
-        const int i = tid + kTopkThreads * j;
-        const int w = wid + 32 * j;  // the word of neurons 32 w .. 32 w + 31: this warp's logits of round j
+        const int i = tid + T * j;
+        const int w = wid + NW * j;  // the word of neurons 32 w .. 32 w + 31: this warp's logits of round j
         const int bn = i < M ? bin_of(__uint_as_float(zb[j])) : -1;
         const uint32_t gt = __ballot_sync(0xffffffffu, bn > bstar);
         if (lane == 0 && w < W) put(w, gt);
@@ -175,9 +215,9 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
       }
       __syncthreads();  // the list is complete; the words stored above are ordered before the bits added below
       TK(6);
-      if (tid < ncand) {  // rank among the keys of the bin: larger key first, then lower index
-        const uint32_t mk = ckey[tid];
-        const int mi = cidx[tid];
+      for (int t = tid; t < ncand; t += T) {  // rank among the keys of the bin: larger key first, then lower index
+        const uint32_t mk = ckey[t];
+        const int mi = cidx[t];
         int rank = 0;
         for (int q = 0; q < ncand; ++q) {
           const uint32_t qk = ckey[q];
@@ -192,7 +232,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
       return;
     }
     __syncthreads();  // heavy ties: the general path reuses the histogram and the per-word array
-    for (int w = tid; w < W; w += kTopkThreads) wsm[w] = 0;
+    for (int w = tid; w < W; w += T) wsm[w] = 0;
   }
 
   // ---- general path: radix select on the keys --------------------------------------------
@@ -208,8 +248,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
     // pass 0: one histogram of 256 bins per warp (8192 ints); passes 1 and 2: one of 4096 bins
     int4* h4 = reinterpret_cast<int4*>(hist);
     __syncthreads();
-    h4[tid] = make_int4(0, 0, 0, 0);
-    if (pass == 0) h4[tid + kTopkThreads] = make_int4(0, 0, 0, 0);
+    const int nz = (pass == 0 ? NW * 256 : 4096) / 4;
+    for (int i = tid; i < nz; i += T) h4[i] = make_int4(0, 0, 0, 0);
     __syncthreads();
     const uint32_t prefix = s_prefix;
     const int remaining = s_remaining;
@@ -217,7 +257,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
       const uint32_t key = order_key(zb[j]);
-      const bool in = tid + kTopkThreads * j < M && (key & mask) == prefix;
+      const bool in = tid + T * j < M && (key & mask) == prefix;
       // lanes with the same digit add once
       const uint32_t d = in ? (key >> shift) & dmask : 0xffffffffu;
       const uint32_t peers = __match_any_sync(0xffffffffu, d);
@@ -225,28 +265,30 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
     }
     __syncthreads();
     // the bin of the remaining-th largest key: thread t takes the highest bins not taken by the threads below it
-    int c[4] = {0, 0, 0, 0};
+    constexpr int BPP = 4096 / T;
+    int c[BPP];
+#pragma unroll
+    for (int i = 0; i < BPP; ++i) c[i] = 0;
     int top;
     if (pass == 0) {
       top = 255 - tid;
       if (tid < 256) {
 #pragma unroll 8
-        for (int w = 0; w < 32; ++w) c[0] += hist[w * 256 + top];
+        for (int w = 0; w < NW; ++w) c[0] += hist[w * 256 + top];
       }
     } else {
-      top = 4095 - 4 * tid;
-      const int4 v = h4[1023 - tid];  // bins top - 3 .. top
-      c[0] = v.w;
-      c[1] = v.z;
-      c[2] = v.y;
-      c[3] = v.x;
+      top = 4095 - BPP * tid;
+#pragma unroll
+      for (int i = 0; i < BPP; ++i) c[i] = hist[top - i];
     }
-    const int mine = c[0] + c[1] + c[2] + c[3];
-    const int above = block_inclusive_scan_1024(mine, wsum, lane, wid) - mine;  // keys with a higher digit
+    int mine = 0;
+#pragma unroll
+    for (int i = 0; i < BPP; ++i) mine += c[i];
+    const int above = block_inclusive_scan<T>(mine, wsum, lane, wid) - mine;  // keys with a higher digit
     if (above < remaining && remaining <= above + mine) {  // exactly one thread
       int acc = above, bin = top, cnt = c[0];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
+      for (int i = 0; i < BPP - 1; ++i) {
         if (remaining > acc + c[i] && bin == top - i) {
           acc += c[i];
           bin = top - i - 1;
@@ -268,16 +310,16 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   if (surplus) {  // block-uniform: ranks of the equal keys in index order
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
-      const int w = wid + 32 * j;
-      const uint32_t eq = __ballot_sync(0xffffffffu, tid + kTopkThreads * j < M && order_key(zb[j]) == thr);
+      const int w = wid + NW * j;
+      const uint32_t eq = __ballot_sync(0xffffffffu, tid + T * j < M && order_key(zb[j]) == thr);
       if (lane == 0 && w < W) wsm[w] = __popc(eq);
     }
     block_exclusive_scan(wsm, W, hist);
   }
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
-    const int w = wid + 32 * j;
-    const bool valid = tid + kTopkThreads * j < M;
+    const int w = wid + NW * j;
+    const bool valid = tid + T * j < M;
     const uint32_t key = order_key(zb[j]);
     const uint32_t gt = __ballot_sync(0xffffffffu, valid && key > thr);
     const uint32_t eq = __ballot_sync(0xffffffffu, valid && key == thr);
@@ -287,11 +329,11 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const float* __restrict__
   }
 }
 
-template <int KPT>
+template <int T, int KPT>
 static cudaError_t topk_launch(const Dims& d, const float* logits, int B, uint32_t* bitmap, uint32_t* bitmap2, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(d.L, B);
-  cfg.blockDim = dim3(kTopkThreads);
+  cfg.blockDim = dim3(T);
   cfg.dynamicSmemBytes = (size_t)d.W * 4;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -299,22 +341,32 @@ static cudaError_t topk_launch(const Dims& d, const float* logits, int B, uint32
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_topk<KPT>, logits, bitmap, bitmap2, d.L, d.M, d.k, B > 1 ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, k_topk<T, KPT>, logits, bitmap, bitmap2, d.L, d.M, d.k, B > 1 ? 1 : 0);
 }
 
 cudaError_t launch_topk(const Dims& d, const float* logits, int B, uint32_t* bitmap, uint32_t* bitmap2, bool cleared,
-                        cudaStream_t s) {
+                        cudaStream_t s, int sm_count) {
   if (B > 1 && !cleared) {
     const size_t bytes = (size_t)d.L * d.W * 4;
     cudaError_t e = cudaMemsetAsync(bitmap, 0, bytes, s);
     if (e == cudaSuccess && bitmap2) e = cudaMemsetAsync(bitmap2, 0, bytes, s);
     if (e != cudaSuccess) return e;
   }
-  const int kpt = (d.M + kTopkThreads - 1) / kTopkThreads;
-  if (kpt <= 12) return topk_launch<12>(d, logits, B, bitmap, bitmap2, s);
-  if (kpt <= 16) return topk_launch<16>(d, logits, B, bitmap, bitmap2, s);
-  if (kpt <= 28) return topk_launch<28>(d, logits, B, bitmap, bitmap2, s);
-  if (kpt <= 40) return topk_launch<40>(d, logits, B, bitmap, bitmap2, s);
+  // More jobs than SMs: blocks of 512 threads, of which two share an SM's registers where one of 1024 fills them; a job is a
+  // chain of block-wide steps, and two chains side by side take little longer than one (np_predict for sixteen sequences of
+  // the 7B shape, 512 jobs: 82 us against 86).  With a job per SM at most the wider block is the shorter chain (one
+  // sequence on its own: 79 us against 83).
+  if (d.L * B > sm_count) {
+    const int kpt = (d.M + 511) / 512;
+    if (kpt <= 12) return topk_launch<512, 12>(d, logits, B, bitmap, bitmap2, s);
+    if (kpt <= 22) return topk_launch<512, 22>(d, logits, B, bitmap, bitmap2, s);
+    if (kpt <= 28) return topk_launch<512, 28>(d, logits, B, bitmap, bitmap2, s);
+  }
+  const int kpt = (d.M + 1023) / 1024;
+  if (kpt <= 12) return topk_launch<1024, 12>(d, logits, B, bitmap, bitmap2, s);
+  if (kpt <= 16) return topk_launch<1024, 16>(d, logits, B, bitmap, bitmap2, s);
+  if (kpt <= 28) return topk_launch<1024, 28>(d, logits, B, bitmap, bitmap2, s);
+  if (kpt <= 40) return topk_launch<1024, 40>(d, logits, B, bitmap, bitmap2, s);
   return cudaErrorInvalidValue;  // d_ffn > 40960 is rejected by np_init
 }
 

@@ -51,3 +51,25 @@ def test_bitmap_handed_out_is_the_one_kept(B, k):
                 assert (active == np.flatnonzero(O.bitmap_to_bool(got[l], M))).all(), (t, l)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("M,k", [(32, 5), (512, 511), (544, 100), (6144, 600), (6176, 1), (11264, 1100), (14336, 2000), (14368, 2000)])
+def test_more_selections_than_sms(M, k):
+    """Blocks of 512 threads take a job each where there are more jobs than SMs: row counts around their keys per thread,
+    ordinary logits, heavy ties and infinities."""
+    L, B = 10, 16
+    p = Pair(synth.StackConfig("tk", L, 16, M, 8, 25, 50, 1, 45, 0.5), max_batch=B, k=k, C=M, with_oracle=False)
+    try:
+        g = torch.Generator().manual_seed(M)
+        z = torch.randn((B, L, M), generator=g)
+        z[:, 1] = torch.randint(0, 3, (B, M), generator=g).float()      # ties: more keys in the deciding bin than are ranked
+        z[:, 2, ::7] = float("inf")
+        z[:, 3] = 0.25
+        words = torch.full((L, M // 32), -1, dtype=torch.int32, device="cuda")
+        nb.np_topk(p.eng.ctx, z.cuda(), B, words, p.eng.stream)
+        p.eng.stream.synchronize()
+        for l in range(L):
+            want = O.topk_bitmap(z[:, l:l + 1].numpy(), k)[0]
+            assert (words[l].cpu().numpy().view(np.uint32) == want).all(), l
+    finally:
+        p.close()
