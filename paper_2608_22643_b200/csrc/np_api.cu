@@ -189,12 +189,17 @@ struct np_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr}, ev_copied[kStageParts] = {};
   bool half_pending[kStageParts] = {};
   int next_half = 0;
-  cudaEvent_t ev_t[4] = {nullptr, nullptr, nullptr, nullptr};  // compute-stream step timing
-  cudaEvent_t ev_c[2] = {nullptr, nullptr};                    // copy-stream step timing
+  // Step timing.  A timing event between two kernels costs about 2 us and keeps the second from starting early, so there
+  // are few: the delta step's own event ends its stage, and its kernel notes how long it took (Tables::clocks).  (2-layer
+  // stack: 62 us a step with seven events on the compute stream, 52 with four.)
+  cudaEvent_t ev_t[2] = {nullptr, nullptr};  // compute stream: begin and end of the step
+  cudaEvent_t ev_c[2] = {nullptr, nullptr};  // copy stream: begin and end of the install (rows_in_stream: it begins with ev_delta)
+  bool timed_in_stream = false, timed_selected = false;
   bool have_delta = false;
   bool have_spec = false;   // np_speculate has run since the last np_delta
   bool have_pred = false;
   bool have_step = false;
+  bool rows_in_stream = false;      // within np_step: one launch on the compute stream itself pulls the rows
   int step = 0;
   uint64_t launches = 0;
   Pool* pool = nullptr;
@@ -357,12 +362,13 @@ cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
     ctx->mark[l] = ctx->ev_installed[l1 - 1];
     ctx->install_pending[l] = 1;
   }
-  return cudaEventRecord(ctx->ev_installed[l1 - 1], s);
+  return ctx->rows_in_stream ? cudaSuccess : cudaEventRecord(ctx->ev_installed[l1 - 1], s);  // np_step marks those rows itself
 }
 
 // Orders `s` after the install marks of layers [l0, l1); marks that have already completed need no wait, and layers of
 // one launch share theirs.
 cudaError_t wait_installs(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
+  if (ctx->rows_in_stream) return cudaSuccess;
   cudaEvent_t seen = nullptr;
   bool landed = false;
   for (int l = l0; l < l1; ++l) {
@@ -557,7 +563,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   const size_t o_res = take(LW), o_slot = take(LM), o_owner = take(LC), o_stamp = take(LM);
   const size_t o_did = take(LC), o_dsl = take(LC), o_eid = take(LC), o_aid = take(LC), o_asl = take(LC);
   const size_t o_ovf = take(LM), o_cnt = take((size_t)d.L * NP_N_COUNTERS), o_free = take(LC);
-  const size_t o_cid = take(LC), o_ckey = take(LC), o_pred = take(LW), o_stat = take(4), o_bar = take(4);
+  const size_t o_cid = take(LC), o_ckey = take(LC), o_pred = take(LW), o_stat = take(4), o_bar = take(4), o_clk = take(4);
   const size_t o_ident = take(d.dense > 0 ? (size_t)d.M : 1);
   const size_t o_spid = take(LC), o_spsl = take(LC), o_spcnt = take((size_t)d.L * NP_N_COUNTERS), o_spcand = take(LW);
   const size_t o_sfix = take(2 * chain_slices::zfix_words(d)), o_sbar = take(chain_slices::bar_words()), o_sxch = take(2 * chain_slices::xch_words(d, ctx->sm_count));
@@ -585,6 +591,8 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   t.cand_keys = reinterpret_cast<uint32_t*>(base + o_ckey);
   t.pred = reinterpret_cast<uint32_t*>(base + o_pred);
   t.status = reinterpret_cast<int32_t*>(base + o_stat);
+  t.clocks = reinterpret_cast<unsigned long long*>(base + o_clk);
+  NP_INIT_CUDA(cudaMemset(t.clocks, 0, 16));
   t.grid_bar = reinterpret_cast<unsigned int*>(base + o_bar);
   t.identity = reinterpret_cast<int32_t*>(base + o_ident);
   t.spec_ids = reinterpret_cast<int32_t*>(base + o_spid);
@@ -626,7 +634,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   }
   ctx->gu_bytes = 2 * wl.gu_each;
 
-  NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_delta, cudaEventDisableTiming));
+  NP_INIT_CUDA(cudaEventCreate(&ctx->ev_delta));
   NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_spec, cudaEventDisableTiming));
   ctx->ev_installed.assign(d.L, nullptr);
   ctx->mark.assign(d.L, nullptr);
@@ -1105,13 +1113,17 @@ static int install_warnings(np_ctx* ctx, int layer_begin, int layer_end, int* wa
 // eight launches, so that the MLP runs behind them (sparse_runs) can start as their own rows land, but none that is
 // expected to move less than 1 MB (about 20 us of the link): a launch and its mark cost the host and the device several
 // microseconds each.
+static int pull_launches(const np_ctx* ctx, int n) {
+  const size_t expect = ctx->d.rec_bytes * (size_t)std::max(1, ctx->d.k / 8);  // bytes of a layer: an eighth of the set is new
+  const int least = (int)std::min<size_t>(n, ((1u << 20) + expect - 1) / expect);
+  return std::max(1, std::min(8, n / std::max(1, least)));
+}
+
 static int install_pull(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_t cs) {
   const Dims& d = ctx->d;
   const int n = layer_end - layer_begin;
   if (n <= 0) return NP_OK;
-  const size_t expect = d.rec_bytes * (size_t)std::max(1, d.k / 8);  // bytes of a layer: an eighth of the set is new
-  const int least = (int)std::min<size_t>(n, ((1u << 20) + expect - 1) / expect);
-  const int launches = std::max(1, std::min(8, n / std::max(1, least)));
+  const int launches = pull_launches(ctx, n);
   for (int g = 0; g < launches; ++g) {
     const int l0 = layer_begin + (int)((long long)n * g / launches), l1 = layer_begin + (int)((long long)n * (g + 1) / launches);
     NP_LAUNCH(ctx, launch_pull(d, ctx->t, ctx->backing_dev, ctx->bufs.gate_buf, ctx->bufs.up_buf, ctx->bufs.downT_buf, l0, l1,
@@ -1125,6 +1137,8 @@ static int install_pull(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_
 // its bytes cross at 55.1 GB/s, the kernel reads at 51.2: calls pay from about 3.4 MB each.  Runs are that long only where
 // most of a layer arrives at once.
 constexpr size_t kRunBytes = 3400000;
+// whether a layer's lists can hold such a run at all
+static bool runs_can_be_long(const np_ctx* ctx) { return (size_t)ctx->d.C * ctx->d.rec_bytes >= kRunBytes; }
 static bool runs_by_copies(const np_ctx* ctx, int layer_begin, int layer_end) {
   const Dims& d = ctx->d;
   size_t rows = 0, runs = 0;
@@ -1156,7 +1170,7 @@ static int install_enqueue(np_ctx* ctx, int layer_begin, int layer_end, cudaStre
   }
   if (mode == NP_XFER_MEMCPY_RUNS) {
     bool copies = false;
-    if ((size_t)d.C * rec >= kRunBytes) {  // else no run can be long enough, whatever the lists hold
+    if (runs_can_be_long(ctx)) {
       const int rc = install_warnings(ctx, layer_begin, layer_end, warn);
       if (rc < 0) return rc;
       copies = runs_by_copies(ctx, layer_begin, layer_end);
@@ -1287,6 +1301,10 @@ static bool pulls(const np_ctx* ctx) { return ctx->cfg.transfer_mode != NP_XFER_
 // launches than equal runs of a quarter each.
 static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
   const Dims& d = ctx->d;
+  if (ctx->rows_in_stream && ctx->cfg.chain_layers == 0) {  // behind the rows on their stream: one run
+    runs->push_back(d.L - d.dense);
+    return NP_OK;
+  }
   // layers whose rows have all landed already need no run of their own to wait in: they go into one
   // first run (the whole stack when nothing is pending, as in np_mlp_chain on resident rows)
   int landed = d.dense;
@@ -1670,10 +1688,8 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   int rc = NP_OK;
   if (!selected) rc = np_predict(ctx, x_bf16, B, nullptr, nullptr, stream);
   if (rc < 0) return rc;
-  NP_CUDA(ctx, cudaEventRecord(ctx->ev_t[1], s));
   rc = np_delta(ctx, selected, stream);
   if (rc < 0) return rc;
-  NP_CUDA(ctx, cudaEventRecord(ctx->ev_t[2], s));
   // Speculative prefetch behind the step (Section 6's future work).  Its candidates are the rows ranked
   // k+1 .. k+s by this step's own logits (a caller's selection has no ranking to extend: the caller then
   // calls np_speculate itself).  The second selection and the table update run right behind the delta
@@ -1698,17 +1714,36 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
     rc = mlp_chain(ctx, x_bf16, B, x_out, s, kChainHead, true);
     if (rc < 0) return rc;
   }
-  NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_delta, 0));
-  NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[0], cs));
+  // Rows that one launch pulls have no MLP launch to run beside: between the delta step and the chain, on their own stream,
+  // the launch costs the host no waits across streams (2-layer stack, 40 incoming rows in all, three contexts stepping in
+  // turn: 52 us a step with the launch on the copy stream, 47 on the compute stream).
+  const bool in_stream = !head_first && !spec && pulls(ctx) && pull_launches(ctx, d.L) == 1 &&
+                         (ctx->cfg.transfer_mode != NP_XFER_MEMCPY_RUNS || !runs_can_be_long(ctx));
+  const cudaStream_t is = in_stream ? s : cs;
+  ctx->timed_in_stream = in_stream;
+  ctx->timed_selected = selected != nullptr;
+  if (!in_stream) {
+    NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_delta, 0));
+    NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[0], cs));
+  }
   int warn = NP_OK;
   bool late = false;
-  rc = install_enqueue(ctx, 0, d.L, cs, &warn, &late);
+  struct InStream {  // for the length of the install and the chain, whatever way this function is left
+    np_ctx* c;
+    ~InStream() { c->rows_in_stream = false; }
+  } guard = {ctx};
+  ctx->rows_in_stream = in_stream;
+  rc = install_enqueue(ctx, 0, d.L, is, &warn, &late);
   if (rc < 0) return rc;
-  NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[1], cs));
+  NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[1], is));
+  if (in_stream) {
+    std::fill(ctx->mark.begin(), ctx->mark.end(), ctx->ev_c[1]);
+    NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_c[1], 0));  // work queued on it afterwards sees the rows
+  }
 
   rc = mlp_chain(ctx, x_bf16, B, x_out, s, head_first ? kChainTail : kChainAll, true);
   if (rc < 0) return rc;
-  NP_CUDA(ctx, cudaEventRecord(ctx->ev_t[3], s));
+  NP_CUDA(ctx, cudaEventRecord(ctx->ev_t[1], s));
   ctx->have_step = true;
   if (spec) {
     // the guessed rows cross behind the step's own rows, while its MLP launches run
@@ -1736,13 +1771,16 @@ int np_last_step_times(np_ctx* ctx, float* out_us) {
   if (!ctx) return fail(nullptr, NP_E_INVAL, "ctx is NULL");
   if (!out_us) return fail(ctx, NP_E_INVAL, "out is NULL");
   if (!ctx->have_step) return fail(ctx, NP_E_STATE, "no np_step has run");
-  NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_t[3]));
+  NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_t[1]));
   NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_c[1]));
+  unsigned long long clocks[2];
+  NP_CUDA(ctx, cudaMemcpy(clocks, ctx->t.clocks, sizeof clocks, cudaMemcpyDeviceToHost));
   float ms[4];
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[0], ctx->ev_t[0], ctx->ev_t[1]));
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[1], ctx->ev_t[1], ctx->ev_t[2]));
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[2], ctx->ev_c[0], ctx->ev_c[1]));
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[3], ctx->ev_t[2], ctx->ev_t[3]));
+  NP_CUDA(ctx, cudaEventElapsedTime(&ms[0], ctx->ev_t[0], ctx->ev_delta));
+  ms[1] = clocks[1] > clocks[0] ? std::min(ms[0], (float)(clocks[1] - clocks[0]) * 1e-6f) : 0.f;
+  ms[0] = ctx->timed_selected ? 0.f : ms[0] - ms[1];
+  NP_CUDA(ctx, cudaEventElapsedTime(&ms[2], ctx->timed_in_stream ? ctx->ev_delta : ctx->ev_c[0], ctx->ev_c[1]));
+  NP_CUDA(ctx, cudaEventElapsedTime(&ms[3], ctx->ev_delta, ctx->ev_t[1]));
   for (int i = 0; i < 4; ++i) out_us[i] = ms[i] * 1000.f;
   return NP_OK;
 }

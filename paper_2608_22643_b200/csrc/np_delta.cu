@@ -27,6 +27,13 @@ struct DeltaParams {
   int policy, step, check;
 };
 
+// nanoseconds of the device's clock
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+
 // Ascending list of the indices i in [0, n) with flag(i) true; returns the count
 // to every thread.  `red` is shared scratch (>= 40 ints).
 template <typename Flag, typename Emit>
@@ -162,6 +169,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 1) k_delta(DeltaParams p) {
   }
   // No early trigger for the kernel behind this one: whatever follows may read the tables.
   npp::pdl_wait_prior();  // the bitmap may be the previous kernel's
+  if (blockIdx.x == 0 && tid == 0) p.t.clocks[0] = global_ns();
   DK(1);
 
   // ---- 1. diff the bitmaps ------------------------------------------------------------
@@ -497,6 +505,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 1) k_delta(DeltaParams p) {
     v[NP_CNT_RESIDENT] = n_resident;
     v[NP_CNT_STEP] = p.step;
     if (p.check && (n_active > C || n_resident > C || n_evict > C)) atomicOr(p.t.status, kStatBadCount);
+    atomicMax(p.t.clocks + 1, global_ns());
     for (int i = 0; i < NP_N_COUNTERS; ++i) counters[i] = v[i];
     // the host reads its mirror only after an event recorded behind this kernel: no fence needed
     if (h_cnt)
@@ -633,15 +642,9 @@ cudaError_t launch_delta(const Dims& d, const Tables& t, const uint32_t* pred, i
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (sm > 48 * 1024) {
-    static size_t allowed[64] = {};  // per device: the attribute sticks to the function, set it when a launch needs more than before
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_shared(reinterpret_cast<const void*>(k_delta), &done);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || sm > allowed[dev]) {
-      e = cudaFuncSetAttribute(k_delta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) allowed[dev] = sm;
-    }
   }
   return cudaLaunchKernelEx(&cfg, k_delta, p);
 }

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -42,6 +43,7 @@ struct Tables {
   int32_t* spec_ids;      // [L][C]  rows made resident ahead of time by the last np_speculate
   int32_t* spec_slots;    // [L][C]
   int32_t* spec_counters; // [L][NP_N_COUNTERS] their count sits at NP_CNT_DELTA (the install path reads it there)
+  unsigned long long* clocks;  // [2]  start and end of the last delta kernel, nanoseconds (the end only grows)
   uint32_t* spec_cand;    // [L][W]  candidate bitmap of np_step's own speculation
 };
 
@@ -64,6 +66,23 @@ struct Dims {
   int Lp;           // layers the record store holds: layer l reads layer l % Lp of it
   size_t rec_bytes;
 };
+
+// Lets a kernel have all the dynamic shared memory a block can get.  The setting belongs to the function and is shared by
+// every context and thread, so it is made once per device (`done`: one bit each, a static of the caller) and to the same
+// value by all: a launch may then ask for any amount.
+inline cudaError_t allow_shared(const void* fn, std::atomic<uint64_t>* done) {
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (dev < 64 && (done->load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+  cudaFuncAttributes fa;
+  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess && dev < 64) done->fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
 
 // ---- kernel launchers (each in its own .cu) -------------------------------
 cudaError_t launch_tables_reset(const Dims& d, const Tables& t, cudaStream_t s);

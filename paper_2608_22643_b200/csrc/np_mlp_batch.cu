@@ -725,7 +725,8 @@ bool make_plan(const Dims& d, int rows, bool dense, int nsg, int sm_count, Plan*
 template <int NSG, int NP>
 cudaError_t launch_one(const KArgs& ka, size_t sm, int grid, cudaStream_t s) {
   auto kfn = k_mlp_batch<NSG, NP>;
-  cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  static std::atomic<uint64_t> done{0};
+  cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);

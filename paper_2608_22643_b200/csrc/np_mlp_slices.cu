@@ -1060,12 +1060,9 @@ size_t bar_words() { return (size_t)kQ * kBarStride; }
 template <int KS, bool XB>
 static cudaError_t launch_one(const KArgs& ka, size_t sm, int grid_x, cudaStream_t s) {
   auto kfn = k_mlp_slices<KS, XB>;
-  cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  static std::atomic<uint64_t> done{0};
+  cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, kBlock, sm);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid_x);
   cfg.blockDim = dim3(kBlock);

@@ -339,7 +339,8 @@ static cudaError_t l2_dispatch_nb(const uint4* w2, const float* hidden, float* l
 #define NP_L2_LAUNCH(NBV)                                                                             \
   do {                                                                                                \
     auto kfn = k_pred_l2<LPR, CPL, NBV>;                                                              \
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);  \
+    static std::atomic<uint64_t> done{0};                                                             \
+    cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done);                          \
     if (e != cudaSuccess) return e;                                                                   \
     return cudaLaunchKernelEx(&cfg, kfn, w2, hidden, logits, rows, H, B, stage_rows, n_stages, status); \
   } while (0)

@@ -464,7 +464,8 @@ cudaError_t launch_pred_l1_tc(const Dims& d, const PredTcState& st, const void* 
   // x is the caller's buffer: its map is made per call.  The box has 16 rows, the tensor B: rows past the end read zero.
   if (!make_map(&x, x_bf16, (uint64_t)d.D, (uint64_t)B, kTcKBlock, kL1N)) return cudaErrorInvalidValue;
   const size_t smem = (size_t)st.l1_kb_per_block * kL1StageBytes + 1024;
-  cudaError_t e = cudaFuncSetAttribute(k_pred_l1_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static std::atomic<uint64_t> done{0};
+  cudaError_t e = allow_shared(reinterpret_cast<const void*>(k_pred_l1_tc), &done);
   if (e != cudaSuccess) return e;
   k_pred_l1_tc<<<dim3((d.H + kTcTileRows - 1) / kTcTileRows, st.l1_parts), kTcThreads, smem, s>>>(
       w, x, st.l1_part, d.H, (d.D + kTcKBlock - 1) / kTcKBlock, st.l1_kb_per_block, status);
@@ -493,7 +494,8 @@ cudaError_t launch_pred_l2_tc(const Dims& d, const PredTcState& st, float* hidde
                                      static_cast<__nv_bfloat16*>(st.hsplit), d.H, B, l1_parts, hidden, clear, clear2,
                                      clear ? d.L * d.W : 0);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_pred_l2_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)st.smem);
+  static std::atomic<uint64_t> done{0};
+  e = allow_shared(reinterpret_cast<const void*>(k_pred_l2_tc), &done);
   if (e != cudaSuccess) return e;
   const long long rows = (long long)d.L * d.M;
   const long long n_tiles = (rows + kTcTileRows - 1) / kTcTileRows;

@@ -217,7 +217,8 @@ static cudaError_t gemv(const GemvArgs& a, int n_seg, cudaStream_t s, int sm_cou
   const bool wide = max_rows >= 2 * kWarps * sm_count || max_in <= 2048;
   auto kfn = wide ? k_gemv<2, 8> : k_gemv<1, 16>;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<uint64_t> done[2] = {{0}, {0}};
+    cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done[wide]);
     if (e != cudaSuccess) return e;
   }
   const int per_block = kWarps * (wide ? 2 : 1);
