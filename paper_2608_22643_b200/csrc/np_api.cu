@@ -606,7 +606,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   NP_INIT_CUDA(cudaMemset(ctx->slices.zfix, 0, chain_slices::zfix_words(ctx->d) * 8));
   NP_INIT_CUDA(cudaMemset(ctx->slices.bars, 0, chain_slices::bar_words() * 4));
   NP_INIT_CUDA(cudaMemset(ctx->slices.xch, 0, chain_slices::xch_words(ctx->d, ctx->sm_count) * 8));
-  ctx->use_slices = !(cfg->flags & NP_F_ROW_CHAIN) && chain_slices::supported(d, ctx->sm_count);
+  ctx->use_slices = !(cfg->flags & NP_F_ROW_CHAIN) && chain_slices::preferred(d, ctx->sm_count);
   ctx->xterms = base + o_xt;
   ctx->rows.z4 = reinterpret_cast<float*>(base + o_rz);
   ctx->rows.cnt = reinterpret_cast<unsigned int*>(base + o_rcnt);

@@ -224,6 +224,7 @@ struct State {
 };
 bool plan(const Dims& d, int sm_count, Plan* p);
 bool supported(const Dims& d, int sm_count);
+bool preferred(const Dims& d, int sm_count);  // supported, and no other form is faster at this width
 size_t xch_words(const Dims& d, int sm_count);
 bool counted_handover(const Dims& d, int sm_count);  // the sums between layers are counted fixed-point words for this shape
 size_t zfix_words(const Dims& d);

@@ -42,7 +42,7 @@
 //    counted words too, and the blocks of row group 0 wait for them and write the stack's result.
 //
 //    This form is used where a thread owns one or two 4-column granules of the slice (row widths
-//    up to 8192).  Wider slices keep the fp32 form between all layers: 16-byte fp32 reductions into
+//    up to 8192; see preferred() on wider ones).  Wider slices keep the fp32 form between all layers: 16-byte fp32 reductions into
 //    the rotating accumulators (kZRep copies), a fence, one arrival counter per slice that the next
 //    layer's first thread polls, then every thread reads the copies of its columns (the counted
 //    form would hold the previous sums of four granules in registers there).
@@ -238,6 +238,102 @@ __device__ __forceinline__ void wait_group(unsigned int gq, uint64_t* bar, uint3
   wait_or_flag(bar, parity, ok, status);
 }
 
+// A round of the exchange for row groups of more than 32 rows: rows r0 + lane and r0 + 32 + lane of this row group.  Publishes the
+// block's own sums, collects the other slices', leaves the activations as three bf16 terms.  The round of r0 = 0 also
+// collects the sums of squares and leaves inv_rms.
+__device__ __forceinline__ void exchange_rows(const KArgs& a, const float* part, uint16_t* aterm, unsigned long long* mine,
+                                              const unsigned long long* base, int r0, int nrows, int nrows16, int gs, int GW, int apad,
+                                              int q, int lane, unsigned int stamp, float own_ss, float& inv_rms, volatile int* ok) {
+  constexpr int NSET = 2;
+  const int VG = 1 << gs;
+  const bool want_ss = r0 == 0 && lane == 0;
+  // this block's own sums of the rows: the partial sums of the consumer warps (their K blocks)
+  float own_g[NSET], own_u[NSET];
+#pragma unroll
+  for (int t = 0; t < NSET; ++t) {
+    const int row = r0 + 32 * t + lane;
+    own_g[t] = own_u[t] = 0.f;
+    if (row < nrows) {
+      const int v = 2 * row;
+      const float* pp = part + ((size_t)(v >> gs) * GW) * VG + (v & (VG - 1));
+      for (int w = 0; w < GW; ++w) {
+        own_g[t] += pp[w * VG];
+        own_u[t] += pp[w * VG + 1];
+      }
+      st_relaxed_u64(mine + v, stamped(own_g[t], stamp));
+      st_relaxed_u64(mine + v + 1, stamped(own_u[t], stamp));
+    }
+  }
+  // One 16-byte load per row and peer (its gate and up words), issued only by the lanes that
+  // have a row; lane 0 also fetches the peers' sums of squares.  Strong loads are not merged
+  // across lanes, so every load that is not needed costs a request of its own at the L2 (all
+  // blocks poll at about the same moment).
+  float gsum[NSET][kQ], usum[NSET][kQ], ssv[kQ];  // indexed by unrolled constants only (registers)
+  bool done = !*ok;
+  for (uint32_t spin = 0; spin < npp::kSpinLimit && !done; ++spin) {
+    unsigned long long wg[NSET][kQ], wu[NSET][kQ], ws[kQ];  // every load of the round is issued before any is looked at
+#pragma unroll
+    for (int qq = 0; qq < kQ; ++qq) {
+      const unsigned long long* w = base + (size_t)qq * a.xch_stride;
+#pragma unroll
+      for (int t = 0; t < NSET; ++t) {
+        const int row = r0 + 32 * t + lane;
+        wg[t][qq] = wu[t][qq] = (unsigned long long)stamp << 32;
+        if (row < nrows && qq != q) ld_relaxed_v2u64(w + 2 * row, wg[t][qq], wu[t][qq]);
+      }
+      ws[qq] = (unsigned long long)stamp << 32;
+      if (want_ss && qq != q) ws[qq] = ld_relaxed_u64(w + 2 * a.max_rows);
+    }
+    unsigned int bad = 0;
+#pragma unroll
+    for (int qq = 0; qq < kQ; ++qq) {
+#pragma unroll
+      for (int t = 0; t < NSET; ++t) {
+        bad |= ((unsigned int)(wg[t][qq] >> 32) ^ stamp) | ((unsigned int)(wu[t][qq] >> 32) ^ stamp);
+        gsum[t][qq] = __uint_as_float((unsigned int)wg[t][qq]);
+        usum[t][qq] = __uint_as_float((unsigned int)wu[t][qq]);
+      }
+      bad |= (unsigned int)(ws[qq] >> 32) ^ stamp;
+      ssv[qq] = __uint_as_float((unsigned int)ws[qq]);
+    }
+    done = bad == 0;
+  }
+  if (!done) {
+    *ok = 0;
+    atomicOr(a.status, npp::kStatTimeout);
+  }
+  if (r0 == 0) {
+    float ss = 0.f;
+#pragma unroll
+    for (int qq = 0; qq < kQ; ++qq) ss += qq == q ? own_ss : ssv[qq];  // the same order in every block
+    inv_rms = __shfl_sync(0xffffffffu, rsqrtf(ss / (float)a.D + kRmsEps), 0);  // lane 0 holds the peers' sums
+  }
+#pragma unroll
+  for (int t = 0; t < NSET; ++t) {
+    const int row = r0 + 32 * t + lane;
+    if (row < nrows16) {
+      float av = 0.f;  // rows that pad the last 16-row block: zero
+      if (row < nrows) {
+        float gsv = 0.f, usv = 0.f;
+#pragma unroll
+        for (int qq = 0; qq < kQ; ++qq) {
+          gsv += qq == q ? own_g[t] : gsum[t][qq];
+          usv += qq == q ? own_u[t] : usum[t][qq];
+        }
+        // the MLP's input is x_l scaled to unit RMS; the dot products are linear in it
+        gsv *= inv_rms;
+        usv *= inv_rms;
+        av = gsv / (1.f + __expf(-gsv)) * usv;
+      }
+      uint32_t t0, t1, t2;
+      split3(av, t0, t1, t2);
+      aterm[row] = (uint16_t)(t0 >> 16);
+      aterm[apad + row] = (uint16_t)(t1 >> 16);
+      aterm[2 * apad + row] = (uint16_t)(t2 >> 16);
+    }
+  }
+}
+
 // ring slot and use parity of the group with sequence number g (exact for g < 2^32 / ng)
 __device__ __forceinline__ void slot_of(unsigned int g, unsigned int magic, int ng, int& slot, uint32_t& par) {
   const unsigned int qd = __umulhi(g, magic);
@@ -283,7 +379,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
   const int GW = 1 << a.gw_shift;  // consumer warps per gate|up group: each takes every GW-th K block
   float* part = ybuf + Ds;                                           // [groups][GW][VG] partial gate / up sums
   uint16_t* aterm = reinterpret_cast<uint16_t*>(part + (size_t)n_gu_max * GW * VG);  // [3][apad] bf16 terms of a_i
-  int* slot_cache = reinterpret_cast<int*>(aterm + 3 * apad + (apad & 1));
+  uint16_t* slot_cache = aterm + 3 * apad + (apad & 1);  // slots are below the capacity, at most 40960
   volatile int* ok = &s_ok;
   volatile unsigned int* armed = &s_armed;
 
@@ -329,7 +425,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
         atomicOr(a.status, kStatBadSlot);
         slot = 0;
       }
-      slot_cache[lay_pre[li] + i] = slot;
+      slot_cache[lay_pre[li] + i] = (uint16_t)slot;
     }
   }
   __syncthreads();
@@ -417,7 +513,12 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
       if (lane == 0) st_relaxed_u64(mine + 2 * a.max_rows, stamped(own_ss, stamp));
       float inv_rms = 0.f;
       const int nrows16 = (nrows + 15) & ~15;
-      for (int r0 = 0; r0 < nrows16; r0 += 32) {
+      // More than 32 rows: two rows per lane go through one round of polls.  A round is a trip to the L2 and back, whatever it
+      // fetches (39 rows of a block, 70B shape: 1.29 ms per 80 layers with a round per 32 rows, 1.21 with one round).  Up to 32 rows the
+      // form with one row per lane stays: 234 us per 32 layers of the 7B shape against 237 with the other.
+      for (int r0 = 0; nrows16 > 32 && r0 < nrows16; r0 += 64)
+        exchange_rows(a, part, aterm, mine, base, r0, nrows, nrows16, gs, GW, apad, q, lane, stamp, own_ss, inv_rms, ok);
+      for (int r0 = 0; r0 < nrows16 && nrows16 <= 32; r0 += 32) {
         const int row = r0 + lane;
         const bool has_row = row < nrows, want_ss = r0 == 0 && lane == 0;
         // this block's own sums of the row: the partial sums of the consumer warps (their K blocks)
@@ -962,7 +1063,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
   }
 }
 
-bool plan(const Dims& d, int sm_count, Plan* p) {
+// the plan for groups of at most 1 << vg_shift_max vectors; false: it does not fit
+static bool plan_groups(const Dims& d, int sm_count, int vg_shift_max, Plan* p) {
   if (d.D % (16 * kQ) || sm_count < kQ) return false;
   const int Ds = d.D / kQ;
   const int nk = Ds / 16;
@@ -978,7 +1080,7 @@ bool plan(const Dims& d, int sm_count, Plan* p) {
   if (const char* e = getenv("NP_SL_GT")) group_target = (size_t)atoi(e) * 1024;
 #endif
   int vg_shift = 1;
-  while (vg_shift < 4 && ((size_t)2 << vg_shift) * pstride <= group_target) ++vg_shift;
+  while (vg_shift < vg_shift_max && ((size_t)2 << vg_shift) * pstride <= group_target) ++vg_shift;
   const int VG = 1 << vg_shift;
   const size_t group_bytes = (size_t)VG * pstride;
   const size_t budget = 227 * 1024 - 2048;  // static shared memory of the kernel
@@ -1002,14 +1104,17 @@ bool plan(const Dims& d, int sm_count, Plan* p) {
   // everything but the ring and the slot cache; the cache (the slots of a launch's rows) takes a minimum first
   // and, once the ring's slots are counted, whatever is left, so that a launch can span more layers
   const size_t fixed0 = 3 * pstride + (size_t)Ds * 4 + (size_t)n_gu_max * GW * VG * 4 + (size_t)(3 * apad + (apad & 1)) * 2 + 64;
-  const size_t cache_min = std::max<size_t>(4 * (size_t)max_rows, std::min<size_t>(8192, 4 * (size_t)max_rows * 8));
+  // the cache: room for sixteen layers where that takes no more than 8 KB, and less where the ring would otherwise not fit
+  // (8192 columns at a capacity of 11468: 19.8 us per layer in the row-partitioned kernel, 16.2 here)
+  size_t cache_min = std::max<size_t>(2 * (size_t)max_rows, std::min<size_t>(8192, 2 * (size_t)max_rows * 16));
+  while (fixed0 + cache_min + 3 * group_bytes > budget && cache_min > 2 * (size_t)max_rows) cache_min = std::max(cache_min / 2, 2 * (size_t)max_rows);
   if (fixed0 + cache_min + 3 * group_bytes > budget) return false;
   int ng = (int)std::min<size_t>(kMaxGroups, (budget - fixed0 - cache_min) / group_bytes);
   if (d.ring_stages >= 2) ng = std::max(3, std::min(ng, d.ring_stages));
-  const size_t cache_bytes = std::min<size_t>(budget - fixed0 - (size_t)ng * group_bytes, 4 * (size_t)max_rows * kMaxLayers);
-  p->run_layers = (int)std::max<size_t>(1, std::min<size_t>(kMaxLayers, cache_bytes / (4 * (size_t)max_rows)));
+  const size_t cache_bytes = std::min<size_t>(budget - fixed0 - (size_t)ng * group_bytes, 2 * (size_t)max_rows * kMaxLayers);
+  p->run_layers = (int)std::max<size_t>(1, std::min<size_t>(kMaxLayers, cache_bytes / (2 * (size_t)max_rows)));
   p->slot_cache_rows = p->run_layers * max_rows;
-  const size_t fixed = fixed0 + (size_t)p->slot_cache_rows * 4;
+  const size_t fixed = fixed0 + (size_t)p->slot_cache_rows * 2;
   // Groups in flight per block.  Where the hand-over between layers has no fence (counted sums) the producer runs
   // as far ahead as the ring and its pacing history allow (7B shape: 284 us per 32 layers with one group in
   // flight, 274 with five; 13B shape: 390 us per 40 layers against 357).  The fp32 form keeps about 40 KB in
@@ -1033,6 +1138,18 @@ bool plan(const Dims& d, int sm_count, Plan* p) {
   p->group_bytes = group_bytes;
   p->smem = (size_t)ng * group_bytes + fixed;
   return true;
+}
+
+// Groups of eight vectors where the ring would not hold three of sixteen (8192 columns at a capacity of 19456: 17.5 us per
+// layer against 19.9 in the row-partitioned kernel).
+bool plan(const Dims& d, int sm_count, Plan* p) { return plan_groups(d, sm_count, 4, p) || plan_groups(d, sm_count, 3, p); }
+
+// Rows of more than 8192 columns: four granules per thread, fp32 sums between the layers.  The row-partitioned kernel, and
+// above its widths the kernels per layer, are faster at every one of them (100 to 1600 rows of 8256 columns: 9.3 to 26.9 us
+// per layer against 14.6 to 34.0 here; 14336 columns: 11.0 to 36.1 against 15.8 to 59.4); such rows come here only where
+// the stack has dense layers and no other resident kernel covers its width.
+bool preferred(const Dims& d, int sm_count) {
+  return supported(d, sm_count) && (d.D <= 8192 || (d.dense > 0 && !chain_alu::supported(d, sm_count)));
 }
 
 bool supported(const Dims& d, int sm_count) {

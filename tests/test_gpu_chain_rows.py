@@ -1,0 +1,38 @@
+"""The column-sliced MLP kernel where its row groups and its shared memory run out, against the oracle."""
+import pytest
+import torch
+
+from paper_2608_22643_b200 import binding as nb
+from paper_2608_22643_b200 import synth
+from tests.harness import Pair, rel_l2, u16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D,M,k,L", [
+    (256, 4096, 37 * 32, 3),      # a row per lane in every row group of 148 SMs
+    (256, 4096, 37 * 32 + 1, 3),  # one row group of 33
+    (256, 4096, 37 * 64, 3),
+    (256, 4096, 37 * 64 + 1, 3),  # one of 65: a second round of the exchange
+    (256, 4096, 4096, 3),
+    (1216, 2048, 37 * 39, 3),     # 39 rows, 19 K blocks of a slice
+    (8192, 8320, 1040, 1),        # the ring fits beside a smaller slot cache only
+    (8256, 512, 100, 3),          # the narrowest rows that another kernel takes
+])
+def test_chain_row_groups(D, M, k, L):
+    cfg = synth.StackConfig("rows", L, D, M, 32, 25, 50, 3, 23, 0.9)
+    p = Pair(cfg, max_batch=1, k=k, C=M)
+    try:
+        xs = synth.hidden_states(cfg, 3, batch=1)
+        out = torch.empty((1, D), dtype=torch.float32, device="cuda")
+        logits = torch.empty((1, L, M), dtype=torch.float32, device="cuda")
+        for t in range(3):
+            nb.np_predict(p.eng.ctx, xs[t].cuda(), 1, logits, None, p.eng.stream)
+            nb.np_step(p.eng.ctx, xs[t].cuda(), 1, out, p.eng.stream, p.eng.copy_stream)
+            torch.cuda.synchronize()
+            res = p.ora.step(u16(xs[t]), logits_f32=logits.cpu().numpy())
+            p.check_delta_against(res["deltas"])
+            assert rel_l2(out.cpu().numpy()[0], res["x_final"][0]) < 1e-5, t  # fp32 sums of bf16 products: 1e-6
+        p.eng.counters()
+    finally:
+        p.close()
