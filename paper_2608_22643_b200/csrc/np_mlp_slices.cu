@@ -1234,7 +1234,9 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s,
     if (p.ks <= kFixMaxKS) st->bar_base += (nl > 1 || ka.x_out) ? (unsigned int)p.R : 0u;
     else if (nl > 1) st->bar_base += (unsigned int)(nl - 1) * (unsigned int)p.R;
     st->seq_base += (unsigned int)nl + 1u;
-    const bool xb = ((d.D / kQ / 16) >> p.gw_shift) <= 32 && p.ks <= 16;  // phase 1's B operands fit a warp's registers
+    // phase 1's B operands of a warp (one more K block than its partner's where the slice's count is odd) fit its registers
+    const int trip = ((d.D / kQ / 16) + (1 << p.gw_shift) - 1) >> p.gw_shift;
+    const bool xb = trip <= 32 && p.ks <= 16;
     if (p.ks == 8) e = xb ? launch_one<8, true>(ka, p.smem, p.R * kQ, s) : launch_one<8, false>(ka, p.smem, p.R * kQ, s);
     else if (p.ks == 16) e = xb ? launch_one<16, true>(ka, p.smem, p.R * kQ, s) : launch_one<16, false>(ka, p.smem, p.R * kQ, s);
     else e = launch_one<32, false>(ka, p.smem, p.R * kQ, s);

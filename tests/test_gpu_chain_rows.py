@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
     (256, 4096, 37 * 64 + 1, 3),  # one of 65: a second round of the exchange
     (256, 4096, 4096, 3),
     (1216, 2048, 37 * 39, 3),     # 39 rows, 19 K blocks of a slice
+    (4160, 2048, 37 * 39, 2),     # 65 K blocks of a slice over pairs of warps: 33 for one of them
     (8192, 8320, 1040, 1),        # the ring fits beside a smaller slot cache only
     (8256, 512, 100, 3),          # the narrowest rows that another kernel takes
 ])
