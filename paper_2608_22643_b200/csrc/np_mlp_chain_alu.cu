@@ -10,7 +10,7 @@
 // warp and x_l in shared memory as fp32; every block adds its partial vector of all D outputs to
 // one of kZRep accumulator copies and a grid-wide counter barrier publishes x_{l+1}.
 // It takes any row width, and is what runs where the column-sliced kernel (np_mlp_slices.cu)
-// does not apply: row widths that are not a multiple of 64, dense layers without the
+// does not apply: row widths that are not a multiple of 16, dense layers without the
 // direct-load kernel, and NP_F_ROW_CHAIN.  Every wait is bounded (kStatTimeout on expiry).
 #include <algorithm>
 

@@ -341,9 +341,9 @@ __device__ __forceinline__ void slot_of(unsigned int g, unsigned int magic, int 
   par = qd & 1u;
 }
 
-// KS: 16-column tiles (phase 2) per warp: ceil(D / kQ / 16 / kWarps).  XB: a warp has at most 32 K blocks
+// KS: 16-column tiles (phase 2) per warp, at least the widest slice's.  EVEN: the width is a multiple of 64.  XB: a warp has at most 32 K blocks
 // in phase 1 and keeps their B operands (x) in registers for the whole layer.
-template <int KS, bool XB>
+template <int KS, bool XB, bool EVEN>
 __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
   extern __shared__ __align__(128) unsigned char csm[];
   __shared__ __align__(8) uint64_t full_bar[kMaxGroups];   // the group's copies have landed
@@ -358,7 +358,13 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
 
   constexpr bool kFix = KS <= kFixMaxKS;  // counted fixed-point sums between the layers of a launch
   const bool fin = kFix && a.x_out != nullptr;  // ... and behind its last layer: the launch leaves the stack's result itself
-  const int D = a.D, Ds = D / kQ;
+  const int q = blockIdx.x % kQ, r = blockIdx.x / kQ;
+  const int D = a.D;
+  // Slices of whole K blocks, where the width is not a multiple of 64 one more in some of them.  Such widths took 6.2 us per
+  // layer (1008 columns, 156 rows), 8.8 (2384, 600) and 12.1 (4112, 1101) in the row-partitioned kernel and take 5.1, 6.6 and
+  // 8.6 here.  An instance of its own: the arithmetic costs registers (5 % of a layer at the 7B shape).
+  const int kb0 = EVEN ? 0 : q * (D >> 4) / kQ;                                     // first K block of an uneven slice
+  const int Ds = EVEN ? D / kQ : ((q + 1) * (D >> 4) / kQ - kb0) << 4;
   const int nk = Ds >> 4;     // 16-wide K blocks = 16-column tiles of the slice
   const uint32_t piece_bytes = (uint32_t)Ds * 2u;
   const uint32_t pstride = piece_bytes + kPad;  // distance between pieces in shared memory
@@ -368,8 +374,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
   const int ng = a.ng;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int G = gridDim.x, R = G / kQ;
-  const int q = blockIdx.x % kQ, r = blockIdx.x / kQ;
-  const int qoff = q * Ds;  // first column (= first K index) of this slice
+  const int qoff = EVEN ? q * Ds : kb0 << 4;  // first column (= first K index) of this slice
   const int nl = a.l_end - a.l_begin;
   const int apad = ((a.max_rows + 15) & ~15) + 16;  // activations per term, padded so that a 16-row block never runs out
   const int n_gu_max = (2 * a.max_rows + VG - 1) >> gs;
@@ -444,7 +449,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
     // through the L2 do not push out the few hundred KB every layer meets in (exchange words, counted sums,
     // slot lists): 7B shape 236 us per 32 layers against 249, 13B shape 341 us per 40 layers against 358.
     const uint64_t l2_policy = npp::policy_evict_first();
-    const size_t qbytes = (size_t)q * piece_bytes;
+    const size_t qbytes = (size_t)qoff * 2;
     for (int li = 0; li < nl; ++li) {
       const int vbase = lay_pre[li], nrows = lay_pre[li + 1] - vbase;
       const size_t lbase = (size_t)(a.l_begin + li) * layer_bytes + qbytes;
@@ -602,6 +607,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
   const int g8 = lane >> 2, t4 = lane & 3;  // mma fragment coordinates of this lane
   const int m4 = lane >> 3, rr = lane & 7;  // ldmatrix: lanes 8 m4 .. 8 m4 + 7 give the row addresses of 8x8 matrix m4
   const uint32_t ring = npp::smem_addr(csm);
+  constexpr int kStep = KS < 8 ? KS : 8;
   constexpr int J4 = (KS * kWarps * 16 / 4 + kThreads - 1) / kThreads;  // float4 granules of the slice per thread
   const int nf4 = Ds >> 2;
   float4 xown[J4];        // x_l of the columns this thread owns, for the whole run
@@ -931,12 +937,12 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
       // no guard on the tile index: a tile past the slice's end is computed from the last valid
       // tile's bytes and never looked at, which keeps the loop free of branches
 #pragma unroll
-      for (int j0 = 0; j0 < KS; j0 += 8) {  // eight loads, then their eight mma
-        uint32_t af[8][4];
+      for (int j0 = 0; j0 < KS; j0 += kStep) {  // eight loads, then their eight mma
+        uint32_t af[kStep][4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) ldmatrix_x4_trans(af[u], dbase + (uint32_t)min((j0 + u) * kWarps, nk - 1 - wid) * 32u);
+        for (int u = 0; u < kStep; ++u) ldmatrix_x4_trans(af[u], dbase + (uint32_t)min((j0 + u) * kWarps, nk - 1 - wid) * 32u);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) mma_bf16_16816(acc[j0 + u], af[u], b0, b1);
+        for (int u = 0; u < kStep; ++u) mma_bf16_16816(acc[j0 + u], af[u], b0, b1);
       }
       __syncwarp();
       if (lane == 0) npp::mbar_arrive(&empty_bar[slot]);
@@ -1065,9 +1071,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
 
 // the plan for groups of at most 1 << vg_shift_max vectors; false: it does not fit
 static bool plan_groups(const Dims& d, int sm_count, int vg_shift_max, Plan* p) {
-  if (d.D % (16 * kQ) || sm_count < kQ) return false;
-  const int Ds = d.D / kQ;
-  const int nk = Ds / 16;
+  if (d.D % 16 || d.D < 16 * kQ || sm_count < kQ) return false;
+  const int nk = (d.D / 16 + kQ - 1) / kQ;  // of the widest slice
+  const int Ds = nk * 16;
   const int ks = (nk + kWarps - 1) / kWarps;
   if (ks > 32) return false;
   const int R = sm_count / kQ;
@@ -1128,7 +1134,8 @@ static bool plan_groups(const Dims& d, int sm_count, int vg_shift_max, Plan* p) 
   if (getenv("NP_SL_NOFILL")) window = -1;
 #endif
   p->R = R;
-  p->ks = ks <= 8 ? 8 : (ks <= 16 ? 16 : 32);
+  // narrow slices have instances of their own: with eight tiles for the two of 256 columns a layer took 5.2 us, with two 4.8
+  p->ks = ks <= 2 ? 2 : ks <= 4 ? 4 : ks <= 8 ? 8 : ks <= 16 ? 16 : 32;
   p->vg_shift = vg_shift;
   p->gw_shift = gw_shift;
   p->ng = ng;
@@ -1174,9 +1181,9 @@ size_t xch_words(const Dims& d, int sm_count) {
 size_t zfix_words(const Dims& d) { return (size_t)2 * kFixRep * d.D; }
 size_t bar_words() { return (size_t)kQ * kBarStride; }
 
-template <int KS, bool XB>
+template <int KS, bool XB, bool EVEN>
 static cudaError_t launch_one(const KArgs& ka, size_t sm, int grid_x, cudaStream_t s) {
-  auto kfn = k_mlp_slices<KS, XB>;
+  auto kfn = k_mlp_slices<KS, XB, EVEN>;
   static std::atomic<uint64_t> done{0};
   cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done);
   if (e != cudaSuccess) return e;
@@ -1235,11 +1242,17 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s,
     else if (nl > 1) st->bar_base += (unsigned int)(nl - 1) * (unsigned int)p.R;
     st->seq_base += (unsigned int)nl + 1u;
     // phase 1's B operands of a warp (one more K block than its partner's where the slice's count is odd) fit its registers
-    const int trip = ((d.D / kQ / 16) + (1 << p.gw_shift) - 1) >> p.gw_shift;
+    const int trip = ((d.D / 16 + kQ - 1) / kQ + (1 << p.gw_shift) - 1) >> p.gw_shift;
     const bool xb = trip <= 32 && p.ks <= 16;
-    if (p.ks == 8) e = xb ? launch_one<8, true>(ka, p.smem, p.R * kQ, s) : launch_one<8, false>(ka, p.smem, p.R * kQ, s);
-    else if (p.ks == 16) e = xb ? launch_one<16, true>(ka, p.smem, p.R * kQ, s) : launch_one<16, false>(ka, p.smem, p.R * kQ, s);
-    else e = launch_one<32, false>(ka, p.smem, p.R * kQ, s);
+    const bool even = d.D % (16 * kQ) == 0;
+    const int grid = p.R * kQ;
+    if (p.ks == 2) e = launch_one<2, true, false>(ka, p.smem, grid, s);  // at most 16 and 32 K blocks
+    else if (p.ks == 4) e = launch_one<4, true, false>(ka, p.smem, grid, s);
+    else if (p.ks == 8 && even) e = xb ? launch_one<8, true, true>(ka, p.smem, grid, s) : launch_one<8, false, true>(ka, p.smem, grid, s);
+    else if (p.ks == 8) e = xb ? launch_one<8, true, false>(ka, p.smem, grid, s) : launch_one<8, false, false>(ka, p.smem, grid, s);
+    else if (p.ks == 16 && even) e = xb ? launch_one<16, true, true>(ka, p.smem, grid, s) : launch_one<16, false, true>(ka, p.smem, grid, s);
+    else if (p.ks == 16) e = xb ? launch_one<16, true, false>(ka, p.smem, grid, s) : launch_one<16, false, false>(ka, p.smem, grid, s);
+    else e = launch_one<32, false, false>(ka, p.smem, grid, s);
     if (e != cudaSuccess) return e;
   }
   return e;

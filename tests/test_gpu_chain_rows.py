@@ -17,6 +17,10 @@ pytestmark = pytest.mark.gpu
     (256, 4096, 4096, 3),
     (1216, 2048, 37 * 39, 3),     # 39 rows, 19 K blocks of a slice
     (4160, 2048, 37 * 39, 2),     # 65 K blocks of a slice over pairs of warps: 33 for one of them
+    (80, 512, 130, 3),            # slices of one and two K blocks
+    (2384, 4096, 37 * 30, 3),     # slices of 37 and 38
+    (4144, 2048, 37 * 39, 2),     # slices of 64 and 65
+    (8176, 512, 100, 2),          # the widest slice holds a tile more than the others
     (8192, 8320, 1040, 1),        # the ring fits beside a smaller slot cache only
     (8256, 512, 100, 3),          # the narrowest rows that another kernel takes
 ])
