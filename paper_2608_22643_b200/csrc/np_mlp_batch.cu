@@ -700,7 +700,7 @@ struct Plan {
 bool make_plan(const Dims& d, int rows, bool dense, int nsg, int sm_count, Plan* p) {
   if (d.D % 16 || d.C > 65535) return false;
   const int nkt = d.D / 16;
-  int Q = 1;
+  int Q = std::min(4, nkt);
   while (Q <= kMaxQ && (nkt + Q - 1) / Q > kMaxNk) Q *= 2;
   if (Q > kMaxQ || nkt < Q || sm_count < Q) return false;
   const int nk = (nkt + Q - 1) / Q;  // the widest slice
