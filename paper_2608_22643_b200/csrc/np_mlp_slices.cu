@@ -95,7 +95,7 @@ constexpr int kFixMaxKS = 16;          // widest slices (in 16-column tiles per 
 constexpr int kFixRep = NP_SL_FIXREP;  // copies of the counted words (row group r adds to copy r % kFixRep).  One: the 37
                                        // adds to a word cost less than reading more copies (7B shape, 32 layers: 250 us
                                        // with one copy, 252 with two, 262 with four)
-constexpr int kHist = 8;               // pacing history of the producer (> window)
+constexpr int kMaxWindow = 7;          // groups in flight, at most
 constexpr int kGroupTarget = 68 * 1024;  // largest load group: up to 16 vectors, three groups to a ring at least (70B shape:
                                          // 66 KB groups of 16 vectors, 1.39 ms per 80 layers; 33 KB groups of 8: 1.51 ms)
 constexpr int kPad = 16;               // bytes between pieces in shared memory
@@ -441,8 +441,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
     // lanes waiting on different barriers must not be used: the compiler may reconverge the warp
     // after a wait); the copies of a group are then issued by as many lanes as it has pieces,
     // since one lane issuing ninety 2 KB copies per layer sets the pace otherwise.
-    int hist_slot[kHist];
-    uint32_t hist_par[kHist];
     int issued = 0, slot = 0;
     uint32_t par = 0;
     // A row is read once per token: the copies mark their lines evict-first, so that the 27 MB a layer streams
@@ -465,16 +463,16 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(KArgs a) {
             // bytes (HBM is shared by all blocks) but queues in front of the short loads on the
             // layer's critical path (exchange words, barrier counter, accumulators).
             if (a.window > 0 && issued >= a.window) {
-              const int h = (issued - a.window) % kHist;
-              wait_or_flag(&full_bar[hist_slot[h]], hist_par[h], ok, a.status);
+              int before;
+              uint32_t bpar;
+              slot_of((unsigned int)(issued - a.window), a.ng_magic, ng, before, bpar);
+              wait_or_flag(&full_bar[before], bpar, ok, a.status);
             }
             npp::mbar_expect_tx(&full_bar[slot], (uint32_t)npieces * piece_bytes);
             __threadfence_block();
             *armed = (unsigned int)issued + 1u;  // consumers of this group may now test the barrier's parity
           }
           __syncwarp();  // the expect_tx precedes the copies
-          hist_slot[issued % kHist] = slot;
-          hist_par[issued % kHist] = par;
           ++issued;
           unsigned char* dst = csm + (size_t)slot * a.group_bytes;
 #ifdef NP_TUNE
@@ -1122,15 +1120,15 @@ static bool plan_groups(const Dims& d, int sm_count, int vg_shift_max, Plan* p) 
   p->slot_cache_rows = p->run_layers * max_rows;
   const size_t fixed = fixed0 + (size_t)p->slot_cache_rows * 2;
   // Groups in flight per block.  Where the hand-over between layers has no fence (counted sums) the producer runs
-  // as far ahead as the ring and its pacing history allow (7B shape: 284 us per 32 layers with one group in
+  // as far ahead as the ring allows (7B shape: 284 us per 32 layers with one group in
   // flight, 274 with five; 13B shape: 390 us per 40 layers against 357).  The fp32 form keeps about 40 KB in
   // flight: a deeper burst queues in front of its fence and of the short loads behind it (13B shape, when it
   // still used this form: 385 us with one 41 KB group in flight, 411 with two or more).
-  int window = ks <= kFixMaxKS ? std::max(1, std::min(ng - 1, kHist - 1)) : std::max(1, std::min(ng - 1, (int)(40 * 1024 / group_bytes)));
+  int window = ks <= kFixMaxKS ? std::max(1, std::min(ng - 1, kMaxWindow)) : std::max(1, std::min(ng - 1, (int)(40 * 1024 / group_bytes)));
   if (ng <= 3) window = 1;  // a ring of three large groups (70B shape, 66 KB each): 1.36 ms per 80 layers with one in flight, 1.39 with two
 #ifdef NP_TUNE  // development builds only: geometry from the environment
   if (const char* e = getenv("NP_SL_NG")) ng = std::max(2, std::min(ng, atoi(e)));
-  if (const char* e = getenv("NP_SL_WIN")) window = std::min(atoi(e), std::min(kHist - 1, ng - 1));
+  if (const char* e = getenv("NP_SL_WIN")) window = std::min(atoi(e), std::min(kMaxWindow, ng - 1));
   if (getenv("NP_SL_NOFILL")) window = -1;
 #endif
   p->R = R;
