@@ -57,7 +57,7 @@ def parse_args():
     ap.add_argument("--transfer", default="gather", choices=["runs", "gather", "zerocopy", "file"],
                     help="file: the record store is a file, read through io_uring with O_DIRECT (Section 3.5)")
     ap.add_argument("--mapped-staging", action="store_true",
-                    help="gather / file transfer: the scatter kernel reads the pinned staging itself, no staging copy")
+                    help="gather transfer: host threads pack the records, the scatter kernel reads the pinned staging; file transfer: no staging copy")
     ap.add_argument("--store-path", default=None, help="--transfer file: where the store file is written (default: a temp file)")
     ap.add_argument("--io-depth", type=int, default=0, help="--transfer file: reads in flight (0 = 256; -1 = blocking preads)")
     ap.add_argument("--buffered", action="store_true", help="--transfer file: open the store without O_DIRECT")
@@ -84,7 +84,7 @@ def parse_args():
                          "least this many; ms_per_step is the mean over all of them")
     ap.add_argument("--batch", type=int, default=1, help="sequences per step (the metric's workload is 1)")
     ap.add_argument("--gamma", type=float, default=0.9, help="shared-driver weight of batched hidden states")
-    ap.add_argument("--host-threads", type=int, default=0, help="threads packing records (gather transfer)")
+    ap.add_argument("--host-threads", type=int, default=0, help="threads packing records (gather transfer with --mapped-staging)")
     ap.add_argument("--dense-layers", type=int, default=0,
                     help="dense prefix: the first d layers stay whole on the GPU and take no part in selection or install")
     ap.add_argument("--budget-gib", type=float, default=None,
@@ -749,8 +749,8 @@ def cuda_arm(args):
                     "delta_rows_per_layer": float(cnt[:, nb.NP_CNT_DELTA].mean()), "note": note}
 
         result["variants"] = {
-            "transfer=zerocopy": variant("scatter kernel reads the pinned store over PCIe by neuron ID; no host packing, "
-                                         "no staging copy", transfer_mode=nb.NP_XFER_ZERO_COPY),
+            "transfer=zerocopy": variant("rows pulled from the pinned store by neuron ID whatever the flags; the default "
+                                         "gather transfer does the same without --mapped-staging", transfer_mode=nb.NP_XFER_ZERO_COPY),
             "policy=lru": variant("rows stay resident while capacity allows (least recently predicted leave first): "
                                   "fewer incoming rows per step than under Eq. 3's exact replacement",
                                   evict_policy=nb.NP_EVICT_LRU),

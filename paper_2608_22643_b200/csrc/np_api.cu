@@ -183,10 +183,9 @@ struct np_ctx {
   std::vector<cudaEvent_t> mark;      // the event behind a layer's rows: ev_installed of the last layer of its launch
   std::vector<char> install_pending;
   cudaEvent_t ev_half[kStageParts] = {};        // parts of the host / device staging in flight
-  // library-owned side streams of the install path: [0] runs the scatter kernels behind the
-  // staged copies; in zero-copy mode consecutive layers alternate between the two
-  cudaStream_t aux[2] = {nullptr, nullptr};
-  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr}, ev_copied[kStageParts] = {};
+  // library-owned side stream of the install path: the scatter kernels behind the staged copies
+  cudaStream_t aux = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_copied[kStageParts] = {};
   bool half_pending[kStageParts] = {};
   int next_half = 0;
   // Step timing.  A timing event between two kernels costs about 2 us and keeps the second from starting early, so there
@@ -448,10 +447,8 @@ int np_destroy(np_ctx* ctx) {
     if (e) cudaEventDestroy(e);
   for (auto e : ctx->ev_copied)
     if (e) cudaEventDestroy(e);
-  for (int i = 0; i < 2; ++i) {
-    if (ctx->ev_join[i]) cudaEventDestroy(ctx->ev_join[i]);
-    if (ctx->aux[i]) cudaStreamDestroy(ctx->aux[i]);
-  }
+  if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+  if (ctx->aux) cudaStreamDestroy(ctx->aux);
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   for (auto e : ctx->ev_t)
     if (e) cudaEventDestroy(e);
@@ -643,10 +640,8 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
     NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_installed[l], cudaEventDisableTiming));
   for (auto& e : ctx->ev_half) NP_INIT_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   for (auto& e : ctx->ev_copied) NP_INIT_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  for (int i = 0; i < 2; ++i) {
-    NP_INIT_CUDA(cudaStreamCreateWithFlags(&ctx->aux[i], cudaStreamNonBlocking));
-    NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_join[i], cudaEventDisableTiming));
-  }
+  NP_INIT_CUDA(cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking));
+  NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
   NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
   for (auto& e : ctx->ev_t) NP_INIT_CUDA(cudaEventCreate(&e));
   for (auto& e : ctx->ev_c) NP_INIT_CUDA(cudaEventCreate(&e));
@@ -898,18 +893,18 @@ static int install_from_file(np_ctx* ctx, int layer_begin, int layer_end, cudaSt
     } else {
       NP_CUDA(ctx, cudaMemcpyAsync(dbuf, hbuf, (size_t)c.rows * rec, cudaMemcpyHostToDevice, cs));
       NP_CUDA(ctx, cudaEventRecord(ctx->ev_copied[c.h], cs));
-      NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[0], ctx->ev_copied[c.h], 0));
+      NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux, ctx->ev_copied[c.h], 0));
     }
     NP_LAUNCH(ctx, launch_scatter(d, dbuf, ctx->t.delta_slots + (size_t)c.l * d.C,
                                 ctx->t.counters + (size_t)c.l * NP_N_COUNTERS + NP_CNT_DELTA, c.first, c.rows,
                                 static_cast<char*>(ctx->bufs.gate_buf) + (size_t)(c.l - d.dense) * d.C * row_bytes,
                                 static_cast<char*>(ctx->bufs.up_buf) + (size_t)(c.l - d.dense) * d.C * row_bytes,
                                 static_cast<char*>(ctx->bufs.downT_buf) + (size_t)(c.l - d.dense) * d.C * row_bytes,
-                                ctx->t.status, check, ctx->aux[0], ctx->sm_count));
-    NP_CUDA(ctx, cudaEventRecord(ctx->ev_half[c.h], ctx->aux[0]));  // both copies of the part are free again
+                                ctx->t.status, check, ctx->aux, ctx->sm_count));
+    NP_CUDA(ctx, cudaEventRecord(ctx->ev_half[c.h], ctx->aux));  // both copies of the part are free again
     ctx->half_pending[c.h] = true;
     if (c.last) {
-      NP_CUDA(ctx, mark_installed(ctx, c.l, c.l + 1, ctx->aux[0]));
+      NP_CUDA(ctx, mark_installed(ctx, c.l, c.l + 1, ctx->aux));
     }
     return NP_OK;
   };
@@ -930,7 +925,7 @@ static int install_from_file(np_ctx* ctx, int layer_begin, int layer_end, cudaSt
         queued.pop_front();
         if (rc < 0) return give_up(rc);
       }
-      NP_CUDA(ctx, mark_installed(ctx, l, l + 1, ctx->aux[0]));
+      NP_CUDA(ctx, mark_installed(ctx, l, l + 1, ctx->aux));
       continue;
     }
     for (int first = 0; first < n; first += part_rows) {
@@ -1045,13 +1040,13 @@ static int install_packed(np_ctx* ctx, int layer_begin, int layer_end, int* warn
                                     static_cast<char*>(ctx->bufs.gate_buf) + (size_t)(pc.l - d.dense) * d.C * row_bytes,
                                     static_cast<char*>(ctx->bufs.up_buf) + (size_t)(pc.l - d.dense) * d.C * row_bytes,
                                     static_cast<char*>(ctx->bufs.downT_buf) + (size_t)(pc.l - d.dense) * d.C * row_bytes,
-                                    ctx->t.status, check, ctx->aux[0], ctx->sm_count));
+                                    ctx->t.status, check, ctx->aux, ctx->sm_count));
       if (pc.last) {
-        NP_CUDA(ctx, mark_installed(ctx, pc.l, pc.l + 1, ctx->aux[0]));
+        NP_CUDA(ctx, mark_installed(ctx, pc.l, pc.l + 1, ctx->aux));
       }
     }
     if (used > 0) {
-      NP_CUDA(ctx, cudaEventRecord(ctx->ev_half[h], ctx->aux[0]));  // both copies of the part are free again
+      NP_CUDA(ctx, cudaEventRecord(ctx->ev_half[h], ctx->aux));  // both copies of the part are free again
       ctx->half_pending[h] = true;
     }
     batch.clear();
@@ -1212,13 +1207,13 @@ static int install_enqueue(np_ctx* ctx, int layer_begin, int layer_end, cudaStre
   // kernels run on a side stream: ordered after everything the caller's copy stream holds so far, and joined back into it
   // at the end, so the caller sees one stream's worth of ordering.
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, cs));
-  NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[0], ctx->ev_fork, 0));
+  NP_CUDA(ctx, cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0));
   NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_delta));
   const int rc = mode == NP_XFER_FILE ? install_from_file(ctx, layer_begin, layer_end, cs, warn)
                                       : install_packed(ctx, layer_begin, layer_end, warn);
   if (rc < 0) return rc;
-  NP_CUDA(ctx, cudaEventRecord(ctx->ev_join[0], ctx->aux[0]));
-  NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_join[0], 0));
+  NP_CUDA(ctx, cudaEventRecord(ctx->ev_join, ctx->aux));
+  NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_join, 0));
   return NP_OK;
 }
 
