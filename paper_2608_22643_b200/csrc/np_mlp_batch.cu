@@ -700,6 +700,10 @@ struct Plan {
 bool make_plan(const Dims& d, int rows, bool dense, int nsg, int sm_count, Plan* p) {
   if (d.D % 16 || d.C > 65535) return false;
   const int nkt = d.D / 16;
+  // At least four slices: a block's share of x, and of what it adds to x, shrinks with their number (12 layers' mean at
+  // sixteen sequences: 1024 columns and 400 rows 11.1 us with one slice, 9.3 with two, 8.2 with four; 2432 and 619 14.2 with
+  // two, 13.2 with four).  No more than the operands need: the exchange polls four slices at a time (4096 columns and 1101
+  // rows 16.6 us with four, 23.7 with eight).
   int Q = std::min(4, nkt);
   while (Q <= kMaxQ && (nkt + Q - 1) / Q > kMaxNk) Q *= 2;
   if (Q > kMaxQ || nkt < Q || sm_count < Q) return false;
