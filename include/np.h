@@ -342,7 +342,9 @@ int np_install(np_ctx* ctx, int32_t layer_begin, int32_t layer_end, void* copy_s
 int np_sparse_mlp(np_ctx* ctx, int32_t layer, const float* x, int32_t B, float* y, void* stream);
 
 /* One whole decode step: np_predict, np_delta, np_install of every layer on
- * `copy_stream`, and the pre-normalised residual MLP chain
+ * `copy_stream` (a few rows are pulled on `stream`, in the same order with what
+ * `copy_stream` held on entry and with what is queued on it afterwards), and the
+ * pre-normalised residual MLP chain
  *   x_{l+1} = x_l + MLP_l(n_l),  n_l = x_l / sqrt(mean(x_l^2) + 1e-6)
  * on `stream`, x_0 = x_bf16 widened to fp32 (the RMS normalisation with unit gain stands
  * for the per-layer norm in front of every MLP block of the paper's models).

@@ -355,6 +355,15 @@ int check_device_status(np_ctx* ctx, cudaStream_t s) {
   return NP_OK;
 }
 
+// Orders `s` after what `other` holds now; an idle stream needs no event.
+cudaError_t order_after(cudaStream_t s, cudaStream_t other, cudaEvent_t ev) {
+  const cudaError_t q = cudaStreamQuery(other);
+  if (q != cudaErrorNotReady) return q;
+  (void)cudaGetLastError();
+  const cudaError_t e = cudaEventRecord(ev, other);
+  return e == cudaSuccess ? cudaStreamWaitEvent(s, ev, 0) : e;
+}
+
 // marks layers [l0, l1) installed by what `s` holds now
 cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
   for (int l = l0; l < l1; ++l) {
@@ -1717,7 +1726,11 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   const cudaStream_t is = in_stream ? s : cs;
   ctx->timed_in_stream = in_stream;
   ctx->timed_selected = selected != nullptr;
-  if (!in_stream) {
+  if (in_stream) {
+    // the caller's work on copy_stream (a write to the store, a read of the row buffers) comes before these rows, as it
+    // does where they are pulled on copy_stream itself
+    NP_CUDA(ctx, order_after(s, cs, ctx->ev_fork));
+  } else {
     NP_CUDA(ctx, cudaStreamWaitEvent(cs, ctx->ev_delta, 0));
     NP_CUDA(ctx, cudaEventRecord(ctx->ev_c[0], cs));
   }

@@ -1,0 +1,56 @@
+"""What a step promises about the caller's streams: the order of its rows with the caller's own work."""
+import pytest
+import torch
+
+from paper_2608_22643_b200 import binding as nb
+from paper_2608_22643_b200 import synth
+from tests.harness import Pair
+
+pytestmark = pytest.mark.gpu
+
+TINY = synth.CONFIGS["tiny"]      # one launch pulls the rows of a step
+SMALL = synth.CONFIGS["small"]
+MANY = synth.StackConfig("many", 12, 1024, 2048, 64, 30, 60, 4, 51, 0.9)   # several launches on copy_stream
+
+DELAY = 20_000_000                # cycles of a bounded device-side sleep, about 10 ms; a step of these stacks takes 0.1
+
+
+@pytest.mark.parametrize("mode", [nb.NP_XFER_MEMCPY_RUNS, nb.NP_XFER_HOST_GATHER, nb.NP_XFER_ZERO_COPY])
+@pytest.mark.parametrize("cfg", [TINY, SMALL, MANY])
+def test_rows_wait_for_what_copy_stream_holds(cfg, mode):
+    """A write to the store that copy_stream holds when a step is queued is seen by its rows; a copy of the row buffers
+    that copy_stream holds sees the rows of the step before."""
+    p = Pair(cfg, transfer_mode=mode)
+    try:
+        e = p.eng
+        words = synth.random_bitmaps(cfg.n_layers, cfg.d_ffn, p.k, 5, 4, 0.5)
+        x = synth.hidden_states(cfg, 1)[0].cuda()
+        out = torch.empty((1, cfg.d_model), dtype=torch.float32, device="cuda")
+        fresh = torch.randn(p.backing.shape, generator=torch.Generator().manual_seed(3)).to(torch.bfloat16).cuda()
+        snap = torch.empty_like(e.gate)
+        for t in range(4):
+            before = e.gate.clone()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(e.copy_stream):
+                torch.cuda._sleep(DELAY)
+                snap.copy_(e.gate)
+                if t == 2:
+                    p.backing.copy_(fresh, non_blocking=True)
+            assert not e.copy_stream.query()
+            nb.np_step_selected(e.ctx, x, 1, words[t].cuda(), out, e.stream, e.copy_stream)
+            after = torch.empty_like(e.gate)
+            with torch.cuda.stream(e.copy_stream):      # queued behind the step: sees its rows
+                after.copy_(e.gate)
+            torch.cuda.synchronize()
+            assert torch.equal(snap, before), t
+            assert torch.equal(after, e.gate), t
+            if t == 2:                                   # every row of this step is one of the new records
+                c = e.counters()
+                for l in range(cfg.n_layers):
+                    d = e.delta_lists(l, c[l])
+                    assert len(d["delta_ids"]) > 0
+                    want = fresh[l, torch.from_numpy(d["delta_ids"].copy()).cuda().long()]
+                    for i, buf in enumerate((e.gate, e.up, e.downT)):
+                        assert torch.equal(buf[l, torch.from_numpy(d["delta_slots"].copy()).cuda().long()], want[:, i]), (l, i)
+    finally:
+        p.close()
