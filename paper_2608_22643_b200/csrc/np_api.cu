@@ -364,13 +364,24 @@ cudaError_t order_after(cudaStream_t s, cudaStream_t other, cudaEvent_t ev) {
   return e == cudaSuccess ? cudaStreamWaitEvent(s, ev, 0) : e;
 }
 
-// marks layers [l0, l1) installed by what `s` holds now
+// Marks layers [l0, l1) installed by what `s` holds now.  Rows of those layers that an earlier call put on another stream
+// stay covered: the new mark comes behind theirs, and so does the event recorded here where layers in front of l0 still
+// have it for a mark (their launch ended at l1, too).
 cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
+  const cudaEvent_t ev = ctx->ev_installed[l1 - 1];
+  cudaEvent_t seen = nullptr;
+  for (int l = std::max(0, l0 - 1); l < l1; ++l) {
+    const cudaEvent_t m = ctx->mark[l];
+    if (!ctx->install_pending[l] || m == seen || (l < l0 && m != ev)) continue;
+    seen = m;
+    const cudaError_t e = cudaStreamWaitEvent(s, m, 0);
+    if (e != cudaSuccess) return e;
+  }
   for (int l = l0; l < l1; ++l) {
-    ctx->mark[l] = ctx->ev_installed[l1 - 1];
+    ctx->mark[l] = ev;
     ctx->install_pending[l] = 1;
   }
-  return ctx->rows_in_stream ? cudaSuccess : cudaEventRecord(ctx->ev_installed[l1 - 1], s);  // np_step marks those rows itself
+  return ctx->rows_in_stream ? cudaSuccess : cudaEventRecord(ev, s);  // np_step marks those rows itself
 }
 
 // Orders `s` after the install marks of layers [l0, l1); marks that have already completed need no wait, and layers of

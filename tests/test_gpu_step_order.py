@@ -1,10 +1,12 @@
 """What a step promises about the caller's streams: the order of its rows with the caller's own work."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import np_oracle as O
 from paper_2608_22643_b200 import binding as nb
 from paper_2608_22643_b200 import synth
-from tests.harness import Pair
+from tests.harness import Pair, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -52,5 +54,43 @@ def test_rows_wait_for_what_copy_stream_holds(cfg, mode):
                     want = fresh[l, torch.from_numpy(d["delta_ids"].copy()).cuda().long()]
                     for i, buf in enumerate((e.gate, e.up, e.downT)):
                         assert torch.equal(buf[l, torch.from_numpy(d["delta_slots"].copy()).cuda().long()], want[:, i]), (l, i)
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("second", ["last layer", "speculative"])
+def test_marks_survive_an_install_on_another_stream(second):
+    """A layer's MLP waits for its rows on one stream also after another install has marked that layer, or the last
+    layer of its launch, on a second stream."""
+    cfg = SMALL
+    p = Pair(cfg, transfer_mode=nb.NP_XFER_ZERO_COPY)
+    try:
+        e, L, D = p.eng, cfg.n_layers, cfg.d_model
+        other = torch.cuda.Stream()
+        words = synth.random_bitmaps(L, cfg.d_ffn, p.k, 5, 3, 0.3)
+        x = np.random.default_rng(8).standard_normal((1, D)).astype(np.float32)
+        xd = torch.from_numpy(x).cuda()
+        y = torch.empty((L, 1, D), dtype=torch.float32, device="cuda")
+        for t in range(3):
+            nb.np_delta(e.ctx, words[t].cuda(), e.stream)
+            torch.cuda.synchronize()
+            with torch.cuda.stream(e.copy_stream):
+                torch.cuda._sleep(DELAY)
+            nb.np_install(e.ctx, 0, L, e.copy_stream)
+            if second == "speculative":
+                nb.np_speculate(e.ctx, words[(t + 1) % 3].cuda(), 8, e.stream)
+                nb.np_install_speculative(e.ctx, other)
+            else:
+                nb.np_install(e.ctx, L - 1, L, other)
+            for l in range(L):
+                nb.np_sparse_mlp(e.ctx, l, xd, 1, y[l], e.stream)
+            torch.cuda.synchronize()
+            deltas = p.ora.res.delta(words[t].numpy().view(np.uint32))
+            for l, d in enumerate(deltas):
+                O.install(p.store_u16, p.ora.gate, p.ora.up, p.ora.downT, l, d.delta_ids, d.delta_slots)
+                want = O.sparse_mlp(p.ora.gate, p.ora.up, p.ora.downT, l, d.active_slots, x.astype(np.float64))
+                assert rel_l2(y[l].cpu().numpy(), want) < 1e-5, (t, l)    # fp32 sums of bf16 products: 1e-6
+            if second == "speculative":
+                break                          # the oracle above holds no speculative rows
     finally:
         p.close()
