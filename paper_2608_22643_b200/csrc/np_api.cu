@@ -181,7 +181,7 @@ struct np_ctx {
   cudaEvent_t ev_spec = nullptr;      // the lists of the last np_speculate are written
   std::vector<cudaEvent_t> ev_installed;
   std::vector<cudaEvent_t> mark;      // the event behind a layer's rows: ev_installed of the last layer of its launch
-  std::vector<char> install_pending;
+  std::vector<char> install_pending;  // kLanded, kMarked, kMarkedInCapture
   cudaEvent_t ev_half[kStageParts] = {};        // parts of the host / device staging in flight
   // library-owned side stream of the install path: the scatter kernels behind the staged copies
   cudaStream_t aux = nullptr;
@@ -355,14 +355,38 @@ int check_device_status(np_ctx* ctx, cudaStream_t s) {
   return NP_OK;
 }
 
+// Whether work queued on `s` goes into a graph that is being captured.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+// Asks about work outside of any capture, which a capture that is going on (this thread's or another's) would refuse.
+template <typename Query>
+cudaError_t ask(Query query) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t q = query();
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  if (q == cudaErrorNotReady) (void)cudaGetLastError();
+  return q;
+}
+
 // Orders `s` after what `other` holds now; an idle stream needs no event.
 cudaError_t order_after(cudaStream_t s, cudaStream_t other, cudaEvent_t ev) {
-  const cudaError_t q = cudaStreamQuery(other);
+  const cudaError_t q = ask([&] { return cudaStreamQuery(other); });
   if (q != cudaErrorNotReady) return q;
-  (void)cudaGetLastError();
   const cudaError_t e = cudaEventRecord(ev, other);
   return e == cudaSuccess ? cudaStreamWaitEvent(s, ev, 0) : e;
 }
+
+// np_ctx::install_pending: nothing to wait for; behind the layer's mark; behind a mark that belongs to a capture, which
+// may be waited for but not asked
+enum : char { kLanded = 0, kMarked = 1, kMarkedInCapture = 2 };
 
 // Marks layers [l0, l1) installed by what `s` holds now.  Rows of those layers that an earlier call put on another stream
 // stay covered: the new mark comes behind theirs, and so does the event recorded here where layers in front of l0 still
@@ -377,11 +401,18 @@ cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
     const cudaError_t e = cudaStreamWaitEvent(s, m, 0);
     if (e != cudaSuccess) return e;
   }
+  const char how = capturing(s) ? kMarkedInCapture : kMarked;
   for (int l = l0; l < l1; ++l) {
     ctx->mark[l] = ev;
-    ctx->install_pending[l] = 1;
+    ctx->install_pending[l] = how;
   }
   return ctx->rows_in_stream ? cudaSuccess : cudaEventRecord(ev, s);  // np_step marks those rows itself
+}
+
+// cudaSuccess: the layer's rows have landed; cudaErrorNotReady: they may still be on their way
+cudaError_t ask_installed(const np_ctx* ctx, int l) {
+  if (ctx->install_pending[l] == kMarkedInCapture) return cudaErrorNotReady;
+  return ask([&] { return cudaEventQuery(ctx->mark[l]); });
 }
 
 // Orders `s` after the install marks of layers [l0, l1); marks that have already completed need no wait, and layers of
@@ -394,16 +425,15 @@ cudaError_t wait_installs(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
     if (!ctx->install_pending[l]) continue;
     if (ctx->mark[l] != seen) {
       seen = ctx->mark[l];
-      const cudaError_t q = cudaEventQuery(seen);
+      const cudaError_t q = ask_installed(ctx, l);
       if (q != cudaSuccess && q != cudaErrorNotReady) return q;
       landed = q == cudaSuccess;
       if (!landed) {
-        (void)cudaGetLastError();
         const cudaError_t e = cudaStreamWaitEvent(s, seen, 0);
         if (e != cudaSuccess) return e;
       }
     }
-    if (landed) ctx->install_pending[l] = 0;  // later calls need not ask again
+    if (landed) ctx->install_pending[l] = kLanded;  // later calls need not ask again
   }
   return cudaSuccess;
 }
@@ -1327,11 +1357,8 @@ static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
   for (; landed < d.L; ++landed) {
     if (!ctx->install_pending[landed]) continue;
     if (ctx->mark[landed] != ready) {
-      const cudaError_t q = cudaEventQuery(ctx->mark[landed]);
-      if (q == cudaErrorNotReady) {
-        (void)cudaGetLastError();
-        break;
-      }
+      const cudaError_t q = ask_installed(ctx, landed);
+      if (q == cudaErrorNotReady) break;
       if (q != cudaSuccess) return fail(ctx, NP_E_CUDA, "cudaEventQuery failed: %s", cudaGetErrorString(q));
       ready = ctx->mark[landed];
     }
@@ -1459,18 +1486,23 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
 // kChainTail = the sparse layers and the result.
 // `stepping`: a launch of np_step, beside which rows are pulled.
 static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaStream_t s, int part, bool stepping) {
-  if (B >= kTcMinBatch && ctx->use_batch) return batch_chain(ctx, x_bf16, B, x_out, s, part, stepping);
+  // Into a graph go kernels whose launches may be replayed as they are: the resident ones, the row-partitioned kernel
+  // apart, take counter values and stamps that the host counts up from launch to launch.  (A dense prefix has no per-layer
+  // form for one sequence.)
+  const bool alu = chain_alu::supported(ctx->d, ctx->sm_count);
+  const bool counted = !capturing(s) || (B == 1 && ctx->d.dense > 0 && !alu);
+  const bool use_rows = counted && ctx->use_rows, use_slices = counted && ctx->use_slices;
+  if (B >= kTcMinBatch && ctx->use_batch && counted) return batch_chain(ctx, x_bf16, B, x_out, s, part, stepping);
   const Dims& d = ctx->d;
   const size_t n = (size_t)B * d.D;
-  const bool persistent = B == 1 && !(ctx->cfg.flags & (NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES)) &&
-                          (ctx->use_rows || ctx->use_slices || chain_alu::supported(d, ctx->sm_count));
+  const bool persistent = B == 1 && !(ctx->cfg.flags & (NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES)) && (use_rows || use_slices || alu);
   const bool tc_batch = !persistent && ctx->mlp_tc && B >= kTcMinBatch && !(ctx->cfg.flags & NP_F_DIRECT_LOADS);
   if (part != kChainTail) ctx->chain_kernel_launches = 0;
   // the sliced kernel widens the stack's bf16 input itself when it runs layer 0
-  const bool fold_widen = persistent && (ctx->use_rows || ctx->use_slices) && d.dense == 0;
+  const bool fold_widen = persistent && (use_rows || use_slices) && d.dense == 0;
   // Where the sliced kernel hands its sums over as counted words, layer 0's fp32 accumulator is used only by a
   // first launch of one layer that does not end the stack: the clearing waits until the runs are known.
-  const bool lazy_clear = fold_widen && ctx->use_slices && !ctx->use_rows && chain_slices::counted_handover(d, ctx->sm_count);
+  const bool lazy_clear = fold_widen && use_slices && !use_rows && chain_slices::counted_handover(d, ctx->sm_count);
   bool out_written = false;  // the last resident launch left x_out itself
   if (part != kChainTail) {
     if (!fold_widen) NP_LAUNCH(ctx, launch_widen_bf16(x_bf16, ctx->ws.xbuf[1], n, s));
@@ -1529,11 +1561,11 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
       NP_CUDA(ctx, wait_installs(ctx, l0, l1, s));
       a.l_begin = l0;
       a.l_end = l1;
-      if (ctx->use_rows) {
+      if (use_rows) {
         const int rl = chain_rows::run_layers(d, ctx->rows);
         ctx->chain_kernel_launches += (l1 - l0 + rl - 1) / rl;
         NP_LAUNCH(ctx, chain_rows::launch(d, a, &ctx->rows, s));
-      } else if (ctx->use_slices) {
+      } else if (use_slices) {
         const int sms = resident_sms(ctx, beside_pull, chain_slices::supported);
         chain_slices::Plan sp;
         chain_slices::plan(d, sms, &sp);
@@ -1732,7 +1764,7 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   // Rows that one launch pulls have no MLP launch to run beside: between the delta step and the chain, on their own stream,
   // the launch costs the host no waits across streams (2-layer stack, 40 incoming rows in all, three contexts stepping in
   // turn: 52 us a step with the launch on the copy stream, 47 on the compute stream).
-  const bool in_stream = !head_first && !spec && pulls(ctx) && pull_launches(ctx, d.L) == 1 &&
+  const bool in_stream = !head_first && !spec && !capturing(s) && pulls(ctx) && pull_launches(ctx, d.L) == 1 &&
                          (ctx->cfg.transfer_mode != NP_XFER_MEMCPY_RUNS || !runs_can_be_long(ctx));
   const cudaStream_t is = in_stream ? s : cs;
   ctx->timed_in_stream = in_stream;
