@@ -124,8 +124,9 @@ __global__ void k_split_hidden(const float* __restrict__ hidden, __nv_bfloat16* 
       v = hidden[(size_t)b * H + m];
     }
   }
-  const __nv_bfloat16 t0 = __float2bfloat16_rn(v);
-  v -= __bfloat162float(t0);
+  __nv_bfloat16 t0 = __float2bfloat16_rn(v);
+  if (isinf(__bfloat162float(t0))) t0 = __float2bfloat16_rz(v);  // above the largest bf16: the rest goes into the next term
+  v = isfinite(v) ? v - __bfloat162float(t0) : 0.f;              // an infinity is the first term's alone: what is left of it is no number
   const __nv_bfloat16 t1 = __float2bfloat16_rn(v);
   v -= __bfloat162float(t1);
   const __nv_bfloat16 t2 = __float2bfloat16_rn(v);

@@ -73,3 +73,33 @@ def test_more_selections_than_sms(M, k):
             assert (words[l].cpu().numpy().view(np.uint32) == want).all(), l
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("B", [2, 3, 16])
+def test_hidden_values_at_the_end_of_the_range(B):
+    """A hidden value beyond the largest bf16, and one that overflowed to infinity: the scores are those of the product in
+    64 bits (infinite with the sign of the weight), and the other sequences' scores do not change."""
+    L, M, D, H = 2, 64, 128, 64
+    p = Pair(synth.StackConfig("pr", L, D, M, H, 25, 50, 2, 46, 0.9), max_batch=B, with_oracle=False)
+    try:
+        w1, w2 = p.eng.w1.view(H, D), p.eng.w2.view(L * M, H)
+        w1[5, 0], w1[5, 1] = 1.0, 1.0
+        w1[6, 2] = 4.0
+        x = synth.hidden_states(p.cfg, 1, batch=B)[0].cuda()
+        plain = x.clone()
+        x[0] = 0
+        x[0, 0], x[0, 1] = 3.3895e38, 1.0e36          # hidden value 5 is 3.3995e38: finite, and infinite once rounded to bf16
+        x[1] = 0
+        x[1, 2] = 3.0e38                              # hidden value 6 is 1.2e39: infinite
+        got = torch.empty((B, L * M), dtype=torch.float32, device="cuda")
+        rest = torch.empty((B, L * M), dtype=torch.float32, device="cuda")
+        nb.np_predict(p.eng.ctx, x, B, got, None, p.eng.stream)
+        nb.np_predict(p.eng.ctx, plain, B, rest, None, p.eng.stream)
+        p.eng.counters()
+        hidden = (x[0].double() @ w1.double().T).clamp(min=0)
+        assert 3.396e38 < float(hidden[5]) < 3.4e38
+        assert rel_l2(got[0].cpu().numpy(), (w2.double() @ hidden).cpu().numpy()) < 1e-5
+        assert torch.equal(got[1], torch.sign(w2[:, 6].float()) * float("inf"))
+        assert torch.equal(got[2:], rest[2:])
+    finally:
+        p.close()
