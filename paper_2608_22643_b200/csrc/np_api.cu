@@ -177,7 +177,10 @@ struct np_ctx {
   int32_t* host_lists_dev = nullptr;  // device alias
   const char* backing_dev = nullptr;  // device alias of the record store
   char* hstage_dev = nullptr;         // device alias of the pinned staging (NP_F_MAPPED_STAGING)
-  cudaEvent_t ev_delta = nullptr;
+  cudaEvent_t ev_delta = nullptr;     // behind the last np_delta: one of ev_deltas
+  // Two, so that a np_delta of its own leaves the last step's event (ev_deltas[step_delta]) and its clocks to np_last_step_times.
+  cudaEvent_t ev_deltas[2] = {nullptr, nullptr};
+  int cur_delta = 0, step_delta = -1;
   cudaEvent_t ev_spec = nullptr;      // the lists of the last np_speculate are written
   std::vector<cudaEvent_t> ev_installed;
   std::vector<cudaEvent_t> mark;      // the event behind a layer's rows: ev_installed of the last layer of its launch
@@ -189,10 +192,11 @@ struct np_ctx {
   bool half_pending[kStageParts] = {};
   int next_half = 0;
   // Step timing.  A timing event between two kernels costs about 2 us and keeps the second from starting early, so there
-  // are few: the delta step's own event ends its stage, and its kernel notes how long it took (Tables::clocks).  (2-layer
+  // are few: the delta's event, which the install needs anyway, ends its stage, and its kernel notes how long it took
+  // (Tables::clocks).  (2-layer
   // stack: 62 us a step with seven events on the compute stream, 52 with four.)
   cudaEvent_t ev_t[2] = {nullptr, nullptr};  // compute stream: begin and end of the step
-  cudaEvent_t ev_c[2] = {nullptr, nullptr};  // copy stream: begin and end of the install (rows_in_stream: it begins with ev_delta)
+  cudaEvent_t ev_c[2] = {nullptr, nullptr};  // copy stream: begin and end of the install (rows_in_stream: it begins with the delta's event)
   bool timed_in_stream = false, timed_selected = false;
   bool have_delta = false;
   bool have_spec = false;   // np_speculate has run since the last np_delta
@@ -489,7 +493,8 @@ int np_destroy(np_ctx* ctx) {
   ctx->reader.close();  // nothing may be in flight when the pool and the buffers go
   delete ctx->pool;
   if (ctx->slab) cudaFree(ctx->slab);
-  if (ctx->ev_delta) cudaEventDestroy(ctx->ev_delta);
+  for (auto e : ctx->ev_deltas)
+    if (e) cudaEventDestroy(e);
   if (ctx->ev_spec) cudaEventDestroy(ctx->ev_spec);
   for (auto e : ctx->ev_installed)
     if (e) cudaEventDestroy(e);
@@ -610,7 +615,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   const size_t o_res = take(LW), o_slot = take(LM), o_owner = take(LC), o_stamp = take(LM);
   const size_t o_did = take(LC), o_dsl = take(LC), o_eid = take(LC), o_aid = take(LC), o_asl = take(LC);
   const size_t o_ovf = take(LM), o_cnt = take((size_t)d.L * NP_N_COUNTERS), o_free = take(LC);
-  const size_t o_cid = take(LC), o_ckey = take(LC), o_pred = take(LW), o_stat = take(4), o_bar = take(4), o_clk = take(4);
+  const size_t o_cid = take(LC), o_ckey = take(LC), o_pred = take(LW), o_stat = take(4), o_bar = take(4), o_clk = take(8);
   const size_t o_ident = take(d.dense > 0 ? (size_t)d.M : 1);
   const size_t o_spid = take(LC), o_spsl = take(LC), o_spcnt = take((size_t)d.L * NP_N_COUNTERS), o_spcand = take(LW);
   const size_t o_sfix = take(2 * chain_slices::zfix_words(d)), o_sbar = take(chain_slices::bar_words()), o_sxch = take(2 * chain_slices::xch_words(d, ctx->sm_count));
@@ -639,7 +644,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   t.pred = reinterpret_cast<uint32_t*>(base + o_pred);
   t.status = reinterpret_cast<int32_t*>(base + o_stat);
   t.clocks = reinterpret_cast<unsigned long long*>(base + o_clk);
-  NP_INIT_CUDA(cudaMemset(t.clocks, 0, 16));
+  NP_INIT_CUDA(cudaMemset(t.clocks, 0, 32));
   t.grid_bar = reinterpret_cast<unsigned int*>(base + o_bar);
   t.identity = reinterpret_cast<int32_t*>(base + o_ident);
   t.spec_ids = reinterpret_cast<int32_t*>(base + o_spid);
@@ -681,7 +686,8 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   }
   ctx->gu_bytes = 2 * wl.gu_each;
 
-  NP_INIT_CUDA(cudaEventCreate(&ctx->ev_delta));
+  for (auto& e : ctx->ev_deltas) NP_INIT_CUDA(cudaEventCreate(&e));
+  ctx->ev_delta = ctx->ev_deltas[0];
   NP_INIT_CUDA(cudaEventCreateWithFlags(&ctx->ev_spec, cudaEventDisableTiming));
   ctx->ev_installed.assign(d.L, nullptr);
   ctx->mark.assign(d.L, nullptr);
@@ -901,8 +907,12 @@ int np_delta(np_ctx* ctx, const uint32_t* pred_bitmap, void* stream) {
   }
   // the previous step's installs must have landed before tables and slots are reused
   NP_CUDA(ctx, wait_installs(ctx, 0, ctx->d.L, s));
-  std::fill(ctx->install_pending.begin(), ctx->install_pending.end(), 0);
-  NP_LAUNCH(ctx, launch_delta(ctx->d, ctx->t, pred_bitmap, ctx->cfg.evict_policy, ctx->step, ctx->host_lists_dev,
+  std::fill(ctx->install_pending.begin(), ctx->install_pending.end(), kLanded);
+  if (ctx->cur_delta == ctx->step_delta) ctx->cur_delta ^= 1;
+  ctx->ev_delta = ctx->ev_deltas[ctx->cur_delta];
+  Tables t = ctx->t;
+  t.clocks += 2 * ctx->cur_delta;
+  NP_LAUNCH(ctx, launch_delta(ctx->d, t, pred_bitmap, ctx->cfg.evict_policy, ctx->step, ctx->host_lists_dev,
                             ctx->cfg.flags & NP_F_CHECK_BOUNDS, s));
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_delta, s));
   ctx->step += 1;
@@ -1737,6 +1747,7 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   if (rc < 0) return rc;
   rc = np_delta(ctx, selected, stream);
   if (rc < 0) return rc;
+  ctx->step_delta = ctx->cur_delta;
   // Speculative prefetch behind the step (Section 6's future work).  Its candidates are the rows ranked
   // k+1 .. k+s by this step's own logits (a caller's selection has no ranking to extend: the caller then
   // calls np_speculate itself).  The second selection and the table update run right behind the delta
@@ -1824,14 +1835,16 @@ int np_last_step_times(np_ctx* ctx, float* out_us) {
   if (!ctx->have_step) return fail(ctx, NP_E_STATE, "no np_step has run");
   NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_t[1]));
   NP_CUDA(ctx, cudaEventSynchronize(ctx->ev_c[1]));
-  unsigned long long clocks[2];
-  NP_CUDA(ctx, cudaMemcpy(clocks, ctx->t.clocks, sizeof clocks, cudaMemcpyDeviceToHost));
+  unsigned long long clocks[2];  // read on the library's own stream: other streams of the program are not waited for
+  NP_CUDA(ctx, cudaMemcpyAsync(clocks, ctx->t.clocks + 2 * ctx->step_delta, sizeof clocks, cudaMemcpyDeviceToHost, ctx->aux));
+  NP_CUDA(ctx, cudaStreamSynchronize(ctx->aux));
+  const cudaEvent_t ev_delta = ctx->ev_deltas[ctx->step_delta];
   float ms[4];
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[0], ctx->ev_t[0], ctx->ev_delta));
+  NP_CUDA(ctx, cudaEventElapsedTime(&ms[0], ctx->ev_t[0], ev_delta));
   ms[1] = clocks[1] > clocks[0] ? std::min(ms[0], (float)(clocks[1] - clocks[0]) * 1e-6f) : 0.f;
   ms[0] = ctx->timed_selected ? 0.f : ms[0] - ms[1];
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[2], ctx->timed_in_stream ? ctx->ev_delta : ctx->ev_c[0], ctx->ev_c[1]));
-  NP_CUDA(ctx, cudaEventElapsedTime(&ms[3], ctx->ev_delta, ctx->ev_t[1]));
+  NP_CUDA(ctx, cudaEventElapsedTime(&ms[2], ctx->timed_in_stream ? ev_delta : ctx->ev_c[0], ctx->ev_c[1]));
+  NP_CUDA(ctx, cudaEventElapsedTime(&ms[3], ev_delta, ctx->ev_t[1]));
   for (int i = 0; i < 4; ++i) out_us[i] = ms[i] * 1000.f;
   return NP_OK;
 }

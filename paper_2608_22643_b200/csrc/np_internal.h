@@ -43,7 +43,7 @@ struct Tables {
   int32_t* spec_ids;      // [L][C]  rows made resident ahead of time by the last np_speculate
   int32_t* spec_slots;    // [L][C]
   int32_t* spec_counters; // [L][NP_N_COUNTERS] their count sits at NP_CNT_DELTA (the install path reads it there)
-  unsigned long long* clocks;  // [2]  start and end of the last delta kernel, nanoseconds (the end only grows)
+  unsigned long long* clocks;  // [2][2]  start and end of a delta kernel, nanoseconds (the end only grows); np_delta takes a pair
   uint32_t* spec_cand;    // [L][W]  candidate bitmap of np_step's own speculation
 };
 

@@ -94,3 +94,34 @@ def test_marks_survive_an_install_on_another_stream(second):
                 break                          # the oracle above holds no speculative rows
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("cfg", [TINY, MANY])
+def test_step_times_are_those_of_the_step(cfg):
+    """np_last_step_times after other calls, one of them not finished, reports what it reported right behind the step, and
+    waits for no work of the program's own."""
+    p = Pair(cfg, with_oracle=False)
+    try:
+        e = p.eng
+        words = synth.random_bitmaps(cfg.n_layers, cfg.d_ffn, p.k, 5, 4, 0.5)
+        x = synth.hidden_states(cfg, 1)[0].cuda()
+        out = torch.empty((1, cfg.d_model), dtype=torch.float32, device="cuda")
+        later = words[1:].cuda()
+        for t in range(3):
+            nb.np_step(e.ctx, x, 1, out, e.stream, e.copy_stream)
+            first = nb.np_last_step_times(e.ctx)
+            assert (first > 0).all(), t
+            nb.np_delta(e.ctx, words[t].cuda(), e.stream)
+            nb.np_install(e.ctx, 0, cfg.n_layers, e.copy_stream)
+            assert (nb.np_last_step_times(e.ctx) == first).all(), t
+            torch.cuda.synchronize()
+            torch.cuda._sleep(10 * DELAY)
+            with torch.cuda.stream(e.stream):
+                torch.cuda._sleep(DELAY)
+            nb.np_delta(e.ctx, later[t], e.stream)
+            assert (nb.np_last_step_times(e.ctx) == first).all(), t
+            assert not torch.cuda.default_stream().query() and not e.stream.query(), t
+            torch.cuda.synchronize()
+            nb.np_install(e.ctx, 0, cfg.n_layers, e.copy_stream)
+    finally:
+        p.close()
