@@ -1411,7 +1411,8 @@ static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
 }
 
 // SMs for a resident launch.  One that runs while rows are pulled leaves the pull kernel its SMs: on all of them it would
-// not start before the last row has landed.  Every launch of a step does so, also those that no pull of the same step runs
+// not start before the last row has landed.  The run that ends the stack has waited for its context's rows and, outside a
+// step, takes all SMs whatever is in flight when it is queued (a chain in one launch gives the same bits each time).  Every launch of a step does so, also those that no pull of the same step runs
 // beside: other contexts pull, too, and a launch on all SMs would wait for them (2.7 % of the SMs; a step of the 7B shape
 // with 24 dense layers is 1.22 ms this way and 1.25 with the dense layers cut in two launches, the second on all SMs).
 static int resident_sms(const np_ctx* ctx, bool beside_pull, bool (*fits)(const Dims&, int)) {
@@ -1476,13 +1477,12 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
   std::vector<int> runs;
   int rc = sparse_runs(ctx, &runs);
   if (rc < 0) return rc;
-  const bool beside_pull = stepping || ctx->install_pending[d.L - 1];
   int l0 = d.dense;
   for (const int n : runs) {
     NP_CUDA(ctx, wait_installs(ctx, l0, l0 + n, s));
     a.l_begin = l0;
     a.l_end = l0 += n;
-    rc = batch_run(ctx, a, x, B, beside_pull, s);
+    rc = batch_run(ctx, a, x, B, stepping || (l0 < d.L && ctx->install_pending[d.L - 1]), s);
     if (rc < 0) return rc;
   }
   NP_LAUNCH(ctx, chain_batch::launch_out(d, x, x_out, B, s));
@@ -1564,11 +1564,11 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
       const int rc = sparse_runs(ctx, &runs);
       if (rc < 0) return rc;
     }
-    const bool beside_pull = stepping || ctx->install_pending[d.L - 1];
     int l0 = d.dense;
     for (size_t ri = 0; ri < runs.size() && part != kChainHead; ++ri) {
       const int l1 = l0 + runs[ri];
       NP_CUDA(ctx, wait_installs(ctx, l0, l1, s));
+      const bool beside_pull = stepping || (l1 < d.L && ctx->install_pending[d.L - 1]);
       a.l_begin = l0;
       a.l_end = l1;
       if (use_rows) {

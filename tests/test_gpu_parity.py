@@ -347,6 +347,29 @@ def test_chain_in_one_launch_is_reproducible_bit_for_bit():
         p.close()
 
 
+def test_chain_in_one_launch_does_not_depend_on_rows_in_flight():
+    """The launch waits for every row, so whether they had landed when it was queued shows in no bit."""
+    cfg = DENSE
+    p = Pair(cfg, chain_layers=cfg.n_layers, transfer_mode=nb.NP_XFER_ZERO_COPY, with_oracle=False)
+    try:
+        words = synth.random_bitmaps(cfg.n_layers, cfg.d_ffn, p.k, 5, 3, 0.5)
+        x = synth.hidden_states(cfg, 1)[0].cuda()
+        outs = torch.empty((2, 1, cfg.d_model), dtype=torch.float32, device="cuda")
+        for t in range(3):
+            nb.np_delta(p.eng.ctx, words[t].cuda(), p.eng.stream)
+            torch.cuda.synchronize()
+            with torch.cuda.stream(p.eng.copy_stream):
+                torch.cuda._sleep(20_000_000)             # about 10 ms: the rows are on their way when the chain is queued
+            nb.np_install(p.eng.ctx, 0, cfg.n_layers, p.eng.copy_stream)
+            for o in outs:
+                nb.np_mlp_chain(p.eng.ctx, x, 1, o, p.eng.stream)
+                assert nb.np_chain_launches(p.eng.ctx) == 1
+                torch.cuda.synchronize()
+            assert torch.equal(outs[0].view(torch.int32), outs[1].view(torch.int32)), t
+    finally:
+        p.close()
+
+
 def test_partial_sums_beyond_the_counted_words_range_are_reported():
     """Between the layers of a launch the resident kernel hands the MLP's partial sums over as counted
     fixed-point words (|sum| < 2^19 per block).  Down rows of 3e6 push layer 0 far past that: the launch
