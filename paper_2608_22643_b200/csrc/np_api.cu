@@ -1174,6 +1174,20 @@ static int pull_launches(const np_ctx* ctx, int n) {
   return std::max(1, std::min(8, n / std::max(1, least)));
 }
 
+// Whether a dense prefix takes longer than the rows of `ns` layers do (an eighth of a set per layer at 50 GB/s, half as much
+// again; a dense layer streams at 6 TB/s).
+static bool rows_hide_behind_dense(const np_ctx* ctx, int ns) {
+  const Dims& d = ctx->d;
+  const double pull_s = 1.5 * ns * (d.k / 8.0) * (double)d.rec_bytes / 50e9, dense_s = d.dense * ((double)d.M * 6.0 * d.D / 6e12);
+  return pull_s < dense_s;
+}
+
+// SMs of a pull (k_pull_rows): two for bf16 records; four for 8-bit ones, where anything waits for them.  (7B shape, 24 dense
+// layers and 8-bit records, three such stacks stepping in turn: 1.32 ms a step with four, 1.26 with two.)
+static int pull_blocks(const np_ctx* ctx) {
+  return ctx->d.rec_int8 && !rows_hide_behind_dense(ctx, ctx->d.L - ctx->d.dense) ? 4 : 2;
+}
+
 static int install_pull(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_t cs) {
   const Dims& d = ctx->d;
   const int n = layer_end - layer_begin;
@@ -1182,7 +1196,7 @@ static int install_pull(np_ctx* ctx, int layer_begin, int layer_end, cudaStream_
   for (int g = 0; g < launches; ++g) {
     const int l0 = layer_begin + (int)((long long)n * g / launches), l1 = layer_begin + (int)((long long)n * (g + 1) / launches);
     NP_LAUNCH(ctx, launch_pull(d, ctx->t, ctx->backing_dev, ctx->bufs.gate_buf, ctx->bufs.up_buf, ctx->bufs.downT_buf, l0, l1,
-                               ctx->cfg.flags & NP_F_CHECK_BOUNDS, cs));
+                               pull_blocks(ctx), ctx->cfg.flags & NP_F_CHECK_BOUNDS, cs));
     NP_CUDA(ctx, mark_installed(ctx, l0, l1, cs));
   }
   return NP_OK;
@@ -1375,16 +1389,12 @@ static int sparse_runs(np_ctx* ctx, std::vector<int>* runs) {
     ctx->install_pending[landed] = 0;
   }
   const int ns = d.L - landed;  // layers that still wait for rows
-  // Behind a dense prefix that takes longer than the rows do (an eighth of a set per layer at 50 GB/s, half as much again;
-  // a dense layer streams at 6 TB/s) there is nothing to wait for either.  (7B shape, 24 dense layers: 1.195 ms a step with
-  // one run, 1.215 with three; three such stacks stepping in turn 1.26 and 1.41: a resident launch of one context delays
-  // those of the others.)
-  if (pulls(ctx) && d.dense > 0 && ctx->cfg.chain_layers == 0 && d.dense < d.L) {
-    const double pull_s = 1.5 * ns * (d.k / 8.0) * (double)d.rec_bytes / 50e9, dense_s = d.dense * ((double)d.M * 6.0 * d.D / 6e12);
-    if (pull_s < dense_s) {
-      runs->push_back(d.L - d.dense);
-      return NP_OK;
-    }
+  // Behind a dense prefix that takes longer than the rows do there is nothing to wait for either.  (7B shape, 24 dense
+  // layers: 1.195 ms a step with one run, 1.215 with three; three such stacks stepping in turn 1.26 and 1.41: a resident
+  // launch of one context delays those of the others.)
+  if (pulls(ctx) && d.dense > 0 && ctx->cfg.chain_layers == 0 && d.dense < d.L && rows_hide_behind_dense(ctx, ns)) {
+    runs->push_back(d.L - d.dense);
+    return NP_OK;
   }
   if (ctx->cfg.chain_layers > 0) {
     const int run = ctx->cfg.chain_layers;

@@ -138,8 +138,8 @@ cudaError_t launch_scatter(const Dims& d, const void* src, const int32_t* slots,
                            cudaStream_t s, int sm_count);
 // the incoming rows of layers [l_begin, l_end), read from the pinned store by neuron ID and placed
 cudaError_t launch_pull(const Dims& d, const Tables& t, const char* store_dev, void* gate, void* up, void* downT, int l_begin,
-                        int l_end, int check, cudaStream_t s);
-// SMs that resident kernels leave free where rows are pulled beside them: room for the pulls of two contexts
+                        int l_end, int blocks, int check, cudaStream_t s);
+// SMs that resident kernels leave free where rows are pulled beside them: room for the pulls of two contexts (of one, 8-bit records)
 constexpr int kPullReserve = 4;
 
 cudaError_t launch_dequant_dense_layer(const Dims& d, const void* store_l, const int32_t* identity, void* dense_l,

@@ -152,21 +152,29 @@ cudaError_t launch_scatter(const Dims& d, const void* src, const int32_t* slots,
 // ---------------------------------------------------------------------------------------
 // Transfer and placement in one: the incoming rows of several layers, read by neuron ID from the pinned store.
 //
-// What bounds it is the host link.  Reads of 128-byte lines, 512 bytes a warp instruction, 150 to 250 KB in flight over
-// the machine, reach 51.2 GB/s on random 24 KB records where one contiguous copy of the same bytes reaches 55.1; more in
-// flight gives nothing.  Packing the records with the host's cores and copying the packed parts gives 39 to 48 depending
-// on the host (the packing reads and writes every byte in host memory beside the copy's own reads), and a copy call per
-// record 5.4.  A step of the 7B shape (145 MB of incoming rows): 3.16 ms packed and copied, 2.97 pulled.
+// What bounds it is the host link, and in front of that the reads in flight: 128-byte lines, 512 bytes a warp instruction,
+// about 4.5 us each.  The 147 MB of incoming rows of a 7B-shaped step, one context on its own (one contiguous copy of the
+// same bytes: 55.1 GB/s; the store's size, 8.7 GB or an eighth of that, makes no difference):
 //
-// Two SMs are enough for that, with 1024 threads each and six loads in flight per lane (four: 3.00 ms; one SM: 4.4 ms;
-// four SMs: 2.97 as well).  The others are left to the resident MLP kernels, which are launched narrower while rows are on
-// their way (kPullReserve).  A kernel on all SMs, small enough to fit beside the resident blocks, was no faster, and the
-// resident kernels lost 7 % by giving up the registers.  A piece is 384 units of 16 bytes (two rounds of loads), taken
-// from the 128-byte line the record starts in, so that a warp's accesses are whole lines also for records that are not a
-// multiple of 128 bytes; the last piece takes what is left.
+//   two SMs of 1024 threads, six loads in flight per lane   44.4 GB/s    301 steps/s
+//   two SMs, eight loads per lane                           49.6         332
+//   three SMs, six / eight                                  46.9 / 50.0  316 / 337
+//   four / six SMs, six loads                               48.1 / 49.0  324 / 330
+//
+// Two SMs with eight loads it is: every further SM is one less for the resident MLP kernels, which are launched narrower
+// while rows are on their way (kPullReserve; two such kernels fit, and two contexts stepping in turn reach 51 GB/s with
+// six or eight loads).  Packing the records with the host's cores and copying the packed parts gives 40 to 47 depending
+// on the host (304 to 315 steps/s; the packing reads and writes every byte in host memory beside the copy's own reads),
+// and a copy call per record 4.8.  A kernel on all SMs, small enough to fit beside the resident blocks, was no faster, and
+// the resident kernels lost 7 % by giving up the registers.
+//
+// 8-bit records: a lane's dequantising adds to the trip of its loads, and there are no registers for eight (25.9 GB/s with
+// them, 26.5 with six, 357 steps/s).  They take four SMs: 44.6 GB/s, 573 steps/s (pull_blocks on where they do not).
+//
+// A piece is 384 units of 16 bytes, taken from the 128-byte line the record starts in, so that a warp's accesses are whole
+// lines also for records that are not a multiple of 128 bytes; the last piece takes what is left.
 // ---------------------------------------------------------------------------------------
 constexpr int kPullThreads = 1024;
-constexpr int kPullBlocks = 2;
 constexpr int kPullUnits = 384;
 
 struct PullArgs {
@@ -184,7 +192,7 @@ struct PullArgs {
 
 template <bool kInt8>
 __global__ void __launch_bounds__(kPullThreads) k_pull_rows(PullArgs a) {
-  constexpr int U = 6;  // loads a lane has in flight
+  constexpr int U = kInt8 ? 6 : 8;  // loads a lane has in flight
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (kPullThreads / 32);
   const int row_units = kInt8 ? a.D >> 4 : a.D >> 3;             // 16-byte units of a source row
@@ -254,7 +262,7 @@ __global__ void __launch_bounds__(kPullThreads) k_pull_rows(PullArgs a) {
 }
 
 cudaError_t launch_pull(const Dims& d, const Tables& t, const char* store_dev, void* gate, void* up, void* downT, int l_begin,
-                        int l_end, int check, cudaStream_t s) {
+                        int l_end, int blocks, int check, cudaStream_t s) {
   PullArgs a;
   a.store = store_dev;
   a.ids = t.delta_ids;
@@ -273,8 +281,8 @@ cudaError_t launch_pull(const Dims& d, const Tables& t, const char* store_dev, v
   a.C = d.C;
   a.Lp = d.Lp;
   a.check = check;
-  if (d.rec_int8) k_pull_rows<true><<<kPullBlocks, kPullThreads, 0, s>>>(a);
-  else k_pull_rows<false><<<kPullBlocks, kPullThreads, 0, s>>>(a);
+  if (d.rec_int8) k_pull_rows<true><<<blocks, kPullThreads, 0, s>>>(a);
+  else k_pull_rows<false><<<blocks, kPullThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
