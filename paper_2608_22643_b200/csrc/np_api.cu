@@ -185,6 +185,7 @@ struct np_ctx {
   std::vector<cudaEvent_t> ev_installed;
   std::vector<cudaEvent_t> mark;      // the event behind a layer's rows: ev_installed of the last layer of its launch
   std::vector<char> install_pending;  // kLanded, kMarked, kMarkedInCapture
+  bool in_call = false, capturing = false;  // see Call
   cudaEvent_t ev_half[kStageParts] = {};        // parts of the host / device staging in flight
   // library-owned side stream of the install path: the scatter kernels behind the staged copies
   cudaStream_t aux = nullptr;
@@ -359,31 +360,34 @@ int check_device_status(np_ctx* ctx, cudaStream_t s) {
   return NP_OK;
 }
 
-// Whether work queued on `s` goes into a graph that is being captured.
-bool capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return false;
-  }
-  return st != cudaStreamCaptureStatusNone;
-}
-
-// Asks about work outside of any capture, which a capture that is going on (this thread's or another's) would refuse.
-template <typename Query>
-cudaError_t ask(Query query) {
+// A call of the library that queues work on `s`: whether that work goes into a graph that is being captured, asked once, and
+// the leave to ask streams and events about work outside of any capture, which a capture that is going on (this thread's or
+// another's) would refuse.  Calls within a call take the outer one's answers: with every part asking for itself a short step
+// took 2 to 6 % longer (20 layers, three contexts stepping in turn: 150 us).
+struct Call {
+  np_ctx* ctx = nullptr;
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  (void)cudaThreadExchangeStreamCaptureMode(&mode);
-  const cudaError_t q = query();
-  (void)cudaThreadExchangeStreamCaptureMode(&mode);
-  if (q == cudaErrorNotReady) (void)cudaGetLastError();
-  return q;
-}
+  Call(np_ctx* c, cudaStream_t s) {
+    if (c->in_call) return;
+    ctx = c;
+    ctx->in_call = true;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) (void)cudaGetLastError();
+    ctx->capturing = st != cudaStreamCaptureStatusNone;
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  ~Call() {
+    if (!ctx) return;
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    ctx->in_call = ctx->capturing = false;
+  }
+};
 
 // Orders `s` after what `other` holds now; an idle stream needs no event.
 cudaError_t order_after(cudaStream_t s, cudaStream_t other, cudaEvent_t ev) {
-  const cudaError_t q = ask([&] { return cudaStreamQuery(other); });
+  const cudaError_t q = cudaStreamQuery(other);
   if (q != cudaErrorNotReady) return q;
+  (void)cudaGetLastError();
   const cudaError_t e = cudaEventRecord(ev, other);
   return e == cudaSuccess ? cudaStreamWaitEvent(s, ev, 0) : e;
 }
@@ -405,10 +409,9 @@ cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
     const cudaError_t e = cudaStreamWaitEvent(s, m, 0);
     if (e != cudaSuccess) return e;
   }
-  const char how = capturing(s) ? kMarkedInCapture : kMarked;
   for (int l = l0; l < l1; ++l) {
     ctx->mark[l] = ev;
-    ctx->install_pending[l] = how;
+    ctx->install_pending[l] = ctx->capturing ? kMarkedInCapture : kMarked;
   }
   return ctx->rows_in_stream ? cudaSuccess : cudaEventRecord(ev, s);  // np_step marks those rows itself
 }
@@ -416,7 +419,9 @@ cudaError_t mark_installed(np_ctx* ctx, int l0, int l1, cudaStream_t s) {
 // cudaSuccess: the layer's rows have landed; cudaErrorNotReady: they may still be on their way
 cudaError_t ask_installed(const np_ctx* ctx, int l) {
   if (ctx->install_pending[l] == kMarkedInCapture) return cudaErrorNotReady;
-  return ask([&] { return cudaEventQuery(ctx->mark[l]); });
+  const cudaError_t q = cudaEventQuery(ctx->mark[l]);
+  if (q == cudaErrorNotReady) (void)cudaGetLastError();
+  return q;
 }
 
 // Orders `s` after the install marks of layers [l0, l1); marks that have already completed need no wait, and layers of
@@ -897,6 +902,7 @@ int np_delta(np_ctx* ctx, const uint32_t* pred_bitmap, void* stream) {
     pred_bitmap = ctx->t.pred;
   }
   cudaStream_t s = as_stream(stream);
+  const Call call(ctx, s);
   if (ctx->d.dense > 0 && pred_bitmap != ctx->t.pred) {
     // a caller's bitmap may name rows of dense layers; those layers select nothing
     const size_t skip = (size_t)ctx->d.dense * ctx->d.W;
@@ -1299,6 +1305,7 @@ int np_install(np_ctx* ctx, int32_t layer_begin, int32_t layer_end, void* copy_s
   int warn = NP_OK;
   bool late = false;
   NP_CUDA(ctx, cudaStreamWaitEvent(as_stream(copy_stream), ctx->ev_delta, 0));
+  const Call call(ctx, as_stream(copy_stream));  // behind the wait, which takes the stream into the capture of the delta step
   int rc = install_enqueue(ctx, layer_begin, layer_end, as_stream(copy_stream), &warn, &late);
   if (rc >= 0 && late) rc = install_warnings(ctx, layer_begin, layer_end, &warn);
   return rc < 0 ? rc : warn;
@@ -1509,13 +1516,13 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
   // Into a graph go kernels whose launches may be replayed as they are: the resident ones, the row-partitioned kernel
   // apart, take counter values and stamps that the host counts up from launch to launch.  (A dense prefix has no per-layer
   // form for one sequence.)
-  const bool alu = chain_alu::supported(ctx->d, ctx->sm_count);
-  const bool counted = !capturing(s) || (B == 1 && ctx->d.dense > 0 && !alu);
+  const auto alu = [&] { return chain_alu::supported(ctx->d, ctx->sm_count); };
+  const bool counted = !ctx->capturing || (B == 1 && ctx->d.dense > 0 && !alu());
   const bool use_rows = counted && ctx->use_rows, use_slices = counted && ctx->use_slices;
   if (B >= kTcMinBatch && ctx->use_batch && counted) return batch_chain(ctx, x_bf16, B, x_out, s, part, stepping);
   const Dims& d = ctx->d;
   const size_t n = (size_t)B * d.D;
-  const bool persistent = B == 1 && !(ctx->cfg.flags & (NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES)) && (use_rows || use_slices || alu);
+  const bool persistent = B == 1 && !(ctx->cfg.flags & (NP_F_DIRECT_LOADS | NP_F_LAYER_LAUNCHES)) && (use_rows || use_slices || alu());
   const bool tc_batch = !persistent && ctx->mlp_tc && B >= kTcMinBatch && !(ctx->cfg.flags & NP_F_DIRECT_LOADS);
   if (part != kChainTail) ctx->chain_kernel_launches = 0;
   // the sliced kernel widens the stack's bf16 input itself when it runs layer 0
@@ -1637,6 +1644,7 @@ int np_mlp_chain(np_ctx* ctx, const void* x_bf16, int32_t B, float* x_out, void*
   if ((uintptr_t)x_out % 16) return fail(ctx, NP_E_INVAL, "x_out must be 16-byte aligned");
   if (B < 1 || B > ctx->d.Bmax) return fail(ctx, NP_E_INVAL, "B=%d outside [1, max_batch=%d]", B, ctx->d.Bmax);
   if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_mlp_chain needs a prior np_delta");
+  const Call call(ctx, as_stream(stream));
   return mlp_chain(ctx, x_bf16, B, x_out, as_stream(stream), kChainAll, false);
 }
 
@@ -1654,6 +1662,7 @@ int np_speculate(np_ctx* ctx, const uint32_t* cand_bitmap, int32_t budget, void*
   if (budget < 0) return fail(ctx, NP_E_INVAL, "budget must be >= 0");
   if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_speculate needs a prior np_delta");
   cudaStream_t s = as_stream(stream);
+  const Call call(ctx, s);
   // rows brought in ahead of time by an earlier call must have landed before their tables move again
   if (ctx->have_spec) NP_CUDA(ctx, wait_installs(ctx, 0, ctx->d.L, s));
   NP_LAUNCH(ctx, launch_speculate(ctx->d, ctx->t, cand_bitmap, std::min(budget, ctx->d.C),
@@ -1735,6 +1744,7 @@ int np_sparse_mlp(np_ctx* ctx, int32_t layer, const float* x, int32_t B, float* 
   if (B < 1 || B > d.Bmax) return fail(ctx, NP_E_INVAL, "B=%d outside [1, max_batch=%d]", B, d.Bmax);
   if (!ctx->have_delta) return fail(ctx, NP_E_STATE, "np_sparse_mlp needs a prior np_delta");
   cudaStream_t s = as_stream(stream);
+  const Call call(ctx, s);
   NP_CUDA(ctx, cudaMemsetAsync(y, 0, (size_t)B * d.D * 4, s));
   if (ctx->mlp_tc && B >= kTcMinBatch) NP_CUDA(ctx, cudaMemsetAsync(ctx->ws.gu[0], 0, ctx->gu_bytes / 2, s));
   return mlp_layer(ctx, layer, x, nullptr, y, nullptr, nullptr, B, 0, -1, s);
@@ -1751,6 +1761,7 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   if (stream == copy_stream) return fail(ctx, NP_E_INVAL, "a step needs two different streams");
   const Dims& d = ctx->d;
   cudaStream_t s = as_stream(stream), cs = as_stream(copy_stream);
+  const Call call(ctx, s);
   NP_CUDA(ctx, cudaEventRecord(ctx->ev_t[0], s));
   int rc = NP_OK;
   if (!selected) rc = np_predict(ctx, x_bf16, B, nullptr, nullptr, stream);
@@ -1785,7 +1796,7 @@ static int step_impl(np_ctx* ctx, const void* x_bf16, int32_t B, const uint32_t*
   // Rows that one launch pulls have no MLP launch to run beside: between the delta step and the chain, on their own stream,
   // the launch costs the host no waits across streams (2-layer stack, 40 incoming rows in all, three contexts stepping in
   // turn: 52 us a step with the launch on the copy stream, 47 on the compute stream).
-  const bool in_stream = !head_first && !spec && !capturing(s) && pulls(ctx) && pull_launches(ctx, d.L) == 1 &&
+  const bool in_stream = !head_first && !spec && !ctx->capturing && pulls(ctx) && pull_launches(ctx, d.L) == 1 &&
                          (ctx->cfg.transfer_mode != NP_XFER_MEMCPY_RUNS || !runs_can_be_long(ctx));
   const cudaStream_t is = in_stream ? s : cs;
   ctx->timed_in_stream = in_stream;
