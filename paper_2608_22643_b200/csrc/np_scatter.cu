@@ -175,7 +175,7 @@ cudaError_t launch_scatter(const Dims& d, const void* src, const int32_t* slots,
 // lines also for records that are not a multiple of 128 bytes; the last piece takes what is left.
 // ---------------------------------------------------------------------------------------
 constexpr int kPullThreads = 1024;
-constexpr int kPullUnits = 384;
+constexpr int kPullLoads = 6;  // loads a lane has in flight
 
 struct PullArgs {
   const char* store;        // device alias of the pinned store
@@ -188,76 +188,81 @@ struct PullArgs {
   int32_t* status;
   size_t rec_bytes;
   int l_begin, l_end, dense, D, M, C, Lp, check;
+  int pieces, piece;  // pieces of a record, 16-byte units of a piece
 };
 
 template <bool kInt8>
 __global__ void __launch_bounds__(kPullThreads) k_pull_rows(PullArgs a) {
-  constexpr int U = kInt8 ? 6 : 8;  // loads a lane has in flight
+  constexpr int U = kPullLoads;
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (kPullThreads / 32);
   const int row_units = kInt8 ? a.D >> 4 : a.D >> 3;             // 16-byte units of a source row
-  const int pieces = max(1, (3 * row_units + kPullUnits / 2) / kPullUnits);  // per record
-  // the first piece of the layer that is this warp's: the deal goes on where it stopped in the layer before
+  const int pieces = a.pieces;
+  auto pieces_of = [&](int l) { return min(max(a.counters[(size_t)l * NP_N_COUNTERS + NP_CNT_DELTA], 0), a.C) * pieces; };
+  // this warp's pieces are every nw-th of all layers' in a row: i counts from the start of layer l
+  int l = a.l_begin, total = pieces_of(l), id = 0, slot = 0;
   int i = blockIdx.x * (kPullThreads / 32) + (threadIdx.x >> 5);
-  for (int l = a.l_begin; l < a.l_end; ++l) {
-    const int total = min(max(a.counters[(size_t)l * NP_N_COUNTERS + NP_CNT_DELTA], 0), a.C) * pieces;
-    const int32_t* ids = a.ids + (size_t)l * a.C;
-    const int32_t* slots = a.slots + (size_t)l * a.C;
-    int next_id = 0, next_slot = 0;
-    if (i < total) next_id = ids[i / pieces], next_slot = slots[i / pieces];
-    for (; i < total; i += nw) {
-      const int p = i % pieces;
-      const int id = next_id, slot = next_slot;
-      if (i + nw < total) next_id = ids[(i + nw) / pieces], next_slot = slots[(i + nw) / pieces];  // on their way beside the rows
-      if (a.check && (id < 0 || id >= a.M || slot < 0 || slot >= a.C)) {
-        if (lane == 0) atomicOr(a.status, id < 0 || id >= a.M ? kStatBadNeuron : kStatBadSlot);
-        continue;
-      }
-      const char* rec = a.store + ((size_t)(l % a.Lp) * a.M + id) * a.rec_bytes;
-      const size_t dst = ((size_t)(l - a.dense) * a.C + slot) * a.D * 2;
-      const int mis = (int)((reinterpret_cast<uintptr_t>(rec) >> 4) & 7);  // units between the line's start and the record
-      const int end = p + 1 < pieces ? (p + 1) * kPullUnits - mis : 3 * row_units;
-      float sc[3];
-      if (kInt8) {
-        const uint4 s4 = ldg_stream(rec + (size_t)3 * a.D);
-        sc[0] = __uint_as_float(s4.x), sc[1] = __uint_as_float(s4.y), sc[2] = __uint_as_float(s4.z);
-      }
-#pragma unroll 1
-      for (int v0 = p * kPullUnits - mis + lane; v0 < end; v0 += U * 32) {
-        uint4 x[U];
+  auto settle = [&] {  // to the layer that holds piece i, and its list entry
+    while (i >= total) {
+      i -= total;
+      if (++l == a.l_end) return;
+      total = pieces_of(l);
+    }
+    id = a.ids[(size_t)l * a.C + i / pieces];
+    slot = a.slots[(size_t)l * a.C + i / pieces];
+  };
+  settle();
+  while (l < a.l_end) {
+    const int p = i % pieces;
+    if (a.check && (id < 0 || id >= a.M || slot < 0 || slot >= a.C)) {
+      if (lane == 0) atomicOr(a.status, id < 0 || id >= a.M ? kStatBadNeuron : kStatBadSlot);
+      i += nw;
+      settle();
+      continue;
+    }
+    const char* rec = a.store + ((size_t)(l % a.Lp) * a.M + id) * a.rec_bytes;
+    const size_t dst = ((size_t)(l - a.dense) * a.C + slot) * a.D * 2;
+    const int mis = (int)((reinterpret_cast<uintptr_t>(rec) >> 4) & 7);  // units between the line's start and the record
+    const int end = min((p + 1) * a.piece - mis, 3 * row_units);
+    const int v0 = p * a.piece - mis + lane;
+    float sc[3];
+    if (kInt8) {
+      const uint4 s4 = ldg_stream(rec + (size_t)3 * a.D);
+      sc[0] = __uint_as_float(s4.x), sc[1] = __uint_as_float(s4.y), sc[2] = __uint_as_float(s4.z);
+    }
+    uint4 x[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-          const int v = v0 + 32 * j;
-          if (v >= 0 && v < end) x[j] = ldg_stream(rec + (size_t)v * 16);
-        }
+    for (int j = 0; j < U; ++j) {
+      const int v = v0 + 32 * j;
+      if (v >= 0 && v < end) x[j] = ldg_stream(rec + (size_t)v * 16);
+    }
+    i += nw;
+    settle();  // the next piece's list entry comes while the rows are on their way
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-          int v = v0 + 32 * j;
-          if (v >= 0 && v < end) {
-            char* row = a.gate;
-            float scale = kInt8 ? sc[0] : 0.f;
-            if (v >= row_units) {
-              v -= row_units;
-              row = a.up;
-              if (kInt8) scale = sc[1];
-              if (v >= row_units) {
-                v -= row_units;
-                row = a.downT;
-                if (kInt8) scale = sc[2];
-              }
-            }
-            if (kInt8) {
-              uint4* o = reinterpret_cast<uint4*>(row + dst) + 2 * v;
-              o[0] = make_uint4(dequant2(x[j].x, 0, scale), dequant2(x[j].x, 16, scale), dequant2(x[j].y, 0, scale), dequant2(x[j].y, 16, scale));
-              o[1] = make_uint4(dequant2(x[j].z, 0, scale), dequant2(x[j].z, 16, scale), dequant2(x[j].w, 0, scale), dequant2(x[j].w, 16, scale));
-            } else {
-              reinterpret_cast<uint4*>(row + dst)[v] = x[j];
-            }
+    for (int j = 0; j < U; ++j) {
+      int v = v0 + 32 * j;
+      if (v >= 0 && v < end) {
+        char* row = a.gate;
+        float scale = kInt8 ? sc[0] : 0.f;
+        if (v >= row_units) {
+          v -= row_units;
+          row = a.up;
+          if (kInt8) scale = sc[1];
+          if (v >= row_units) {
+            v -= row_units;
+            row = a.downT;
+            if (kInt8) scale = sc[2];
           }
+        }
+        if (kInt8) {
+          uint4* o = reinterpret_cast<uint4*>(row + dst) + 2 * v;
+          o[0] = make_uint4(dequant2(x[j].x, 0, scale), dequant2(x[j].x, 16, scale), dequant2(x[j].y, 0, scale), dequant2(x[j].y, 16, scale));
+          o[1] = make_uint4(dequant2(x[j].z, 0, scale), dequant2(x[j].z, 16, scale), dequant2(x[j].w, 0, scale), dequant2(x[j].w, 16, scale));
+        } else {
+          reinterpret_cast<uint4*>(row + dst)[v] = x[j];
         }
       }
     }
-    i -= total;  // >= 0 here; what is left of the round belongs to the next layer
   }
 }
 
@@ -281,6 +286,11 @@ cudaError_t launch_pull(const Dims& d, const Tables& t, const char* store_dev, v
   a.C = d.C;
   a.Lp = d.Lp;
   a.check = check;
+  // whole lines, and no more units than one round of a warp's loads; a record starts up to `mis` units into its first line
+  const int units = 3 * d.D / (d.rec_int8 ? 16 : 8), most = 32 * kPullLoads;
+  const int mis = d.rec_bytes % 128 == 0 ? (int)((reinterpret_cast<uintptr_t>(store_dev) >> 4) & 7) : 7;
+  a.pieces = (units + mis + most - 1) / most;
+  a.piece = ((units + mis + a.pieces - 1) / a.pieces + 7) & ~7;
   if (d.rec_int8) k_pull_rows<true><<<blocks, kPullThreads, 0, s>>>(a);
   else k_pull_rows<false><<<blocks, kPullThreads, 0, s>>>(a);
   return cudaGetLastError();
