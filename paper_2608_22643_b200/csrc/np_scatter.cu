@@ -198,7 +198,19 @@ __global__ void __launch_bounds__(kPullThreads) k_pull_rows(PullArgs a) {
   const int nw = gridDim.x * (kPullThreads / 32);
   const int row_units = kInt8 ? a.D >> 4 : a.D >> 3;             // 16-byte units of a source row
   const int pieces = a.pieces;
-  auto pieces_of = [&](int l) { return min(max(a.counters[(size_t)l * NP_N_COUNTERS + NP_CNT_DELTA], 0), a.C) * pieces; };
+  // pieces of a layer: the lanes hold 32 layers' counts, read at once (a launch without rows is as long as these reads)
+  int base = a.l_begin, held = 0;
+  auto read_counts = [&] {
+    held = base + lane < a.l_end ? min(max(a.counters[(size_t)(base + lane) * NP_N_COUNTERS + NP_CNT_DELTA], 0), a.C) * pieces : 0;
+  };
+  auto pieces_of = [&](int l) {
+    if (l - base >= 32) {
+      base = l;
+      read_counts();
+    }
+    return __shfl_sync(0xffffffffu, held, l - base);
+  };
+  read_counts();
   // this warp's pieces are every nw-th of all layers' in a row: i counts from the start of layer l
   int l = a.l_begin, total = pieces_of(l), id = 0, slot = 0;
   int i = blockIdx.x * (kPullThreads / 32) + (threadIdx.x >> 5);
