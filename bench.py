@@ -594,9 +594,9 @@ def cuda_arm(args):
     s.synchronize()
     n_launch = nb.np_chain_launches(eng.ctx)                        # resident launches the chain was cut into
     if n_launch <= 0:
-        n_launch = L - nd                                           # per-layer (or batch) kernels
+        n_launch = L - nd                                           # kernels per layer
     mlp_kernel = nb.np_mlp_kernel_name(eng.ctx, Bq)       # the kernel the library chose for this shape and batch
-    if Bq > 1:
+    if "+" in mlp_kernel:
         mlp_kernel += " (the launches of one layer)"
     mlp_us = k0.elapsed_time(k1) * 1000.0 / (reps * n_launch)      # per launch, gaps included
     p0, p1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)

@@ -1448,10 +1448,12 @@ static int dense_run_layers(const np_ctx* ctx) {
   return std::max(3, std::min(12, 2 * d.dense / (d.L - d.dense)));
 }
 
-static int batch_run(np_ctx* ctx, const ChainArgs& a, float* x, int B, bool beside_pull, cudaStream_t s) {
+// `made` (may be NULL) counts the launches
+static int batch_run(np_ctx* ctx, const ChainArgs& a, float* x, int B, bool beside_pull, cudaStream_t s, int* made) {
   int n = 0;
   NP_CUDA(ctx, chain_batch::launch(ctx->d, a, x, B, &ctx->batch, s, resident_sms(ctx, beside_pull, chain_batch::supported), &n));
   ctx->launches += n;
+  if (made) *made += n;
   return NP_OK;
 }
 
@@ -1479,7 +1481,7 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
       for (int l0 = 0; l0 < d.dense; l0 += dense_run) {
         a.l_begin = l0;
         a.l_end = std::min(d.dense, l0 + dense_run);
-        const int rc = batch_run(ctx, a, x, B, stepping, s);
+        const int rc = batch_run(ctx, a, x, B, stepping, s, nullptr);
         if (rc < 0) return rc;
       }
     }
@@ -1499,7 +1501,7 @@ static int batch_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cud
     NP_CUDA(ctx, wait_installs(ctx, l0, l0 + n, s));
     a.l_begin = l0;
     a.l_end = l0 += n;
-    rc = batch_run(ctx, a, x, B, stepping || (l0 < d.L && ctx->install_pending[d.L - 1]), s);
+    rc = batch_run(ctx, a, x, B, stepping || (l0 < d.L && ctx->install_pending[d.L - 1]), s, &ctx->chain_kernel_launches);
     if (rc < 0) return rc;
   }
   NP_LAUNCH(ctx, chain_batch::launch_out(d, x, x_out, B, s));
@@ -1721,9 +1723,9 @@ const char* np_mlp_kernel_name(np_ctx* ctx, int32_t B) {
     if (ctx->use_slices) return "k_mlp_slices";
     if (chain_alu::supported(d, ctx->sm_count)) return "k_mlp_chain_alu";
   }
+  if (ctx->use_batch && B >= kTcMinBatch) return "k_mlp_batch";
   if (ctx->mlp_tc && B >= kTcMinBatch && !(flags & NP_F_DIRECT_LOADS))
     return ((flags & NP_F_TCGEN05_BATCH) && mlp_tc_up_on_tcgen05(d, ctx->sm_count)) ? "k_mlp_up5 + k_mlp_tc_down" : "k_mlp_tc_up + k_mlp_tc_down";
-  if (ctx->use_batch && B >= kTcMinBatch) return "k_mlp_batch";  // widths the pair does not cover
   return (flags & NP_F_DIRECT_LOADS) ? "k_sparse_mlp" : "k_sparse_mlp_pipe";
 }
 

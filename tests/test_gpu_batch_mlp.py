@@ -88,16 +88,28 @@ def test_chain_matches_oracle(cfg, B, flags):
         p.close()
 
 
-def test_kernel_choice_follows_the_flag():
-    """The library names the kernels it launches for a batch: the tcgen05 up kernel only with its flag and only for
-    row widths it covers."""
-    for cfg, flags, want in [(DENSE, TC, "k_mlp_tc_up + k_mlp_tc_down"), (DENSE, TC5, "k_mlp_up5 + k_mlp_tc_down"),
-                             (ODD, TC5, "k_mlp_tc_up + k_mlp_tc_down")]:
-        p = Pair(cfg, max_batch=16, flags=flags)
-        try:
-            assert nb.np_mlp_kernel_name(p.eng.ctx, 16) == want, (cfg.name, flags)
-        finally:
-            p.close()
+@pytest.mark.parametrize("cfg,flags,want", [
+    (DENSE, TC, "k_mlp_batch"), (ODD, TC, "k_mlp_batch"), (DENSE, nb.NP_F_LAYER_LAUNCHES, "k_mlp_tc_up + k_mlp_tc_down"),
+    (DENSE, TC5, "k_mlp_up5 + k_mlp_tc_down"), (ODD, TC5, "k_mlp_tc_up + k_mlp_tc_down"), (DENSE, ALU, "k_sparse_mlp_pipe"),
+])
+def test_kernel_choice_follows_the_flag(cfg, flags, want):
+    """The library names the kernels it launches for a batch, the tcgen05 up kernel only with its flag and only for row
+    widths it covers; what it launches is counted: a resident kernel as runs of layers, the others per layer."""
+    p = Pair(cfg, max_batch=16, flags=flags, C=cfg.d_ffn, with_oracle=False)
+    try:
+        assert nb.np_mlp_kernel_name(p.eng.ctx, 16) == want
+        x = synth.hidden_states(cfg, 1, batch=16)[0].cuda()
+        out = torch.empty((16, cfg.d_model), dtype=torch.float32, device="cuda")
+        nb.np_step(p.eng.ctx, x, 16, out, p.eng.stream, p.eng.copy_stream)
+        torch.cuda.synchronize()
+        before = nb.np_launch_count(p.eng.ctx)
+        nb.np_mlp_chain(p.eng.ctx, x, 16, out, p.eng.stream)
+        p.eng.counters()
+        made = nb.np_launch_count(p.eng.ctx) - before
+        assert nb.np_chain_launches(p.eng.ctx) == (1 if want == "k_mlp_batch" else 0)     # every row is resident: one run
+        assert made == 3 if want == "k_mlp_batch" else made >= 2 + cfg.n_layers     # x in, the run, x out
+    finally:
+        p.close()
 
 
 @pytest.mark.parametrize("B", [3, 16])

@@ -138,12 +138,12 @@ def test_larger_shapes_few_layers(name, n_layers, mode, chain_layers):
         p.close()
 
 
-@pytest.mark.parametrize("flags,kernel", [(0, "k_mlp_tc_up + k_mlp_tc_down"),
+@pytest.mark.parametrize("flags,kernel", [(0, "k_mlp_batch"), (nb.NP_F_LAYER_LAUNCHES, "k_mlp_tc_up + k_mlp_tc_down"),
                                           (nb.NP_F_TCGEN05_BATCH, "k_mlp_up5 + k_mlp_tc_down")])
 def test_stress_shape_batch16_few_layers(flags, kernel):
     """Sixteen sequences at the 7B row shape (the delta-stress workload) on four layers: the
     tensor-core predictor and the tensor-core batch MLP in the configuration bench.py --batch 16
-    times (and with the up phase on tcgen05); unions of the per-sequence sets, tables bit-exact,
+    times (the resident kernel, the pair of kernels per layer, and the pair with the up phase on tcgen05); unions of the per-sequence sets, tables bit-exact,
     chain within tolerance."""
     cfg = synth.CONFIGS["stress"].with_(n_layers=4)
     L, M, D, B = cfg.n_layers, cfg.d_ffn, cfg.d_model, 16
