@@ -53,11 +53,15 @@ extern "C" {
 #define NP_E_NOMEM     -4   /* allocation of library-owned state failed */
 #define NP_E_DEVICE    -5   /* a kernel recorded a status bit (np_last_error prints them): 1 slot, 2 neuron id or
                                4 count out of range; 8 a bounded wait ran out; 16 a block's partial MLP sum was
-                               not finite or reached 2^19 in magnitude (the resident one-sequence kernel hands
-                               sums between layers in fixed point, resolution 2^-30); state is suspect */
+                               not finite or reached 2^19 in magnitude (k_mlp_slices hands sums between layers
+                               in fixed point, resolution 2^-30: one sequence, row widths of 64 to 8192 that
+                               are a multiple of 16, where np_mlp_kernel_name names it; every other kernel
+                               keeps them in fp32); state is suspect */
 #define NP_E_IO        -6   /* a read of the store file failed or came up short */
 #define NP_W_OVERFLOW   1   /* some layer's predicted set did not fit capacity */
-#define NP_W_CHUNKED    2   /* some layer's delta is larger than the staging (rows that are staged were split) */
+#define NP_W_CHUNKED    2   /* some layer's delta has more rows than the staging holds (with HOST_GATHER and FILE: than a
+                               part of it, staging_rows over two to four).  Rows that are staged were split into chunks;
+                               rows that are pulled were not, and the warning only says that the count was that high */
 
 /* eviction policies (np_config.evict_policy) */
 #define NP_EVICT_EXACT  0   /* Eq. 3: every row leaving the predicted set frees its slot */
@@ -66,7 +70,8 @@ extern "C" {
 
 /* how np_install moves records (np_config.transfer_mode).  The three modes with a pinned store differ in what the host
    does; short runs of rows are pulled by a kernel that reads the store by neuron ID and places the rows (the paper's
-   mapped-staging idea without the staging: 51 GB/s on scattered records, on two SMs, no host core busy) in all of them. */
+   mapped-staging idea without the staging: 50 GB/s on scattered 24 KB records, on two SMs, four with 8-bit records,
+   no host core busy) in all of them. */
 #define NP_XFER_MEMCPY_RUNS  0  /* one cudaMemcpyAsync per run of adjacent neuron IDs into device staging, then the
                                    scatter kernel, where the runs are long enough to pay a copy call (3.4 MB on
                                    average); pulled otherwise */
@@ -144,11 +149,12 @@ typedef struct np_config {
   int32_t capacity;       /* C, 1 <= C <= M */
   int32_t max_batch;      /* largest B any call will pass, 1..16 */
   int32_t evict_policy;   /* NP_EVICT_* */
-  int32_t staging_rows;   /* records the staging buffer holds (>= 1); larger deltas are
-                             split into chunks (Section 3.5, bounded staging) */
+  int32_t staging_rows;   /* records the staging buffer holds (>= 1; >= 2 with HOST_GATHER and FILE); larger
+                             deltas that are staged are split into chunks (Section 3.5, bounded staging) */
   int32_t transfer_mode;  /* NP_XFER_* */
   int32_t flags;          /* NP_F_* */
-  int32_t host_threads;   /* worker threads for NP_XFER_HOST_GATHER (0 = pick) */
+  int32_t host_threads;   /* worker threads that pack records (HOST_GATHER with NP_F_MAPPED_STAGING) or read them
+                             (FILE without io_uring); 0 = pick.  Other contexts start none */
   int32_t chain_layers;   /* layers per resident MLP kernel in np_step / np_mlp_chain (0 = runs that
                              shrink towards the end: the last run is an eighth of the stack, the one
                              before it a quarter, the first takes the rest) */
@@ -198,7 +204,8 @@ typedef struct np_buffers {
   void* gate_buf;          /* dev  */
   void* up_buf;            /* dev  */
   void* downT_buf;         /* dev  */
-  void* staging;           /* dev; unused (may be NULL) with NP_XFER_ZERO_COPY */
+  void* staging;           /* dev; may be NULL with NP_XFER_ZERO_COPY and NP_F_MAPPED_STAGING.  HOST_GATHER without
+                              that flag asks for it (and for host_staging) but pulls its rows past both */
   void* host_staging;      /* pinned host, staging_bytes; only for NP_XFER_HOST_GATHER and
                               NP_XFER_FILE */
   void* workspace;         /* dev, 256-byte aligned */
@@ -416,15 +423,17 @@ int np_install_speculative(np_ctx* ctx, void* copy_stream);
  * and their count.  Valid until the next np_speculate. */
 int np_get_speculative(np_ctx* ctx, int32_t layer, const int32_t** ids, const int32_t** slots, const int32_t** count);
 
-/* Launches of the resident MLP kernel (sparse layers, one sequence) made by the last np_mlp_chain / np_step:
- * the runs the chain was cut into.  0 when that call ran per-layer or batch kernels.  For reports. */
+/* Launches of the resident MLP kernel (sparse layers) made by the last np_mlp_chain / np_step: the runs the chain was
+ * cut into.  0 when that call ran kernels per layer.  For reports. */
 int np_chain_launches(np_ctx* ctx, int32_t* out);
 
 /* Name of the kernel np_mlp_chain / np_step run the sparse layers' MLP with for B sequences in this
- * context (a static string: "k_mlp_slices", "k_mlp_chain_alu", "k_mlp_tc_up + k_mlp_tc_down",
- * "k_sparse_mlp_pipe" or "k_sparse_mlp").  "k_mlp_tc_up + k_mlp_tc_down" names the tensor-core form for batches: its
- * two phases run as one resident kernel ("k_mlp_batch", the name for widths that only it covers) where that applies, as
- * two kernels per layer elsewhere.  For reports; NULL if ctx is NULL or B is out of range. */
+ * context (a static string: "k_mlp_slices", "k_mlp_rows", "k_mlp_chain_alu", "k_mlp_batch" (two to sixteen
+ * sequences, both phases of a run of layers), "k_mlp_tc_up + k_mlp_tc_down" or "k_mlp_up5 + k_mlp_tc_down" (a pair per
+ * layer: NP_F_LAYER_LAUNCHES, NP_F_TCGEN05_BATCH and shapes the resident kernel does not hold), "k_sparse_mlp_pipe" or
+ * "k_sparse_mlp").  A chain that is captured into a graph runs the row-partitioned or the per-layer kernels instead of
+ * the others: their launches carry counts that a replay would repeat.  For reports; NULL if ctx is NULL or B is out of
+ * range. */
 const char* np_mlp_kernel_name(np_ctx* ctx, int32_t B);
 
 /* Timing of the last np_step in microseconds, host float [4]: predict+top-k,
