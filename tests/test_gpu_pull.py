@@ -38,18 +38,53 @@ def test_record_sizes(D, records, mode):
         p.close()
 
 
-def test_runs_by_copies_and_by_pulls():
+@pytest.mark.parametrize("records,M,staging_rows", [
+    (nb.NP_REC_BF16, 256, 200),    # 24 KB records: 256 adjacent ones are longer than the shortest run that pays a copy
+    (nb.NP_REC_BF16, 256, 60),     # five chunks a layer
+    (nb.NP_REC_INT8, 512, 512),    # 12 KB records, a chunk a layer
+    (nb.NP_REC_INT8, 512, 150),    # four
+])
+def test_runs_by_copies_and_by_pulls(records, M, staging_rows):
     """Whole layers arrive as one long run each (copy engine), scattered rows are pulled; both leave the same bytes."""
-    L, M, D = 2, 256, 4096     # 24 KB records: 256 adjacent ones are longer than the shortest run that pays a copy
+    L, D = 2, 4096
     cfg = synth.StackConfig("runs", L, D, M, 16, 25, 50, 3, 48, 0.9)
-    p = Pair(cfg, k=M, C=M, transfer_mode=nb.NP_XFER_MEMCPY_RUNS, staging_rows=200)
+    p = Pair(cfg, k=M, C=M, transfer_mode=nb.NP_XFER_MEMCPY_RUNS, staging_rows=staging_rows, record_format=records)
     try:
         full = torch.full((L, M // 32), -1, dtype=torch.int32)
-        some = synth.random_bitmaps(L, M, 90, 9, 1, 0.5)[0]
-        for words, warn in ((full, nb.NP_W_CHUNKED), (some, nb.NP_OK), (full, nb.NP_OK)):
+        none = torch.zeros((L, M // 32), dtype=torch.int32)
+        some = synth.random_bitmaps(L, M, min(90, staging_rows), 9, 1, 0.5)[0]
+        chunked = nb.NP_W_CHUNKED if M > staging_rows else nb.NP_OK
+        rest = nb.NP_W_CHUNKED if M - min(90, staging_rows) > staging_rows else nb.NP_OK
+        for words, warn, scatters in ((full, chunked, True), (some, nb.NP_OK, False), (full, rest, False), (none, nb.NP_OK, False),
+                                      (some, nb.NP_OK, False), (none, nb.NP_OK, False), (full, chunked, True)):
             nb.np_delta(p.eng.ctx, words.cuda(), p.eng.stream)
+            before = nb.np_launch_count(p.eng.ctx)
             assert nb.np_install(p.eng.ctx, 0, L, p.eng.copy_stream) == warn
+            # a scatter kernel per chunk of a layer behind its copies
+            if scatters:
+                assert nb.np_launch_count(p.eng.ctx) - before == L * -(-M // staging_rows)
             p.check_resident_bytes()
             p.check_delta_against(p.ora.res.delta(words.numpy().view(np.uint32)))
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("records", [nb.NP_REC_BF16, nb.NP_REC_INT8])
+@pytest.mark.parametrize("staging_rows", [None, 2, 9])
+def test_packed_records_in_chunks(records, staging_rows):
+    """Host threads pack the records into parts of the pinned staging however few rows a part holds."""
+    cfg = synth.CONFIGS["small"]
+    p = Pair(cfg, transfer_mode=nb.NP_XFER_HOST_GATHER, staging_rows=staging_rows, record_format=records,
+             flags=nb.NP_F_CHECK_BOUNDS | nb.NP_F_MAPPED_STAGING)
+    try:
+        words = synth.random_bitmaps(cfg.n_layers, cfg.d_ffn, p.k, 5, 4, 0.8)
+        words[:, :, 3] = -1                       # adjacent records
+        for t in range(4):
+            nb.np_delta(p.eng.ctx, words[t].cuda(), p.eng.stream)
+            rc = nb.np_install(p.eng.ctx, 0, cfg.n_layers, p.eng.copy_stream)
+            if staging_rows is not None and t == 0:
+                assert rc == nb.NP_W_CHUNKED
+            p.check_resident_bytes()
+            p.check_delta_against(p.ora.res.delta(words[t].numpy().view(np.uint32)))
     finally:
         p.close()
