@@ -156,23 +156,24 @@ cudaError_t launch_scatter(const Dims& d, const void* src, const int32_t* slots,
 // about 4.5 us each.  The 147 MB of incoming rows of a 7B-shaped step, one context on its own (one contiguous copy of the
 // same bytes: 55.1 GB/s; the store's size, 8.7 GB or an eighth of that, makes no difference):
 //
-//   two SMs of 1024 threads, six loads in flight per lane   44.4 GB/s    301 steps/s
-//   two SMs, eight loads per lane                           49.6         332
-//   three SMs, six / eight                                  46.9 / 50.0  316 / 337
-//   four / six SMs, six loads                               48.1 / 49.0  324 / 330
+//   two SMs of 1024 threads, six loads per lane, pieces of 384 units in rounds   44.4 GB/s    301 steps/s
+//   the same with eight loads per lane                                           49.6         332
+//   three SMs, six / eight loads                                                 46.9 / 50.0  316 / 337
+//   four / six SMs, six loads                                                    48.1 / 49.0  324 / 330
+//   two SMs, six loads, pieces of one round                                      50.1         337
 //
-// Two SMs with eight loads it is: every further SM is one less for the resident MLP kernels, which are launched narrower
-// while rows are on their way (kPullReserve; two such kernels fit, and two contexts stepping in turn reach 51 GB/s with
-// six or eight loads).  Packing the records with the host's cores and copying the packed parts gives 40 to 47 depending
-// on the host (304 to 315 steps/s; the packing reads and writes every byte in host memory beside the copy's own reads),
-// and a copy call per record 4.8.  A kernel on all SMs, small enough to fit beside the resident blocks, was no faster, and
-// the resident kernels lost 7 % by giving up the registers.
+// A piece of a record is what one round of a warp's loads takes, all pieces of a record alike and whole 128-byte lines from
+// the line the record starts in, so that no round is nearly empty; the next piece's layer and list entry are read while
+// the rows are on their way.  More in flight than this gives nothing alone, and where two contexts pull at a time (51 GB/s
+// together) it only delays what else crosses the link: seven or eight loads per lane cost three stacks of 20 layers that
+// select and step in turn 2 to 3 %.  Every further SM is one less for the resident MLP kernels, which are launched
+// narrower while rows are on their way (kPullReserve; two pulls fit).  Packing the records with the host's cores and
+// copying the packed parts gives 40 to 47 GB/s depending on the host (304 to 317 steps/s; the packing reads and writes
+// every byte in host memory beside the copy's own reads), and a copy call per record 4.8.  A kernel on all SMs, small
+// enough to fit beside the resident blocks, was no faster, and the resident kernels lost 7 % by giving up the registers.
 //
-// 8-bit records: a lane's dequantising adds to the trip of its loads, and there are no registers for eight (25.9 GB/s with
-// them, 26.5 with six, 357 steps/s).  They take four SMs: 44.6 GB/s, 573 steps/s (pull_blocks on where they do not).
-//
-// A piece is 384 units of 16 bytes, taken from the 128-byte line the record starts in, so that a warp's accesses are whole
-// lines also for records that are not a multiple of 128 bytes; the last piece takes what is left.
+// 8-bit records: a lane's dequantising adds to the trip of its loads.  Two SMs read 27 GB/s (361 steps/s), four 47 (606;
+// eight loads per lane 597): they take four (pull_blocks on where they do not).
 // ---------------------------------------------------------------------------------------
 constexpr int kPullThreads = 1024;
 constexpr int kPullLoads = 6;  // loads a lane has in flight
