@@ -663,7 +663,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   NP_INIT_CUDA(cudaMemset(ctx->slices.zfix, 0, chain_slices::zfix_words(ctx->d) * 8));
   NP_INIT_CUDA(cudaMemset(ctx->slices.bars, 0, chain_slices::bar_words() * 4));
   NP_INIT_CUDA(cudaMemset(ctx->slices.xch, 0, chain_slices::xch_words(ctx->d, ctx->sm_count) * 8));
-  ctx->use_slices = !(cfg->flags & NP_F_ROW_CHAIN) && chain_slices::preferred(d, ctx->sm_count);
+  ctx->use_slices = !(cfg->flags & NP_F_ROW_CHAIN) && chain_slices::supported(d, ctx->sm_count);
   ctx->xterms = base + o_xt;
   ctx->rows.z4 = reinterpret_cast<float*>(base + o_rz);
   ctx->rows.cnt = reinterpret_cast<unsigned int*>(base + o_rcnt);
@@ -756,6 +756,7 @@ int np_init(np_ctx** out, const np_config* cfg, const np_buffers* b) {
   if (d.dense > 0) {
     Dims dd = d;
     dd.k = dd.C = d.M;
+    dd.dense = 0;
     if ((!dense_chain::supported(d, ctx->sm_count) && !chain_alu::supported(dd, ctx->sm_count)) || (d.dense < d.L && !chain_slices::supported(d, ctx->sm_count) && !chain_alu::supported(d, ctx->sm_count))) {
       np_destroy(ctx);
       return fail(nullptr, NP_E_INVAL, "dense_layers > 0: this shape is outside what the resident MLP kernels cover");
@@ -1531,7 +1532,7 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
   const bool fold_widen = persistent && (use_rows || use_slices) && d.dense == 0;
   // Where the sliced kernel hands its sums over as counted words, layer 0's fp32 accumulator is used only by a
   // first launch of one layer that does not end the stack: the clearing waits until the runs are known.
-  const bool lazy_clear = fold_widen && use_slices && !use_rows && chain_slices::counted_handover(d, ctx->sm_count);
+  const bool lazy_clear = fold_widen && use_slices && !use_rows;
   bool out_written = false;  // the last resident launch left x_out itself
   if (part != kChainTail) {
     if (!fold_widen) NP_LAUNCH(ctx, launch_widen_bf16(x_bf16, ctx->ws.xbuf[1], n, s));
@@ -1596,11 +1597,10 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
         NP_LAUNCH(ctx, chain_rows::launch(d, a, &ctx->rows, s));
       } else if (use_slices) {
         const int sms = resident_sms(ctx, beside_pull, chain_slices::supported);
-        chain_slices::Plan sp;
-        chain_slices::plan(d, sms, &sp);
-        ctx->chain_kernel_launches += (l1 - l0 + sp.run_layers - 1) / sp.run_layers;
+        constexpr int run = chain_slices::kMaxLayers;
+        ctx->chain_kernel_launches += (l1 - l0 + run - 1) / run;
         a.x_out = l1 == d.L ? x_out : nullptr;  // the run that ends the stack may leave the result itself
-        if (lazy_clear && l0 == 0 && std::min(l1, sp.run_layers) == 1 && l1 != d.L)
+        if (lazy_clear && l0 == 0 && std::min(l1, run) == 1 && l1 != d.L)
           NP_CUDA(ctx, cudaMemsetAsync(ctx->ws.zbuf[0], 0, (size_t)kZRep * d.D * 4, s));
         NP_LAUNCH(ctx, chain_slices::launch(d, a, &ctx->slices, s, sms));
         out_written = a.x_out && ctx->slices.wrote_out;

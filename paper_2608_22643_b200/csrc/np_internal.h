@@ -209,10 +209,10 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, cudaStream_t s, int sm_cou
 }  // namespace chain_alu
 
 namespace chain_slices {  // column-sliced resident form for one sequence (np_mlp_slices.cu); same hand-over of x
-struct Plan {
-  int R, ks, vg_shift, gw_shift, ng, window, run_layers, slot_cache_rows, max_rows, xch_stride;
-  size_t group_bytes, smem;
-};
+// Widest rows.  Wider ones are the row-partitioned kernel's, and above its widths the kernels per layer take them: both were
+// faster there (100 to 1600 rows of 8256 columns 9.3 to 26.9 us per layer against 14.6 to 34.0 here).
+constexpr int kMaxD = 8192;
+constexpr int kMaxLayers = 128;  // layers per launch
 // Library-owned device words and the host's running record of them: the counted sums and the
 // exchange stamps only ever grow, so nothing has to be cleared between launches.
 struct State {
@@ -222,11 +222,8 @@ struct State {
   unsigned int bar_base, seq_base;
   int wrote_out;             // the last launch left the stack's result in ChainArgs::x_out
 };
-bool plan(const Dims& d, int sm_count, Plan* p);
 bool supported(const Dims& d, int sm_count);
-bool preferred(const Dims& d, int sm_count);  // supported, and no other form is faster at this width
 size_t xch_words(const Dims& d, int sm_count);
-bool counted_handover(const Dims& d, int sm_count);  // the sums between layers are counted fixed-point words for this shape
 size_t zfix_words(const Dims& d);
 size_t bar_words();
 cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s, int sm_count);

@@ -437,6 +437,8 @@ static bool alu_plan(const Dims& d, int sm_count, AluPlan* p) {
   const int per_block = (int)std::max<long long>(1, (expect + sm_count - 1) / sm_count);
   const int max_per_block = d.C / sm_count + 2;   // whatever the active count turns out to be
   p->run_layers = std::max(1, std::min(kChainMaxLayers, 16384 / (4 * max_per_block)));
+  // Behind a dense prefix there is no other kernel for the widest rows: fewer layers' slots rather than none of them.
+  while (d.dense > 0 && (size_t)d.D * 4 + (size_t)p->run_layers * max_per_block * 4 + 2 * rec > 227 * 1024 - 4096 && p->run_layers > 1) p->run_layers /= 2;
   p->slot_cache_rows = p->run_layers * max_per_block;
   const size_t fixed = (size_t)d.D * 4 + (size_t)p->slot_cache_rows * 4;
   const size_t budget = 227 * 1024 - 4096;  // static shared memory and the driver's reserve
@@ -475,7 +477,10 @@ bool supported(const Dims& d, int sm_count) {
 
 cudaError_t launch(const Dims& d_in, const ChainArgs& a, cudaStream_t s, int sm_count) {
   Dims d = d_in;
-  if (a.dense_rows > 0) d.k = d.C = a.dense_rows;  // plan for layers whose every row is active
+  if (a.dense_rows > 0) {  // plan for layers whose every row is active
+    d.k = d.C = a.dense_rows;
+    d.dense = 0;
+  }
   AluPlan p;
   if (!alu_plan(d, sm_count, &p)) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;

@@ -63,6 +63,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
+// A bounded wait on an mbarrier for blocks that drain after a time-out: once any wait of the block has run out (*ok == 0)
+// every later one is skipped.  One loop around one try_wait, not unrolled: with the unrolled loops of mbar_wait at every wait
+// the resident kernels had 80 to 150 KB of code, missed the instruction cache on every layer (195 times at 256 columns) and
+// spent a sixth of their issue slots waiting for instructions.
+__device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
+  uint32_t spin = 0;
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity)) {
+    if (!*ok) return;
+    if (++spin == kSpinLimit) {
+      *ok = 0;
+      atomicOr(status, kStatTimeout);
+    }
+  }
+}
+
 // 1-D bulk copy global -> this CTA's shared memory; completion is reported to
 // `bar` in bytes.  Both addresses 16-byte aligned, `bytes` a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {

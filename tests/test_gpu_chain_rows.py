@@ -41,3 +41,40 @@ def test_chain_row_groups(D, M, k, L):
         p.eng.counters()
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("D,M,k,L", [
+    (64, 512, 60, 130),           # one K block per slice, a single warp; more layers than a launch covers
+    (128, 512, 10, 3),            # two K blocks, row groups without rows
+    (512, 2048, 37 * 16 + 1, 3),  # a down tile of one row in one row group
+    (576, 1024, 100, 3),          # nine K blocks of a slice on five warps of two: a ragged last warp
+    (2064, 1024, 37 * 8, 3),      # slices of 32 and 33 K blocks: a warp without any in three of them
+    (5120, 2048, 37 * 48, 2),     # rounds of the exchange of 48 rows: one full
+    (5120, 2048, 37 * 48 + 1, 2), # a second round of one row
+    (6144, 2560, 37 * 65, 2),     # two rounds of 64 rows, two buffers
+    (8192, 2560, 37 * 33, 2),     # two tiles held at a time, an odd number of them
+    (8176, 2048, 37 * 17, 2),     # the same at uneven slices
+])
+def test_chain_tiles(D, M, k, L):
+    cfg = synth.StackConfig("tiles", L, D, M, 32, 25, 50, 2, 29, 0.9)
+    p = Pair(cfg, max_batch=1, k=k, C=max(k, M // 2))
+    try:
+        xs = synth.hidden_states(cfg, 2, batch=1)
+        out = torch.empty((1, D), dtype=torch.float32, device="cuda")
+        logits = torch.empty((1, L, M), dtype=torch.float32, device="cuda")
+        for t in range(2):
+            x = xs[t].cuda()
+            nb.np_predict(p.eng.ctx, x, 1, logits, None, p.eng.stream)
+            nb.np_step(p.eng.ctx, x, 1, out, p.eng.stream, p.eng.copy_stream)
+            torch.cuda.synchronize()
+            res = p.ora.step(u16(xs[t]), logits_f32=logits.cpu().numpy())
+            # fp32 sums of bf16 products: 1e-6 over a few layers; layers past 20 add in proportion
+            tol = 1e-5 * max(1.0, L / 20)
+            assert rel_l2(out.cpu().numpy()[0], res["x_final"][0]) < tol, t
+            nb.np_mlp_chain(p.eng.ctx, x, 1, out, p.eng.stream)      # resident rows: one run, as few launches as there can be
+            torch.cuda.synchronize()
+            assert rel_l2(out.cpu().numpy()[0], res["x_final"][0]) < tol, t
+            assert nb.np_chain_launches(p.eng.ctx) == (L + 127) // 128
+        p.eng.counters()
+    finally:
+        p.close()
