@@ -100,12 +100,13 @@ bool pred_l2_ring_fits(int H, int B);
 constexpr int kPredTcMinBatch = 2;
 constexpr int kPredL1Parts = 16;  // K ranges (partial sums) of the tensor-core layer 1, at most
 struct PredTcState {
-  alignas(64) unsigned char map_w2[128];  // CUtensorMap of W2 [L*M][H]
+  alignas(64) unsigned char map_w2[128];  // CUtensorMap of W2 [L*M][H], boxes of bt tiles
+  alignas(64) unsigned char map_tile[128];  // the same, boxes of one tile
   alignas(64) unsigned char map_h[128];   // CUtensorMap of the split hidden terms [48][H]
   alignas(64) unsigned char map_w1[128];  // CUtensorMap of W1 [H][D]
   void* hsplit;                           // device bf16 [48][H] (workspace)
   float* l1_part;                         // device fp32 [kPredL1Parts][16][H]: layer 1's partial sums per K range
-  int n_stages;
+  int n_stages, bt;
   size_t smem;
   int ready;
   int l1_ready, l1_parts, l1_kb_per_block;

@@ -103,3 +103,26 @@ def test_hidden_values_at_the_end_of_the_range(B):
         assert torch.equal(got[2:], rest[2:])
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("H", [64, 896, 960, 1024])   # 896 and 960: the widest with two tiles to a stage, 1024: one
+@pytest.mark.parametrize("L,M", [
+    (1, 128),       # a block with one tile: the pair's second is missing
+    (37, 1024),     # 296 tiles: a pair for each of 148 SMs
+    (38, 1024),     # 304: pairs, and pairs with a tile behind them
+    (37, 1056),     # 305.25: the last tile is a quarter
+    (75, 1024),     # 600: two pairs and an odd tile on some SMs
+])
+def test_pairs_of_row_tiles(L, M, H):
+    B = 3
+    p = Pair(synth.StackConfig("pt", L, 64, M, H, 25, 50, 1, 47, 0.9), max_batch=B, k=1, C=32, with_oracle=False, store_layers=1,
+             gen_device="cuda")
+    try:
+        x = synth.hidden_states(p.cfg, 1, batch=B)[0]
+        logits = torch.full((B, L, M), 7.0, dtype=torch.float32, device="cuda")
+        nb.np_predict(p.eng.ctx, x.cuda(), B, logits, None, p.eng.stream)
+        p.eng.counters()
+        z = O.predict(u16(p.w1_cpu), u16(p.w2_cpu), u16(x), L, M)
+        assert rel_l2(logits.cpu().numpy(), z) < 1e-5    # fp32 accumulation of at most 1024 products: below 1e-6
+    finally:
+        p.close()
