@@ -469,8 +469,10 @@ bool pred_tc_prepare(const Dims& d, const void* w1, const void* w2, void* hsplit
   // Two tiles to a stage where four such stages fit: a copy instruction costs the SM's copy unit some 80 cycles whatever it
   // brings (13B shape, three sequences: 176 us a pass with boxes of 32 rows, 138 with 128, 129 with 256; 7B shape, sixteen
   // sequences, passes of several contexts in turn: 79.8 us with 128, 75.8 with 256).  With three stages the stream runs dry
-  // (70B shape, 1024 wide: 915 us against 885 with one tile to a stage).
-  st->bt = h_bytes + 4 * 2 * kTcTileBytes <= budget ? 2 : 1;
+  // (70B shape, 1024 wide: 915 us against 885 with one tile to a stage), and where rows do not start on 128-byte lines the next
+  // K block comes for the other part of a line too late (eight sequences, 552 wide, 65 layers of 16384 rows: 246 us
+  // against 236).
+  st->bt = d.H % kTcKBlock == 0 && h_bytes + 4 * 2 * kTcTileBytes <= budget ? 2 : 1;
   st->n_stages = (int)std::min<size_t>(kTcMaxStages, (budget - h_bytes) / (st->bt * kTcTileBytes));
   st->smem = (size_t)st->n_stages * st->bt * kTcTileBytes + h_bytes + 1024;
   if (!make_map(&a, w2, (uint64_t)d.H, rows, kTcKBlock, st->bt * kTcTileRows)) return false;
