@@ -801,11 +801,6 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, float* x, int B, State* st
     ka.ng = p.ng;
     ka.max_rows = p.max_rows;
     ka.slot_bytes = p.slot_bytes;
-    const unsigned int nl = (unsigned int)(ka.l_end - ka.l_begin);
-    // counters and stamps only ever grow; the next launch starts where this one ends
-    st->read_base += nl * (unsigned int)p.R;
-    st->add_base += nl * (unsigned int)(p.R * kWarps);
-    st->seq_base += nl * (unsigned int)((p.max_rows + kChunk - 1) / kChunk) + 1u;
     const int grid = p.R * p.Q;
     cudaError_t e;
     if (nsg == 1) {
@@ -820,6 +815,11 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, float* x, int B, State* st
       else e = launch_one<2, 10>(ka, p.smem, grid, s);
     }
     if (e != cudaSuccess) return e;
+    // Counters and stamps only ever grow; the next launch starts where this one ends.  (A launch that failed counts nothing.)
+    const unsigned int nl = (unsigned int)(ka.l_end - ka.l_begin);
+    st->read_base += nl * (unsigned int)p.R;
+    st->add_base += nl * (unsigned int)(p.R * kWarps);
+    st->seq_base += nl * (unsigned int)((p.max_rows + kChunk - 1) / kChunk) + 1u;
     *launches += 1;
   }
   return cudaSuccess;

@@ -882,7 +882,6 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s,
     for (int i = 0; i < 2; ++i) ka.xbuf[i] = a.xbuf[i];
     // the launch that ends the stack leaves the result itself
     ka.x_out = std::min(a.l_end, l0 + kMaxLayers) == a.l_end ? a.x_out : nullptr;
-    st->wrote_out = ka.x_out != nullptr;
     for (int i = 0; i < 3; ++i) ka.zbuf[i] = a.zbuf[i];
     ka.zfix = st->zfix;
     ka.bars = st->bars;
@@ -902,11 +901,6 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s,
     ka.max_rows = p.max_rows;
     ka.part_bufs = p.part_bufs;
     ka.slot_bytes = (uint32_t)p.slot_bytes;
-    const unsigned int nl = (unsigned int)(ka.l_end - ka.l_begin);
-    // the counters and stamps only ever grow; the next launch starts where this one ends
-    st->bar_base += (nl > 1 || ka.x_out) ? (unsigned int)p.R : 0u;
-    const int chunk_rows = tiles_chunk(p.kb) * 8;
-    st->seq_base += nl * (unsigned int)((p.max_rows + chunk_rows - 1) / chunk_rows) + 1u;
     const int grid = p.R * kQ;
     cudaError_t e;
 #define NP_SLICES(kb) \
@@ -926,6 +920,12 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s,
     }
 #undef NP_SLICES
     if (e != cudaSuccess) return e;
+    // The counters and stamps only ever grow; the next launch starts where this one ends.  (A launch that failed counts nothing.)
+    const unsigned int nl = (unsigned int)(ka.l_end - ka.l_begin);
+    const int chunk_rows = tiles_chunk(p.kb) * 8;
+    st->bar_base += (nl > 1 || ka.x_out) ? (unsigned int)p.R : 0u;
+    st->seq_base += nl * (unsigned int)((p.max_rows + chunk_rows - 1) / chunk_rows) + 1u;
+    st->wrote_out = ka.x_out != nullptr;
   }
   return cudaSuccess;
 }

@@ -1,0 +1,76 @@
+"""A small library over the internal launch functions of libnp.so, compiled against the internal header, for tests that hand a
+resident kernel its device words themselves."""
+import ctypes as C
+import os
+import subprocess
+import tempfile
+
+from paper_2608_22643_b200 import build as nbuild
+
+_SOURCE = r"""
+#include "np_internal.h"
+using namespace npi;
+static Dims dims(int D, int C, int k, int L) {
+  Dims d = {};
+  d.L = d.Lp = L; d.D = D; d.M = C; d.H = 64; d.k = k; d.C = C; d.W = C / 32; d.Bmax = 16;
+  return d;
+}
+// ptr: gate, up, downT, slots, counters, x (bf16), xbuf[2], zbuf[3], x_out, status, zfix, bars, xch
+extern "C" int t_slices(int D, int C, int k, int L, int sms, void* const* ptr, unsigned int* base, void* stream) {
+  const Dims d = dims(D, C, k, L);
+  ChainArgs a = {};
+  a.gate = ptr[0]; a.up = ptr[1]; a.downT = ptr[2];
+  a.active_slots = static_cast<const int32_t*>(ptr[3]);
+  a.counters = static_cast<const int32_t*>(ptr[4]);
+  a.x_bf16 = ptr[5];
+  for (int i = 0; i < 2; ++i) a.xbuf[i] = static_cast<float*>(ptr[6 + i]);
+  for (int i = 0; i < 3; ++i) a.zbuf[i] = static_cast<float*>(ptr[8 + i]);
+  a.x_out = static_cast<float*>(ptr[11]);
+  a.status = static_cast<int32_t*>(ptr[12]);
+  a.l_end = L;
+  a.check = 1;
+  chain_slices::State st = {};
+  st.zfix = static_cast<unsigned long long*>(ptr[13]);
+  st.bars = static_cast<unsigned int*>(ptr[14]);
+  st.xch = static_cast<unsigned long long*>(ptr[15]);
+  st.bar_base = base[0]; st.seq_base = base[1];
+  const int e = (int)chain_slices::launch(d, a, &st, static_cast<cudaStream_t>(stream), sms);
+  base[0] = st.bar_base; base[1] = st.seq_base; base[2] = (unsigned int)st.wrote_out;
+  return e;
+}
+extern "C" void t_slices_words(int D, int C, int k, int sms, unsigned long long* n) {
+  const Dims d = dims(D, C, k, 1);
+  n[0] = chain_slices::zfix_words(d); n[1] = chain_slices::bar_words(); n[2] = chain_slices::xch_words(d, sms);
+}
+extern "C" int t_batch(int D, int C, int k, int L, int B, int sms, void* stream, unsigned int* base) {
+  const Dims d = dims(D, C, k, L);
+  ChainArgs a = {};
+  a.l_end = L;
+  chain_batch::State st = {};
+  st.read_base = base[0]; st.add_base = base[1]; st.seq_base = base[2];
+  int n = 0;
+  const int e = (int)chain_batch::launch(d, a, nullptr, B, &st, static_cast<cudaStream_t>(stream), sms, &n);
+  base[0] = st.read_base; base[1] = st.add_base; base[2] = st.seq_base;
+  return e;
+}
+"""
+
+
+def load():
+    lib = nbuild.build()
+    out = tempfile.mkdtemp(prefix="np_internals_")
+    src, so = os.path.join(out, "t.cpp"), os.path.join(out, "t.so")
+    with open(src, "w") as f:
+        f.write(_SOURCE)
+    cuda = os.path.join(os.path.dirname(os.path.dirname(nbuild._nvcc())), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", nbuild.CSRC, "-I", nbuild.INCLUDE, "-I", cuda, src,
+                    lib, "-Wl,-rpath," + os.path.dirname(lib), "-o", so], check=True)
+    return C.CDLL(so)
+
+
+def uints(*v):
+    return (C.c_uint * len(v))(*v)
+
+
+def pointers(*v):
+    return (C.c_void_p * len(v))(*v)
