@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kChainBlock, 1) k_mlp_chain(ChainKernelArgs a)
           ++use;
         }
       }
+      npp::drain_ring(full_bar, n_stages, s, use & 1u, a.status);
     }
     return;
   }

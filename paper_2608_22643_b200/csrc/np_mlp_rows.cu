@@ -372,8 +372,15 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
           npp::bulk_g2s_stream(csm + (size_t)s * pstride, src, row_bytes, &full_bar[s], npp::policy_evict_first());
         }
       }
-      good = __all_sync(0xffffffffu, good);
-      v0 += (unsigned int)cnt;
+      const bool all = __all_sync(0xffffffffu, good);
+      if (!all && good && lane < cnt) {  // a copy of a round that could not go out whole
+        int s;
+        uint32_t par;
+        slot_of(v0 + (unsigned int)lane, a.ns_magic, ns, s, par);
+        if (!npp::mbar_wait(&full_bar[s], par)) atomicOr(a.status, npp::kStatTimeout);
+      }
+      good = all;
+      if (good) v0 += (unsigned int)cnt;
     };
     for (int li = 0; li < nl && good; ++li) {
       const int vrow0 = lay_pre[li], nrows = min(lay_pre[li + 1], total_rows) - vrow0;
@@ -384,6 +391,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
       if (nrows > 0) issue(src, 2 * nrows);
       PK(0, 0);
     }
+    // nobody leaves before its copies have landed, also after a time-out: a lane waits for the last use of its slots
+    for (unsigned int s = (unsigned int)lane; s < (unsigned int)ns; s += 32)
+      if (v0 > s && !npp::mbar_wait(&full_bar[s], ((v0 - 1u - s) / (unsigned int)ns) & 1u)) atomicOr(a.status, npp::kStatTimeout);
   } else if (wid == kWarps + 1) {
     // =========================== mover warp ===========================
     // The down rows do not fit into the ring beside the gate and up rows (a block's rows of a layer are about 216 KB),
@@ -449,6 +459,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
             npp::mbar_arrive(&tm_full[buf]);
           }
         }
+      }
+      // after a time-out: the copies on their way into the staging pieces, then those out of them (k of them went out)
+      for (unsigned int s = 0; s < (unsigned int)kDS && !good; ++s) {
+        if (kn > s && !npp::mbar_wait(&ds_full[s], ((kn - 1u - s) / kDS) & 1u)) atomicOr(a.status, npp::kStatTimeout);
+        if (k > s && !npp::mbar_wait(&ds_free[s], ((k - 1u - s) / kDS) & 1u)) atomicOr(a.status, npp::kStatTimeout);
       }
     }
   } else {

@@ -64,17 +64,37 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // A bounded wait on an mbarrier for blocks that drain after a time-out: once any wait of the block has run out (*ok == 0)
-// every later one is skipped.  One loop around one try_wait, not unrolled: with the unrolled loops of mbar_wait at every wait
-// the resident kernels had 80 to 150 KB of code, missed the instruction cache on every layer (195 times at 256 columns) and
-// spent a sixth of their issue slots waiting for instructions.
-__device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
+// every later one is skipped.  True: the phase is complete.  One loop around one try_wait, not unrolled: with the unrolled
+// loops of mbar_wait at every wait k_mlp_slices had 90 to 150 KB of code, missed the instruction cache on every layer (195
+// times at 256 columns) and spent a sixth of its issue slots waiting for instructions.
+__device__ __forceinline__ bool wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
   uint32_t spin = 0;
 #pragma unroll 1
   while (!mbar_try_wait(bar, parity)) {
-    if (!*ok) return;
+    if (!*ok) return false;
     if (++spin == kSpinLimit) {
       *ok = 0;
       atomicOr(status, kStatTimeout);
+    }
+  }
+  return true;
+}
+
+// A block may leave only when the copies it has asked for have landed: after a time-out nobody else waits for them, and they
+// would write to shared memory that is another block's by then.  For the one lane that fills a ring of `n` slots in turn, at
+// its end: `next` is the slot it would fill next, in the use with parity `par`; the slots before it were filled in that use,
+// the others in the one before (or never: the wait for a use before the first returns at once).
+__device__ __forceinline__ void drain_ring(uint64_t* full, int n, int next, uint32_t par, int32_t* status) {
+#pragma unroll 1
+  for (int s = 0; s < n; ++s) {
+    const uint32_t p = s < next ? par : par ^ 1u;
+    uint32_t spin = 0;
+#pragma unroll 1
+    while (!mbar_try_wait(&full[s], p)) {
+      if (++spin == kSpinLimit) {
+        atomicOr(status, kStatTimeout);
+        break;
+      }
     }
   }
 }

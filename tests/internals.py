@@ -42,16 +42,41 @@ extern "C" void t_slices_words(int D, int C, int k, int sms, unsigned long long*
   const Dims d = dims(D, C, k, 1);
   n[0] = chain_slices::zfix_words(d); n[1] = chain_slices::bar_words(); n[2] = chain_slices::xch_words(d, sms);
 }
-extern "C" int t_batch(int D, int C, int k, int L, int B, int sms, void* stream, unsigned int* base) {
+// ptr: gate, up, downT, slots, counters, x (bf16 [B][D]), x as the kernel keeps it, result, status, cnt, xch
+extern "C" int t_batch(int D, int C, int k, int L, int B, int sms, void* const* ptr, unsigned int* base, void* stream) {
   const Dims d = dims(D, C, k, L);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
   ChainArgs a = {};
+  a.gate = ptr[0]; a.up = ptr[1]; a.downT = ptr[2];
+  a.active_slots = static_cast<const int32_t*>(ptr[3]);
+  a.counters = static_cast<const int32_t*>(ptr[4]);
+  a.status = static_cast<int32_t*>(ptr[8]);
   a.l_end = L;
+  a.check = 1;
   chain_batch::State st = {};
+  st.cnt = static_cast<unsigned int*>(ptr[9]);
+  st.xch = static_cast<unsigned long long*>(ptr[10]);
   st.read_base = base[0]; st.add_base = base[1]; st.seq_base = base[2];
+  float* x = static_cast<float*>(ptr[6]);
   int n = 0;
-  const int e = (int)chain_batch::launch(d, a, nullptr, B, &st, static_cast<cudaStream_t>(stream), sms, &n);
+  int e = (int)chain_batch::launch_in(d, ptr[5], x, B, s);
+  if (!e) e = (int)chain_batch::launch(d, a, x, B, &st, s, sms, &n);
+  if (!e) e = (int)chain_batch::launch_out(d, x, static_cast<float*>(ptr[7]), B, s);
   base[0] = st.read_base; base[1] = st.add_base; base[2] = st.seq_base;
   return e;
+}
+extern "C" int t_batch_record(unsigned int* base) {  // a launch that the caller knows to fail
+  chain_batch::State st = {};
+  st.read_base = base[0]; st.add_base = base[1]; st.seq_base = base[2];
+  ChainArgs a = {};
+  a.l_end = 3;
+  int n = 0;
+  const int e = (int)chain_batch::launch(dims(256, 512, 60, 3), a, nullptr, 4, &st, nullptr, 148, &n);
+  base[0] = st.read_base; base[1] = st.add_base; base[2] = st.seq_base;
+  return e;
+}
+extern "C" void t_batch_words(int sms, unsigned long long* n) {
+  n[0] = chain_batch::cnt_words(); n[1] = chain_batch::xch_words(sms);
 }
 """
 
