@@ -129,14 +129,13 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
 }
 
 // One lane's bounded wait on an mbarrier; after the block's first time-out nothing waits any more.
-// True: the phase is complete.
-__device__ __forceinline__ bool wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
-  if (npp::mbar_try_wait(bar, parity)) return true;
-  if (!*ok) return false;
-  if (npp::mbar_wait(bar, parity)) return true;
-  *ok = 0;
-  atomicOr(status, npp::kStatTimeout);
-  return false;
+__device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
+  if (npp::mbar_try_wait(bar, parity)) return;
+  if (!*ok) return;
+  if (!npp::mbar_wait(bar, parity)) {
+    *ok = 0;
+    atomicOr(status, npp::kStatTimeout);
+  }
 }
 __device__ __forceinline__ void warp_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status, int lane) {
   if (lane == 0) wait_or_flag(bar, parity, ok, status);
@@ -443,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     if (wid == kProducer) {
       // ---- producer: gate|up tiles of a layer (8 records), its down tiles (16), the next layer's, in the order of use ----
       int slot = 0;
-      uint32_t par = 0;
+      uint32_t par = 0, patience = npp::kSpinLimit;
       const uint64_t pol = npp::policy_evict_first();  // a row is read once per token
       const size_t qoff = (size_t)k0 * 32;
       for (int li = 0; li < nl; ++li) {
@@ -453,16 +452,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           const int step = pass == 0 ? 8 : 16;
           for (int r0 = 0; r0 < nrows; r0 += step) {
             const int n = min(step, nrows - r0);
-            bool free = true;
             if (lane == 0) {
-              free = wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status);
-              if (free) npp::mbar_expect_tx(&full_bar[slot], (uint32_t)(pass == 0 ? 2 * n : n) * piece_bytes);
+              wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status);
+              npp::mbar_expect_tx(&full_bar[slot], (uint32_t)(pass == 0 ? 2 * n : n) * piece_bytes);
             }
             __syncwarp();
-            if (!__shfl_sync(0xffffffffu, free, 0)) {  // after a time-out: no copy into a slot that is still full
-              if (lane == 0) npp::drain_ring(full_bar, a.ng, slot, par, a.status);
-              return;
-            }
             const int i = pass == 0 ? (lane & 7) : lane;
             if (lane < 16 && i < n) {
               const int row = r0 + i;
@@ -478,7 +472,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           }
         }
       }
-      if (lane == 0) npp::drain_ring(full_bar, a.ng, slot, par, a.status);
+      // Nobody leaves before the copies have landed.  (After a time-out the producer has not waited for free slots, and a slot's
+      // barrier may have lost count of two uses that overlapped: then a time that is far longer than any copy's.)
+      if (lane == 0) npp::drain_ring(full_bar, a.ng, slot, par, patience);
+      if (!*ok) __nanosleep(500000);
     } else if (wid == kSync) {
       // ---- synchroniser: the two counters of the slice ----
       if (lane == 0) {

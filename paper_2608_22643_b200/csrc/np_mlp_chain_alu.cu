@@ -179,7 +179,8 @@ __global__ void __launch_bounds__(kChainBlock, 1) k_mlp_chain(ChainKernelArgs a)
           ++use;
         }
       }
-      npp::drain_ring(full_bar, n_stages, s, use & 1u, a.status);
+      uint32_t patience = npp::kSpinLimit;
+      npp::drain_ring(full_bar, n_stages, s, use & 1u, patience);
     }
     return;
   }

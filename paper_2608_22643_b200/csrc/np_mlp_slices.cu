@@ -58,7 +58,7 @@
 //
 // Every wait (mbarrier, exchange words, counted sums) is bounded; once one has run out the block
 // records kStatTimeout and skips all later waits, so the kernel drains; the blocks that depend on it
-// follow at their next wait.  The producer stops and stays until its copies have landed.
+// follow at their next wait.  The producer stays until its copies have landed.
 #include <algorithm>
 
 #include "np_device.cuh"
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     // after a wait); a slot's copies are then issued by as many lanes as it has pieces.  The slots of a layer's rows
     // are fetched a layer ahead.
     int slot = 0;
-    uint32_t par = 0;
+    uint32_t par = 0, patience = npp::kSpinLimit;
     // A row is read once per token: the copies mark their lines evict-first, so that the 27 MB a layer streams
     // through the L2 do not push out the few hundred KB every layer meets in (exchange words, counted sums).
     const uint64_t l2_policy = npp::policy_evict_first();
@@ -371,16 +371,12 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 #pragma unroll 1
         for (int r0 = 0; r0 < nrows; r0 += step) {
           const int npieces = min(step, nrows - r0) << (pass == 0 ? 1 : 0);
-          bool free = true;
           if (lane == 0) {
-            free = npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status);
-            if (free) npp::mbar_expect_tx(&full_bar[slot], (uint32_t)npieces * piece_bytes);
+            // (after a time-out the slot may be taken from its readers, not from the copies under way)
+            if (!npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status)) npp::wait_landed(&full_bar[slot], par ^ 1u, patience);
+            npp::mbar_expect_tx(&full_bar[slot], (uint32_t)npieces * piece_bytes);
           }
           __syncwarp();  // the expect_tx precedes the copies
-          if (!__shfl_sync(0xffffffffu, free, 0)) {  // after a time-out: no copy into a slot that is still full
-            if (lane == 0) npp::drain_ring(full_bar, ng, slot, par, a.status);
-            return;
-          }
           if (lane < npieces) {
             int s = rows[r0 + (pass == 0 ? lane >> 1 : lane)];
             if (a.check && (s < 0 || s >= a.C)) {
@@ -398,7 +394,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
         }
       }
     }
-    if (lane == 0) npp::drain_ring(full_bar, ng, slot, par, a.status);
+    if (lane == 0) npp::drain_ring(full_bar, ng, slot, par, patience);
     return;
   }
 

@@ -81,22 +81,17 @@ __device__ __forceinline__ bool wait_or_flag(uint64_t* bar, uint32_t parity, vol
 }
 
 // A block may leave only when the copies it has asked for have landed: after a time-out nobody else waits for them, and they
-// would write to shared memory that is another block's by then.  For the one lane that fills a ring of `n` slots in turn, at
-// its end: `next` is the slot it would fill next, in the use with parity `par`; the slots before it were filled in that use,
-// the others in the one before (or never: the wait for a use before the first returns at once).
-__device__ __forceinline__ void drain_ring(uint64_t* full, int n, int next, uint32_t par, int32_t* status) {
+// would write to shared memory that is another block's by then.  `patience`: polls left to the block for all of this.
+__device__ __forceinline__ void wait_landed(uint64_t* full, uint32_t parity, uint32_t& patience) {
 #pragma unroll 1
-  for (int s = 0; s < n; ++s) {
-    const uint32_t p = s < next ? par : par ^ 1u;
-    uint32_t spin = 0;
+  while (patience > 0 && !mbar_try_wait(full, parity)) --patience;
+}
+// For the one lane that fills a ring of `n` slots in turn, at its end: `next` is the slot it would fill next, in the use with
+// parity `par`; the slots before it were filled in that use, the others in the one before (or never: the wait for a use before
+// the first returns at once).
+__device__ __forceinline__ void drain_ring(uint64_t* full, int n, int next, uint32_t par, uint32_t& patience) {
 #pragma unroll 1
-    while (!mbar_try_wait(&full[s], p)) {
-      if (++spin == kSpinLimit) {
-        atomicOr(status, kStatTimeout);
-        break;
-      }
-    }
-  }
+  for (int s = 0; s < n; ++s) wait_landed(&full[s], s < next ? par : par ^ 1u, patience);
 }
 
 // 1-D bulk copy global -> this CTA's shared memory; completion is reported to
