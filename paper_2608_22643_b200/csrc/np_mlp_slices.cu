@@ -491,9 +491,9 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
         seen ^= p0.x ^ p0.y ^ p1.x ^ p1.y;
       }
     }
-    // Every value has arrived (it is stored, to words that hold nothing yet) before the block counts itself in: only then may
-    // any block of the slice add to these words.
-    static_cast<volatile uint32_t*>(bs)[lane] = (uint32_t)(seen >> 32) ^ (uint32_t)seen;
+    // Every value has arrived (it is compared, to no effect) before the block counts itself in: only then may any block of the
+    // slice add to these words.
+    if (seen == 0xffffffffffffffffull) static_cast<volatile uint32_t*>(bs)[lane] = 0u;
     asm volatile("bar.sync 1, %0;" ::"r"(a.nw * 32) : "memory");
     if (tid == 0) atomicAdd(a.bars + q * kBarStride, 1u);
   }
