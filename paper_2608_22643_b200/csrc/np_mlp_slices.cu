@@ -196,17 +196,20 @@ __device__ __forceinline__ void exchange_rows(const KArgs& a, const float* part,
                                               int q, int lane, unsigned int stamp, uint64_t* ss_bar, uint32_t ss_par, float& inv_rms, volatile int* ok) {
   const int row = row0 + lane;
   const bool has_row = row < rows, want_ss = first && lane == 0;
-  float own_g = 0.f, own_u = 0.f, own_ss = 0.f;
+  float own_ss = 0.f;
   const float2* pp = reinterpret_cast<const float2*>(part) + row;
   float2 pv[kWarps];
 #pragma unroll
   for (int w = 0; w < kWarps; ++w)  // rows past the round's: whatever is there, not looked at
     pv[w] = w < a.nw ? pp[w * (kChunkVec / 2)] : make_float2(0.f, 0.f);
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    own_g += pv[w].x;
-    own_u += pv[w].y;
-  }
+  for (int o = kWarps / 2; o > 0; o >>= 1)  // in pairs: three roundings of a sum where one after the other takes seven
+#pragma unroll
+    for (int w = 0; w < o; ++w) {
+      pv[w].x += pv[w + o].x;
+      pv[w].y += pv[w + o].y;
+    }
+  const float own_g = pv[0].x, own_u = pv[0].y;
   if (has_row) st_relaxed_v2u64(mine + 2 * row, stamped(own_g, stamp), stamped(own_u, stamp));
   if (first) {  // the sums of squares come behind the dot products
     npp::wait_or_flag(ss_bar, ss_par, ok, a.status);
@@ -657,16 +660,22 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
       float* pw = part + ((size_t)(nx & (unsigned int)(a.part_bufs - 1)) * a.nw + wid) * kChunkVec + tc * 16 + g8 + 8 * (t4 & 1);
 #pragma unroll
       for (int u = 0; u < PT; u += 2) {
-        float c[2][4];
+        float c[2][2][4];  // a tile's odd K blocks add up beside its even ones: half the roundings of one chain
 #pragma unroll
-        for (int v = 0; v < 2; ++v) c[v][0] = c[v][1] = c[v][2] = c[v][3] = 0.f;
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) c[v][0][e] = c[v][1][e] = 0.f;
 #pragma unroll
         for (int i = 0; i < KB; ++i)
 #pragma unroll
           for (int v = 0; v < 2 && u + v < PT; ++v)
-            if (FULL || i < nkb) mma_bf16_16816(c[v], af[u + v][i], xb[i >> 1][(i & 1) * 2], xb[i >> 1][(i & 1) * 2 + 1]);
-        const float lo = t4 < 2 ? c[0][0] + c[0][1] : c[1][0] + c[1][1];
-        const float hi = t4 < 2 ? c[0][2] + c[0][3] : c[1][2] + c[1][3];
+            if (FULL || i < nkb) mma_bf16_16816(c[v][i & 1], af[u + v][i], xb[i >> 1][(i & 1) * 2], xb[i >> 1][(i & 1) * 2 + 1]);
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) c[v][0][e] += c[v][1][e];
+        const float lo = t4 < 2 ? c[0][0][0] + c[0][0][1] : c[1][0][0] + c[1][0][1];
+        const float hi = t4 < 2 ? c[0][0][2] + c[0][0][3] : c[1][0][2] + c[1][0][3];
         const float other = __shfl_xor_sync(0xffffffffu, (t4 & 1) ? lo : hi, 1);
         const int tile = u + (t4 >> 1);
         if (tile < PT && t0 + tile < nt) pw[tile * 16] = ((t4 & 1) ? hi : lo) + other;

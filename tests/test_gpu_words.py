@@ -14,10 +14,10 @@ TIMEOUT = 8     # the status bit of a wait that ran out
 class Words:
     """A small stack whose rows are resident, and the words a launch meets its other blocks in."""
 
-    def __init__(self, lib, D, C, k, L, B=1):
+    def __init__(self, lib, D, C, k, L, B=1, seed=3):
         self.lib, self.shape, self.B = lib, (D, C, k, L), B
         self.sms = torch.cuda.get_device_properties(0).multi_processor_count
-        g = torch.Generator(device="cuda").manual_seed(3)
+        g = torch.Generator(device="cuda").manual_seed(seed)
         self.rows = [(torch.randn(L, C, D, generator=g, device="cuda") * 0.02).to(torch.bfloat16) for _ in range(3)]
         self.slots = torch.stack([torch.randperm(C, generator=g, device="cuda") for _ in range(L)]).to(torch.int32)
         self.counters = torch.zeros(L, nb.NP_N_COUNTERS, dtype=torch.int32, device="cuda")
@@ -100,3 +100,18 @@ def test_a_wait_that_runs_out(lib, B, D):
     w.clear()
     got, status = w.run()
     assert status == 0 and w.error(got) < 1e-5
+
+
+# A multiplication that adds to a long chain truncates at every step.  Mean of four inputs with one chain per tile and the warps'
+# sums added one after the other 3.06e-7, 7.41e-7, 8.53e-7; two chains and sums in pairs 2.74e-7, 5.84e-7, 6.67e-7.  The same
+# inputs give the same bits, so a limit between them tells them apart.
+@pytest.mark.parametrize("D,k,most", [(2384, 600, 2.9e-7), (4112, 1101, 6.6e-7), (5120, 1382, 7.6e-7)])
+def test_error_of_the_sums(lib, D, k, most):
+    """20 layers against 64-bit sums."""
+    errors = []
+    for seed in range(4):
+        w = Words(lib, D, k + 100, k, 20, seed=seed)
+        got, status = w.run()
+        assert status == 0
+        errors.append(w.error(got))
+    assert sum(errors) / 4 < most
