@@ -23,7 +23,7 @@
 //          block-wide barrier, and x is never read from another warp's part of shared memory.  (With
 //          the rows dealt to the warps instead, eight of them, x went through shared memory and a
 //          barrier to all, and every warp read half of it back: 7.3 us per layer at the 7B shape, 5.4 now;
-//          13B 8.1 and 7.0, 70B 15.1 and 12.5, 256 columns and 60 rows 4.7 and 2.9.)
+//          13B 8.1 and 7.0, 70B 15.1 and 12.1, 256 columns and 60 rows 4.7 and 2.9.)
 // rows     What a phase multiplies is in registers as A fragments before its operand arrives: gate
 //          and up tiles are loaded while the sums of the layer before are on their way, down tiles
 //          during the exchange.  A tile's ring slot is free as soon as it is loaded, so the registers
@@ -77,6 +77,7 @@ constexpr int kBlock = (kWarps + 4) * 32;  // plus the producer warp, two exchan
 constexpr int kConsumerRegs = 208;     // 256 x 208 + 128 x 88 = 384 x 168, what the block is launched with
 constexpr int kOtherRegs = 88;
 constexpr int kExchWarps = 2;              // each takes 32 rows of a round
+constexpr int kSlotPieces = 16;        // pieces of a ring slot: an MMA tile.  (Slots of 8 or 4: 7B shape 210 and 288 us where 16 took 204.)
 constexpr int kMaxSlots = 32;          // ring slots
 constexpr int kBarStride = 32;         // one 128-byte line per counter
 constexpr int kFixShift = 30;          // fixed-point position of the counted sums
@@ -117,7 +118,7 @@ struct KArgs {
   unsigned int seq_base;       // stamp of the launch's first exchange minus one
   int l_begin, l_end, D, C, check;
   int nw, kw;                  // consumer warps that own columns, K blocks of each (the last may have fewer)
-  int vg_shift, ng;            // log2 of the pieces per ring slot, ring slots
+  int ng;                      // ring slots
   int max_rows;                // most rows a block can have in a layer
   int part_bufs;               // rounds of partial dot products held (1 or 2)
   uint32_t slot_bytes;
@@ -182,7 +183,9 @@ __device__ __forceinline__ unsigned long long stamped(float v, unsigned int stam
   return ((unsigned long long)stamp << 32) | (unsigned long long)__float_as_uint(v);
 }
 
-// An arrival that waits for a loaded register.
+// An arrival whose address is formed with a loaded register.  The order of the loads and what is written behind the arrival does
+// not need it (__syncwarp and the arrival's release give that); it keeps the compiler from moving loads across the arrival:
+// with a plain one the instances with sixteen K blocks spill 104 to 148 bytes (70B shape 1046 us per 80 layers against 968).
 __device__ __forceinline__ void mbar_arrive_after(uint64_t* bar, uint32_t loaded) {
   asm volatile("{\n\t.reg .b32 t;\n\tand.b32 t, %1, 0;\n\tadd.u32 t, t, %0;\n\tmbarrier.arrive.shared::cta.b64 _, [t];\n\t}" ::"r"(npp::smem_addr(bar)), "r"(loaded)
                : "memory");
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
   const int nk = (q + 1) * (D >> 4) / Q - kq0;     // 16-wide K blocks = 16-column tiles of the slice
   const uint32_t piece_bytes = (uint32_t)nk * 32u;
   const uint32_t pstride = piece_bytes + kPad;     // distance between pieces in shared memory
-  const int gs = a.vg_shift, VG = 1 << gs, ng = a.ng;
+  const int ng = a.ng;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int nl = a.l_end - a.l_begin;
   const int apad = ((a.max_rows + 15) & ~15) + 16;  // activations per term, padded so that a 16-row block never runs out
@@ -311,7 +314,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
   uint32_t* bstage = reinterpret_cast<uint32_t*>(csm + (size_t)ng * a.slot_bytes);         // [nw][bstage_words]
   float* part = reinterpret_cast<float*>(bstage + (size_t)a.nw * bstage_words(KB));        // [part_bufs][nw][kChunkVec]
   uint16_t* aterm = reinterpret_cast<uint16_t*>(part + (size_t)a.part_bufs * a.nw * kChunkVec);  // [3][apad] bf16 terms of a_i
-  int32_t* slot_buf = reinterpret_cast<int32_t*>(aterm + 3 * apad + (apad & 1));           // [2][max_rows]
+  int32_t* slot_buf = reinterpret_cast<int32_t*>(aterm + 3 * apad);                        // [2][max_rows]
   volatile int* ok = &s_ok;
 
   // ---- this row group's share of every layer of the run ----
@@ -367,10 +370,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
       const int nrows = lay_n[li];
       const int32_t* rows = slot_buf + (size_t)(li & 1) * a.max_rows;
       const size_t lbase = (size_t)(a.l_begin + li) * layer_bytes + (size_t)kq0 * 32;
-      // pass 0: gate|up pieces (VG / 2 rows a slot, two pieces each); pass 1: down pieces (VG rows)
+      // pass 0: gate|up pieces (8 rows a slot, two pieces each); pass 1: down pieces (16 rows)
 #pragma unroll 1
       for (int pass = 0; pass < 2; ++pass) {
-        const int step = pass == 0 ? VG >> 1 : VG;
+        const int step = pass == 0 ? kSlotPieces / 2 : kSlotPieces;
 #pragma unroll 1
         for (int r0 = 0; r0 < nrows; r0 += step) {
           const int npieces = min(step, nrows - r0) << (pass == 0 ? 1 : 0);
@@ -419,8 +422,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
         const unsigned long long* base = a.xch + ((size_t)(nx & 1u) * G + (size_t)r * Q) * kXchStride;
         const float* pt = part + (size_t)(nx & (unsigned int)(a.part_bufs - 1)) * a.nw * kChunkVec;
         const int rows = min(CT * 8, nrows - c0);
-        // (a warp without rows now may have some in a later round: it needs the sum of squares, too)
-        if (32 * e < rows || nrows > c0 + rows) exchange_rows(a, pt, ssq_part, aterm + c0, apad, mine, base, 32 * e, rows, c0 == 0, q, lane, stamp, &ss_bar, nss & 1u, inv_rms, ok);
+        // (a warp without rows in the first round has none in a later one, for which it would need the sum of squares)
+        if (32 * e < rows) exchange_rows(a, pt, ssq_part, aterm + c0, apad, mine, base, 32 * e, rows, c0 == 0, q, lane, stamp, &ss_bar, nss & 1u, inv_rms, ok);
         __syncwarp();
         if (lane == 0) npp::mbar_arrive(&act_bar);
         ++nx;
@@ -451,22 +454,22 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     int s = slot;
     uint32_t p = par;
 #pragma unroll 1
-    for (; n > 0; n -= VG) {
+    for (; n > 0; n -= kSlotPieces) {
       npp::wait_or_flag(&full_bar[s], p, ok, a.status);
       if (++s == ng) s = 0, p ^= 1u;
     }
   };
-  // address of piece i of the group
-  auto piece = [&](int i) -> uint32_t {
-    int s = slot + (i >> gs);
+  // address of tile u of the group: a slot each
+  auto tile_at = [&](int u) -> uint32_t {
+    int s = slot + u;
     if (s >= ng) s -= ng;
-    return ring + (uint32_t)s * a.slot_bytes + (uint32_t)(i & (VG - 1)) * pstride;
+    return ring + (uint32_t)s * a.slot_bytes;
   };
-  // gives the group's slots back; `last`: a register of its last load, which has arrived before that
+  // gives the group's slots back; `last`: a register loaded from its last tile
   auto group_release = [&](int n, uint32_t last) {
     __syncwarp();  // every lane has loaded its part
 #pragma unroll 1
-    for (; n > 0; n -= VG) {
+    for (; n > 0; n -= kSlotPieces) {
       if (lane == 0) mbar_arrive_after(&empty_bar[slot], last);
       if (++slot == ng) slot = 0, par ^= 1u;
     }
@@ -501,7 +504,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     if (tid == 0) atomicAdd(a.bars + q * kBarStride, 1u);
   }
 
-#pragma unroll 1
   // x += the sums in the set at `zw`, once every row group has added its part.  Two pairs of columns are polled together.
   auto add_sums = [&](const unsigned long long* zw) {
 #pragma unroll
@@ -544,6 +546,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     }
   };
 
+#pragma unroll 1
   for (int li = 0; li < nl; ++li) {
     const int l = a.l_begin + li;
     const int nrows = lay_n[li], nvec = 2 * nrows;
@@ -564,7 +567,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 #pragma unroll
         for (int u = 0; u < WT && v + u < PT; ++u) {
           if (16 * u < n) {
-            const uint32_t p = piece(min(16 * u + rr + 8 * (m4 & 1), n - 1)) + (uint32_t)(m4 >> 1) * 16u;
+            const uint32_t p = tile_at(u) + (uint32_t)min(rr + 8 * (m4 & 1), n - 1 - 16 * u) * pstride + (uint32_t)(m4 >> 1) * 16u;
 #pragma unroll
             for (int i = 0; i < KB; ++i) {
               if (FULL || i < nkb) ldmatrix_x4(af[v + u][i], p + (uint32_t)i * 32u);
@@ -712,7 +715,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 #pragma unroll
         for (int u = 0; u < PD; ++u) {
           if (16 * u < n) {
-            const uint32_t p = piece(min(16 * u + rr + 8 * (m4 >> 1), n - 1)) + (uint32_t)(m4 & 1) * 16u;
+            const uint32_t p = tile_at(u) + (uint32_t)min(rr + 8 * (m4 >> 1), n - 1 - 16 * u) * pstride + (uint32_t)(m4 & 1) * 16u;
 #pragma unroll
             for (int j = 0; j < KH; ++j) {
               if (FULL || j0 + j < nkb) ldmatrix_x4_trans(df[u][j], p + (uint32_t)(j0 + j) * 32u);
@@ -800,7 +803,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 
 namespace {
 struct Plan {
-  int R, kb, kw, nw, vg_shift, ng, max_rows, part_bufs;
+  int R, kb, kw, nw, ng, max_rows, part_bufs;
   bool full;  // every warp of every slice has kb K blocks
   size_t slot_bytes, smem;
 };
@@ -823,24 +826,17 @@ bool plan(const Dims& d, int sm_count, Plan* p) {
   p->part_bufs = expect > tiles_chunk(KB) * 8 ? 2 : 1;  // rounds follow each other where a share has more rows than one
   const int apad = ((p->max_rows + 15) & ~15) + 16;
   const size_t fixed = (size_t)p->nw * bstage_words(KB) * 4 + (size_t)p->part_bufs * p->nw * kChunkVec * 4 +
-                       (size_t)(3 * apad + (apad & 1)) * 2 + (size_t)2 * p->max_rows * 4 + 128;
+                       (size_t)(3 * apad) * 2 + (size_t)2 * p->max_rows * 4 + 128;
   const size_t budget = 227 * 1024 - 2560;  // static shared memory of the kernel
   const size_t pstride = (size_t)nk * 32 + kPad;
-  int vg = 4;
-  // slots of 16 pieces, of fewer where the ring would hold no more than the tiles a warp loads at a time
-  const int least = 16 * std::max(tiles_up(KB), tiles_down(KB));  // pieces
-  for (; vg >= 1; --vg) {
-    const size_t slot_bytes = pstride << vg;
-    const int ng_min = (least >> vg) + (vg > 2 ? 1 : 0);
-    if (fixed + ng_min * slot_bytes > budget) continue;
-    p->vg_shift = vg;
-    p->slot_bytes = slot_bytes;
-    p->ng = (int)std::min<size_t>(kMaxSlots, (budget - fixed) / slot_bytes);
-    if (d.ring_stages >= 2) p->ng = std::max(ng_min, std::min(p->ng, d.ring_stages));
-    p->smem = (size_t)p->ng * slot_bytes + fixed;
-    return true;
-  }
-  return false;
+  // the tiles a warp loads at a time and one more (every width to 8192 and capacity to 40960 has room for that on 100 SMs and more)
+  const int ng_min = std::max(tiles_up(KB), tiles_down(KB)) + 1;
+  p->slot_bytes = pstride * kSlotPieces;
+  if (fixed + ng_min * p->slot_bytes > budget) return false;
+  p->ng = (int)std::min<size_t>(kMaxSlots, (budget - fixed) / p->slot_bytes);
+  if (d.ring_stages >= 2) p->ng = std::max(ng_min, std::min(p->ng, d.ring_stages));
+  p->smem = (size_t)p->ng * p->slot_bytes + fixed;
+  return true;
 }
 }  // namespace
 
@@ -907,7 +903,6 @@ cudaError_t launch(const Dims& d, const ChainArgs& a, State* st, cudaStream_t s,
     ka.check = a.check;
     ka.nw = p.nw;
     ka.kw = p.kw;
-    ka.vg_shift = p.vg_shift;
     ka.ng = p.ng;
     ka.max_rows = p.max_rows;
     ka.part_bufs = p.part_bufs;

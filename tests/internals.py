@@ -38,6 +38,7 @@ extern "C" int t_slices(int D, int C, int k, int L, int sms, void* const* ptr, u
   base[0] = st.bar_base; base[1] = st.seq_base; base[2] = (unsigned int)st.wrote_out;
   return e;
 }
+extern "C" int t_slices_supported(int D, int C, int k, int sms) { return chain_slices::supported(dims(D, C, k, 1), sms); }
 extern "C" void t_slices_words(int D, int C, int k, int sms, unsigned long long* n) {
   const Dims d = dims(D, C, k, 1);
   n[0] = chain_slices::zfix_words(d); n[1] = chain_slices::bar_words(); n[2] = chain_slices::xch_words(d, sms);
