@@ -1605,8 +1605,9 @@ static int mlp_chain(np_ctx* ctx, const void* x_bf16, int B, float* x_out, cudaS
         NP_LAUNCH(ctx, chain_slices::launch(d, a, &ctx->slices, s, sms));
         out_written = a.x_out && ctx->slices.wrote_out;
       } else {
-        ctx->chain_kernel_launches += 1;
-        NP_LAUNCH(ctx, chain_alu::launch(d, a, s, resident_sms(ctx, beside_pull, chain_alu::supported)));
+        const int sms = resident_sms(ctx, beside_pull, chain_alu::supported), run = chain_alu::run_layers(d, sms);
+        ctx->chain_kernel_launches += (l1 - l0 + run - 1) / run;
+        NP_LAUNCH(ctx, chain_alu::launch(d, a, s, sms));
       }
       l0 = l1;
     }

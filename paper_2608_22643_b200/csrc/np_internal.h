@@ -206,6 +206,7 @@ cudaError_t launch(const Dims& d, const void* rec0, int rows, float* const xbuf[
 }  // namespace dense_chain
 namespace chain_alu {  // row-partitioned resident kernel (np_mlp_chain_alu.cu): any row width; the sliced kernel's fallback
 bool supported(const Dims& d, int sm_count);
+int run_layers(const Dims& d, int sm_count);  // layers per launch
 cudaError_t launch(const Dims& d, const ChainArgs& a, cudaStream_t s, int sm_count);
 }  // namespace chain_alu
 

@@ -477,6 +477,11 @@ bool supported(const Dims& d, int sm_count) {
   return alu_plan(d, sm_count, &p);
 }
 
+int run_layers(const Dims& d, int sm_count) {
+  AluPlan p;
+  return alu_plan(d, sm_count, &p) ? p.run_layers : 0;
+}
+
 cudaError_t launch(const Dims& d_in, const ChainArgs& a, cudaStream_t s, int sm_count) {
   Dims d = d_in;
   if (a.dense_rows > 0) {  // plan for layers whose every row is active

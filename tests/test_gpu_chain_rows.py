@@ -99,3 +99,21 @@ def test_chain_tiles(D, M, k, L):
         p.eng.counters()
     finally:
         p.close()
+
+
+def test_launches_of_the_row_partitioned_kernel():
+    """More layers than one of its launches covers: both are counted."""
+    cfg = synth.StackConfig("long", 130, 64, 128, 32, 25, 50, 1, 31, 0.9)
+    p = Pair(cfg, max_batch=1, flags=nb.NP_F_CHECK_BOUNDS | nb.NP_F_ROW_CHAIN, with_oracle=False)
+    try:
+        assert nb.np_mlp_kernel_name(p.eng.ctx, 1) == "k_mlp_chain_alu"
+        x = synth.hidden_states(cfg, 1)[0].cuda()
+        out = torch.empty((1, cfg.d_model), dtype=torch.float32, device="cuda")
+        nb.np_step(p.eng.ctx, x, 1, out, p.eng.stream, p.eng.copy_stream)
+        torch.cuda.synchronize()
+        nb.np_mlp_chain(p.eng.ctx, x, 1, out, p.eng.stream)
+        torch.cuda.synchronize()
+        assert nb.np_chain_launches(p.eng.ctx) == 2
+        p.eng.counters()
+    finally:
+        p.close()
