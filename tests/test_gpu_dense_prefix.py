@@ -90,6 +90,38 @@ def test_dense_layers_at_other_row_widths(cfg, d):
         p.close()
 
 
+def test_the_widest_rows_behind_a_dense_layer():
+    """13264 columns: the sparse layers' slots have room beside the ring only for half the layers a launch otherwise takes."""
+    L, D, M, C, k = 3, 13264, 11424, 4448, 300
+    cfg = synth.StackConfig("wide", L, D, M, 32, 0, 0, 2, 41, 0.9)
+    p = Pair(cfg, k=k, C=C, transfer_mode=nb.NP_XFER_HOST_GATHER, staging_rows=64, dense_layers=1, store_layers=1, gen_device="cuda",
+             with_oracle=False)
+    try:
+        assert nb.np_mlp_kernel_name(p.eng.ctx, 1) == "k_mlp_chain_alu"
+        xs = synth.hidden_states(cfg, 2)
+        out = torch.empty((1, D), dtype=torch.float32, device="cuda")
+        for t in range(2):
+            nb.np_step(p.eng.ctx, xs[t].cuda(), 1, out, p.eng.stream, p.eng.copy_stream)
+            torch.cuda.synchronize()
+            cnt = p.eng.counters()
+            want = xs[t, 0].cuda().double()
+            for l in range(L):
+                if l == 0:
+                    rows = p.eng.dense[0].unbind(1)
+                else:
+                    slots = torch.as_tensor(p.eng.delta_lists(l, cnt[l])["active_slots"].astype("int64")).cuda()
+                    assert len(slots) == k
+                    rows = [b[l - 1][slots] for b in (p.eng.gate, p.eng.up, p.eng.downT)]
+                n = want / torch.sqrt((want * want).mean() + 1e-6)
+                g, u = (torch.cat([part.double() @ n for part in r.split(1024)]) for r in rows[:2])
+                h = g / (1 + torch.exp(-g)) * u
+                want = want + sum(a @ part.double() for a, part in zip(h.split(1024), rows[2].split(1024)))
+            assert rel_l2(out.cpu().numpy()[0], want.cpu().numpy()) < 1e-5, t    # fp32 sums of up to 13264 products: 1e-6
+        p.check_resident_bytes()
+    finally:
+        p.close()
+
+
 def test_all_layers_dense():
     cfg = TINY
     p = Pair(cfg, dense_layers=cfg.n_layers)
