@@ -12,13 +12,13 @@
 // still bound by the single pass over W2:
 //
 //   * W2 tiles [128 rows x 64 k] come in by tiled TMA (128-byte swizzle, the layout the MMA
-//     shared-memory descriptor expects), two tiles to a copy, through a ring of 32 KB stages, one producer lane.
+//     shared-memory descriptor expects), one or two tiles to a copy, through a ring of 16 or 32 KB stages, one producer lane.
 //   * hidden is fp32; to keep fp32 accuracy it is split into three bf16 terms
 //     (h = h0 + h1 + h2 exactly up to 2^-24), which become 48 N-columns; the three partial
 //     products are added in the epilogue.  The extra MMA work is free under the W2 stream.
 //   * one lane issues the MMAs (4 per tile and stage, K = 16 each) and commits each stage back to the
-//     producer and each finished pair of tiles to the epilogue; two pairs of 64-column accumulators in
-//     tensor memory let the epilogue of pair i overlap the MMAs of pair i+1.
+//     producer and each finished tile or pair to the epilogue; two pairs of 64-column accumulators in
+//     tensor memory let the epilogue of group i overlap the MMAs of group i+1.
 //   * 4 epilogue warps read their 32 TMEM lanes (tcgen05.ld), add the three terms and store
 //     coalesced fp32 logits.
 //
@@ -466,13 +466,14 @@ bool pred_tc_prepare(const Dims& d, const void* w1, const void* w2, void* hsplit
   const size_t h_bytes = (size_t)((d.H + kTcKBlock - 1) / kTcKBlock) * kTcN * kTcKBlock * 2;
   const size_t budget = 220 * 1024 - 1024;  // alignment slack
   if (h_bytes + 2 * kTcTileBytes > budget) return false;
-  // Two tiles to a stage where four such stages fit: a copy instruction costs the SM's copy unit some 80 cycles whatever it
-  // brings (13B shape, three sequences: 176 us a pass with boxes of 32 rows, 138 with 128, 129 with 256; 7B shape, sixteen
-  // sequences, passes of several contexts in turn: 79.8 us with 128, 75.8 with 256).  With three stages the stream runs dry
-  // (70B shape, 1024 wide: 915 us against 885 with one tile to a stage), and where rows do not start on 128-byte lines the next
-  // K block comes for the other part of a line too late (eight sequences, 552 wide, 65 layers of 16384 rows: 246 us
-  // against 236).
-  st->bt = d.H % kTcKBlock == 0 && h_bytes + 4 * 2 * kTcTileBytes <= budget ? 2 : 1;
+  // Two tiles to a stage for narrow hidden vectors: a tile is then a handful of K blocks, and what it costs is the hand-over of
+  // its stages and accumulator.  Wider ones reach the copy rate with one tile and lose with two, whose stages are half as many
+  // and twice as coarse.  A pass alone on its stream, one tile and two: 136 wide, 60 layers of 3072 rows, three sequences 42 and
+  // 38 us; 256, 60 of 5824, three 61 and 56, sixteen 76 and 74; 320, 60 of 7296, three 81 and 76, sixteen 101 and 101; 376, 40 of
+  // 8576, three 76 and 76, sixteen 96 and 100; 512, 32 of 11008, sixteen 101 and 108; 896, 60 of 20384, three 377 and 408, sixteen
+  // 451 and 479.  (Passes of several contexts on streams of their own overlap, and the last two hide it: 512 wide and sixteen
+  // sequences 77.0 and 75.5.)
+  st->bt = d.H <= 320 ? 2 : 1;
   st->n_stages = (int)std::min<size_t>(kTcMaxStages, (budget - h_bytes) / (st->bt * kTcTileBytes));
   st->smem = (size_t)st->n_stages * st->bt * kTcTileBytes + h_bytes + 1024;
   if (!make_map(&a, w2, (uint64_t)d.H, rows, kTcKBlock, st->bt * kTcTileRows)) return false;

@@ -105,7 +105,7 @@ def test_hidden_values_at_the_end_of_the_range(B):
         p.close()
 
 
-@pytest.mark.parametrize("H", [64, 896, 960, 1024])   # 896 and 960: the widest with two tiles to a stage, 1024: one
+@pytest.mark.parametrize("H", [64, 264, 320, 328, 384, 896, 960, 1024])   # 320: the widest with two tiles to a stage
 @pytest.mark.parametrize("L,M", [
     (1, 128),       # a block with one tile: the pair's second is missing
     (37, 1024),     # 296 tiles: a pair for each of 148 SMs
