@@ -466,14 +466,15 @@ bool pred_tc_prepare(const Dims& d, const void* w1, const void* w2, void* hsplit
   const size_t h_bytes = (size_t)((d.H + kTcKBlock - 1) / kTcKBlock) * kTcN * kTcKBlock * 2;
   const size_t budget = 220 * 1024 - 1024;  // alignment slack
   if (h_bytes + 2 * kTcTileBytes > budget) return false;
-  // Two tiles to a stage for narrow hidden vectors: a tile is then a handful of K blocks, and what it costs is the hand-over of
-  // its stages and accumulator.  Wider ones reach the copy rate with one tile and lose with two, whose stages are half as many
-  // and twice as coarse.  A pass alone on its stream, one tile and two: 136 wide, 60 layers of 3072 rows, three sequences 42 and
-  // 38 us; 256, 60 of 5824, three 61 and 56, sixteen 76 and 74; 320, 60 of 7296, three 81 and 76, sixteen 101 and 101; 376, 40 of
-  // 8576, three 76 and 76, sixteen 96 and 100; 512, 32 of 11008, sixteen 101 and 108; 896, 60 of 20384, three 377 and 408, sixteen
-  // 451 and 479.  (Passes of several contexts on streams of their own overlap, and the last two hide it: 512 wide and sixteen
-  // sequences 77.0 and 75.5.)
-  st->bt = d.H <= 320 ? 2 : 1;
+  // Two tiles to a stage where the ring holds all K blocks of a pair at once (up to 320 columns): a row's bytes are then asked for
+  // together, and a copy instruction, which costs the SM's copy unit some 80 cycles whatever it brings, brings 32 KB.  Where a pair
+  // is longer than the ring, every row is come back to for its later K blocks, and the stream is slower than with one tile.  A
+  // pass alone on its stream, one tile and two: 136 wide, 60 layers of 3072 rows, three sequences 42 and 38 us; 256, 60 of 5824,
+  // three 61 and 56, sixteen 76 and 74; 320, 60 of 7296, three 81 and 76, sixteen 101 and 101; 376, 40 of 8576, three 76 and 76,
+  // sixteen 96 and 100; 512, 32 of 11008, sixteen 101 and 108; 896, 60 of 20384, three 377 and 408, sixteen 451 and 479.  (Passes
+  // of several contexts on streams of their own overlap, and that hides it: 512 wide and sixteen sequences 77.0 and 75.5.)
+  const size_t n_kb = (d.H + kTcKBlock - 1) / kTcKBlock;
+  st->bt = n_kb * kTcMaxBt * kTcTileBytes + h_bytes <= budget ? kTcMaxBt : 1;
   st->n_stages = (int)std::min<size_t>(kTcMaxStages, (budget - h_bytes) / (st->bt * kTcTileBytes));
   st->smem = (size_t)st->n_stages * st->bt * kTcTileBytes + h_bytes + 1024;
   if (!make_map(&a, w2, (uint64_t)d.H, rows, kTcKBlock, st->bt * kTcTileRows)) return false;
