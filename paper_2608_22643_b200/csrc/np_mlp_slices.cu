@@ -226,7 +226,7 @@ __device__ __forceinline__ void exchange_rows(const KArgs& a, const float* part,
   // across lanes, so every load that is not needed costs a request of its own at the L2 (all
   // blocks poll at about the same moment).
   float gsum[kQ], usum[kQ], ssv[kQ];  // indexed by unrolled constants only (registers)
-  bool done = !*ok;
+  bool done = __any_sync(0xffffffffu, !*ok);
 #pragma unroll 1
   for (uint32_t spin = 0; spin < npp::kSpinLimit && !done; ++spin) {
     unsigned long long wg[kQ], wu[kQ], ws[kQ];  // every load of the round is issued before any is looked at
@@ -246,7 +246,9 @@ __device__ __forceinline__ void exchange_rows(const KArgs& a, const float* part,
       usum[qq] = __uint_as_float((unsigned int)wu[qq]);
       ssv[qq] = __uint_as_float((unsigned int)ws[qq]);
     }
-    done = bad == 0;
+    // The lanes leave together: with an exit of its own for each the warp runs on in pieces (256 columns 59.6 us per 20 layers, 56.4
+    // with the vote; 7B shape 172.0 per 32 and 170.2).
+    done = __all_sync(0xffffffffu, bad == 0);
   }
   if (!done && *ok) {
     *ok = 0;
@@ -259,26 +261,24 @@ __device__ __forceinline__ void exchange_rows(const KArgs& a, const float* part,
     for (int qq = 0; qq < kQ; ++qq) ss += qq == q ? own_ss : ssv[qq];  // the same order in every block
     inv_rms = __shfl_sync(0xffffffffu, rsqrtf(ss / (float)a.D + kRmsEps), 0);  // lane 0 holds the peers' sums
   }
-  if (row < ((rows + 15) & ~15)) {
-    float av = 0.f;  // rows that pad the last 16-row block: zero
-    if (has_row) {
-      float gsv = 0.f, usv = 0.f;
+  // All lanes form an activation, those without a row a zero: the last 16-row block is padded with some of them, the others lie
+  // behind the last round's end.  (With branches around the lanes that have a row 256 columns take 55.7 us per 20 layers, 54.4
+  // without; 7B shape 171.0 per 32 and 170.1.)
+  float gsv = 0.f, usv = 0.f;
 #pragma unroll
-      for (int qq = 0; qq < kQ; ++qq) {
-        gsv += qq == q ? own_g : gsum[qq];
-        usv += qq == q ? own_u : usum[qq];
-      }
-      // the MLP's input is x_l scaled to unit RMS; the dot products are linear in it
-      gsv *= inv_rms;
-      usv *= inv_rms;
-      av = gsv / (1.f + __expf(-gsv)) * usv;
-    }
-    uint32_t tt[3];
-    split3(av, tt);
-    aterm[row] = (uint16_t)(tt[0] >> 16);
-    aterm[apad + row] = (uint16_t)(tt[1] >> 16);
-    aterm[2 * apad + row] = (uint16_t)(tt[2] >> 16);
+  for (int qq = 0; qq < kQ; ++qq) {
+    gsv += qq == q ? own_g : gsum[qq];
+    usv += qq == q ? own_u : usum[qq];
   }
+  // the MLP's input is x_l scaled to unit RMS; the dot products are linear in it
+  gsv *= inv_rms;
+  usv *= inv_rms;
+  const float av = has_row ? gsv / (1.f + __expf(-gsv)) * usv : 0.f;
+  uint32_t tt[3];
+  split3(av, tt);
+  aterm[row] = (uint16_t)(tt[0] >> 16);
+  aterm[apad + row] = (uint16_t)(tt[1] >> 16);
+  aterm[2 * apad + row] = (uint16_t)(tt[2] >> 16);
 }
 
 // KB: K blocks (16 columns) of a warp.  FULL: every warp of every slice has exactly KB.
