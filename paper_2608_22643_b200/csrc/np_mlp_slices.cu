@@ -124,8 +124,10 @@ struct KArgs {
   uint32_t slot_bytes;
 };
 
-// 32-bit words a consumer warp's B operand takes: [K block pair][term][lane of the quad][K block of the pair][half]
-__host__ __device__ constexpr int bstage_words(int KB) { return (KB + 1) / 2 * 48; }
+// 32-bit words a consumer warp's B operand takes: [K block pair][term][lane of the quad][K block of the pair][half].  A fourth, zero
+// "term" stands in the columns that have none: every lane loads its column, and no branch parts the warp between x and the
+// multiplications.  (7B shape 170.1 us per 32 layers with a branch around those lanes, 166.9 without; 13B 278.9 and 272.3.)
+__host__ __device__ constexpr int bstage_words(int KB) { return (KB + 1) / 2 * 64; }
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm(
@@ -477,6 +479,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 
   // counted sums: what the words of this lane's columns held when their set was last complete
   // (zprev: the set read next, zprev2: the other one; they trade places after every read)
+  for (int i = lane; i < bstage_words(KB); i += 32) bs[i] = 0u;  // the fourth term stays zero
+  __syncwarp();
   float2 xown[J];  // x_l of the columns this lane owns, for the whole run
   unsigned long long zprev[J][2], zprev2[J][2];
 #pragma unroll
@@ -623,7 +627,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
             split3(xown[j].x, p0);
             split3(xown[j].y, p1);
             // columns 2 c, 2 c + 1: K block c >> 3, half (c >> 2) & 1 of it, lane c & 3 of the quad
-            uint32_t* w = bs + (c >> 4) * 48 + (c & 3) * 4 + ((c >> 3) & 1) * 2 + ((c >> 2) & 1);
+            uint32_t* w = bs + (c >> 4) * 64 + (c & 3) * 4 + ((c >> 3) & 1) * 2 + ((c >> 2) & 1);
 #pragma unroll
             for (int e = 0; e < 3; ++e) w[e * 16] = pack_hi16(p0[e], p1[e]);
             if (r == 0 && l == l_last) *reinterpret_cast<float2*>(a.xbuf[l & 1] + col0 + 2 * c) = xown[j];  // x for the next launch
@@ -646,8 +650,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < (KB + 1) / 2; ++i) {
-          uint4 v = make_uint4(0u, 0u, 0u, 0u);
-          if (term < 3) v = *reinterpret_cast<const uint4*>(bs + i * 48 + term * 16 + t4 * 4);
+          const uint4 v = *reinterpret_cast<const uint4*>(bs + i * 64 + term * 16 + t4 * 4);
           xb[i][0] = v.x, xb[i][1] = v.y, xb[i][2] = v.z, xb[i][3] = v.w;
         }
       }
@@ -735,12 +738,11 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 #pragma unroll
         for (int u = 0; u < PD; ++u) {
           if (16 * u < n) {
-            uint32_t b0 = 0u, b1 = 0u;
-            if (term < 3) {
-              const uint16_t* ap = aterm + (size_t)term * apad + r0 + 16 * u + 2 * t4;
-              b0 = *reinterpret_cast<const uint32_t*>(ap);
-              b1 = *reinterpret_cast<const uint32_t*>(ap + 8);
-            }
+            // (loaded by all lanes here, too: 7B shape 166.9 and 164.1, 70B 958 and 940; with a fourth term in shared memory instead
+            // of the selection 167.5 and 939)
+            const uint16_t* ap = aterm + (size_t)(term < 3 ? term : 0) * apad + r0 + 16 * u + 2 * t4;
+            uint32_t b0 = *reinterpret_cast<const uint32_t*>(ap), b1 = *reinterpret_cast<const uint32_t*>(ap + 8);
+            if (term == 3) b0 = b1 = 0u;
 #pragma unroll
             for (int j = 0; j < KH; ++j)
               if (FULL || j0 + j < nkb) mma_bf16_16816(acc[j0 + j], df[u][j], b0, b1);
