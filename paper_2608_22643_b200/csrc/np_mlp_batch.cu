@@ -137,6 +137,10 @@ __device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, vol
     atomicOr(status, npp::kStatTimeout);
   }
 }
+__device__ __forceinline__ void all_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
+  npp::wait_or_flag(bar, parity, ok, status);
+  __syncwarp();
+}
 __device__ __forceinline__ void warp_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status, int lane) {
   if (lane == 0) wait_or_flag(bar, parity, ok, status);
   __syncwarp();
@@ -269,11 +273,8 @@ __device__ __forceinline__ void exchange_chunk(const KArgs& a, const float4* par
 #pragma unroll
   for (int i = 0; i < NPAIR; ++i) {
     const int row = row0 + i * row_step;
-    float h = 0.f;  // rows and sequences that pad a tile: zero
-    if (live && row < rows) {
-      const float gs = g[i] * inv, us = u[i] * inv;
-      h = gs / (1.f + __expf(-gs)) * us;
-    }
+    const float gs = g[i] * inv, us = u[i] * inv;
+    const float h = live && row < rows ? gs / (1.f + __expf(-gs)) * us : 0.f;  // rows and sequences that pad a tile: zero
     uint32_t tr[3];
     split3(h, tr);
     // A fragment of m16n8k16: element (m, k) is half k & 1 of register (m >> 3) + 2 (k >> 3) of lane 4 (m & 7) + (k & 7) / 2
@@ -338,10 +339,8 @@ __device__ __forceinline__ void down_reds(const float (&acc)[2 * PN][4], float* 
         const float ra = __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[2], 1), rb = __shfl_xor_sync(0xffffffffu, odd ? v[1] : v[3], 1);
         const int seq = odd ? 8 + g8 : g8;
         float* dst = tile + (size_t)j * NS * 8 + seq * 8 + (t4 >> 1) * 4;
-        if (seq < B) {
-          if (odd) red_add_v4(dst, ra, rb, v[2], v[3]);
-          else red_add_v4(dst, v[0], v[1], ra, rb);
-        }
+        const float o0 = odd ? ra : v[0], o1 = odd ? rb : v[1], o2 = odd ? v[2] : ra, o3 = odd ? v[3] : rb;
+        if (seq < B) red_add_v4(dst, o0, o1, o2, o3);
       }
     } else {
       // rows g8 and g8 + 8 belong to one sequence; even lanes take the pair's first tile, odd lanes its second
@@ -349,10 +348,8 @@ __device__ __forceinline__ void down_reds(const float (&acc)[2 * PN][4], float* 
       const float b0 = acc[2 * p + 1][0] + acc[2 * p + 1][2], b1 = acc[2 * p + 1][1] + acc[2 * p + 1][3];
       const float ra = __shfl_xor_sync(0xffffffffu, odd ? a0 : b0, 1), rb = __shfl_xor_sync(0xffffffffu, odd ? a1 : b1, 1);
       float* dst = tile + (size_t)(odd ? 1 : 0) * NS * 8 + g8 * 8 + (t4 >> 1) * 4;
-      if (g8 < B) {
-        if (odd) red_add_v4(dst, ra, rb, b0, b1);
-        else red_add_v4(dst, a0, a1, ra, rb);
-      }
+      const float o0 = odd ? ra : a0, o1 = odd ? rb : a1, o2 = odd ? b0 : ra, o3 = odd ? b1 : rb;
+      if (g8 < B) red_add_v4(dst, o0, o1, o2, o3);
     }
   }
 }
@@ -497,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           const unsigned int n = nx + (unsigned int)c;
           if (n % kExchGroups != (unsigned int)e) continue;
           const unsigned int buf = n & 1u, use = n >> 1, turn = n / kExchGroups;
-          warp_wait(&part_full[buf], use & 1u, ok, a.status, lane);
+          all_wait(&part_full[buf], use & 1u, ok, a.status);
           const unsigned int area = (unsigned int)e * 2u + (turn & 1u), stamp = a.seq_base + 1u + n;
           const float4* pt = part + (size_t)buf * kPart;
           uint16_t* hc = hs + (size_t)c * HT * 256;
@@ -538,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     // ---- x_l: this warp's K blocks wid, wid + 8, ..., straight into B fragments ----
     uint32_t xb[NP][NSG][3][2];
     {
-      warp_wait(&x_ready, (uint32_t)li & 1u, ok, a.status, lane);
+      all_wait(&x_ready, (uint32_t)li & 1u, ok, a.status);
       float2 lo[NP][NSG], hi[NP][NSG];
       const float* xp = xs + (size_t)g8 * 8 + 2 * t4;
 #pragma unroll
@@ -636,18 +633,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     auto chunk_wait = [&](int c, int sl, uint32_t pr) {
       const unsigned int n = nx + (unsigned int)c;
       if (!__all_sync(0xffffffffu, acts_there(n))) {
-        if (lane == 0) {
-          bool there = false;
-          for (uint32_t spin = 0; spin < npp::kSpinLimit * 16u && !there && *ok; ++spin) there = acts_there(n);
-          if (!there && *ok) {
-            *ok = 0;
-            atomicOr(a.status, npp::kStatTimeout);
-          }
+        bool there = false;
+#pragma unroll 1
+        for (uint32_t spin = 0; spin < npp::kSpinLimit * 16u && !there && *ok; ++spin) there = __all_sync(0xffffffffu, acts_there(n));
+        if (!there && *ok) {
+          *ok = 0;
+          atomicOr(a.status, npp::kStatTimeout);
         }
         __syncwarp();
       }
       __threadfence_block();
-      if (!__all_sync(0xffffffffu, mbar_test(&full_bar[sl], pr))) warp_wait(&full_bar[sl], pr, ok, a.status, lane);
+      if (!__all_sync(0xffffffffu, mbar_test(&full_bar[sl], pr))) all_wait(&full_bar[sl], pr, ok, a.status);
     };
     {
       float acc[2 * NP][4];
@@ -661,7 +657,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
         next_slot();
       }
       // x += y in place, once every block of the slice has read x_l
-      warp_wait(&may_add, (uint32_t)li & 1u, ok, a.status, lane);
+      all_wait(&may_add, (uint32_t)li & 1u, ok, a.status);
       if (nrows > 0) down_reds<NSG, NP>(acc, xs, wid, nk, a.B, lane);
     }
     nx += (unsigned int)nch;
