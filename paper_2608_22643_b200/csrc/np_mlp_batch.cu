@@ -449,10 +449,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           const int step = pass == 0 ? 8 : 16;
           for (int r0 = 0; r0 < nrows; r0 += step) {
             const int n = min(step, nrows - r0);
-            if (lane == 0) {
-              wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status);
-              npp::mbar_expect_tx(&full_bar[slot], (uint32_t)(pass == 0 ? 2 * n : n) * piece_bytes);
-            }
+            // (After a time-out the slot may be taken from its readers, not from the copies under way.)
+            if (!npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status)) npp::wait_landed(&full_bar[slot], par ^ 1u, patience);
+            if (lane == 0) npp::mbar_expect_tx(&full_bar[slot], (uint32_t)(pass == 0 ? 2 * n : n) * piece_bytes);
             __syncwarp();
             const int i = pass == 0 ? (lane & 7) : lane;
             if (lane < 16 && i < n) {
@@ -469,10 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           }
         }
       }
-      // Nobody leaves before the copies have landed.  (After a time-out the producer has not waited for free slots, and a slot's
-      // barrier may have lost count of two uses that overlapped: then a time that is far longer than any copy's.)
-      if (lane == 0) npp::drain_ring(full_bar, a.ng, slot, par, patience);
-      if (!*ok) __nanosleep(500000);
+      if (lane == 0) npp::drain_ring(full_bar, a.ng, slot, par, patience);  // nobody leaves before the copies have landed
     } else if (wid == kSync) {
       // ---- synchroniser: the two counters of the slice ----
       if (lane == 0) {
