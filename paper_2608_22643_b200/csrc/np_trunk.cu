@@ -22,12 +22,16 @@ namespace npi {
 using namespace npd;
 namespace trunk {
 
-constexpr int kWarps = 16;
+// Two blocks to an SM: the next kernel's first blocks load their weights where this one's have left.  With the LayerNorm read into
+// registers once (it was read from the L2 three times) a pass at the paper's sizes takes 99.9 us back to back (32 sparse layers;
+// blocks of sixteen warps 101.6) and 113.7 cold (115.7); one block of eight warps to an SM takes 122.
+constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
 // a warp works on kRows rows side by side with kPieces 16-byte pieces of each in flight per lane:
 // (2, 8) where there are rows enough for every warp of the device, (1, 16) for the short matrices
 // of the trunk, so that they spread over all SMs and a row of 8 KB is one round of loads
 constexpr int kMaxSegs = 8;
+constexpr int kMaxLn = 4096;      // values of a normalised input, at most (4 T)
 constexpr float kLnEps = 1e-5f;   // the LayerNorm epsilon (the paper does not state one)
 
 struct Seg {
@@ -70,9 +74,14 @@ __device__ __forceinline__ float dot8(const uint4& w, const float4& x0, const fl
   return acc;
 }
 
+__device__ __forceinline__ void cp_async4(float* dst_smem, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(npp::smem_addr(dst_smem)), "l"(src) : "memory");
+}
+
 template <int kRows, int kPieces>
-__global__ void __launch_bounds__(kThreads, 1) k_gemv(GemvArgs a) {
-  extern __shared__ __align__(16) float xs[];  // the input: even 4-float granules first, then the odd ones
+__global__ void __launch_bounds__(kThreads, 2) k_gemv(GemvArgs a) {
+  // the input: even 4-float granules first, then the odd ones; behind it gain and bias of a LayerNorm
+  extern __shared__ __align__(16) float xs[];
   __shared__ float red[kWarps];
   const Seg& s = a.seg[blockIdx.y];
   const int in_dim = s.in_dim, chunks = in_dim >> 3, rows = s.rows;
@@ -92,32 +101,53 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemv(GemvArgs a) {
     }
   };
   if (r0 < rows) load(r0, lane);  // the weights do not depend on the previous kernel; the input does
+  const bool ln = s.ln_gain != nullptr;
+  float* const gain = xs + in_dim;
+  if (ln) {
+    for (int i = tid; i < in_dim; i += kThreads) {
+      cp_async4(gain + i, s.ln_gain + i);
+      cp_async4(gain + in_dim + i, s.ln_bias + i);
+    }
+  }
   npp::pdl_wait_prior();
 
   // ---- the input vector, normalised and activated if asked for ----
-  float mean = 0.f, rstd = 1.f;
-  const bool ln = s.ln_gain != nullptr;
   const uint16_t* xr = s.x ? nullptr : s.x_rows + (size_t)(*s.x_row) * in_dim;
   auto xin = [&](int i) { return s.x ? __ldcg(s.x + i) : __uint_as_float((uint32_t)xr[i] << 16); };
-  if (ln) {
-    float t = 0.f;
-    for (int i = tid; i < in_dim; i += kThreads) t += xin(i);
-    mean = block_sum(t, red) / (float)in_dim;
-    t = 0.f;
-    for (int i = tid; i < in_dim; i += kThreads) {
-      const float dv = xin(i) - mean;
-      t += dv * dv;
-    }
-    rstd = rsqrtf(block_sum(t, red) / (float)in_dim + kLnEps);
-  }
-  for (int i = tid; i < in_dim; i += kThreads) {
-    float v = xin(i);
-    if (ln) {
-      v = (v - mean) * rstd * s.ln_gain[i] + s.ln_bias[i];
-      v = v / (1.f + __expf(-v));
-    }
+  auto put = [&](int i, float v) {
     const int g = i >> 2;  // granule
     xs[((g & 1) * chunks + (g >> 1)) * 4 + (i & 3)] = v;
+  };
+  if (ln) {  // read once, into registers (a normalised input has kMaxLn values at most)
+    float x[kMaxLn / kThreads], t = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMaxLn / kThreads; ++k) {
+      const int i = tid + k * kThreads;
+      x[k] = i < in_dim ? xin(i) : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < kMaxLn / kThreads; ++k) t += x[k];
+    const float mean = block_sum(t, red) / (float)in_dim;
+    t = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMaxLn / kThreads; ++k)
+      if (tid + k * kThreads < in_dim) {
+        x[k] -= mean;
+        t += x[k] * x[k];
+      }
+    const float rstd = rsqrtf(block_sum(t, red) / (float)in_dim + kLnEps);
+    asm volatile("cp.async.wait_all;" ::: "memory");  // a thread reads what it has copied itself
+#pragma unroll
+    for (int k = 0; k < kMaxLn / kThreads; ++k) {
+      const int i = tid + k * kThreads;
+      if (i < in_dim) {
+        const float v = x[k] * rstd * gain[i] + gain[in_dim + i];
+        put(i, v / (1.f + __expf(-v)));
+      }
+    }
+  } else {
+#pragma unroll 8
+    for (int i = tid; i < in_dim; i += kThreads) put(i, xin(i));
   }
   __syncthreads();
 
@@ -206,15 +236,16 @@ static cudaError_t launch_pdl(K kfn, dim3 grid, size_t smem, cudaStream_t s, con
 }
 
 static cudaError_t gemv(const GemvArgs& a, int n_seg, cudaStream_t s, int sm_count) {
-  int max_in = 8, max_rows = 1;
+  int max_in = 8, max_rows = 1, floats = 8;
   for (int i = 0; i < n_seg; ++i) {
     max_in = std::max(max_in, a.seg[i].in_dim);
+    floats = std::max(floats, a.seg[i].in_dim * (a.seg[i].ln_gain ? 3 : 1));
     max_rows = std::max(max_rows, a.seg[i].rows);
   }
-  const size_t smem = (size_t)max_in * 4;
+  const size_t smem = (size_t)floats * 4;
   // two rows per warp where every warp of the device gets two, and where a row is so short that
   // one row's pieces would leave half of a lane's loads unused
-  const bool wide = max_rows >= 2 * kWarps * sm_count || max_in <= 2048;
+  const bool wide = max_rows >= 4 * kWarps * sm_count || max_in <= 2048;
   auto kfn = wide ? k_gemv<2, 8> : k_gemv<1, 16>;
   if (smem > 48 * 1024) {
     static std::atomic<uint64_t> done[2] = {{0}, {0}};
@@ -223,7 +254,7 @@ static cudaError_t gemv(const GemvArgs& a, int n_seg, cudaStream_t s, int sm_cou
   }
   const int per_block = kWarps * (wide ? 2 : 1);
   const int want = (max_rows + per_block - 1) / per_block;
-  return launch_pdl(kfn, dim3(std::max(1, std::min(want, sm_count)), n_seg), smem, s, a);
+  return launch_pdl(kfn, dim3(std::max(1, std::min(want, 2 * sm_count)), n_seg), smem, s, a);
 }
 
 }  // namespace trunk
