@@ -22,8 +22,8 @@
 //          the same columns.  Nothing but the partial dot products crosses between the warps: no
 //          block-wide barrier, and x is never read from another warp's part of shared memory.  (With
 //          the rows dealt to the warps instead, eight of them, x went through shared memory and a
-//          barrier to all, and every warp read half of it back: 7.3 us per layer at the 7B shape, 5.4 now;
-//          13B 8.1 and 7.0, 70B 15.1 and 12.1, 256 columns and 60 rows 4.7 and 2.9.)
+//          barrier to all, and every warp read half of it back: 7.3 us per layer at the 7B shape, 5.1 now;
+//          13B 8.1 and 6.6, 70B 15.1 and 11.4, 256 columns and 60 rows 4.7 and 2.7.)
 // rows     What a phase multiplies is in registers as A fragments before its operand arrives: gate
 //          and up tiles are loaded while the sums of the layer before are on their way, down tiles
 //          during the exchange.  A tile's ring slot is free as soon as it is loaded, so the registers
@@ -49,6 +49,9 @@
 // 0-2.  Phase 2: A = 16 output columns x 16 down rows (ldmatrix.trans of the row-major pieces), B =
 // the activations as three bf16 terms.  In both, columns 4-6 of B repeat columns 0-2, so that the
 // upper two lanes of a quad hold a second tile's sums without a shuffle.
+//
+// On the way from the sums to the next layer's sums nothing parts a warp: a branch around some lanes, or a loop that lanes leave one by
+// one, costs it hundreds of cycles per layer (each such place says what).
 //
 // Shared memory is one ring of load groups in the order they are consumed: the gate|up pieces of a
 // layer's rows, then its down pieces, then the next layer's.  A producer warp fills it with 1-D bulk
@@ -96,6 +99,11 @@ __host__ __device__ constexpr int tiles_down(int KB) { return KB <= 4 ? 4 : KB <
 // layers with one wait for all four, 78 with two), a late return leaves the ring full (7B shape 185 us with one wait, 173 with
 // two; 3000 rows of 4096 columns 177 and 160 us per 12 layers).
 __host__ __device__ constexpr int tiles_wait(int KB) { return KB <= 4 ? 4 : tiles_up(KB) > 2 ? 2 : tiles_up(KB); }
+// Whether the producer's wait for a free slot is lane 0's or the whole warp's.  What lies between a free slot and its copies sets the
+// stream's pace, so the rows' addresses are formed before the wait; which wait is shorter then differs by instance (us per stack, all
+// lanes / lane 0 / before, lane 0 with the addresses behind the wait: 256 columns 54.1 / 54.6 / 54.9, 7B shape 162.3 / 172.7 / 164.0,
+// 13B 267.1 / 264.6 / 266.6, 6144 149.6 / 156.3 / 155.0, 70B 1006 / 909 / 945).
+__host__ __device__ constexpr bool lane0_waits(int KB) { return KB == 10 || KB == 16; }
 // tiles of a round of the exchange: whole groups of tiles_up
 __host__ __device__ constexpr int tiles_chunk(int KB) { return kChunkVec / 16 / tiles_up(KB) * tiles_up(KB); }
 
@@ -347,9 +355,8 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 
   if (wid == kWarps) {
     // =========================== producer warp ===========================
-    // The groups are requested in the order they are consumed.  The waits are lane 0's (several
-    // lanes waiting on different barriers must not be used: the compiler may reconverge the warp
-    // after a wait); a slot's copies are then issued by as many lanes as it has pieces.  The slots of a layer's rows
+    // The groups are requested in the order they are consumed.  (Lanes that wait on different barriers must not be used: the compiler
+    // may reconverge the warp after a wait.)  A slot's copies are issued by as many lanes as it has pieces.  The slots of a layer's rows
     // are fetched a layer ahead.
     int slot = 0;
     uint32_t par = 0, patience = npp::kSpinLimit;
@@ -379,21 +386,21 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
 #pragma unroll 1
         for (int r0 = 0; r0 < nrows; r0 += step) {
           const int npieces = min(step, nrows - r0) << (pass == 0 ? 1 : 0);
-          if (lane == 0) {
-            // (after a time-out the slot may be taken from its readers, not from the copies under way)
-            if (!npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status)) npp::wait_landed(&full_bar[slot], par ^ 1u, patience);
-            npp::mbar_expect_tx(&full_bar[slot], (uint32_t)npieces * piece_bytes);
-          }
-          __syncwarp();  // the expect_tx precedes the copies
+          const unsigned char* src = nullptr;
           if (lane < npieces) {
-            int s = rows[r0 + (pass == 0 ? lane >> 1 : lane)];
-            if (a.check && (s < 0 || s >= a.C)) {
+            int sl = rows[r0 + (pass == 0 ? lane >> 1 : lane)];
+            if (a.check && (sl < 0 || sl >= a.C)) {
               atomicOr(a.status, kStatBadSlot);
-              s = 0;
+              sl = 0;
             }
-            const unsigned char* src = (pass == 0 ? ((lane & 1) ? a.up : a.gate) : a.downT) + lbase + (size_t)s * row_bytes;
-            npp::bulk_g2s_stream(csm + (size_t)slot * a.slot_bytes + (size_t)lane * pstride, src, piece_bytes, &full_bar[slot], l2_policy);
+            src = (pass == 0 ? ((lane & 1) ? a.up : a.gate) : a.downT) + lbase + (size_t)sl * row_bytes;
           }
+          // (after a time-out the slot may be taken from its readers, not from the copies under way)
+          if (!lane0_waits(KB) || lane == 0)
+            if (!npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status)) npp::wait_landed(&full_bar[slot], par ^ 1u, patience);
+          if (lane == 0) npp::mbar_expect_tx(&full_bar[slot], (uint32_t)npieces * piece_bytes);
+          __syncwarp();  // the expect_tx precedes the copies
+          if (src) npp::bulk_g2s_stream(csm + (size_t)slot * a.slot_bytes + (size_t)lane * pstride, src, piece_bytes, &full_bar[slot], l2_policy);
           __syncwarp();
           if (++slot == ng) {
             slot = 0;
