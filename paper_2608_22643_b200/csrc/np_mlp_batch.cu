@@ -137,6 +137,10 @@ __device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, vol
     atomicOr(status, npp::kStatTimeout);
   }
 }
+// A warp's wait, by all lanes or by lane 0.  The latter parts the warp and brings it together again, some 300 cycles where the phase
+// is long complete, so what lies on the way of x is waited for by all lanes (sixteen sequences of 1024 columns 83 us per 12 layers,
+// 90 with lane 0's waits; two of the 7B shape 319 per 32 and 337).  The waits inside the up phase's loop are lane 0's: by all lanes
+// they cost the widest rows more than they give the others (13B shape, eight sequences, 581 us per 40 layers against 560).
 __device__ __forceinline__ void all_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
   npp::wait_or_flag(bar, parity, ok, status);
   __syncwarp();
@@ -629,10 +633,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     auto chunk_wait = [&](int c, int sl, uint32_t pr) {
       const unsigned int n = nx + (unsigned int)c;
       if (!__all_sync(0xffffffffu, acts_there(n))) {
-        bool there = false;
+        bool done = false;  // the same in all lanes
 #pragma unroll 1
-        for (uint32_t spin = 0; spin < npp::kSpinLimit * 16u && !there && *ok; ++spin) there = __all_sync(0xffffffffu, acts_there(n));
-        if (!there && *ok) {
+        for (uint32_t spin = 0; spin < npp::kSpinLimit * 16u && !done; ++spin) done = __all_sync(0xffffffffu, acts_there(n) || !*ok);
+        if (!done) {
           *ok = 0;
           atomicOr(a.status, npp::kStatTimeout);
         }
