@@ -121,6 +121,16 @@ def test_topk_paths_of_the_selection_kernel():
         p.close()
 
 
+@pytest.mark.parametrize("L,M,B", [(2, 32, 1), (2, 1056, 2), (2, 1504, 1), (80, 1568, 2), (1, 32800, 1), (1, 40960, 2)])
+def test_topk_words_of_every_round(L, M, B):
+    """A lane holds the word of a round (of two, from 33 rounds on): one round, a last round of few warps, both block widths."""
+    p = Pair(TINY.with_(n_layers=L, d_ffn=M), max_batch=B, k=M // 3, C=M, with_oracle=False)
+    try:
+        _topk_case(p, np.random.default_rng(M).standard_normal((B, L, M)).astype(np.float32))
+    finally:
+        p.close()
+
+
 @pytest.mark.parametrize("policy", [nb.NP_EVICT_EXACT, nb.NP_EVICT_LRU])
 @pytest.mark.parametrize("cfg,n_set,C,persist", [
     (TINY, 102, 205, 0.8), (TINY, 102, 102, 0.6), (SMALL, 208, 520, 0.83), (SMALL, 700, 520, 0.7),
