@@ -34,7 +34,8 @@
 // have read x_l, and may read x_{l+1} once all R have added.  Two counters per slice say so (they only grow; the host
 // tracks their value); a warp of its own waits on them.
 //
-// Every wait is bounded (np_pipe.cuh); once one has run out the block records kStatTimeout and skips all later waits.
+// Every wait is bounded (np_pipe.cuh); once one has run out the block records kStatTimeout and skips all later waits except
+// those for its ring (np_ring.h).
 #include <algorithm>
 
 #include "np_device.cuh"
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
   __shared__ __align__(8) uint64_t part_full[2], part_empty[2];
   __shared__ __align__(8) uint64_t x_ready, x_read, may_add;
   __shared__ float ssq_part[kWarps * 16];
-  __shared__ int s_ok;
+  __shared__ int s_ok[2];  // no wait has run out; the ring was given up
   __shared__ unsigned int s_act[kExchGroups * kExchWarps];  // chunks each exchange warp has finished, ever growing
   __shared__ int lay_rb[kMaxLayers], lay_n[kMaxLayers], lay_pre[kMaxLayers + 1];
 
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
   float4* part = reinterpret_cast<float4*>(csm + (size_t)a.ng * a.slot_bytes);           // [2][2 tiles][NSG][8 warps][32]
   uint16_t* hs = reinterpret_cast<uint16_t*>(part + 2 * kPart);                // [max_chunks][HT][32][4] words
   uint16_t* slot_cache = hs + (size_t)max_chunks * HT * 256;
-  volatile int* ok = &s_ok;
+  volatile int* ok = s_ok;
   unsigned int* cnt_read = a.cnt + (size_t)q * kCntStride;
   unsigned int* cnt_add = a.cnt + (size_t)(kMaxQ + q) * kCntStride;
 
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     npp::mbar_init(&x_read, kWarps);
     npp::mbar_init(&may_add, 1);
     npp::fence_barrier_init();
-    s_ok = 1;
+    s_ok[0] = 1, s_ok[1] = 0;
     for (int i = 0; i < kExchGroups * kExchWarps; ++i) s_act[i] = 0;
   }
   // The tiles are read whole: rows that no copy fills meet zero activations, so what they hold must be finite.
@@ -443,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     if (wid == kProducer) {
       // ---- producer: gate|up tiles of a layer (8 records), its down tiles (16), the next layer's, in the order of use ----
       int slot = 0;
-      uint32_t par = 0, patience = npp::kSpinLimit;
+      uint32_t par = 0;
       const uint64_t pol = npp::policy_evict_first();  // a row is read once per token
       const size_t qoff = (size_t)k0 * 32;
       for (int li = 0; li < nl; ++li) {
@@ -453,8 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           const int step = pass == 0 ? 8 : 16;
           for (int r0 = 0; r0 < nrows; r0 += step) {
             const int n = min(step, nrows - r0);
-            // (After a time-out the slot may be taken from its readers, not from the copies under way.)
-            if (!npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status)) npp::wait_landed(&full_bar[slot], par ^ 1u, patience);
+            npp::ring_wait(&empty_bar[slot], par ^ 1u, ok, a.status);
             if (lane == 0) npp::mbar_expect_tx(&full_bar[slot], (uint32_t)(pass == 0 ? 2 * n : n) * piece_bytes);
             __syncwarp();
             const int i = pass == 0 ? (lane & 7) : lane;
@@ -472,6 +472,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
           }
         }
       }
+      uint32_t patience = npp::kSpinLimit;
       if (lane == 0) npp::drain_ring(full_bar, a.ng, slot, par, patience);  // nobody leaves before the copies have landed
     } else if (wid == kSync) {
       // ---- synchroniser: the two counters of the slice ----
@@ -580,7 +581,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
     uint32_t rdy = mbar_test(&full_bar[slot], par);
     for (int t = 0; t < n_up; ++t) {
       const unsigned int n = nx + (unsigned int)(t >> 1), buf = n & 1u;
-      if (!__all_sync(0xffffffffu, rdy)) warp_wait(&full_bar[slot], par, ok, a.status, lane);
+      if (!__all_sync(0xffffffffu, rdy)) {
+        if (lane == 0) npp::ring_wait(&full_bar[slot], par, ok, a.status);
+        __syncwarp();
+      }
       const uint32_t ap = ring + (uint32_t)slot * a.slot_bytes + up_off;
       uint64_t* const done_bar = &empty_bar[slot];
       next_slot();
@@ -643,7 +647,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
         __syncwarp();
       }
       __threadfence_block();
-      if (!__all_sync(0xffffffffu, mbar_test(&full_bar[sl], pr))) all_wait(&full_bar[sl], pr, ok, a.status);
+      if (!__all_sync(0xffffffffu, mbar_test(&full_bar[sl], pr))) {
+        npp::ring_wait(&full_bar[sl], pr, ok, a.status);
+        __syncwarp();
+      }
     };
     {
       float acc[2 * NP][4];

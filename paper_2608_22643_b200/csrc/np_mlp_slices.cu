@@ -60,8 +60,9 @@
 // exchange warp adds the warps' partial dot products, trades them and leaves the activations.
 //
 // Every wait (mbarrier, exchange words, counted sums) is bounded; once one has run out the block
-// records kStatTimeout and skips all later waits, so the kernel drains; the blocks that depend on it
-// follow at their next wait.  The producer stays until its copies have landed.
+// records kStatTimeout and skips all later waits except those for its ring (np_ring.h), so the kernel
+// drains; the blocks that depend on it follow at their next wait.  The producer stays until its copies
+// have landed.
 #include <algorithm>
 
 #include "np_device.cuh"
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
   __shared__ __align__(8) uint64_t ss_bar;                // ... and its sum of x_l^2
   __shared__ __align__(8) uint64_t act_bar;               // the exchange warp has left the round's activations
   __shared__ float ssq_part[kWarps];                      // per-warp sums of x_l^2
-  __shared__ int s_ok;
+  __shared__ int s_ok[2];                                 // no wait has run out; the ring was given up
   __shared__ int lay_rb[kMaxLayers];  // first active-list index of this block's row group, per layer
   __shared__ int lay_n[kMaxLayers];   // rows of this row group
 
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
   float* part = reinterpret_cast<float*>(bstage + (size_t)a.nw * bstage_words(KB));        // [part_bufs][nw][kChunkVec]
   uint16_t* aterm = reinterpret_cast<uint16_t*>(part + (size_t)a.part_bufs * a.nw * kChunkVec);  // [3][apad] bf16 terms of a_i
   int32_t* slot_buf = reinterpret_cast<int32_t*>(aterm + 3 * apad);                        // [2][max_rows]
-  volatile int* ok = &s_ok;
+  volatile int* ok = s_ok;
 
   // ---- this row group's share of every layer of the run ----
   if (tid < nl) {
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     npp::mbar_init(&ss_bar, (uint32_t)a.nw);
     npp::mbar_init(&act_bar, kExchWarps);
     npp::fence_barrier_init();
-    s_ok = 1;
+    s_ok[0] = 1, s_ok[1] = 0;
   }
   __syncthreads();
   if (wid >= kWarps) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     // may reconverge the warp after a wait.)  A slot's copies are issued by as many lanes as it has pieces.  The slots of a layer's rows
     // are fetched a layer ahead.
     int slot = 0;
-    uint32_t par = 0, patience = npp::kSpinLimit;
+    uint32_t par = 0;
     // A row is read once per token: the copies mark their lines evict-first, so that the 27 MB a layer streams
     // through the L2 do not push out the few hundred KB every layer meets in (exchange words, counted sums).
     const uint64_t l2_policy = npp::policy_evict_first();
@@ -395,9 +396,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
             }
             src = (pass == 0 ? ((lane & 1) ? a.up : a.gate) : a.downT) + lbase + (size_t)sl * row_bytes;
           }
-          // (after a time-out the slot may be taken from its readers, not from the copies under way)
-          if (!lane0_waits(KB) || lane == 0)
-            if (!npp::wait_or_flag(&empty_bar[slot], par ^ 1u, ok, a.status)) npp::wait_landed(&full_bar[slot], par ^ 1u, patience);
+          if (!lane0_waits(KB) || lane == 0) npp::ring_wait(&empty_bar[slot], par ^ 1u, ok, a.status);
           if (lane == 0) npp::mbar_expect_tx(&full_bar[slot], (uint32_t)npieces * piece_bytes);
           __syncwarp();  // the expect_tx precedes the copies
           if (src) npp::bulk_g2s_stream(csm + (size_t)slot * a.slot_bytes + (size_t)lane * pstride, src, piece_bytes, &full_bar[slot], l2_policy);
@@ -409,6 +408,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
         }
       }
     }
+    uint32_t patience = npp::kSpinLimit;
     if (lane == 0) npp::drain_ring(full_bar, ng, slot, par, patience);
     return;
   }
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_slices(const __grid_constant_
     uint32_t p = par;
 #pragma unroll 1
     for (; n > 0; n -= kSlotPieces) {
-      npp::wait_or_flag(&full_bar[s], p, ok, a.status);
+      npp::ring_wait(&full_bar[s], p, ok, a.status);
       if (++s == ng) s = 0, p ^= 1u;
     }
   };

@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "np_ring.h"
+
 namespace npp {
 
 constexpr int kStatTimeout = 8;           // a bounded wait ran out
@@ -64,7 +66,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // A bounded wait on an mbarrier for blocks that drain after a time-out: once any wait of the block has run out (*ok == 0)
-// every later one is skipped.  True: the phase is complete.  One loop around one try_wait, not unrolled: with the unrolled
+// every later one of these is skipped.  True: the phase is complete.  One loop around one try_wait, not unrolled: with the unrolled
 // loops of mbar_wait at every wait k_mlp_slices had 90 to 150 KB of code, missed the instruction cache on every layer (195
 // times at 256 columns) and spent a sixth of its issue slots waiting for instructions.
 __device__ __forceinline__ bool wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
@@ -78,6 +80,28 @@ __device__ __forceinline__ bool wait_or_flag(uint64_t* bar, uint32_t parity, vol
     }
   }
   return true;
+}
+
+// A wait on a ring's own barriers, which the flag does not end (np_ring.h).  `ok` points to the flag and, behind it, to whether the
+// ring was given up.
+struct RingBlock {
+  volatile int* ok;
+  int32_t* status;
+  __device__ __forceinline__ bool stands() { return ok[0] != 0; }
+  __device__ __forceinline__ void lower() {
+    ok[0] = 0;
+    atomicOr(status, kStatTimeout);
+  }
+  __device__ __forceinline__ void pause() { __nanosleep(4000); }
+  __device__ __forceinline__ bool given_up() { return ok[1] != 0; }
+  __device__ __forceinline__ void give_up() { ok[1] = 1; }
+};
+__device__ __forceinline__ void ring_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
+  RingBlock b = {ok, status};
+  uint32_t polls = 0;
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity))
+    if (ring_wait_step<kSpinLimit>(polls, b)) return;
 }
 
 // A block may leave only when the copies it has asked for have landed: after a time-out nobody else waits for them, and they

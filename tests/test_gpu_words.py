@@ -115,3 +115,17 @@ def test_error_of_the_sums(lib, D, k, most):
         assert status == 0
         errors.append(w.error(got))
     assert sum(errors) / 4 < most
+
+
+@pytest.mark.parametrize("B,D,rows", [(1, 4096, 37 * 64), (1, 8192, 37 * 64), (3, 4096, 37 * 80), (16, 2048, 37 * 80)])
+def test_a_wait_that_runs_out_laps_before_the_end(lib, B, D, rows):
+    """The same with several laps of a block's ring left when the wait runs out: none of its slots is filled any more."""
+    w = Words(lib, D, 3072, rows, 4, B)
+    want, status = w.run()
+    assert status == 0 and w.error(want) < 1e-5
+    w.base[0] += 1
+    _, status = w.run()
+    assert status == TIMEOUT
+    w.clear()
+    got, status = w.run()
+    assert status == 0 and w.error(got) < 1e-5
