@@ -84,6 +84,9 @@ inline cudaError_t allow_shared(const void* fn, std::atomic<uint64_t>* done) {
   return e;
 }
 
+// Dynamic shared memory that needs no allow_shared: 48 KB hold a kernel's static variables, too (of the kernels that ask, 2 KB at most).
+constexpr size_t kPlainShared = 46 * 1024;
+
 // ---- kernel launchers (each in its own .cu) -------------------------------
 cudaError_t launch_tables_reset(const Dims& d, const Tables& t, cudaStream_t s);
 

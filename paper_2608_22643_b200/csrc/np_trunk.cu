@@ -238,6 +238,7 @@ static cudaError_t launch_pdl(K kfn, dim3 grid, size_t smem, cudaStream_t s, con
 static cudaError_t gemv(const GemvArgs& a, int n_seg, cudaStream_t s, int sm_count) {
   int max_in = 8, max_rows = 1, floats = 8;
   for (int i = 0; i < n_seg; ++i) {
+    if (a.seg[i].ln_gain && a.seg[i].in_dim > kMaxLn) return cudaErrorInvalidValue;
     max_in = std::max(max_in, a.seg[i].in_dim);
     floats = std::max(floats, a.seg[i].in_dim * (a.seg[i].ln_gain ? 3 : 1));
     max_rows = std::max(max_rows, a.seg[i].rows);
@@ -247,7 +248,7 @@ static cudaError_t gemv(const GemvArgs& a, int n_seg, cudaStream_t s, int sm_cou
   // one row's pieces would leave half of a lane's loads unused
   const bool wide = max_rows >= 4 * kWarps * sm_count || max_in <= 2048;
   auto kfn = wide ? k_gemv<2, 8> : k_gemv<1, 16>;
-  if (smem > 48 * 1024) {
+  if (smem > kPlainShared) {
     static std::atomic<uint64_t> done[2] = {{0}, {0}};
     cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done[wide]);
     if (e != cudaSuccess) return e;

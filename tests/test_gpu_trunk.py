@@ -57,6 +57,18 @@ def test_forward_at_the_papers_sizes():
     assert _run(512, (4096, 4096, 128, 1), 512, 2048, 4, 31, 512, seed=12, tokens=2) < 2e-5
 
 
+@pytest.mark.parametrize("shape", [
+    (1024, (8, 16, 8, 1), 5, 8, 1, 2, 6),      # the largest T: a LayerNorm's input, gain and bias take 48 KB
+    (1016, (8, 16, 8, 1), 5, 8, 2, 1, 5),
+    (72, (40, 16, 8, 1), 5, 24, 2, 2, 6),      # normalised inputs that are no multiple of a block's threads
+    (8, (12288, 8, 8, 1), 5, 8, 1, 2, 6),      # an input of 48 KB
+    (8, (12280, 8, 16384, 1), 5, 8, 1, 2, 6),  # the widest
+])
+def test_forward_where_its_shared_memory_ends(shape):
+    T, dims, K0, E, nblk, nh, K = shape
+    assert _run(T, dims, K0, E, nblk, nh, K, seed=14, tokens=1) < 2e-5
+
+
 def test_heads_feed_the_centroid_selection():
     """Head logits [n_heads][2][K] are the layout np_centroid_select reads for one sequence."""
     cfg = synth.StackConfig("sel", 3, 64, 256, 16, 10, 25, 2, 51, 0.9)
