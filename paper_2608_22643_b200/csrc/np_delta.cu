@@ -641,7 +641,7 @@ cudaError_t launch_delta(const Dims& d, const Tables& t, const uint32_t* pred, i
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (sm > 48 * 1024) {
+  if (sm > kPlainShared) {
     static std::atomic<uint64_t> done{0};
     const cudaError_t e = allow_shared(reinterpret_cast<const void*>(k_delta), &done);
     if (e != cudaSuccess) return e;

@@ -524,10 +524,9 @@ template <int NB, int COLS>
 static cudaError_t mlp_launch_cols(const MlpKernelArgs& ka, int groups, int grid_x, cudaStream_t s) {
   const size_t sm = ((size_t)NB * ka.D + (size_t)NB * kTileRows * kMaxSeg * 2 + NB * kTileRows) * 4;
   auto kfn = k_sparse_mlp<NB, COLS>;
-  // set on every launch: the attribute belongs to the current device's context, and a cache in
-  // this function would be shared by all devices and threads of the process
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (sm > kPlainShared) {
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_shared(reinterpret_cast<const void*>(kfn), &done);
     if (e != cudaSuccess) return e;
   }
   dim3 grid(grid_x, groups);
