@@ -24,7 +24,7 @@
 // The rows come through a ring of row-sized pieces in shared memory, filled by 1-D bulk
 // copies from a producer lane: gate and up rows of a tile of 8 rows, then the layer's down
 // rows.  Cooperative launch with clusters: every block is resident.  Every wait is bounded
-// (kStatTimeout on expiry); after one has run out the later ones are skipped, and every
+// (kStatTimeout on expiry); after one has run out those for other clusters are skipped, and every
 // block still meets its cluster at the end, so no block leaves while a peer may write to it.
 #include <algorithm>
 
@@ -198,23 +198,15 @@ __device__ __forceinline__ uint4 tc_ld4(uint32_t taddr) {
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Bounded waits.  Once any wait of the block has run out (*ok == 0) every later wait is
-// skipped, so no barrier is ever left short of threads.
-__device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
-  if (npp::mbar_try_wait(bar, parity)) return;  // the usual case: already complete
-  if (!*ok) return;
-  if (!npp::mbar_wait(bar, parity)) {
-    *ok = 0;
-    atomicOr(status, npp::kStatTimeout);
-  }
-}
-__device__ __forceinline__ void wait_cluster_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
-  if (mbar_try_wait_cluster(bar, parity)) return;
-  if (!*ok) return;
-  for (uint32_t i = 0; i < npp::kSpinLimit; ++i)
-    if (mbar_try_wait_cluster(bar, parity)) return;
-  *ok = 0;
-  atomicOr(status, npp::kStatTimeout);
+// Every wait is bounded.  Once one has run out (*ok == 0) the block no longer waits for its range's counter; all other waits are for
+// copies, for warps of the block and for blocks of the cluster, which get on without it, and go on (np_ring.h): no barrier is
+// armed over copies under way, and nobody leaves before what the others send it has arrived.
+__device__ __forceinline__ void ring_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
+  npp::RingBlock b = {ok, status};
+  uint32_t polls = 0;
+#pragma unroll 1
+  while (!mbar_try_wait_cluster(bar, parity))
+    if (npp::ring_wait_step<npp::kSpinLimit>(polls, b)) return;
 }
 
 // ring slot and use parity of piece number v of the launch (exact for v < 2^32 / ns)
@@ -257,7 +249,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
   __shared__ float act[kMaxRows];                         // a_i of the block's rows
   __shared__ __align__(16) float ssq_part[kCS][kWarps / kCS][4];  // sum(x^2) by column range and warp of its owner (16-byte granules: first float)
   __shared__ __align__(16) float ag_ssq[kWarps / kCS][4];         // this block's own, on their way to the cluster
-  __shared__ int s_ok;
+  __shared__ int s_ok[2];                                 // no wait has run out; waits for copies were given up
   __shared__ int lay_rb[kMaxLayers];       // first active-list index of this block, per layer
   __shared__ int lay_pre[kMaxLayers + 1];  // rows of this block before each layer (virtual row index)
 
@@ -285,7 +277,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
   unsigned char* ag_own = reinterpret_cast<unsigned char*>(y_stage + (size_t)(kCS - 1) * seg);
   unsigned char* ag_stage = kCS >= 4 ? reinterpret_cast<unsigned char*>(rs_buf) : ag_own;  // [3][seg * 2]
   int* slot_cache = reinterpret_cast<int*>(ag_own + (kCS >= 4 ? 0 : 3 * (size_t)seg * 2));  // this block's slots, virtual row order
-  volatile int* ok = &s_ok;
+  volatile int* ok = s_ok;
 
   // ---- this block's share of every layer of the run ----
   if (tid < nl) {
@@ -316,7 +308,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
     npp::mbar_init(&rs_bar, 1);  // armed by this block once per layer with the bytes it expects
     npp::mbar_init(&ag_bar, 1);
     npp::fence_barrier_init();
-    s_ok = 1;
+    s_ok[0] = 1, s_ok[1] = 0;
   }
   if (wid == kWarps + 1) {  // tensor memory: all of it (this kernel has the SM to itself); the address lands in shared memory
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(npp::smem_addr(&s_tmem_base)), "r"(kTmemCols) : "memory");
@@ -356,7 +348,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
     // its up rows.  A layer goes out at once, a lane per piece (one lane alone spends over 0.1 us per request).  A lane waits for its own slot: the slots of a batch are released in order by consumers that need
     // nothing from this batch, so the lanes may wait for one another at the end of a batch.
     unsigned int v0 = 0;
-    bool good = true;
     // lane i < cnt requests the piece v0 + i from src
     auto issue = [&](const unsigned char* src, int cnt) {
       if (lane < cnt) {
@@ -364,25 +355,14 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
         uint32_t par;
         const unsigned int v = v0 + (unsigned int)lane;
         slot_of(v, a.ns_magic, ns, s, par);
-        if (v >= (unsigned int)ns && !npp::mbar_wait(&empty_bar[s], par ^ 1u)) {
-          atomicOr(a.status, npp::kStatTimeout);
-          good = false;
-        } else {
-          npp::mbar_expect_tx(&full_bar[s], row_bytes);
-          npp::bulk_g2s_stream(csm + (size_t)s * pstride, src, row_bytes, &full_bar[s], npp::policy_evict_first());
-        }
+        if (v >= (unsigned int)ns) npp::ring_wait(&empty_bar[s], par ^ 1u, ok, a.status);
+        npp::mbar_expect_tx(&full_bar[s], row_bytes);
+        npp::bulk_g2s_stream(csm + (size_t)s * pstride, src, row_bytes, &full_bar[s], npp::policy_evict_first());
       }
-      const bool all = __all_sync(0xffffffffu, good);
-      if (!all && good && lane < cnt) {  // a copy of a round that could not go out whole
-        int s;
-        uint32_t par;
-        slot_of(v0 + (unsigned int)lane, a.ns_magic, ns, s, par);
-        if (!npp::mbar_wait(&full_bar[s], par)) atomicOr(a.status, npp::kStatTimeout);
-      }
-      good = all;
-      if (good) v0 += (unsigned int)cnt;
+      __syncwarp();
+      v0 += (unsigned int)cnt;
     };
-    for (int li = 0; li < nl && good; ++li) {
+    for (int li = 0; li < nl; ++li) {
       const int vrow0 = lay_pre[li], nrows = min(lay_pre[li + 1], total_rows) - vrow0;
       const size_t lbase = (size_t)(a.l_begin + li) * layer_bytes;
       // a layer's pieces: its gate rows, then its up rows, a lane each
@@ -403,7 +383,6 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
     // request row k + 1, wait for row k, copy it on (4 copies of 2 KB), commit: the commit frees the staging piece,
     // and after a layer's last row it tells the consumers.
     if (lane == 0) {
-      bool good = true;
       int li_n = 0, r_n = 0;    // the next row to request
       unsigned int kn = 0;      // its number within the launch
       auto rows_of = [&](int li) { return min(min(lay_pre[li + 1], total_rows) - lay_pre[li], kTmemRows); };
@@ -414,11 +393,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
         }
         if (li_n >= nl) return;
         const int s = (int)(kn % kDS);
-        if (kn >= (unsigned int)kDS && !npp::mbar_wait(&ds_free[s], ((kn / kDS) & 1u) ^ 1u)) {
-          atomicOr(a.status, npp::kStatTimeout);
-          good = false;
-          return;
-        }
+        if (kn >= (unsigned int)kDS) npp::ring_wait(&ds_free[s], ((kn / kDS) & 1u) ^ 1u, ok, a.status);
         npp::mbar_expect_tx(&ds_full[s], row_bytes);
         npp::bulk_g2s_stream(dstage + (size_t)s * pstride,
                              a.downT + (size_t)(a.l_begin + li_n) * layer_bytes + (size_t)slot_cache[lay_pre[li_n] + r_n] * row_bytes,
@@ -428,22 +403,17 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
       };
       request();
       unsigned int k = 0;
-      for (int li = 0; li < nl && good; ++li) {
+      for (int li = 0; li < nl; ++li) {
         const int nrows = rows_of(li), buf = li & 1;
-        for (int r = 0; r < nrows && good; ++r, ++k) {
+        // the buffer's readers of two layers ago
+        auto buffer_free = [&] {
+          if (li >= 2) npp::ring_wait(&tm_empty[buf], (uint32_t)((li >> 1) - 1) & 1u, ok, a.status);
+        };
+        for (int r = 0; r < nrows; ++r, ++k) {
           request();  // the row after this one
-          if (!good) break;
           const int s = (int)(k % kDS);
-          if (!npp::mbar_wait(&ds_full[s], (k / kDS) & 1u)) {
-            atomicOr(a.status, npp::kStatTimeout);
-            good = false;
-            break;
-          }
-          if (r == 0 && li >= 2 && !npp::mbar_wait(&tm_empty[buf], (uint32_t)((li >> 1) - 1) & 1u)) {  // the buffer's readers of two layers ago
-            atomicOr(a.status, npp::kStatTimeout);
-            good = false;
-            break;
-          }
+          npp::ring_wait(&ds_full[s], (k / kDS) & 1u, ok, a.status);
+          if (r == 0) buffer_free();
           tc_fence_after();
           const uint32_t col = (uint32_t)(buf * (kTmemCols / 2) + r * 16);
           for (uint32_t j = 0; j < row_bytes / 2048u; ++j)
@@ -451,19 +421,10 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
           tc_commit(&ds_free[s]);
           if (r == nrows - 1) tc_commit(&tm_full[buf]);
         }
-        if (nrows == 0 && good) {  // nothing to copy: the consumers still wait for the buffer's turn
-          if (li >= 2 && !npp::mbar_wait(&tm_empty[buf], (uint32_t)((li >> 1) - 1) & 1u)) {
-            atomicOr(a.status, npp::kStatTimeout);
-            good = false;
-          } else {
-            npp::mbar_arrive(&tm_full[buf]);
-          }
+        if (nrows == 0) {  // nothing to copy: the consumers still wait for the buffer's turn
+          buffer_free();
+          npp::mbar_arrive(&tm_full[buf]);
         }
-      }
-      // after a time-out: the copies on their way into the staging pieces, then those out of them (k of them went out)
-      for (unsigned int s = 0; s < (unsigned int)kDS && !good; ++s) {
-        if (kn > s && !npp::mbar_wait(&ds_full[s], ((kn - 1u - s) / kDS) & 1u)) atomicOr(a.status, npp::kStatTimeout);
-        if (k > s && !npp::mbar_wait(&ds_free[s], ((k - 1u - s) / kDS) & 1u)) atomicOr(a.status, npp::kStatTimeout);
       }
     }
   } else {
@@ -512,7 +473,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
 
     for (int li = 0; li < nl; ++li) {
       RK(0);
-      if (li > 0) wait_cluster_or_flag(&ag_bar, (uint32_t)(li - 1) & 1u, ok, a.status);  // x_l and its sums are here
+      if (li > 0) ring_wait_cluster(&ag_bar, (uint32_t)(li - 1) & 1u, ok, a.status);  // x_l and its sums are here
       RK(1);
       AK(0);
       if (wid == 0) PK(1, 20);
@@ -532,7 +493,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
           int s;
           uint32_t par;
           slot_of(pbase + (unsigned int)lane, a.ns_magic, ns, s, par);
-          wait_or_flag(&full_bar[s], par, ok, a.status);
+          npp::ring_wait(&full_bar[s], par, ok, a.status);
         }
         __syncwarp();
         RK(16);
@@ -656,7 +617,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
       };
       {
         const int buf = li & 1;
-        if (lane == 0) wait_or_flag(&tm_full[buf], (uint32_t)(li >> 1) & 1u, ok, a.status);
+        if (lane == 0) npp::ring_wait(&tm_full[buf], (uint32_t)(li >> 1) & 1u, ok, a.status);
         __syncwarp();
         tc_fence_after();
         RK(18);
@@ -701,7 +662,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
       float* zl = a.z4 + (size_t)((a.seq + (unsigned int)li) & 3u) * kZR * D + (size_t)rank * seg;  // copy 0 of this layer's accumulator, this block's range
       RK(7);
       if (own) {
-        wait_cluster_or_flag(&rs_bar, (uint32_t)li & 1u, ok, a.status);
+        ring_wait_cluster(&rs_bar, (uint32_t)li & 1u, ok, a.status);
         RK(8);
         AK(3);
 #pragma unroll
@@ -740,7 +701,7 @@ __global__ void __launch_bounds__(kBlock, 1) k_mlp_rows(KArgs a) {
           }
           if (!there) {
             atomicOr(a.status, npp::kStatTimeout);
-            s_ok = 0;
+            s_ok[0] = 0;
           }
         }
       }

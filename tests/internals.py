@@ -76,6 +76,29 @@ extern "C" int t_batch_record(unsigned int* base) {  // a launch that the caller
   base[0] = st.read_base; base[1] = st.add_base; base[2] = st.seq_base;
   return e;
 }
+// ptr: as for t_slices up to the status, then accumulators, counters; the result is in xbuf[(L - 1) & 1]
+extern "C" int t_rows(int D, int C, int k, int L, int sms, void* const* ptr, unsigned int* base, void* stream) {
+  const Dims d = dims(D, C, k, L);
+  ChainArgs a = {};
+  a.gate = ptr[0]; a.up = ptr[1]; a.downT = ptr[2];
+  a.active_slots = static_cast<const int32_t*>(ptr[3]);
+  a.counters = static_cast<const int32_t*>(ptr[4]);
+  a.x_bf16 = ptr[5];
+  for (int i = 0; i < 2; ++i) a.xbuf[i] = static_cast<float*>(ptr[6 + i]);
+  for (int i = 0; i < 3; ++i) a.zbuf[i] = static_cast<float*>(ptr[8 + i]);
+  a.status = static_cast<int32_t*>(ptr[12]);
+  a.l_end = L;
+  a.check = 1;
+  chain_rows::State st = {};
+  st.z4 = static_cast<float*>(ptr[13]);
+  st.cnt = static_cast<unsigned int*>(ptr[14]);
+  st.cnt_base = base[0]; st.seq = base[1];
+  if (!chain_rows::prepare(d, sms, &st) || chain_rows::run_layers(d, st) < L) return -1;
+  const int e = (int)chain_rows::launch(d, a, &st, static_cast<cudaStream_t>(stream));
+  base[0] = st.cnt_base; base[1] = st.seq;
+  return e;
+}
+extern "C" unsigned long long t_rows_words(int D) { return chain_rows::z_floats(dims(D, 1024, 1, 1)); }
 extern "C" void t_batch_words(int sms, unsigned long long* n) {
   n[0] = chain_batch::cnt_words(); n[1] = chain_batch::xch_words(sms);
 }

@@ -129,3 +129,31 @@ def test_a_wait_that_runs_out_laps_before_the_end(lib, B, D, rows):
     w.clear()
     got, status = w.run()
     assert status == 0 and w.error(got) < 1e-5
+
+
+@pytest.mark.parametrize("D,k", [(1024, 1500), (4096, 1100)])
+def test_a_wait_that_runs_out_in_a_cluster(lib, D, k):
+    """The same for the kernel that deals whole rows to the blocks of clusters."""
+    L = 7                                           # several laps of its ring
+    w = Words(lib, D, k + 100, k, L)
+    acc = torch.zeros(int(lib.t_rows_words(D)), device="cuda")
+    cnt = torch.zeros(4, dtype=torch.int32, device="cuda")
+    t = [*w.rows, w.slots, w.counters, w.x, *w.acc, w.out, w.status, acc, cnt]
+
+    def run():
+        stream = internals.C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        rc = lib.t_rows(*w.shape, w.sms, internals.pointers(*[v.data_ptr() for v in t]), w.base, stream)
+        torch.cuda.synchronize()
+        assert rc == 0
+        return w.acc[(L - 1) & 1, :D].clone().view(1, D), int(w.status[0])
+
+    want, status = run()
+    assert status == 0 and w.error(want) < 1e-5
+    w.base[0] += 1
+    _, status = run()
+    assert status == TIMEOUT
+    for v in (acc, cnt, w.acc):
+        v.zero_()
+    w.clear()
+    got, status = run()
+    assert status == 0 and w.error(got) < 1e-5
