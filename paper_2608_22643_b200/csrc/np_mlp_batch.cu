@@ -129,15 +129,6 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// One lane's bounded wait on an mbarrier; after the block's first time-out nothing waits any more.
-__device__ __forceinline__ void wait_or_flag(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
-  if (npp::mbar_try_wait(bar, parity)) return;
-  if (!*ok) return;
-  if (!npp::mbar_wait(bar, parity)) {
-    *ok = 0;
-    atomicOr(status, npp::kStatTimeout);
-  }
-}
 // A warp's wait, by all lanes or by lane 0.  The latter parts the warp and brings it together again, some 300 cycles where the phase
 // is long complete, so what lies on the way of x is waited for by all lanes (sixteen sequences of 1024 columns 83 us per 12 layers,
 // 90 with lane 0's waits; two of the 7B shape 319 per 32 and 337).  The waits inside the up phase's loop are lane 0's: by all lanes
@@ -147,7 +138,7 @@ __device__ __forceinline__ void all_wait(uint64_t* bar, uint32_t parity, volatil
   __syncwarp();
 }
 __device__ __forceinline__ void warp_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status, int lane) {
-  if (lane == 0) wait_or_flag(bar, parity, ok, status);
+  if (lane == 0) npp::wait_or_flag(bar, parity, ok, status);
   __syncwarp();
 }
 // Whether the phase of that parity is complete, without waiting.  The consumers ask early and look at the answer when they
@@ -480,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_batch(KArgs a) {
         for (int li = 0; li < nl; ++li) {
           if (li > 0) wait_count(cnt_add, a.add_base + (unsigned int)li * (unsigned int)(R * kWarps), ok, a.status);
           npp::mbar_arrive(&x_ready);
-          wait_or_flag(&x_read, (uint32_t)li & 1u, ok, a.status);
+          npp::wait_or_flag(&x_read, (uint32_t)li & 1u, ok, a.status);
           asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt_read) : "memory");
           wait_count(cnt_read, a.read_base + (unsigned int)(li + 1) * (unsigned int)R, ok, a.status);
           npp::mbar_arrive(&may_add);
