@@ -130,9 +130,10 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
 }
 
 // A warp's wait, by all lanes or by lane 0.  The latter parts the warp and brings it together again, some 300 cycles where the phase
-// is long complete, so what lies on the way of x is waited for by all lanes (sixteen sequences of 1024 columns 83 us per 12 layers,
+// is long complete, so the barriers on the way of x are waited for by all lanes (sixteen sequences of 1024 columns 83 us per 12 layers,
 // 90 with lane 0's waits; two of the 7B shape 319 per 32 and 337).  The waits inside the up phase's loop are lane 0's: by all lanes
-// they cost the widest rows more than they give the others (13B shape, eight sequences, 581 us per 40 layers against 560).
+// they cost the widest rows more than they give the others (13B shape, eight sequences, 581 us per 40 layers against 560).  (The polls of
+// the exchange's words still end lane by lane.)
 __device__ __forceinline__ void all_wait(uint64_t* bar, uint32_t parity, volatile int* ok, int32_t* status) {
   npp::wait_or_flag(bar, parity, ok, status);
   __syncwarp();

@@ -50,8 +50,9 @@
 // the activations as three bf16 terms.  In both, columns 4-6 of B repeat columns 0-2, so that the
 // upper two lanes of a quad hold a second tile's sums without a shuffle.
 //
-// On the way from the sums to the next layer's sums nothing parts a warp: a branch around some lanes, or a loop that lanes leave one by
-// one, costs it hundreds of cycles per layer (each such place says what).
+// On the way from the sums to the next layer's sums a branch around some lanes, or a loop that lanes leave one by one, parts a warp and
+// costs it hundreds of cycles per layer: where those were taken out, the place says what it gave.  Two are left: the poll of the sums
+// themselves (add_sums), which every lane leaves when its own columns are there, and lane 0's wait for arrivals in a launch's first layer.
 //
 // Shared memory is one ring of load groups in the order they are consumed: the gate|up pieces of a
 // layer's rows, then its down pieces, then the next layer's.  A producer warp fills it with 1-D bulk
@@ -101,9 +102,12 @@ __host__ __device__ constexpr int tiles_down(int KB) { return KB <= 4 ? 4 : KB <
 // two; 3000 rows of 4096 columns 177 and 160 us per 12 layers).
 __host__ __device__ constexpr int tiles_wait(int KB) { return KB <= 4 ? 4 : tiles_up(KB) > 2 ? 2 : tiles_up(KB); }
 // Whether the producer's wait for a free slot is lane 0's or the whole warp's.  What lies between a free slot and its copies sets the
-// stream's pace, so the rows' addresses are formed before the wait; which wait is shorter then differs by instance (us per stack, all
-// lanes / lane 0 / before, lane 0 with the addresses behind the wait: 256 columns 54.1 / 54.6 / 54.9, 7B shape 162.3 / 172.7 / 164.0,
-// 13B 267.1 / 264.6 / 266.6, 6144 149.6 / 156.3 / 155.0, 70B 1006 / 909 / 945).
+// stream's pace, so the rows' addresses are formed before the wait (behind it, lane 0's: 7B shape 164.0 us per 32 layers where all
+// lanes' took 162.3 in front, 70B 945 per 80 where lane 0's took 909).  Which wait is shorter is measured, not understood.  us per 20 layers, all
+// lanes / lane 0, with a tenth of the neurons active: below eight K blocks alike (256 columns 54.2 / 54.2, 1536 68.0 / 68.1, 2560 84.7 /
+// 84.8, 3072 87.8 / 87.9), eight 104.8 / 106.7, ten 163.1 / 157.9 (4464 columns 167.5 / 165.3), twelve 203.6 / 219.2 (5296 columns 192.3 /
+// 189.4).  At sixteen it turns with the rows of a block: 39 rows, the 70B shape, 998 / 908 per 80 layers; 60 rows of 8192 columns 358.8 / 364.2, 52 of
+// 7008 297.2 / 309.4.  There the line follows the shape that the kernel meets in the configurations.
 __host__ __device__ constexpr bool lane0_waits(int KB) { return KB == 10 || KB == 16; }
 // tiles of a round of the exchange: whole groups of tiles_up
 __host__ __device__ constexpr int tiles_chunk(int KB) { return kChunkVec / 16 / tiles_up(KB) * tiles_up(KB); }
@@ -135,7 +139,10 @@ struct KArgs {
 
 // 32-bit words a consumer warp's B operand takes: [K block pair][term][lane of the quad][K block of the pair][half].  A fourth, zero
 // "term" stands in the columns that have none: every lane loads its column, and no branch parts the warp between x and the
-// multiplications.  (7B shape 170.1 us per 32 layers with a branch around those lanes, 166.9 without; 13B 278.9 and 272.3.)
+// multiplications.  (7B shape 170.1 us per 32 layers with a branch around those lanes, 166.9 without; 13B 278.9 and 272.3.)  The zeros
+// take a slot of the ring at one width in twenty.  With 16 bytes of zeros per block in their place the slot is there and gives nothing,
+// and the step from pair to pair costs: us per 20 layers, as it is / so, all of widths that lose a slot: 6496 columns 263.4 / 262.1, 6416
+// 260.7 / 260.4, 6432 with few rows 177.5 / 181.0, 5296 191.8 / 195.8, 4464 166.4 / 166.5, 3840 109.8 / 110.2, 3008 94.4 / 93.6.
 __host__ __device__ constexpr int bstage_words(int KB) { return (KB + 1) / 2 * 64; }
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
